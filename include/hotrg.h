@@ -48,7 +48,10 @@ typedef enum hotrg_status {
 } hotrg_status;
 
 typedef enum hotrg_precision {
-  HOTRG_FP64 = 0,   /* every contraction in FP64 on the CUDA cores */
+  HOTRG_FP64 = 0,   /* every contraction in FP64. The squeeze products run on the tensor cores from exact integer
+                       slices (each operand row as a 63-bit fixed-point number, 36 digit products, exact sums, one
+                       rounding) where the shape takes them (P >= 128, chi P >= 256, row length at most 16320, and a
+                       workspace up to 128 GiB), on the CUDA cores elsewhere; the rest on the CUDA cores */
   HOTRG_BF16X3 = 1, /* squeeze GEMM on tcgen05 tensor cores with split operands x = hi + lo
                        (bf16 each); products hi*hi + hi*lo + lo*hi accumulate in FP32 (TMEM):
                        O(2^-16) relative error per product. Gram matrices, eigensolver, norms
@@ -319,6 +322,16 @@ int hotrg_gemm_split_noalloc(const float *A, long long lda, const float *Bt, lon
 int hotrg_gemm_split_f16(const float *A, long long lda, const float *Bt, long long ldb, float *C,
                          long long ldc, long long M, long long N, long long K, int npass, int kblock,
                          int fold_group, void *scratch, size_t scratch_bytes, void *stream);
+
+/* The FP64 squeeze product of the flow on its own, for tests and benchmarks: C = A Bt^T in double precision, computed
+ * on the tensor cores from exact integer slices (see HOTRG_FP64). A (M x lda), Bt (N x ldb) and C (M x ldc) are device
+ * arrays; M >= 128, N >= 256, 64 <= K <= 16320. cta_group: 1 or 2 CTAs per output tile (identical results). `scratch`:
+ * device, 256-B aligned, >= hotrg_gemm_f64_scratch_bytes(M, N, K) bytes (0 for a shape it does not take); its first
+ * word is the status (hotrg_gemm_status). Enqueued on `stream`; not synchronised. Errors: EINVAL, EDEVICE. */
+size_t hotrg_gemm_f64_scratch_bytes(long long M, long long N, long long K);
+int hotrg_gemm_f64(const double *A, long long lda, const double *Bt, long long ldb, double *C, long long ldc,
+                   long long M, long long N, long long K, int cta_group, void *scratch, size_t scratch_bytes,
+                   void *stream);
 
 /* Failure-detection probe of the bounded device-side waits (the paper has no counterpart): two
  * launches of the tensor-core GEMM (BF16X3, one output tile: first on one CTA, then on a CTA pair)

@@ -70,6 +70,9 @@ _SIGS = {
     "hotrg_gemm_split_f16": (c_int, [c_void_p, c_longlong, c_void_p, c_longlong, c_void_p, c_longlong,
                                      c_longlong, c_longlong, c_longlong, c_int, c_int, c_int, c_void_p, c_size_t,
                                      c_void_p]),
+    "hotrg_gemm_f64_scratch_bytes": (c_size_t, [c_longlong, c_longlong, c_longlong]),
+    "hotrg_gemm_f64": (c_int, [c_void_p, c_longlong, c_void_p, c_longlong, c_void_p, c_longlong,
+                               c_longlong, c_longlong, c_longlong, c_int, c_void_p, c_size_t, c_void_p]),
     "hotrg_gemm_status": (c_int, [c_void_p, c_void_p]),
     "hotrg_gemm_wait_probe_bytes": (c_size_t, []),
     "hotrg_gemm_wait_probe": (c_int, [c_double, c_void_p, c_size_t, c_void_p]),

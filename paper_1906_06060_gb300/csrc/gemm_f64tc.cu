@@ -1,0 +1,576 @@
+// FP64 squeeze products on the 5th-generation tensor cores: C[m][n] = sum_k A[m][k] Bt[n][k] in double precision
+// from exact integer slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
+//
+// GB300 has no fast FP64 unit (1.25 TFLOP/s nominal, 4 flop per clock and SM), its fp16 tensor cores run at
+// 8192 flop per clock and SM. Every row of an operand is scaled by a power of two 2^-e that brings its largest entry
+// below 1 and rounded to a 55-bit fixed-point number, which is cut into 7 balanced digits of 8 bits,
+//   x 2^-e = sum_i q_i 2^-(7 + 8 i),  -128 <= q_i <= 128,
+// each stored as an fp16 integer (exact). The product is the sum over the digit pairs with i + j <= 6 (28 products),
+// grouped by level s = i + j:
+//   C[m][n] 2^-(eA + eB) = sum_s L_s 2^-(14 + 8 s),  L_s = sum_{i <= s} sum_k qA_i qB_{s-i}.
+// Exactness: |qA qB| <= 2^14, so a chain of 16 x 64 products stays within 2^24 and the tensor cores' FP32 accumulator
+// holds it exactly; every chain is added into an int32 register accumulator (|L_s| <= (s + 1) K 2^14 < 2^31 for
+// K <= 16320). Level 6 is folded into level 5
+// with a rounding shift, and the six level sums are combined exactly and rounded once. The error of a result is one
+// rounding plus about sqrt(K) 2^-56 of the two rows' largest entries (entries within 1/4 of their row's largest are
+// held exactly), where a chain of K FP64 operations rounds every partial sum to 2^-53 of its size. Rows holding NaN or
+// infinity give NaN.
+//
+// Work: 28 tensor products of 2 M N K flops against one on the FP64 units at 1/2000 of the rate.
+// Kernel structure, ring and bounded waits as k_gemm_split (gemm_tc.cu): warp 0 copies, warp 1 issues MMAs, warps
+// 2-9 fold. Per output tile the levels run one after the other, least significant first, each over all k-blocks; a
+// ring stage holds one digit tile of A and one of B. A finished level sum goes to a per-CTA scratch area in global
+// memory (L2), one 16-byte access per thread and four columns, coalesced; the last level combines them in registers.
+#include "tc_ptx.cuh"
+
+namespace hotrg {
+
+namespace {
+
+constexpr int NSL = kSliceCount;      // digits per entry
+constexpr int kSliceBits = 8 * NSL - 1;  // bits of the fixed-point rows
+constexpr int CHAIN = 16;             // 64-wide k steps per accumulator chain
+constexpr int SC_PLANES = 6;          // level sums parked in scratch: levels 5 (with 6), 4, 3, 2, 1, 0
+constexpr int kExpNaN = 0x40000000;   // row exponent of a row with a non-finite entry
+constexpr int SBK = 64;
+
+template <int CG>
+struct SCfg {
+  static constexpr uint32_t A_TILE = TC_BM * SBK * 2;
+  static constexpr uint32_t B_TILE = (TC_BN / CG) * SBK * 2;
+  static constexpr uint32_t STAGE_BYTES = A_TILE + B_TILE;
+  static constexpr int STAGES = CG == 2 ? 6 : 4;
+  static constexpr size_t SMEM = 1024 + STAGES * STAGE_BYTES + 256;
+};
+
+struct SliceMaps {
+  CUtensorMap a, b;
+};
+
+struct SliceParams {
+  long long M, N, K;
+  int num_kb, group_m, batch;
+  double* C;
+  long long ldc, c_inst;
+  const int* ea;  // row exponents of A and of Bt, instance strides ea_inst, eb_inst
+  const int* eb;
+  long long ea_inst, eb_inst;
+  int4* scratch;
+  int* status;
+  unsigned long long timeout_ns;
+  const GemmBlocks* blk;
+  uint32_t idesc;
+  int accumulate;  // C += instead of C =
+  int vec;         // entries per store: 4 (32-byte aligned rows) or 1
+};
+
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
+                                            int w) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
+      "[%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
+      : "memory");
+}
+// issued by the first CTA of a pair for either CTA (see tma_load_3d_pair)
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
+                                                 int z, int w) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+      "{%3, %4, %5, %6}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
+      : "memory");
+}
+
+// (hi 2^24 + lo) 2^e as a double, rounded once (to nearest, ties to even), in integer arithmetic: the FP64 unit's two
+// operations a clock would make the tile's 32768 conversions and scalings cost more than its copies. |hi| < 2^45,
+// |lo| < 2^47.
+__device__ __forceinline__ double assemble(long long hi, long long lo, int e) {
+  const bool wide = hi > (1LL << 38) || hi < -(1LL << 38);
+  if (wide || e < -900 || e > 900)  // beyond 64 bits, or near the ends of the exponent range
+    return ldexp(fma((double)hi, 16777216.0, (double)lo), e);
+  const long long v = (hi << 24) + lo;  // |v| < 2^62 + 2^47
+  const unsigned long long u = v < 0 ? 0ULL - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << (lz & 63);
+  const unsigned long long kept = m >> 11;  // 53 bits, the leading one included: it adds 1 to the exponent field below
+  const unsigned rest = (unsigned)m & 0x7FFu;
+  const unsigned up = (rest + (unsigned)(kept & 1)) > 0x400u;
+  const unsigned long long bits = ((unsigned long long)(unsigned)(1023 + 62 - lz + e) << 52) + kept + up;
+  return __longlong_as_double((long long)(u ? bits | ((unsigned long long)v & 0x8000000000000000ULL) : 0ULL));
+}
+
+template <int CG>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+    k_gemm_slices(const __grid_constant__ SliceMaps maps, SliceParams p) {
+  using C = SCfg<CG>;
+  constexpr int STAGES = C::STAGES;
+  constexpr uint32_t A_TILE = C::A_TILE, STAGE_BYTES = C::STAGE_BYTES;
+  constexpr int B_ROWS = TC_BN / CG;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const uint32_t full0 = smem_u32(bars);
+  const uint32_t empty0 = full0 + 8 * STAGES;
+  const uint32_t tfull0 = empty0 + 8 * STAGES;
+  const uint32_t tempty0 = tfull0 + 16;
+  const uint32_t final_bar = tempty0 + 16;
+  const uint32_t rank = CG == 2 ? cluster_rank() : 0u;
+  const bool leader = rank == 0;
+  const int cta0 = (int)blockIdx.x / CG, ncta = (int)gridDim.x / CG;
+
+  __shared__ int s_prefix[kMaxGemmBatch + 1];
+  __shared__ int s_total;
+  if (threadIdx.x == 0) {
+    Blk b[2];
+    if (p.blk) {
+      int t = 0;
+      for (int i = 0; i < p.batch; ++i) {
+        s_prefix[i] = t;
+        const int nb = load_blocks<SBK, CG>(p, i, b);
+        t += b[0].tiles + (nb > 1 ? b[1].tiles : 0);
+      }
+      s_prefix[p.batch] = t;
+      s_total = t;
+    } else {
+      load_blocks<SBK, CG>(p, 0, b);
+      s_total = b[0].tiles * p.batch;
+    }
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(tfull0 + 8 * b, 1);
+      mbar_init(tempty0 + 8 * b, CG * TC_FOLD_THREADS / 32);
+    }
+    mbar_init(final_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0 && lane < 2) {
+    const CUtensorMap* m = lane ? &maps.b : &maps.a;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+  }
+  if (warp == 1) {
+    if constexpr (CG == 1) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  if constexpr (CG == 1) __syncthreads();
+  else cluster_sync();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const int total = s_total;
+
+  if (warp == 0) {
+    if (lane == 0 && leader) {
+      int stage = 0;
+      uint32_t phase = 0;
+      long long issued = 0;
+      bool ok = true;
+      for (int tile = cta0; tile < total && ok; tile += ncta) {
+        int inst, mt, nt;
+        Blk bk;
+        locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
+        const int arow = bk.m0 + mt * TC_BM * CG;
+        const int brow = bk.n0 + nt * TC_BN;
+        for (int s = NSL - 1; s >= 0 && ok; --s)
+          for (int kb = 0; kb < bk.num_kb && ok; ++kb) {
+            const int kx = bk.k0 + kb * SBK;
+            for (int i = 0; i <= s; ++i) {
+              if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.timeout_ns)) { ok = false; break; }
+              const uint32_t fb = full0 + 8 * stage;
+              const uint32_t sa = smem_u32(smem + stage * STAGE_BYTES), sb = sa + A_TILE;
+              mbar_expect_tx(fb, CG * STAGE_BYTES);
+              if constexpr (CG == 1) {
+                tma_load_4d(sa, &maps.a, fb, kx, arow, i, inst);
+                tma_load_4d(sb, &maps.b, fb, kx, brow, s - i, inst);
+              } else {
+                tma_load_4d_pair(sa, &maps.a, fb, kx, arow, i, inst);
+                tma_load_4d_pair(sb, &maps.b, fb, kx, brow, s - i, inst);
+                tma_load_4d_pair(mapa_rank(sa, 1), &maps.a, fb, kx, arow + TC_BM, i, inst);
+                tma_load_4d_pair(mapa_rank(sb, 1), &maps.b, fb, kx, brow + B_ROWS, s - i, inst);
+              }
+              ++issued;
+              if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+          }
+      }
+      // drain the copies in flight on every exit path (see k_gemm_split)
+      for (long long i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i)
+        mbar_wait(full0 + 8 * (int)(i % STAGES), (uint32_t)((i / STAGES) & 1), abort_flag, drain_ns(p.timeout_ns),
+                  false);
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && leader) {
+      int stage = 0, buf = 0;
+      uint32_t phase = 0, bphase = 0;
+      bool ok = true;
+      const uint64_t desc_base = smem_desc<SBK>(smem_u32(smem));
+      for (int tile = cta0; tile < total && ok; tile += ncta) {
+        int inst_, mt_, nt_;
+        Blk bk;
+        locate<SBK, CG>(p, s_prefix, tile, inst_, bk, mt_, nt_);
+        for (int s = NSL - 1; s >= 0 && ok; --s) {
+          const int steps = bk.num_kb * (s + 1);
+          for (int t0 = 0; t0 < steps && ok; t0 += CHAIN) {
+            const int g = min(CHAIN, steps - t0);
+            if (!mbar_wait(tempty0 + 8 * buf, bphase ^ 1, abort_flag, p.timeout_ns)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * TC_BN);
+            for (int t = 0; t < g; ++t) {
+              if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.timeout_ns)) { ok = false; break; }
+              tc_fence_after();
+              const uint64_t da = desc_base + ((uint32_t)stage * STAGE_BYTES >> 4);
+              const uint64_t db = da + (A_TILE >> 4);
+#pragma unroll
+              for (int k = 0; k < SBK / 16; ++k)
+                mma_f16<CG>(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), p.idesc, (t | k) ? 1u : 0u);
+              mma_commit_local<CG>(empty0 + 8 * stage);
+              if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            if (!ok) break;
+            mma_commit<CG>(tfull0 + 8 * buf);
+            if (++buf == 2) { buf = 0; bphase ^= 1; }
+          }
+        }
+      }
+      mma_commit_local<CG>(final_bar);
+      mbar_wait(final_bar, 0, abort_flag, drain_ns(p.timeout_ns), false);
+    }
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int ftid = (int)threadIdx.x - 64;
+    int4* const park = p.scratch + (size_t)blockIdx.x * (SC_PLANES * 32 * TC_FOLD_THREADS) + ftid;
+    const uint32_t tempty_dst = CG == 2 && !leader ? mapa_rank(tempty0, 0) : tempty0;
+    int buf = 0;
+    uint32_t bphase = 0;
+    bool ok = true;
+    for (int tile = cta0; tile < total && ok; tile += ncta) {
+      int num_kb;
+      {
+        int inst, mt, nt;
+        Blk bk;
+        locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
+        num_kb = bk.num_kb;
+      }
+      int acc[128];
+#pragma unroll
+      for (int j = 0; j < 128; ++j) acc[j] = 0;
+      for (int s = NSL - 1; s >= 0 && ok; --s) {
+        const int chains = (num_kb * (s + 1) + CHAIN - 1) / CHAIN;
+        for (int t = 0; t < chains; ++t) {
+          int w = 1;
+          if (lane == 0) w = mbar_wait(tfull0 + 8 * buf, bphase, abort_flag, p.timeout_ns) ? 1 : 0;
+          w = __shfl_sync(0xffffffffu, w, 0);
+          if (!w) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * TC_BN + half * 128);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            // one 32-column load at a time: two would not fit beside the 128 sums
+            uint32_t r[32];
+            tmem_ld32(taddr + c * 32, r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) acc[c * 32 + j] += __float2int_rn(__uint_as_float(r[j]));
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            const uint32_t bar = tempty_dst + 8 * buf;
+            if constexpr (CG == 1) mbar_arrive(bar);
+            else if (leader) mbar_arrive(bar);
+            else mbar_arrive_remote(bar);
+          }
+          if (++buf == 2) { buf = 0; bphase ^= 1; }
+        }
+        if (!ok) break;
+        if (s > 5) {
+          // carry into the next level's unit, rounded
+#pragma unroll
+          for (int j = 0; j < 128; ++j) acc[j] = (acc[j] + 128) >> 8;
+        } else {
+          int4* dst = park + (size_t)(5 - s) * 32 * TC_FOLD_THREADS;
+#pragma unroll
+          for (int j = 0; j < 128; j += 4) {
+            dst[(j / 4) * TC_FOLD_THREADS] =
+                make_int4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+            acc[j] = acc[j + 1] = acc[j + 2] = acc[j + 3] = 0;
+          }
+        }
+      }
+      if (!ok) break;
+      int inst, mt, nt;
+      Blk bk;
+      locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
+      const long long row = (long long)bk.m0 + (long long)mt * TC_BM * CG + (long long)rank * TC_BM + q * 32 + lane;
+      const long long col0 = (long long)bk.n0 + (long long)nt * TC_BN + half * 128;
+      const long long row_end = (long long)bk.m0 + bk.mc, col_end = (long long)bk.n0 + bk.nc;
+      if (row < row_end && col0 < col_end) {
+        const int ea = p.ea[(long long)inst * p.ea_inst + row];
+        const int* eb = p.eb + (long long)inst * p.eb_inst + col0;
+        double* dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
+        const bool v4 = p.vec == 4 && (bk.n0 & 3) == 0 && col0 + 128 <= col_end;
+        // every level comes back from the scratch area (this thread's own stores): a rolled loop over four columns,
+        // since 128 unrolled assemblies from registers (300 KB of code) ran from the instruction cache's misses
+        auto value = [&](const int4* l, int u, int ebj) -> double {
+          auto at = [&](int k) { return (long long)reinterpret_cast<const int*>(l + k)[u]; };
+          if (ea == kExpNaN || ebj == kExpNaN) return nan("");
+          return assemble((at(5) << 16) + (at(4) << 8) + at(3), (at(2) << 16) + (at(1) << 8) + at(0), ea + ebj - 54);
+        };
+#pragma unroll 2
+        for (int j = 0; j < 128; j += 4) {
+          if (col0 + j >= col_end) break;
+          int4 l[SC_PLANES];
+#pragma unroll
+          for (int k = 0; k < SC_PLANES; ++k) l[k] = park[(k * 32 + j / 4) * TC_FOLD_THREADS];
+          double v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = col0 + j + u < col_end ? value(l, u, eb[j + u]) : 0.0;
+          if (v4) {
+            if (p.accumulate) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u) v[u] += dst[j + u];
+            }
+            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + j), "d"(v[0]), "d"(v[1]), "d"(v[2]),
+                         "d"(v[3])
+                         : "memory");
+          } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (col0 + j + u < col_end) dst[j + u] = p.accumulate ? dst[j + u] + v[u] : v[u];
+          }
+        }
+      }
+    }
+  }
+  if constexpr (CG == 1) {
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) atomic_status(p.status, ST_TIMEOUT);
+    if (warp == 1) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+                   : "memory");
+    }
+  } else {
+    __syncwarp();
+    cluster_sync();
+    if (threadIdx.x == 0 && *abort_flag) atomic_status(p.status, ST_TIMEOUT);
+    if (warp == 1) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+                   : "memory");
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------- slicing
+// One block per row: the row's largest magnitude gives its exponent, then every entry becomes NSL fp16 digits. Rows are
+// read twice (the second time from L1 / L2), the digits written two columns per thread (4-byte stores, coalesced).
+// Zero-field operands (L != null): row r belongs to a parity class that holds entries only in the columns
+// [kstart, kstart + ncls) of its k class; the columns up to the next multiple of 64 get zeros (the GEMM's k-blocks run
+// over them). which = 0: row r of Bt, k class = its column group; which = 1: row r of A, k class = its row class ^ *pi.
+__global__ void __launch_bounds__(128) k_slice_rows(const double* __restrict__ X, long long ldx, long long K, __half* out,
+                                                    long long ld, long long plane, int* __restrict__ exps,
+                                                    const Z2Layout* __restrict__ L, const int* __restrict__ pi, int which,
+                                                    long long x_inst, long long o_inst, long long e_inst) {
+  __shared__ double red[4];
+  const long long row = blockIdx.x;
+  X += (long long)blockIdx.y * x_inst + row * ldx;
+  out += (long long)blockIdx.y * o_inst + row * ld;
+  long long c0 = 0, kc = K, kpad = K;
+  if (L) {
+    const int ck = which == 0 ? (row >= L->goff[1] ? 1 : 0) : ((row >= L->ncls[0] ? 1 : 0) ^ *pi);
+    c0 = L->kstart[ck];
+    kc = L->ncls[ck];
+    kpad = (kc + 63) / 64 * 64;
+  }
+  double m = 0.0;
+  bool bad = false;
+  for (long long k = threadIdx.x; k < kc; k += 128) {
+    const double a = fabs(X[c0 + k]);
+    bad |= !(a < INFINITY);
+    m = fmax(m, a);
+  }
+  if (bad) m = INFINITY;
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = m;
+  __syncthreads();
+  m = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
+  const bool finite = m < INFINITY;
+  int e = 0;
+  if (finite && m > 0.0) frexp(m, &e);
+  if (threadIdx.x == 0) exps[(long long)blockIdx.y * e_inst + row] = finite ? e : kExpNaN;
+  // x 2^(kSliceBits - e), in two exact factors where one would leave the exponent range
+  const int sh = kSliceBits - e;
+  const int h1 = sh / 2, h2 = sh - h1;
+  const bool one = sh < 1000 && sh > -1000;
+  const double f1 = one ? ldexp(1.0, sh) : ldexp(1.0, h1), f2 = ldexp(1.0, h2);
+  for (long long k = 2 * threadIdx.x; k < kpad; k += 256) {
+    long long v[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      double x = (finite && k + u < kc) ? X[c0 + k + u] : 0.0;
+      x *= f1;
+      if (!one) x *= f2;
+      v[u] = __double2ll_rn(x);
+    }
+    const bool both = k + 1 < kpad;
+#pragma unroll
+    for (int i = NSL - 1; i >= 0; --i) {
+      __half h[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int dgt = i ? (int)(signed char)(v[u] & 255) : (int)v[u];
+        if (i) v[u] = (v[u] - dgt) >> 8;
+        // 1024 + (d + 128) is an fp16 whose low bits hold d + 128
+        h[u] = __hsub(__ushort_as_half((unsigned short)(0x6400 + dgt + 128)), __ushort_as_half(0x6480));
+      }
+      __half* dst = out + (long long)i * plane + c0 + k;
+      if (both) *reinterpret_cast<__half2*>(dst) = __halves2half2(h[0], h[1]);
+      else dst[0] = h[0];
+    }
+  }
+}
+
+bool slice_map(CUtensorMap* m, const __half* ptr, long long rows, long long cols, long long ld, long long plane, int batch,
+               long long inst, int box_rows) {
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)NSL, (cuuint64_t)batch};
+  cuuint64_t strides[3] = {(cuuint64_t)ld * 2, (cuuint64_t)plane * 2, (cuuint64_t)inst * 2};
+  cuuint32_t box[4] = {SBK, (cuuint32_t)box_rows, 1, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<__half*>(ptr), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int CG>
+int launch_slices_variant(long long tiles, const SliceOperand& A, const SliceOperand& B, const SliceParams& p,
+                          cudaStream_t s) {
+  using Cf = SCfg<CG>;
+  SliceMaps maps;
+  std::memset(&maps, 0, sizeof(maps));
+  if (!slice_map(&maps.a, A.p, p.M, p.K, A.ld, A.plane, p.batch, A.inst, TC_BM) ||
+      !slice_map(&maps.b, B.p, p.N, p.K, B.ld, B.plane, p.batch, B.inst, TC_BN / CG))
+    return HOTRG_EDEVICE;
+  auto kern = k_gemm_slices<CG>;
+  static std::atomic<int> resident[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return HOTRG_EDEVICE;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CG;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.blockDim = dim3(TC_THREADS);
+  cfg.dynamicSmemBytes = Cf::SMEM;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = CG > 1 ? 1 : 0;
+  int n = resident[dev].load();
+  if (n <= 0) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cf::SMEM) != cudaSuccess)
+      return HOTRG_EDEVICE;
+    if (CG == 1) {
+      n = num_sms();
+    } else {
+      cfg.gridDim = dim3((unsigned)(CG * std::max(1, num_sms() / CG)));
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
+        cudaGetLastError();
+        return HOTRG_EDEVICE;
+      }
+    }
+    resident[dev].store(n);
+  }
+  // the scratch area holds kSliceCtas CTAs
+  const long long units = std::max(1LL, std::min({tiles, (long long)n, (long long)(kSliceCtas / CG)}));
+  cfg.gridDim = dim3((unsigned)(units * CG));
+  if (cudaLaunchKernelEx(&cfg, kern, maps, p) != cudaSuccess) {
+    cudaGetLastError();
+    return HOTRG_EDEVICE;
+  }
+  return HOTRG_OK;
+}
+
+long long slice_tiles(long long M, long long N, int cg) {
+  return ((M + TC_BM * cg - 1) / (TC_BM * cg)) * ((N + TC_BN - 1) / TC_BN);
+}
+
+}  // namespace
+
+bool slices_take(long long M, long long N, long long K) {
+  return M >= TC_BM && N >= TC_BN && K >= 64 && K <= 16320 && M <= 0x7fffffffLL && N <= 0x7fffffffLL;
+}
+
+size_t slice_scratch_bytes(long long M, long long N, int batch) {
+  // at most kSliceCtas CTAs, and at most one (or a pair) per tile of up to two blocks per instance
+  const long long t = std::min<long long>(kSliceCtas, 4 * slice_tiles(M, N, 1) * batch);
+  return (size_t)t * SC_PLANES * 128 * TC_FOLD_THREADS * sizeof(int);
+}
+
+void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
+                       long long x_inst, cudaStream_t s, const Z2Layout* L, const int* pi, int which) {
+  k_slice_rows<<<dim3((unsigned)rows, (unsigned)batch), 128, 0, s>>>(X, ldx, K, out.p, out.ld, out.plane, out.exps, L, pi,
+                                                                     which, x_inst, out.inst, out.exp_inst);
+  count_launches(1);
+}
+
+int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,
+                       long long K, int* scratch, int* status, double timeout_s, cudaStream_t s, const GemmBlocks* blk,
+                       const GemmBatch* bat, bool accumulate, int cta_group) {
+  if (!slices_take(M, N, K)) return HOTRG_EINVAL;
+  const int batch = bat ? bat->batch : 1;
+  if (batch < 1 || batch > kMaxGemmBatch || (A.ld % 8) || (B.ld % 8) || A.ld < K || B.ld < K || ldc < N)
+    return HOTRG_EINVAL;
+  if ((reinterpret_cast<uintptr_t>(A.p) | reinterpret_cast<uintptr_t>(B.p)) & 15) return HOTRG_EINVAL;
+  if ((A.plane % 8) || (B.plane % 8) || (A.inst % 8) || (B.inst % 8)) return HOTRG_EINVAL;
+  SliceParams p;
+  p.M = M;
+  p.N = N;
+  p.K = K;
+  p.num_kb = (int)((K + SBK - 1) / SBK);
+  p.group_m = 16;
+  p.batch = batch;
+  p.C = C;
+  p.ldc = ldc;
+  p.c_inst = bat ? bat->c_inst : 0;
+  p.ea = A.exps;
+  p.eb = B.exps;
+  p.ea_inst = A.exp_inst;
+  p.eb_inst = B.exp_inst;
+  p.scratch = reinterpret_cast<int4*>(scratch);
+  p.status = status;
+  p.timeout_ns = (unsigned long long)(timeout_s * 1e9);
+  p.blk = blk;
+  p.accumulate = accumulate ? 1 : 0;
+  p.vec = (ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(C) & 31) == 0 && (p.c_inst % 4) == 0 ? 4 : 1;
+  p.idesc = idesc_for(true, cta_group);
+  long long t = slice_tiles(M, N, cta_group) * batch;
+  if (t > 0x3fffffffLL) return HOTRG_EINVAL;
+  if (blk) t *= 2;  // the two blocks' tiles are counted on the device
+  const int rc = cta_group == 2 ? launch_slices_variant<2>(t, A, B, p, s) : launch_slices_variant<1>(t, A, B, p, s);
+  if (rc) return rc;
+  count_launches(1);
+  return HOTRG_OK;
+}
+
+}  // namespace hotrg

@@ -96,6 +96,12 @@ struct hotrg_ctx {
   // instances squeezed together (one GEMM launch per chunk for all of them): every per-step buffer
   // holds `group` slots, st_* bytes apart
   int group = 1;
+  // FP64 products on the tensor cores (gemm_f64tc.cu): the Y and Bt buffers then hold digit planes. yt: the A operand
+  // in double before slicing (the B operand is built in O, free until the first chunk), ey / eb: row exponents,
+  // slice_scratch: level sums of the running launch
+  bool slices = true;
+  void *yt = nullptr, *ey = nullptr, *eb = nullptr, *slice_scratch = nullptr;
+  size_t sz_yt = 0, sz_ey = 0, sz_eb = 0, sz_scr = 0, st_yt = 0, st_ey = 0, st_eb = 0;
   size_t st_Tt = 0, st_Bt = 0, st_X = 0, st_Y = 0, st_O = 0, st_R1 = 0, st_R2 = 0, st_Tnext = 0;
   long long spec_stride = 0;  // doubles per instance in spec_log
   // phase timing (hotrg_timing_start/stop): CUDA events recorded on `stream`
@@ -150,13 +156,22 @@ constexpr int kSpecCap = kMaxGram;  // eigenvalues stored per (step, axis)
 
 long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
 
+// Row stride of a chunk's GEMM output: the slice GEMM stores 32 bytes (four doubles) at a time.
+long long output_ld(long long n, bool slices) { return slices ? round_up(n, 4) : n; }
+
 // Sizes (bytes) of the per-step scratch buffers for one configuration.
 struct StepNeeds {
-  size_t Tt, Bt, X, Y, O, R1, R2;
+  size_t Tt = 0, Bt = 0, X = 0, Y = 0, O = 0, R1 = 0, R2 = 0;
+  size_t yt = 0, ey = 0, eb = 0, scr = 0;  // FP64 products on slices
 };
 
-// mixed: 0 = FP64 path, 2 or 3 = tensor-core path with that many bf16 planes per operand
-StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes) {
+// Contexts whose workspace would pass this size with the digit planes (twice the bytes of FP64 operands) keep the FP64
+// operands and the FP64 units: what fitted the card before still does.
+constexpr size_t kSliceWorkspaceLimit = (size_t)128 << 30;
+
+// planes: 0 = FP64 path, 2 or 3 = tensor-core path with that many 16-bit planes per operand. slices: FP64 products
+// run on digit slices where their shape takes it, over groups of `group` instances.
+StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool slices, int group) {
   const bool mixed = planes > 0;
   Geom g = make_geom(d, dims);
   const long long P = g.P;
@@ -178,10 +193,19 @@ StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes) {
   const size_t es = mixed ? 4 : 8;  // intermediate element size (float / double)
   StepNeeds n;
   n.Tt = (size_t)(P * P) * es;
-  n.Bt = (size_t)(chi3 * P * ldk) * (mixed ? 2 * planes : 8);  // bf16 planes, or double
+  const bool sl = !mixed && slices && slices_take(P, chi3 * P, ldk);
+  const size_t op = mixed ? 2 * planes : (sl ? 2 * kSliceCount : 8);  // bytes of an operand entry
+  n.Bt = (size_t)(chi3 * P * ldk) * op;
   n.X = (size_t)(P * P) * es;
-  n.Y = (size_t)(P * ldk) * (mixed ? 2 * planes : 8);
-  n.O = (size_t)(P * chi3 * P) * es;
+  n.Y = (size_t)(P * ldk) * op;
+  n.O = (size_t)(P * output_ld(chi3 * P, sl)) * es;
+  if (sl) {
+    n.O = std::max(n.O, (size_t)(chi3 * P * ldk) * 8);
+    n.yt = (size_t)(P * ldk) * 8;
+    n.ey = (size_t)P * sizeof(int);
+    n.eb = (size_t)(chi3 * P) * sizeof(int);
+    n.scr = slice_scratch_bytes(P, chi3 * P, group);
+  }
   // epilogue intermediates: contract the other transverse axes in order
   long long cur = P * chi3 * P;
   size_t r[2] = {0, 0};
@@ -203,6 +227,10 @@ void max_into(StepNeeds& acc, const StepNeeds& n) {
   acc.O = std::max(acc.O, n.O);
   acc.R1 = std::max(acc.R1, n.R1);
   acc.R2 = std::max(acc.R2, n.R2);
+  acc.yt = std::max(acc.yt, n.yt);
+  acc.ey = std::max(acc.ey, n.ey);
+  acc.eb = std::max(acc.eb, n.eb);
+  acc.scr = std::max(acc.scr, n.scr);
 }
 
 // Workspace plan: the per-step buffers must hold every step a context can take. The bond
@@ -245,7 +273,7 @@ bool f16_planes(int precision, int planes) {
   return planes == 2 && (precision == HOTRG_FP16X3 || precision == HOTRG_FP16X4);
 }
 
-StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int max_steps,
+StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int max_steps, bool slices, int group,
                long long* Pmax_out) {
   // breadth-first: minimal number of steps after which each bond-dimension state is reached
   std::vector<std::vector<int>> states{std::vector<int>(d, 2)};
@@ -262,7 +290,7 @@ StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int
       }
     }
   }
-  StepNeeds acc{0, 0, 0, 0, 0, 0, 0};
+  StepNeeds acc;
   long long Pmax = 1;
   for (size_t i = 0; i < states.size(); ++i) {
     long long P = 1;
@@ -274,7 +302,7 @@ StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int
       for (int step : {first, fp64_steps + 1, x6_steps + 1, max_steps})
         if (step >= first && step <= max_steps)
           max_into(acc, needs_for(d, states[i].data(), a, Dcut,
-                                  planes_for_step(precision, step, fp64_steps, x6_steps, P)));
+                                  planes_for_step(precision, step, fp64_steps, x6_steps, P), slices, group));
   }
   *Pmax_out = Pmax;
   return acc;
@@ -294,7 +322,7 @@ struct Carver {
 // Lay out every buffer; with base == nullptr only the total size is computed.
 size_t carve(hotrg_ctx* c, char* base) {
   long long Pmax = 1;
-  StepNeeds n = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, &Pmax);
+  StepNeeds n = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, c->slices, c->group, &Pmax);
   c->Pmax = Pmax;
   const long long P2 = Pmax * Pmax;
   const int nr_max = kMaxGram;
@@ -377,6 +405,13 @@ size_t carve(hotrg_ctx* c, char* base) {
   c->O = slots(n.O, c->sz_O, c->st_O);
   c->R1 = slots(n.R1, c->sz_R1, c->st_R1);
   c->R2 = slots(n.R2, c->sz_R2, c->st_R2);
+  if (n.scr) {
+    c->yt = slots(n.yt, c->sz_yt, c->st_yt);
+    c->ey = slots(n.ey * blk, c->sz_ey, c->st_ey);
+    c->eb = slots(n.eb * blk, c->sz_eb, c->st_eb);
+    c->sz_scr = n.scr;
+    c->slice_scratch = k.take<char>(n.scr);
+  }
   if (c->deriv) {
     c->Tt2 = k.take<char>(n.Tt);
     c->dX1[0] = k.take<char>(n.X);
@@ -387,6 +422,17 @@ size_t carve(hotrg_ctx* c, char* base) {
     c->dR2 = k.take<char>(n.R2 ? n.R2 : 256);
   }
   return k.off;
+}
+
+// Workspace bytes, with digit slices for the FP64 products unless that would pass kSliceWorkspaceLimit.
+size_t plan_workspace(hotrg_ctx* c) {
+  c->slices = true;
+  size_t n = carve(c, nullptr);
+  if (n > kSliceWorkspaceLimit) {
+    c->slices = false;
+    n = carve(c, nullptr);
+  }
+  return n;
 }
 
 int cuda_err(hotrg_ctx* c) {
@@ -615,7 +661,8 @@ struct Tangents {
 // holds opts.group slots of each).
 struct Slot {
   void *Tt, *Bt, *X1, *X2, *Y, *O, *R1, *R2;
-  double* Tnext;
+  double *Tnext, *yt;
+  int *ey, *eb;
   unsigned* amax;  // [0] bound of the B operand's source, [1] of the A operand's (fp16 planes)
   int *z2rank, *z2kcol, *z2colpos, *z2pi;
   GemmBlocks* z2blk;
@@ -635,6 +682,9 @@ Slot slot(const hotrg_ctx* c, int j) {
   q.R1 = at(c->R1, c->st_R1);
   q.R2 = at(c->R2, c->st_R2);
   q.Tnext = static_cast<double*>(at(c->Tnext, c->st_Tnext));
+  q.yt = static_cast<double*>(at(c->yt, c->st_yt));
+  q.ey = static_cast<int*>(at(c->ey, c->st_ey));
+  q.eb = static_cast<int*>(at(c->eb, c->st_eb));
   q.amax = c->amax + 2 * j;
   q.z2rank = c->z2rank ? c->z2rank + c->Pmax * j : nullptr;
   q.z2kcol = c->z2kcol ? c->z2kcol + c->Pmax * j : nullptr;
@@ -662,6 +712,24 @@ struct Group {
   }
 };
 
+bool slices_fit(const hotrg_ctx* c, const StepNeeds& need, int nblk) {
+  return need.yt <= c->sz_yt && need.ey * nblk <= c->sz_ey && need.eb * nblk <= c->sz_eb && need.scr <= c->sz_scr;
+}
+
+// An operand on digit slices: column block `blk` (of ldk columns) of the planes at `base`, its row exponents the
+// blk-th run of `rows` entries of `exps`.
+SliceOperand slice_operand(void* base, long long plane, long long ld, long long ldk, int blk, int* exps, long long rows,
+                           size_t inst_bytes, size_t exp_inst_bytes) {
+  SliceOperand o;
+  o.p = static_cast<__half*>(base) + blk * ldk;
+  o.ld = ld;
+  o.plane = plane;
+  o.inst = (long long)(inst_bytes / sizeof(__half));
+  o.exps = exps + blk * rows;
+  o.exp_inst = (long long)(exp_inst_bytes / sizeof(int));
+  return o;
+}
+
 // planes: 0 = FP64 path (TC = double), 2 / 3 = tensor-core path (TC = float) with 3 / 6 passes.
 template <class TC>
 // Coarse-grained tensor of the pair (T1 lower site, T2 upper site along a) into `out` (new
@@ -683,19 +751,20 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
   const int ng = G.n;
   if (ng < 1 || ng > c->group || (tg.n && ng != 1)) return HOTRG_ESTATE;
   const long long P = g.P;
-  const long long ldk = mixed ? round_up(P, 64) : P;
   const int nblk = tg.n ? 3 : 1;
-  const long long ld = nblk * ldk;
   const int fwd_blk = tg.n ? 1 : 0;
   const int c3 = nt ? trans[nt - 1] : -1;
   const int chi3 = c3 >= 0 ? chi[c3] : 1;
   auto Ub = [&](const double* base, int b) { return base + (long long)b * kMaxBond * kMaxGram; };
   // bounds of this step's buffers against the plan
-  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes);
+  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes, c->slices, c->group);
   if (need.Tt > c->sz_Tt || need.Bt * nblk > c->sz_Bt || need.X > c->sz_X || need.Y * nblk > c->sz_Y ||
-      need.O > c->sz_O || need.R1 > c->sz_R1 || need.R2 > c->sz_R2)
+      need.O > c->sz_O || need.R1 > c->sz_R1 || need.R2 > c->sz_R2 || !slices_fit(c, need, nblk))
     return HOTRG_ENOMEM;
+  const bool sl = need.scr > 0;  // FP64 products on digit slices
   if (tg.n && (!c->Tt2 || !c->dO || tg.n > 2)) return HOTRG_ESTATE;
+  const long long ldk = mixed || sl ? round_up(P, 64) : P;
+  const long long ld = nblk * ldk;
   const int nparts = mixed ? planes : 1;
   const long long bt_plane = (long long)chi3 * P * ld, y_plane = P * ld;
   // fp16 planes (FP16 modes; the forward squeeze only, tangents keep bf16): each operand's scale
@@ -723,6 +792,41 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
   auto gemm_a_blk = [](int p) { return p == 0 ? 0 : 1; };
   auto gemm_b_blk = [](int p) { return p == 0 ? 1 : 0; };
   const Slot S0 = slot(c, 0);
+  auto slice_y = [&](const Slot& S, int blk) {
+    return slice_operand(S.Y, y_plane, ld, ldk, blk, S.ey, P, c->st_Y, c->st_ey);
+  };
+  auto slice_bt = [&](const Slot& S, int blk) {
+    return slice_operand(S.Bt, bt_plane, ld, ldk, blk, S.eb, (long long)chi3 * P, c->st_Bt, c->st_eb);
+  };
+  // the operands in double before slicing: B in O (free until the first chunk's GEMM), A in yt, rows of P entries
+  auto dense_plane = [&](void* base) {
+    Planes<Op> q;
+    q.nparts = 1;
+    for (int k = 0; k < 3; ++k) q.p[k] = static_cast<Op*>(base);
+    return q;
+  };
+  auto build_bt = [&](const Slot& S, const TC* src, int blk, int which, const double* U, const TC* src2,
+                      const double* U2) {
+    if constexpr (!mixed) {
+      if (sl) {
+        launch_build_bt<TC, Op>(src, dense_plane(S.O), P, g, c3, U, chi3, s, src2, U2);
+        launch_slice_rows(static_cast<double*>(S.O), P, (long long)chi3 * P, P, slice_bt(S, blk), 1, 0, s);
+        return;
+      }
+    }
+    launch_build_bt<TC, Op>(src, blocks(S.Bt, bt_plane, blk, which, S.amax), ld, g, c3, U, chi3, s, src2, U2);
+  };
+  auto build_y = [&](const Slot& S, auto* src, int blk, int which) {
+    using Tin = typename std::remove_const<typename std::remove_pointer<decltype(src)>::type>::type;
+    if constexpr (!mixed) {
+      if (sl) {
+        launch_build_y<Tin, Op>(src, dense_plane(S.yt), P, g, a, s);
+        launch_slice_rows(S.yt, P, P, P, slice_y(S, blk), 1, 0, s);
+        return;
+      }
+    }
+    launch_build_y<Tin, Op>(src, blocks(S.Y, y_plane, blk, which, S.amax), ld, g, a, s);
+  };
   // B operand(s), one per instance
   PhaseScope* ops_scope = new PhaseScope(c, PH_OPERANDS);
   if (tg.n && mixed && ldk != P) {
@@ -735,20 +839,19 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
     TC* Tt = static_cast<TC*>(S.Tt);
     launch_transpose<TC>(G.T2[j], Tt, P, s);
     if (f16) launch_absmax<TC>(Tt, P, P, P, S.amax + 0, s);
-    launch_build_bt<TC, Op>(Tt, blocks(S.Bt, bt_plane, fwd_blk, 0, S.amax), ld, g, c3,
-                            c3 >= 0 ? Ub(G.U[j], c3) : nullptr, chi3, s);
+    build_bt(S, Tt, fwd_blk, 0, c3 >= 0 ? Ub(G.U[j], c3) : nullptr, nullptr, nullptr);
   }
   for (int p = 0; p < tg.n; ++p) {
     TC* dTt = static_cast<TC*>(c->Tt2);
     launch_transpose<TC>(tg.dT[p], dTt, P, s);
     const bool two = tg.dU[p] && c3 >= 0;
-    launch_build_bt<TC, Op>(dTt, blocks(S0.Bt, bt_plane, dbt_blk(p)), ld, g, c3, c3 >= 0 ? Ub(G.U[0], c3) : nullptr,
-                            chi3, s, two ? static_cast<TC*>(S0.Tt) : nullptr, two ? Ub(tg.dU[p], c3) : nullptr);
+    build_bt(S0, dTt, dbt_blk(p), -1, c3 >= 0 ? Ub(G.U[0], c3) : nullptr, two ? static_cast<TC*>(S0.Tt) : nullptr,
+             two ? Ub(tg.dU[p], c3) : nullptr);
   }
   delete ops_scope;
   TC* O = static_cast<TC*>(S0.O);
   TC* dO = static_cast<TC*>(c->dO);
-  const long long ldO = (long long)chi3 * P;
+  const long long N = (long long)chi3 * P, ldO = output_ld(N, sl);
   // chunks over the other transverse axes
   const int no = nt > 0 ? nt - 1 : 0;
   int kcnt[kMaxD] = {0, 0, 0, 0};
@@ -768,17 +871,26 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
     if constexpr (mixed) {
       const int rc = launch_gemm_split(blocks(S0.Y, y_plane, ablk, 1, S0.amax), ld,
                                        blocks(S0.Bt, bt_plane, bblk, 0, S0.amax), ld, reinterpret_cast<float*>(C),
-                                       ldO, P, ldO, K, npass, c->status, c->timeout_s, s, c->kblock, c->group_m,
+                                       ldO, P, N, K, npass, c->status, c->timeout_s, s, c->kblock, c->group_m,
                                        fold_group_for(c, npass), nullptr, batp, false, c->cta_group);
       if (rc) return rc;
-      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)ldO * K * npass * ng;
+      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * npass * ng;
+    } else if (sl) {
+      // the concatenated k range of a tangent runs as two products: the row exponents belong to one block each
+      for (int h = 0; h < (K > P ? 2 : 1); ++h) {
+        const int rc = launch_gemm_slices(slice_y(S0, ablk + h), slice_bt(S0, bblk + h), reinterpret_cast<double*>(C),
+                                          ldO, P, N, P, static_cast<int*>(c->slice_scratch), c->status, c->timeout_s, s,
+                                          nullptr, batp, h == 1);
+        if (rc) return rc;
+      }
+      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * kSliceProducts * ng;
     } else {
-      launch_gemm_f64(blocks(S0.Y, y_plane, ablk).p[0], ld, blocks(S0.Bt, bt_plane, bblk).p[0], ld, C, ldO, P, ldO,
+      launch_gemm_f64(blocks(S0.Y, y_plane, ablk).p[0], ld, blocks(S0.Bt, bt_plane, bblk).p[0], ld, C, ldO, P, N,
                       K, s, nullptr, batp);
-      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)ldO * K * ng;
+      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * ng;
     }
     if (c->timing) {
-      c->t_gemm_flops += 2.0 * P * (double)ldO * K * ng;
+      c->t_gemm_flops += 2.0 * P * (double)N * K * ng;
       ++c->t_gemm_launches;
     }
     return HOTRG_OK;
@@ -797,9 +909,8 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
       const double* U = G.U[j];
       if (no == 0) {
         if (f16) launch_absmax<double>(T1, P, P, P, S.amax + 1, s);
-        launch_build_y<double, Op>(T1, blocks(S.Y, y_plane, fwd_blk, 1, S.amax), ld, g, a, s);
-        for (int p = 0; p < tg.n; ++p)
-          launch_build_y<double, Op>(tg.dT[p], blocks(S.Y, y_plane, dy_blk(p)), ld, g, a, s);
+        build_y(S, T1, fwd_blk, 1);
+        for (int p = 0; p < tg.n; ++p) build_y(S, tg.dT[p], dy_blk(p), -1);
       } else {
         TC* X1 = static_cast<TC*>(S.X1);
         TC* X2 = static_cast<TC*>(S.X2);
@@ -818,7 +929,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
                                        f16 ? S.amax + 1 : nullptr);
           X = X2;
         }
-        launch_build_y<TC, Op>(X, blocks(S.Y, y_plane, fwd_blk, 1, S.amax), ld, g, a, s);
+        build_y(S, X, fwd_blk, 1);
         for (int p = 0; p < tg.n; ++p) {
           const TC* dX = static_cast<TC*>(c->dX1[p]);
           if (no >= 2) {
@@ -827,7 +938,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
                                          tg.dU[p] ? X1 : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[1]) : nullptr);
             dX = dX2;
           }
-          launch_build_y<TC, Op>(dX, blocks(S.Y, y_plane, dy_blk(p)), ld, g, a, s);
+          build_y(S, dX, dy_blk(p), -1);
         }
       }
     }
@@ -838,7 +949,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
       const int rc = gemm(fwd_blk, fwd_blk, O, P);
       if (rc) return rc;
       c->last_gemm.M = P;
-      c->last_gemm.N = ldO;
+      c->last_gemm.N = N;
       c->last_gemm.K = P;
       c->last_gemm.ldk = ld;
       c->last_gemm.npass = npass;
@@ -927,10 +1038,11 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
   const int c3 = trans[nt - 1];
   const int chi3 = chi[c3];
   auto Ub = [&](int j, int b) { return G.U[j] + (long long)b * kMaxBond * kMaxGram; };
-  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes);
+  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes, c->slices, c->group);
   if (need.Tt > c->sz_Tt || need.Bt > c->sz_Bt || need.X > c->sz_X || need.Y > c->sz_Y || need.O > c->sz_O ||
-      need.R1 > c->sz_R1 || need.R2 > c->sz_R2 || P > c->Pmax)
+      need.R1 > c->sz_R1 || need.R2 > c->sz_R2 || P > c->Pmax || !slices_fit(c, need, 1))
     return HOTRG_ENOMEM;
+  const bool sl = need.scr > 0;  // FP64 products on digit slices
   const int nparts = mixed ? planes : 1;
   const long long bt_plane = (long long)chi3 * P * ldz, y_plane = P * ldz;
   // fp16 planes in the FP16 modes, with the scale bounds of squeeze<TC> (B: sqrt(D_c3) max|Tt|)
@@ -947,8 +1059,14 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
     }
     return q;
   };
-  const long long ldO = (long long)chi3 * P;
+  const long long N = (long long)chi3 * P, ldO = output_ld(N, sl);
   const Slot S0 = slot(c, 0);
+  auto slice_y = [&](const Slot& S) {
+    return slice_operand(S.Y, y_plane, ldz, ldz, 0, S.ey, P, c->st_Y, c->st_ey);
+  };
+  auto slice_bt = [&](const Slot& S) {
+    return slice_operand(S.Bt, bt_plane, ldz, ldz, 0, S.eb, (long long)chi3 * P, c->st_Bt, c->st_eb);
+  };
   PhaseScope* ops_scope = new PhaseScope(c, PH_OPERANDS);
   for (int j = 0; j < ng; ++j) {
     const Slot S = slot(c, j);
@@ -956,14 +1074,18 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
     Z2Layout* L = c->z2L + inst;
     launch_z2_layout(c->z2ev + inst * kMaxD, c->z2ev_new + inst * kMaxD, 1, g, c3, chi3, L, s);
     launch_z2_tables(L, P, chi3, S.z2rank, S.z2kcol, S.z2colpos, s);
-    // zeros between and after the k classes (the GEMM's k-blocks run over them)
-    cudaMemsetAsync(S.Bt, 0, sizeof(Op) * nparts * bt_plane, s);
-    cudaMemsetAsync(S.Y, 0, sizeof(Op) * nparts * y_plane, s);
+    // zeros between and after the k classes (the GEMM's k-blocks run over them; slicing writes its own)
+    if (!sl) {
+      cudaMemsetAsync(S.Bt, 0, sizeof(Op) * nparts * bt_plane, s);
+      cudaMemsetAsync(S.Y, 0, sizeof(Op) * nparts * y_plane, s);
+    }
     TC* Tt = static_cast<TC*>(S.Tt);
     launch_transpose<TC>(G.T2[j], Tt, P, s);
     if (f16) launch_absmax<TC>(Tt, P, P, P, S.amax + 0, s);
-    launch_build_bt_z2<TC, Op>(Tt, pl(S.Bt, bt_plane, 0, S.amax), ldz, g, c3, Ub(j, c3), chi3, S.z2rank, S.z2kcol,
-                               S.z2colpos, L, s);
+    launch_build_bt_z2<TC, Op>(Tt, pl(sl ? S.O : S.Bt, bt_plane, 0, S.amax), ldz, g, c3, Ub(j, c3), chi3, S.z2rank,
+                               S.z2kcol, S.z2colpos, L, s);
+    if (sl)
+      launch_slice_rows(static_cast<double*>(S.O), ldz, (long long)chi3 * P, ldz, slice_bt(S), 1, 0, s, L, S.z2pi, 0);
   }
   delete ops_scope;
   const int no = nt - 1;
@@ -990,11 +1112,11 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
       const int inst = G.inst[j];
       const Z2Layout* L = c->z2L + inst;
       launch_z2_chunk(L, c->z2ev_new + inst * kMaxD, no, no > 0 ? trans[0] : 0, kcnt[0], no > 1 ? trans[1] : 0,
-                      kcnt[1], ldO, S.z2blk, S.z2pi, c->z2flops, mixed ? npass : 1, s);
+                      kcnt[1], N, S.z2blk, S.z2pi, c->z2flops, mixed ? npass : (sl ? kSliceProducts : 1), s);
       if (no == 0) {
         if (f16) launch_absmax<double>(G.T1[j], P, P, P, S.amax + 1, s);
-        launch_build_y_z2<double, Op>(G.T1[j], pl(S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol, L,
-                                      S.z2pi, s);
+        launch_build_y_z2<double, Op>(G.T1[j], pl(sl ? S.yt : S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol,
+                                      L, S.z2pi, s);
       } else {
         TC* X1 = static_cast<TC*>(S.X1);
         TC* X2 = static_cast<TC*>(S.X2);
@@ -1008,8 +1130,10 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
                                        f16 ? S.amax + 1 : nullptr);
           X = X2;
         }
-        launch_build_y_z2<TC, Op>(X, pl(S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol, L, S.z2pi, s);
+        launch_build_y_z2<TC, Op>(X, pl(sl ? S.yt : S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol, L, S.z2pi,
+                                  s);
       }
+      if (sl) launch_slice_rows(S.yt, ldz, P, ldz, slice_y(S), 1, 0, s, L, S.z2pi, 1);
     }
     if (no > 0) prev_k0 = kcnt[0];
     delete ops_scope;
@@ -1017,13 +1141,13 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
       PhaseScope gemm_scope(c, PH_GEMM);
       if constexpr (mixed) {
         const int rc = launch_gemm_split(pl(S0.Y, y_plane, 1, S0.amax), ldz, pl(S0.Bt, bt_plane, 0, S0.amax), ldz,
-                                         static_cast<float*>(S0.O), ldO, P, ldO, ldz, npass, c->status, c->timeout_s,
+                                         static_cast<float*>(S0.O), ldO, P, N, ldz, npass, c->status, c->timeout_s,
                                          s, c->kblock, c->group_m, fold_group_for(c, npass), S0.z2blk, batp, false,
                                          c->cta_group);
         if (rc) return rc;
         // what the autotuner replays: slot 0's operands and block descriptor of this chunk
         c->last_gemm.M = P;
-        c->last_gemm.N = ldO;
+        c->last_gemm.N = N;
         c->last_gemm.K = ldz;
         c->last_gemm.ldk = ldz;
         c->last_gemm.npass = npass;
@@ -1031,9 +1155,14 @@ int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int 
         c->last_gemm.fmt = f16 ? 1 : 0;
         c->last_gemm.mult_b = bt_mult;
         c->last_gemm.blk = S0.z2blk;
+      } else if (sl) {
+        const int rc = launch_gemm_slices(slice_y(S0), slice_bt(S0), static_cast<double*>(S0.O), ldO, P, N, ldz,
+                                          static_cast<int*>(c->slice_scratch), c->status, c->timeout_s, s, S0.z2blk,
+                                          batp);
+        if (rc) return rc;
       } else {
         launch_gemm_f64(pl(S0.Y, y_plane, 1, S0.amax).p[0], ldz, pl(S0.Bt, bt_plane, 0, S0.amax).p[0], ldz,
-                        static_cast<double*>(S0.O), ldO, P, ldO, ldz, s, S0.z2blk, batp);
+                        static_cast<double*>(S0.O), ldO, P, N, ldz, s, S0.z2blk, batp);
       }
       // the blocks' flops are counted on the device (k_z2_chunk)
       if (c->timing) {
@@ -1113,7 +1242,7 @@ int hotrg_workspace_size(int d, int Dcut, const hotrg_opts* opt, size_t* bytes) 
   c.impure = opt->impurities != 0;
   c.z2 = opt->z2 != 0;
   c.group = group_for(opt);
-  *bytes = carve(&c, nullptr);
+  *bytes = plan_workspace(&c);
   return HOTRG_OK;
 }
 
@@ -1175,7 +1304,7 @@ int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const ho
   c->stream = static_cast<cudaStream_t>(opt->stream);
   c->beta = vb;
   c->h = vh;
-  const size_t need = carve(c, nullptr);
+  const size_t need = plan_workspace(c);
   if (!opt->workspace || opt->workspace_bytes < need ||
       (reinterpret_cast<uintptr_t>(opt->workspace) % kAlign)) {
     delete c;
@@ -2038,6 +2167,42 @@ int hotrg_gemm_split_f16(const float* A, long long lda, const float* Bt, long lo
   launch_split_rows(Bt, ldb, N, K, Bp, ld, s);
   const int fg = fold_group > 0 ? fold_group : 1;
   const int rc = launch_gemm_split(Ap, ld, Bp, ld, C, ldc, M, N, K, npass, status, 4.0, s, kblock, 16, fg);
+  if (rc) return rc;
+  return cudaGetLastError() == cudaSuccess ? HOTRG_OK : HOTRG_EDEVICE;
+}
+
+// scratch: status word (256 bytes), row exponents, digit planes and level sums of the launch
+size_t hotrg_gemm_f64_scratch_bytes(long long M, long long N, long long K) {
+  if (!slices_take(M, N, K)) return 0;
+  const long long ld = round_up(K, 64);
+  return (size_t)(kAlign + round_up((M + N) * (long long)sizeof(int), kAlign) + round_up(2 * kSliceCount * M * ld, kAlign) +
+                  round_up(2 * kSliceCount * N * ld, kAlign)) +
+         slice_scratch_bytes(M, N, 1);
+}
+
+int hotrg_gemm_f64(const double* A, long long lda, const double* Bt, long long ldb, double* C, long long ldc, long long M,
+                   long long N, long long K, int cta_group, void* scratch, size_t scratch_bytes, void* stream) {
+  if (!A || !Bt || !C || !scratch || lda < K || ldb < K || ldc < N || (cta_group != 1 && cta_group != 2))
+    return HOTRG_EINVAL;
+  if (!slices_take(M, N, K) || scratch_bytes < hotrg_gemm_f64_scratch_bytes(M, N, K) ||
+      (reinterpret_cast<uintptr_t>(scratch) % kAlign))
+    return HOTRG_EINVAL;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const long long ld = round_up(K, 64);
+  char* p = static_cast<char*>(scratch);
+  int* status = reinterpret_cast<int*>(p);
+  p += kAlign;
+  int* exps = reinterpret_cast<int*>(p);
+  p += round_up((M + N) * (long long)sizeof(int), kAlign);
+  const SliceOperand a = slice_operand(p, M * ld, ld, ld, 0, exps, M, 0, 0);
+  p += round_up(2 * kSliceCount * M * ld, kAlign);
+  const SliceOperand b = slice_operand(p, N * ld, ld, ld, 0, exps + M, N, 0, 0);
+  p += round_up(2 * kSliceCount * N * ld, kAlign);
+  if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return HOTRG_EDEVICE;
+  launch_slice_rows(A, lda, M, K, a, 1, 0, s);
+  launch_slice_rows(Bt, ldb, N, K, b, 1, 0, s);
+  const int rc = launch_gemm_slices(a, b, C, ldc, M, N, K, reinterpret_cast<int*>(p), status, 4.0, s, nullptr, nullptr,
+                                    false, cta_group);
   if (rc) return rc;
   return cudaGetLastError() == cudaSuccess ? HOTRG_OK : HOTRG_EDEVICE;
 }

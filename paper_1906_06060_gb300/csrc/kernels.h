@@ -164,6 +164,34 @@ void launch_gemm_f64(const double* A, long long lda, const double* Bt, long long
                      long long ldc, long long M, long long N, long long K, cudaStream_t s,
                      const GemmBlocks* blk = nullptr, const GemmBatch* bat = nullptr);
 
+// ---- gemm_f64tc.cu --------------------------------------------------------------------------
+// FP64 products on the tensor cores from exact integer slices. An operand: kSliceCount planes of fp16 digits (`plane`
+// elements apart, rows of `ld`, instances `inst` apart) and the exponent of every row (instances exp_inst apart).
+constexpr int kSliceCount = 7;
+constexpr int kSliceProducts = kSliceCount * (kSliceCount + 1) / 2;  // digit pairs a product runs
+constexpr int kSliceCtas = 152;  // CTAs of a launch at most (one per SM): the scratch area is sized for them
+struct SliceOperand {
+  __half* p = nullptr;
+  long long ld = 0, plane = 0, inst = 0;
+  int* exps = nullptr;
+  long long exp_inst = 0;
+};
+// Whether a product of this shape can run on slices: at least one 128 x 256 tile and K up to 16320 (the int32 sums).
+bool slices_take(long long M, long long N, long long K);
+// Bytes of the level-sum scratch of a launch over `batch` products of at most M x N.
+size_t slice_scratch_bytes(long long M, long long N, int batch);
+// Digits and row exponents of `rows` x K doubles (row stride ldx; `batch` instances x_inst apart). With L (zero-field
+// operands, one instance) only the columns of each row's parity class, see k_slice_rows.
+struct Z2Layout;
+void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
+                       long long x_inst, cudaStream_t s, const Z2Layout* L = nullptr, const int* pi = nullptr,
+                       int which = 0);
+// C[m][n] (+)= sum_k A[m][k] Bt[n][k]; blk and bat as for launch_gemm_f64. Returns 0 or a hotrg_status.
+int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,
+                       long long K, int* scratch, int* status, double timeout_s, cudaStream_t s,
+                       const GemmBlocks* blk = nullptr, const GemmBatch* bat = nullptr, bool accumulate = false,
+                       int cta_group = 1);
+
 // ---- gemm_tc.cu ----------------------------------------------------------------------------
 // C[m][n] = sum over passes p of sum_k A_{a(p)}[m][k] Bt_{b(p)}[n][k], bf16 operand planes on
 // tcgen05, FP32 accumulation in TMEM. npass = 1: (hi,hi); 3: + (hi,lo), (lo,hi) with 2 planes;
