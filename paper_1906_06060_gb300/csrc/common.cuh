@@ -95,6 +95,11 @@ struct Planes {
   int fmt = 0;
   const unsigned* amax = nullptr;
   float amax_mult = 1.f;
+  // the planes and scale bound of instance i, `stride` elements apart
+  __device__ __forceinline__ void advance(int i, long long stride) {
+    for (int k = 0; k < 3; ++k) p[k] += i * stride;
+    if (amax) amax += i;
+  }
 };
 
 __device__ __forceinline__ float plane_bound(const unsigned* amax, float mult) {

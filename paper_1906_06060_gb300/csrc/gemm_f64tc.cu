@@ -3,20 +3,21 @@
 //
 // GB300 has no fast FP64 unit (1.25 TFLOP/s nominal, 4 flop per clock and SM), its fp16 tensor cores run at
 // 8192 flop per clock and SM. Every row of an operand is scaled by a power of two 2^-e that brings its largest entry
-// below 1 and rounded to a 55-bit fixed-point number, which is cut into 7 balanced digits of 8 bits,
+// below 1 and rounded to a 63-bit fixed-point number, which is cut into 8 balanced digits of 8 bits,
 //   x 2^-e = sum_i q_i 2^-(7 + 8 i),  -128 <= q_i <= 128,
-// each stored as an fp16 integer (exact). The product is the sum over the digit pairs with i + j <= 6 (28 products),
+// each stored as an fp16 integer (exact). The product is the sum over the digit pairs with i + j <= 7 (36 products),
 // grouped by level s = i + j:
 //   C[m][n] 2^-(eA + eB) = sum_s L_s 2^-(14 + 8 s),  L_s = sum_{i <= s} sum_k qA_i qB_{s-i}.
 // Exactness: |qA qB| <= 2^14, so a chain of 16 x 64 products stays within 2^24 and the tensor cores' FP32 accumulator
 // holds it exactly; every chain is added into an int32 register accumulator (|L_s| <= (s + 1) K 2^14 < 2^31 for
-// K <= 16320). Level 6 is folded into level 5
-// with a rounding shift, and the six level sums are combined exactly and rounded once. The error of a result is one
-// rounding plus about sqrt(K) 2^-56 of the two rows' largest entries (entries within 1/4 of their row's largest are
-// held exactly), where a chain of K FP64 operations rounds every partial sum to 2^-53 of its size. Rows holding NaN or
-// infinity give NaN.
+// K <= 16320). Levels 7 and 6 are folded into level 5 with a rounding shift each, and the six level sums are combined
+// exactly and rounded once. Entries within 2^-10 of their row's largest are held exactly; the dropped digit pairs are
+// worth about sqrt(7 K) 2^-65 of the two rows' largest entries. (Seven digits and 28 products, 13 - 22 % faster, drop
+// sqrt(6 K) 2^-57: at K = 4100 on rows that decay, further off than an FP64 product, so they are not taken.) Measured
+// relative error 5e-17 to 7e-17, one rounding, where FP64 products have 3e-16 to 1.1e-15. Rows holding NaN or infinity
+// give NaN.
 //
-// Work: 28 tensor products of 2 M N K flops against one on the FP64 units at 1/2000 of the rate.
+// Work: 36 tensor products of 2 M N K flops against one on the FP64 units at 1/2000 of the rate.
 // Kernel structure, ring and bounded waits as k_gemm_split (gemm_tc.cu): warp 0 copies, warp 1 issues MMAs, warps
 // 2-9 fold. Per output tile the levels run one after the other, least significant first, each over all k-blocks; a
 // ring stage holds one digit tile of A and one of B. A finished level sum goes to a per-CTA scratch area in global
@@ -49,7 +50,7 @@ struct SliceMaps {
 
 struct SliceParams {
   long long M, N, K;
-  int num_kb, group_m, batch;
+  int num_kb, group_m, batch, b_div;  // Bt of product i: instance i / b_div
   double* C;
   long long ldc, c_inst;
   const int* ea;  // row exponents of A and of Bt, instance strides ea_inst, eb_inst
@@ -125,14 +126,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   __shared__ int s_prefix[kMaxGemmBatch + 1];
   __shared__ int s_total;
+  if (p.blk) {
+    for (int i = threadIdx.x; i < p.batch; i += TC_THREADS) {
+      Blk b[2];
+      const int nb = load_blocks<SBK, CG>(p, i, b);
+      s_prefix[i] = b[0].tiles + (nb > 1 ? b[1].tiles : 0);
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     Blk b[2];
     if (p.blk) {
       int t = 0;
       for (int i = 0; i < p.batch; ++i) {
+        const int n = s_prefix[i];
         s_prefix[i] = t;
-        const int nb = load_blocks<SBK, CG>(p, i, b);
-        t += b[0].tiles + (nb > 1 ? b[1].tiles : 0);
+        t += n;
       }
       s_prefix[p.batch] = t;
       s_total = t;
@@ -188,6 +197,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
         const int arow = bk.m0 + mt * TC_BM * CG;
         const int brow = bk.n0 + nt * TC_BN;
+        const int binst = inst / p.b_div;
         for (int s = NSL - 1; s >= 0 && ok; --s)
           for (int kb = 0; kb < bk.num_kb && ok; ++kb) {
             const int kx = bk.k0 + kb * SBK;
@@ -198,12 +208,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               mbar_expect_tx(fb, CG * STAGE_BYTES);
               if constexpr (CG == 1) {
                 tma_load_4d(sa, &maps.a, fb, kx, arow, i, inst);
-                tma_load_4d(sb, &maps.b, fb, kx, brow, s - i, inst);
+                tma_load_4d(sb, &maps.b, fb, kx, brow, s - i, binst);
               } else {
                 tma_load_4d_pair(sa, &maps.a, fb, kx, arow, i, inst);
-                tma_load_4d_pair(sb, &maps.b, fb, kx, brow, s - i, inst);
+                tma_load_4d_pair(sb, &maps.b, fb, kx, brow, s - i, binst);
                 tma_load_4d_pair(mapa_rank(sa, 1), &maps.a, fb, kx, arow + TC_BM, i, inst);
-                tma_load_4d_pair(mapa_rank(sb, 1), &maps.b, fb, kx, brow + B_ROWS, s - i, inst);
+                tma_load_4d_pair(mapa_rank(sb, 1), &maps.b, fb, kx, brow + B_ROWS, s - i, binst);
               }
               ++issued;
               if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -323,7 +333,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const long long row_end = (long long)bk.m0 + bk.mc, col_end = (long long)bk.n0 + bk.nc;
       if (row < row_end && col0 < col_end) {
         const int ea = p.ea[(long long)inst * p.ea_inst + row];
-        const int* eb = p.eb + (long long)inst * p.eb_inst + col0;
+        const int* eb = p.eb + (long long)(inst / p.b_div) * p.eb_inst + col0;
         double* dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
         const bool v4 = p.vec == 4 && (bk.n0 & 3) == 0 && col0 + 128 <= col_end;
         // every level comes back from the scratch area (this thread's own stores): a rolled loop over four columns,
@@ -380,70 +390,70 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------- slicing
-// One block per row: the row's largest magnitude gives its exponent, then every entry becomes NSL fp16 digits. Rows are
-// read twice (the second time from L1 / L2), the digits written two columns per thread (4-byte stores, coalesced).
-// Zero-field operands (L != null): row r belongs to a parity class that holds entries only in the columns
-// [kstart, kstart + ncls) of its k class; the columns up to the next multiple of 64 get zeros (the GEMM's k-blocks run
-// over them). which = 0: row r of Bt, k class = its column group; which = 1: row r of A, k class = its row class ^ *pi.
-__global__ void __launch_bounds__(128) k_slice_rows(const double* __restrict__ X, long long ldx, long long K, __half* out,
-                                                    long long ld, long long plane, int* __restrict__ exps,
-                                                    const Z2Layout* __restrict__ L, const int* __restrict__ pi, int which,
-                                                    long long x_inst, long long o_inst, long long e_inst) {
-  __shared__ double red[4];
-  const long long row = blockIdx.x;
+// One warp per row: the row's largest exponent field gives its scale, then every entry becomes NSL fp16 digits, all in
+// integer arithmetic (in FP64 operations, ten an entry at two a clock and SM, a 10^4 x 10^3 operand took 160 us; its
+// traffic is worth 32). Rows are read twice (the second time from L1 / L2), two columns a lane; digits are stored four
+// bytes a lane, coalesced.
+// Zero-field operands (L != null): row r of slot blockIdx.y (instance blockIdx.y / nb) belongs to a parity class that
+// holds entries only in the columns [kstart, kstart + ncls) of its k class; the columns up to the next multiple of 64 get
+// zeros (the GEMM's k-blocks run over them). which = 0: row r of Bt, k class = its column group; which = 1: row r of A, k
+// class = its row class ^ pi[slot].
+constexpr int SLICE_WARPS = 4;
+__device__ __forceinline__ int exponent_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ long long fixed_point(double x, int top) {
+  // x 2^(kSliceBits - e) with e = top - 1022, rounded half away from zero: the mantissa moved by the fields' difference
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int f = (int)(b >> 52) & 0x7FF;
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | (f ? 1ULL << 52 : 0ULL);
+  const int sh = top - max(f, 1) - (kSliceBits - 53);
+  const unsigned long long v = sh <= 0 ? m << -sh : (sh > 54 ? 0ULL : (m + (1ULL << (sh - 1))) >> sh);
+  return (long long)b < 0 ? -(long long)v : (long long)v;
+}
+__global__ void __launch_bounds__(32 * SLICE_WARPS) k_slice_rows(const double* __restrict__ X, long long ldx,
+                                                                 long long rows, int K, __half* out, long long ld,
+                                                                 long long plane, int* __restrict__ exps,
+                                                                 const Z2Layout* __restrict__ L,
+                                                                 const int* __restrict__ pi, int which, long long x_inst,
+                                                                 long long o_inst, long long e_inst, int nb) {
+  const int lane = threadIdx.x % 32;
+  const long long row = (long long)blockIdx.x * SLICE_WARPS + threadIdx.x / 32;
+  if (row >= rows) return;
   X += (long long)blockIdx.y * x_inst + row * ldx;
   out += (long long)blockIdx.y * o_inst + row * ld;
-  long long c0 = 0, kc = K, kpad = K;
+  int kc = K, kpad = K;
   if (L) {
-    const int ck = which == 0 ? (row >= L->goff[1] ? 1 : 0) : ((row >= L->ncls[0] ? 1 : 0) ^ *pi);
-    c0 = L->kstart[ck];
+    L += blockIdx.y / nb;
+    const int ck = which == 0 ? (row >= L->goff[1] ? 1 : 0) : ((row >= L->ncls[0] ? 1 : 0) ^ pi[blockIdx.y]);
+    X += L->kstart[ck];
+    out += L->kstart[ck];
     kc = L->ncls[ck];
     kpad = (kc + 63) / 64 * 64;
   }
-  double m = 0.0;
-  bool bad = false;
-  for (long long k = threadIdx.x; k < kc; k += 128) {
-    const double a = fabs(X[c0 + k]);
-    bad |= !(a < INFINITY);
-    m = fmax(m, a);
-  }
-  if (bad) m = INFINITY;
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = m;
-  __syncthreads();
-  m = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
-  const bool finite = m < INFINITY;
-  int e = 0;
-  if (finite && m > 0.0) frexp(m, &e);
-  if (threadIdx.x == 0) exps[(long long)blockIdx.y * e_inst + row] = finite ? e : kExpNaN;
-  // x 2^(kSliceBits - e), in two exact factors where one would leave the exponent range
-  const int sh = kSliceBits - e;
-  const int h1 = sh / 2, h2 = sh - h1;
-  const bool one = sh < 1000 && sh > -1000;
-  const double f1 = one ? ldexp(1.0, sh) : ldexp(1.0, h1), f2 = ldexp(1.0, h2);
-  for (long long k = 2 * threadIdx.x; k < kpad; k += 256) {
+  int top = 1;  // (all subnormal: their unit's field)
+#pragma unroll 4
+  for (int k = lane; k < kc; k += 32) top = max(top, exponent_field(X[k]));
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  const bool finite = top < 0x7FF;
+  if (lane == 0) exps[(long long)blockIdx.y * e_inst + row] = finite ? top - 1022 : kExpNaN;
+#pragma unroll 2
+  for (int k = 2 * lane; k < kpad; k += 64) {
     long long v[2];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      double x = (finite && k + u < kc) ? X[c0 + k + u] : 0.0;
-      x *= f1;
-      if (!one) x *= f2;
-      v[u] = __double2ll_rn(x);
-    }
+    for (int u = 0; u < 2; ++u) v[u] = (finite && k + u < kc) ? fixed_point(X[k + u], top) : 0;
     const bool both = k + 1 < kpad;
 #pragma unroll
     for (int i = NSL - 1; i >= 0; --i) {
-      __half h[2];
+      unsigned h = 0;  // 1024 + (d + 128) is an fp16 whose low bits hold d + 128
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int dgt = i ? (int)(signed char)(v[u] & 255) : (int)v[u];
         if (i) v[u] = (v[u] - dgt) >> 8;
-        // 1024 + (d + 128) is an fp16 whose low bits hold d + 128
-        h[u] = __hsub(__ushort_as_half((unsigned short)(0x6400 + dgt + 128)), __ushort_as_half(0x6480));
+        h |= (unsigned)(0x6400 + dgt + 128) << (16 * u);
       }
-      __half* dst = out + (long long)i * plane + c0 + k;
-      if (both) *reinterpret_cast<__half2*>(dst) = __halves2half2(h[0], h[1]);
-      else dst[0] = h[0];
+      const __half2 q = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6480)));
+      __half* dst = out + (long long)i * plane + k;
+      if (both) *reinterpret_cast<__half2*>(dst) = q;
+      else dst[0] = __low2half(q);
     }
   }
 }
@@ -468,7 +478,7 @@ int launch_slices_variant(long long tiles, const SliceOperand& A, const SliceOpe
   SliceMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   if (!slice_map(&maps.a, A.p, p.M, p.K, A.ld, A.plane, p.batch, A.inst, TC_BM) ||
-      !slice_map(&maps.b, B.p, p.N, p.K, B.ld, B.plane, p.batch, B.inst, TC_BN / CG))
+      !slice_map(&maps.b, B.p, p.N, p.K, B.ld, B.plane, p.batch / p.b_div, B.inst, TC_BN / CG))
     return HOTRG_EDEVICE;
   auto kern = k_gemm_slices<CG>;
   static std::atomic<int> resident[kMaxDevices];
@@ -528,9 +538,9 @@ size_t slice_scratch_bytes(long long M, long long N, int batch) {
 }
 
 void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
-                       long long x_inst, cudaStream_t s, const Z2Layout* L, const int* pi, int which) {
-  k_slice_rows<<<dim3((unsigned)rows, (unsigned)batch), 128, 0, s>>>(X, ldx, K, out.p, out.ld, out.plane, out.exps, L, pi,
-                                                                     which, x_inst, out.inst, out.exp_inst);
+                       long long x_inst, cudaStream_t s, const Z2Layout* L, const int* pi, int which, int nb) {
+  k_slice_rows<<<dim3((unsigned)((rows + SLICE_WARPS - 1) / SLICE_WARPS), (unsigned)batch), 32 * SLICE_WARPS, 0, s>>>(
+      X, ldx, rows, (int)K, out.p, out.ld, out.plane, out.exps, L, pi, which, x_inst, out.inst, out.exp_inst, nb);
   count_launches(1);
 }
 
@@ -550,6 +560,8 @@ int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, 
   p.num_kb = (int)((K + SBK - 1) / SBK);
   p.group_m = 16;
   p.batch = batch;
+  p.b_div = bat ? bat->b_div : 1;
+  if (p.b_div < 1 || batch % p.b_div) return HOTRG_EINVAL;
   p.C = C;
   p.ldc = ldc;
   p.c_inst = bat ? bat->c_inst : 0;

@@ -119,11 +119,11 @@ struct TcParams {
   const unsigned* amaxB;
   float multA, multB;
   // batched launch: `batch` independent products of the same shape; instance i reads the operand
-  // planes at z = i of the 3D tensor maps, writes C + i c_inst, takes the descriptor blk[i] and the
-  // scale bounds amax + i amax_inst
+  // planes at z = i (A) and i / b_div (B) of the 3D tensor maps, writes C + i c_inst, takes the descriptor blk[i]
+  // and the scale bounds amaxA[i], amaxB[i / b_div]
   int batch;
   long long c_inst;
-  int amax_inst;
+  int b_div;  // B operand and B scale bound of instance i: i / b_div
   // wait probe: the producer issues no copies, so the first wait for a stage can never be satisfied
   // and must run out (nothing is in flight to drain)
   int stall;
@@ -164,15 +164,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   __shared__ int s_prefix[kMaxGemmBatch + 1];
   __shared__ int s_total;
+  if (p.blk) {
+    // tiles of every instance (block-sparse: the descriptors differ per instance), then their first tiles below
+    for (int i = threadIdx.x; i < p.batch; i += TC_THREADS) {
+      Blk b[2];
+      const int nb = load_blocks<BK, CG>(p, i, b);
+      s_prefix[i] = b[0].tiles + (nb > 1 ? b[1].tiles : 0);
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     Blk b[2];
     if (p.blk) {
-      // first tile of every instance (block-sparse: the descriptors differ per instance)
       int t = 0;
       for (int i = 0; i < p.batch; ++i) {
+        const int n = s_prefix[i];
         s_prefix[i] = t;
-        const int nb = load_blocks<BK, CG>(p, i, b);
-        t += b[0].tiles + (nb > 1 ? b[1].tiles : 0);
+        t += n;
       }
       s_prefix[p.batch] = t;
       s_total = t;
@@ -230,6 +238,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         locate<BK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
         const int arow = bk.m0 + mt * TC_BM * CG + (int)rank * TC_BM;
         const int brow = bk.n0 + nt * TC_BN + (int)rank * B_ROWS;
+        const int binst = inst / p.b_div;
         for (int kb = 0; kb < bk.num_kb; ++kb) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.timeout_ns)) { ok = false; break; }
           const uint32_t fb = full0 + 8 * stage;
@@ -239,7 +248,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
             for (int pl = 0; pl < NPL; ++pl) {
               tma_load_3d(smem_u32(a_tile(stage, pl)), &maps.a[pl], fb, kx, arow, inst);
-              tma_load_3d(smem_u32(b_tile(stage, pl)), &maps.b[pl], fb, kx, brow, inst);
+              tma_load_3d(smem_u32(b_tile(stage, pl)), &maps.b[pl], fb, kx, brow, binst);
             }
           } else {
             // this CTA fills the stage in both CTAs of the pair (the second CTA's copies land at the
@@ -249,9 +258,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int pl = 0; pl < NPL; ++pl) {
               const uint32_t sa = smem_u32(a_tile(stage, pl)), sb = smem_u32(b_tile(stage, pl));
               tma_load_3d_pair(sa, &maps.a[pl], fb, kx, arow, inst);
-              tma_load_3d_pair(sb, &maps.b[pl], fb, kx, brow, inst);
+              tma_load_3d_pair(sb, &maps.b[pl], fb, kx, brow, binst);
               tma_load_3d_pair(mapa_rank(sa, 1), &maps.a[pl], fb, kx, arow + TC_BM, inst);
-              tma_load_3d_pair(mapa_rank(sb, 1), &maps.b[pl], fb, kx, brow + B_ROWS, inst);
+              tma_load_3d_pair(mapa_rank(sb, 1), &maps.b[pl], fb, kx, brow + B_ROWS, binst);
             }
           }
           ++issued;
@@ -390,8 +399,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       if (p.amaxA) {
         // undo the operands' power-of-two scales (exact): the exponents the operand builders used
         const float unscale =
-            pow2f(-(f16_scale_exponent(plane_bound(p.amaxA + (long long)inst * p.amax_inst, p.multA)) +
-                    f16_scale_exponent(plane_bound(p.amaxB + (long long)inst * p.amax_inst, p.multB))));
+            pow2f(-(f16_scale_exponent(plane_bound(p.amaxA + inst, p.multA)) +
+                    f16_scale_exponent(plane_bound(p.amaxB + inst / p.b_div, p.multB))));
 #pragma unroll
         for (int j = 0; j < 128; ++j) acc[j] *= unscale;
       }
@@ -476,7 +485,7 @@ int launch_variant(long long tiles, const Planes<__nv_bfloat16>& A, long long ld
   std::memset(&maps, 0, sizeof(maps));
   for (int i = 0; i < NPL; ++i)
     if (!make_map(&maps.a[i], A.p[i], p.M, p.K, lda, p.batch, a_inst, TC_BM, BK, A.fmt == 1) ||
-        !make_map(&maps.b[i], B.p[i], p.N, p.K, ldb, p.batch, b_inst, TC_BN / CG, BK, B.fmt == 1))
+        !make_map(&maps.b[i], B.p[i], p.N, p.K, ldb, p.batch / p.b_div, b_inst, TC_BN / CG, BK, B.fmt == 1))
       return HOTRG_EDEVICE;
   auto kern = k_gemm_split<BK, NPL, NPASS, FG, CG>;
   // the dynamic shared-memory limit is a per-device attribute of the kernel: set it once on each
@@ -548,8 +557,8 @@ int launch_gemm_split(const Planes<__nv_bfloat16>& A, long long lda, const Plane
   const int batch = bat ? bat->batch : 1;
   const long long a_inst = bat ? bat->a_inst : M * lda, b_inst = bat ? bat->b_inst : N * ldb;
   if (batch < 1 || batch > kMaxGemmBatch) return HOTRG_EINVAL;
-  if (batch > 1 && (a_inst < M * lda || b_inst < N * ldb || (a_inst % 8) || (b_inst % 8) ||
-                    bat->c_inst < M * ldc || bat->amax_inst < 0))
+  if (batch > 1 && (a_inst < M * lda || b_inst < N * ldb || (a_inst % 8) || (b_inst % 8) || bat->c_inst < M * ldc ||
+                    bat->b_div < 1 || batch % bat->b_div))
     return HOTRG_EINVAL;
   TcParams p;
   p.M = M;
@@ -573,7 +582,7 @@ int launch_gemm_split(const Planes<__nv_bfloat16>& A, long long lda, const Plane
   p.multB = B.amax_mult;
   p.batch = batch;
   p.c_inst = bat ? bat->c_inst : 0;
-  p.amax_inst = bat ? bat->amax_inst : 0;
+  p.b_div = bat ? bat->b_div : 1;
   p.stall = stall ? 1 : 0;
   // output tiles: 128 x 256 per CTA, 256 x 256 per CTA pair
   const long long tiles = (long long)((M + (long long)TC_BM * cta_group - 1) / ((long long)TC_BM * cta_group)) *

@@ -26,6 +26,141 @@
 
 using namespace hotrg;
 
+namespace {
+
+constexpr long long kAlign = 256;
+// shape of the wait probe's GEMM launch: one output tile, one k-block
+constexpr long long TC_PROBE_M = 128, TC_PROBE_N = 256, TC_PROBE_K = 64;
+constexpr int kSpecCap = kMaxGram;  // eigenvalues stored per (step, axis)
+
+long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
+
+// Row stride of a chunk's GEMM output: the slice GEMM stores 32 bytes (four doubles) at a time.
+long long output_ld(long long n, bool slices) { return slices ? round_up(n, 4) : n; }
+
+// Bytes a slot of a per-step buffer takes (256-byte aligned: TMA plane starts).
+size_t slot_bytes(size_t n) { return (size_t)round_up((long long)(n ? n : 1), kAlign); }
+
+// Sizes (bytes) of the per-step buffers for one configuration: Tt, Bt, X1, eb per instance of a group, the others per
+// chunk in flight; nb: chunks in flight; yt, ey, eb, scr: FP64 products on digit slices.
+struct StepNeeds {
+  size_t Tt = 0, Bt = 0, X1 = 0, eb = 0;
+  size_t X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0;
+  size_t scr = 0;
+  int nb = 1;
+};
+
+// Bytes per instance of the group that hold every step of a plan.
+struct StepSizes {
+  size_t Tt = 0, Bt = 0, X1 = 0, eb = 0, X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0, scr = 0;
+  static StepSizes of(const StepNeeds& n) {
+    auto chunks = [&](size_t x) { return (size_t)n.nb * slot_bytes(x); };
+    StepSizes z;
+    z.Tt = slot_bytes(n.Tt);
+    z.Bt = slot_bytes(n.Bt);
+    z.X1 = slot_bytes(n.X1);
+    z.eb = slot_bytes(n.eb);
+    z.X2 = chunks(n.X2);
+    z.Y = chunks(n.Y);
+    z.O = chunks(n.O);
+    z.R1 = chunks(n.R1);
+    z.R2 = chunks(n.R2);
+    z.yt = chunks(n.yt);
+    z.ey = chunks(n.ey);
+    z.scr = n.scr;
+    return z;
+  }
+  template <class F>
+  static void each(F f) {
+    for (size_t StepSizes::*m : {&StepSizes::Tt, &StepSizes::Bt, &StepSizes::X1, &StepSizes::eb, &StepSizes::X2,
+                                 &StepSizes::Y, &StepSizes::O, &StepSizes::R1, &StepSizes::R2, &StepSizes::yt,
+                                 &StepSizes::ey, &StepSizes::scr})
+      f(m);
+  }
+  void max_with(const StepSizes& o) {
+    each([&](size_t StepSizes::*m) { this->*m = std::max(this->*m, o.*m); });
+  }
+  bool covers(const StepNeeds& n) const {
+    const StepSizes o = of(n);
+    bool ok = true;
+    each([&](size_t StepSizes::*m) { ok = ok && o.*m <= this->*m; });
+    return ok;
+  }
+};
+
+// Contexts whose workspace would pass this size with the digit planes (16 bytes an entry for FP64's 8) keep the FP64
+// operands and the FP64 units: what fitted the card before still does.
+constexpr size_t kSliceWorkspaceLimit = (size_t)128 << 30;
+
+// Chunks in flight: as many of the `inner` chunks as keep the group's chunk buffers within this size (twice the L2:
+// beyond it a launch fills the chip many times over and batching gains nothing), in equal parts.
+constexpr size_t kChunkBytes = (size_t)256 << 20;
+int chunk_batch(int inner, int group, size_t bytes_per_chunk) {
+  const long long fit = (long long)(kChunkBytes / std::max<size_t>(1, bytes_per_chunk * group));
+  int nb = (int)std::max(1LL, std::min({fit, (long long)inner, (long long)(kMaxGemmBatch / group)}));
+  const int parts = (inner + nb - 1) / nb;
+  return (inner + parts - 1) / parts;
+}
+
+// planes: 0 = FP64 path, 2 or 3 = tensor-core path with that many 16-bit planes per operand. slices: FP64 products
+// run on digit slices where their shape takes it. group: instances squeezed together; nblk: column blocks of an operand
+// row (3 with tangents).
+StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool slices, int group, int nblk,
+                    int most_chunks = kMaxGemmBatch) {
+  const bool mixed = planes > 0;
+  Geom g = make_geom(d, dims);
+  const long long P = g.P;
+  // operand rows: P rounded up to 64, plus one more 64-column block for the zero-field
+  // (parity-blocked) layout, whose two k classes start at 64-aligned columns
+  const long long ldk = round_up(P, 64) + 64;
+  int chi[kMaxD];
+  int trans[kMaxD], nt = 0;
+  for (int b = 0; b < d; ++b) {
+    chi[b] = dims[b];
+    if (b != a) {
+      const long long sq = (long long)dims[b] * dims[b];
+      chi[b] = (int)(sq < Dcut ? sq : Dcut);
+      trans[nt++] = b;
+    }
+  }
+  const int c3 = nt ? trans[nt - 1] : -1, no = nt ? nt - 1 : 0;
+  const long long chi3 = c3 >= 0 ? chi[c3] : 1;
+  const size_t es = mixed ? 4 : 8;  // intermediate element size (float / double)
+  const bool sl = !mixed && slices && slices_take(P, chi3 * P, ldk);
+  const size_t op = mixed ? 2 * planes : (sl ? 2 * kSliceCount : 8);  // bytes of an operand entry
+  StepNeeds n;
+  n.Tt = (size_t)(P * P) * es;
+  n.Bt = (size_t)(chi3 * P * ldk) * op * nblk;
+  n.X1 = no == 2 ? (size_t)(P * P) * es : 0;
+  n.X2 = no >= 1 ? (size_t)(P * P) * es : 0;
+  n.Y = (size_t)(P * ldk) * op * nblk;
+  n.O = (size_t)(P * output_ld(chi3 * P, sl)) * es;
+  if (sl) {
+    n.O = std::max(n.O, (size_t)(chi3 * P * ldk) * 8);
+    n.yt = (size_t)(P * ldk) * 8;
+    n.ey = (size_t)P * sizeof(int) * nblk;
+    n.eb = (size_t)(chi3 * P) * sizeof(int) * nblk;
+  }
+  // epilogue intermediates: contract the other transverse axes in order
+  long long cur = P * chi3 * P;
+  size_t r[2] = {0, 0};
+  for (int i = 0; i < no && i < 2; ++i) {
+    const int b = trans[i];
+    cur = cur / ((long long)dims[b] * dims[b]) * chi[b];
+    r[i] = (size_t)cur * es;
+  }
+  n.R1 = r[0];
+  n.R2 = r[1];
+  const size_t tangent = nblk > 1 ? n.O + n.X2 + n.R1 + n.R2 : 0;
+  n.nb = no ? std::min(most_chunks,
+                       chunk_batch(chi[trans[no - 1]], group, n.X2 + n.Y + n.O + n.R1 + n.R2 + n.yt + tangent))
+            : 1;
+  if (sl) n.scr = slice_scratch_bytes(P, chi3 * P, group * n.nb);
+  return n;
+}
+
+}  // namespace
+
 struct hotrg_ctx {
   int d = 0, Dcut = 0, batch = 1, precision = HOTRG_FP64, fp64_steps = 2, x6_steps = 0, max_steps = 64;
   int kblock = 64;
@@ -92,17 +227,16 @@ struct hotrg_ctx {
   long long q_stride = 0, g_stride = 0, u_stride = 0;  // per-instance strides (doubles)
   void *Tt = nullptr, *Bt = nullptr, *X1 = nullptr, *X2 = nullptr, *Y = nullptr, *O = nullptr;
   void *R1 = nullptr, *R2 = nullptr;
-  size_t sz_Tt = 0, sz_Bt = 0, sz_X = 0, sz_Y = 0, sz_O = 0, sz_R1 = 0, sz_R2 = 0;
-  // instances squeezed together (one GEMM launch per chunk for all of them): every per-step buffer
-  // holds `group` slots, st_* bytes apart
-  int group = 1;
   // FP64 products on the tensor cores (gemm_f64tc.cu): the Y and Bt buffers then hold digit planes. yt: the A operand
   // in double before slicing (the B operand is built in O, free until the first chunk), ey / eb: row exponents,
   // slice_scratch: level sums of the running launch
   bool slices = true;
   void *yt = nullptr, *ey = nullptr, *eb = nullptr, *slice_scratch = nullptr;
-  size_t sz_yt = 0, sz_ey = 0, sz_eb = 0, sz_scr = 0, st_yt = 0, st_ey = 0, st_eb = 0;
-  size_t st_Tt = 0, st_Bt = 0, st_X = 0, st_Y = 0, st_O = 0, st_R1 = 0, st_R2 = 0, st_Tnext = 0;
+  // instances squeezed together (one GEMM launch per chunk batch for all of them): every per-step buffer holds `group`
+  // times the bytes sz lists
+  int group = 1;
+  StepSizes sz;
+  size_t st_Tnext = 0;
   long long spec_stride = 0;  // doubles per instance in spec_log
   // phase timing (hotrg_timing_start/stop): CUDA events recorded on `stream`
   struct Ev {
@@ -149,90 +283,6 @@ struct PhaseScope {
 
 namespace {
 
-constexpr long long kAlign = 256;
-// shape of the wait probe's GEMM launch: one output tile, one k-block
-constexpr long long TC_PROBE_M = 128, TC_PROBE_N = 256, TC_PROBE_K = 64;
-constexpr int kSpecCap = kMaxGram;  // eigenvalues stored per (step, axis)
-
-long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
-
-// Row stride of a chunk's GEMM output: the slice GEMM stores 32 bytes (four doubles) at a time.
-long long output_ld(long long n, bool slices) { return slices ? round_up(n, 4) : n; }
-
-// Sizes (bytes) of the per-step scratch buffers for one configuration.
-struct StepNeeds {
-  size_t Tt = 0, Bt = 0, X = 0, Y = 0, O = 0, R1 = 0, R2 = 0;
-  size_t yt = 0, ey = 0, eb = 0, scr = 0;  // FP64 products on slices
-};
-
-// Contexts whose workspace would pass this size with the digit planes (twice the bytes of FP64 operands) keep the FP64
-// operands and the FP64 units: what fitted the card before still does.
-constexpr size_t kSliceWorkspaceLimit = (size_t)128 << 30;
-
-// planes: 0 = FP64 path, 2 or 3 = tensor-core path with that many 16-bit planes per operand. slices: FP64 products
-// run on digit slices where their shape takes it, over groups of `group` instances.
-StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool slices, int group) {
-  const bool mixed = planes > 0;
-  Geom g = make_geom(d, dims);
-  const long long P = g.P;
-  // operand rows: P rounded up to 64, plus one more 64-column block for the zero-field
-  // (parity-blocked) layout, whose two k classes start at 64-aligned columns
-  const long long ldk = round_up(P, 64) + 64;
-  int chi[kMaxD];
-  int trans[kMaxD], nt = 0;
-  for (int b = 0; b < d; ++b) {
-    chi[b] = dims[b];
-    if (b != a) {
-      const long long sq = (long long)dims[b] * dims[b];
-      chi[b] = (int)(sq < Dcut ? sq : Dcut);
-      trans[nt++] = b;
-    }
-  }
-  const int c3 = nt ? trans[nt - 1] : -1;
-  const long long chi3 = c3 >= 0 ? chi[c3] : 1;
-  const size_t es = mixed ? 4 : 8;  // intermediate element size (float / double)
-  StepNeeds n;
-  n.Tt = (size_t)(P * P) * es;
-  const bool sl = !mixed && slices && slices_take(P, chi3 * P, ldk);
-  const size_t op = mixed ? 2 * planes : (sl ? 2 * kSliceCount : 8);  // bytes of an operand entry
-  n.Bt = (size_t)(chi3 * P * ldk) * op;
-  n.X = (size_t)(P * P) * es;
-  n.Y = (size_t)(P * ldk) * op;
-  n.O = (size_t)(P * output_ld(chi3 * P, sl)) * es;
-  if (sl) {
-    n.O = std::max(n.O, (size_t)(chi3 * P * ldk) * 8);
-    n.yt = (size_t)(P * ldk) * 8;
-    n.ey = (size_t)P * sizeof(int);
-    n.eb = (size_t)(chi3 * P) * sizeof(int);
-    n.scr = slice_scratch_bytes(P, chi3 * P, group);
-  }
-  // epilogue intermediates: contract the other transverse axes in order
-  long long cur = P * chi3 * P;
-  size_t r[2] = {0, 0};
-  for (int i = 0; i < nt - 1 && i < 2; ++i) {
-    const int b = trans[i];
-    cur = cur / ((long long)dims[b] * dims[b]) * chi[b];
-    r[i] = (size_t)cur * es;
-  }
-  n.R1 = r[0];
-  n.R2 = r[1];
-  return n;
-}
-
-void max_into(StepNeeds& acc, const StepNeeds& n) {
-  acc.Tt = std::max(acc.Tt, n.Tt);
-  acc.Bt = std::max(acc.Bt, n.Bt);
-  acc.X = std::max(acc.X, n.X);
-  acc.Y = std::max(acc.Y, n.Y);
-  acc.O = std::max(acc.O, n.O);
-  acc.R1 = std::max(acc.R1, n.R1);
-  acc.R2 = std::max(acc.R2, n.R2);
-  acc.yt = std::max(acc.yt, n.yt);
-  acc.ey = std::max(acc.ey, n.ey);
-  acc.eb = std::max(acc.eb, n.eb);
-  acc.scr = std::max(acc.scr, n.scr);
-}
-
 // Workspace plan: the per-step buffers must hold every step a context can take. The bond
 // dimensions reachable within max_steps steps (any axis sequence, starting from all 2) are
 // enumerated breadth-first; each D_b is 2, min(4, Dcut) or min(16, Dcut). Path of a step: FP64
@@ -273,8 +323,8 @@ bool f16_planes(int precision, int planes) {
   return planes == 2 && (precision == HOTRG_FP16X3 || precision == HOTRG_FP16X4);
 }
 
-StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int max_steps, bool slices, int group,
-               long long* Pmax_out) {
+StepSizes plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int max_steps, bool slices, int group,
+               int nblk, long long* Pmax_out) {
   // breadth-first: minimal number of steps after which each bond-dimension state is reached
   std::vector<std::vector<int>> states{std::vector<int>(d, 2)};
   std::vector<int> depth{0};
@@ -290,7 +340,7 @@ StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int
       }
     }
   }
-  StepNeeds acc;
+  StepSizes acc;
   long long Pmax = 1;
   for (size_t i = 0; i < states.size(); ++i) {
     long long P = 1;
@@ -301,8 +351,9 @@ StepNeeds plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int
     for (int a = 0; a < d; ++a)
       for (int step : {first, fp64_steps + 1, x6_steps + 1, max_steps})
         if (step >= first && step <= max_steps)
-          max_into(acc, needs_for(d, states[i].data(), a, Dcut,
-                                  planes_for_step(precision, step, fp64_steps, x6_steps, P), slices, group));
+          acc.max_with(StepSizes::of(needs_for(d, states[i].data(), a, Dcut,
+                                               planes_for_step(precision, step, fp64_steps, x6_steps, P), slices, group,
+                                               nblk)));
   }
   *Pmax_out = Pmax;
   return acc;
@@ -319,10 +370,26 @@ struct Carver {
   }
 };
 
+// The needs of a step from bond dimensions `dims` within the context's buffers. The plan holds every step of the Ising flow;
+// a tensor set from outside can have any bond dimensions up to Dcut, whose own best chunk batch or digit planes may need
+// more: then fewer chunks at a time, then FP64 operands on the FP64 units. false: does not fit.
+bool step_needs(const hotrg_ctx* c, const int* dims, int a, int planes, StepNeeds* n) {
+  const int nblk = c->deriv ? 3 : 1;
+  for (int sl = c->slices ? 1 : 0; sl >= 0; --sl)
+    for (int most = kMaxGemmBatch;; most = n->nb - 1) {
+      *n = needs_for(c->d, dims, a, c->Dcut, planes, sl != 0, c->group, nblk, most);
+      if (c->sz.covers(*n)) return true;
+      if (n->nb <= 1) break;
+    }
+  return false;
+}
+
 // Lay out every buffer; with base == nullptr only the total size is computed.
 size_t carve(hotrg_ctx* c, char* base) {
   long long Pmax = 1;
-  StepNeeds n = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, c->slices, c->group, &Pmax);
+  // with tangents the operands hold three column blocks per row (see squeeze)
+  c->sz = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, c->slices, c->group,
+               c->deriv ? 3 : 1, &Pmax);
   c->Pmax = Pmax;
   const long long P2 = Pmax * Pmax;
   const int nr_max = kMaxGram;
@@ -341,8 +408,8 @@ size_t carve(hotrg_ctx* c, char* base) {
   c->cval = k.take<double>(sizeof(double) * c->batch);
   c->status = k.take<int>(sizeof(int) * 32);
   c->dstep = k.take<int>(sizeof(int) * 32);
-  c->amax = k.take<unsigned>(sizeof(unsigned) * 2 * G);
-  c->norm_partial = k.take<double>(sizeof(double) * 1024);
+  c->amax = k.take<unsigned>(sizeof(unsigned) * (G + kMaxGemmBatch));
+  c->norm_partial = k.take<double>(sizeof(double) * 1024 * G);
   // Gram matrices and isometries: sized for the largest Gram this Dcut produces (n <= Dcut^2... 256)
   const int nmax = std::min(kMaxGram, std::max(16, c->Dcut * c->Dcut));
   const int nrm = std::min(kMaxGram, std::max(16, c->Dcut * c->Dcut));
@@ -379,8 +446,8 @@ size_t carve(hotrg_ctx* c, char* base) {
     c->z2rank = k.take<int>(sizeof(int) * Pmax * G);
     c->z2kcol = k.take<int>(sizeof(int) * Pmax * G);
     c->z2colpos = k.take<int>(sizeof(int) * Pmax * kMaxBond * G);
-    c->z2blk = k.take<GemmBlocks>(sizeof(GemmBlocks) * G);  // contiguous: the batched GEMM reads blk[j]
-    c->z2pi = k.take<int>(sizeof(int) * G);
+    c->z2blk = k.take<GemmBlocks>(sizeof(GemmBlocks) * kMaxGemmBatch);  // one per slot in flight
+    c->z2pi = k.take<int>(sizeof(int) * kMaxGemmBatch);
     c->z2flops = k.take<double>(sizeof(double) * 4);
   }
   if (c->impure) {
@@ -388,38 +455,30 @@ size_t carve(hotrg_ctx* c, char* base) {
     c->Stmp = k.take<double>(sizeof(double) * 2 * P2);
     c->imp_out = k.take<double>(sizeof(double) * 2 * c->batch);
   }
-  // with tangents the operands hold three column blocks per row (see squeeze)
-  const size_t blk = c->deriv ? 3 : 1;
-  // per-step buffers: `group` slots of each (slot strides 256-byte aligned: TMA plane starts)
-  auto slots = [&](size_t bytes, size_t& sz, size_t& st) {
-    sz = bytes;
-    st = (size_t)round_up((long long)(bytes ? bytes : 256), kAlign);
-    return k.take<char>(st * G);
-  };
-  size_t st_x2 = 0;
-  c->Tt = slots(n.Tt, c->sz_Tt, c->st_Tt);
-  c->Bt = slots(n.Bt * blk, c->sz_Bt, c->st_Bt);
-  c->X1 = slots(n.X, c->sz_X, c->st_X);
-  c->X2 = slots(n.X, c->sz_X, st_x2);
-  c->Y = slots(n.Y * blk, c->sz_Y, c->st_Y);
-  c->O = slots(n.O, c->sz_O, c->st_O);
-  c->R1 = slots(n.R1, c->sz_R1, c->st_R1);
-  c->R2 = slots(n.R2, c->sz_R2, c->st_R2);
-  if (n.scr) {
-    c->yt = slots(n.yt, c->sz_yt, c->st_yt);
-    c->ey = slots(n.ey * blk, c->sz_ey, c->st_ey);
-    c->eb = slots(n.eb * blk, c->sz_eb, c->st_eb);
-    c->sz_scr = n.scr;
-    c->slice_scratch = k.take<char>(n.scr);
+  // per-step buffers: for every instance of the group
+  const StepSizes& z = c->sz;
+  c->Tt = k.take<char>(z.Tt * G);
+  c->Bt = k.take<char>(z.Bt * G);
+  c->X1 = k.take<char>(z.X1 * G);
+  c->X2 = k.take<char>(z.X2 * G);
+  c->Y = k.take<char>(z.Y * G);
+  c->O = k.take<char>(z.O * G);
+  c->R1 = k.take<char>(z.R1 * G);
+  c->R2 = k.take<char>(z.R2 * G);
+  if (z.scr) {
+    c->yt = k.take<char>(z.yt * G);
+    c->ey = k.take<char>(z.ey * G);
+    c->eb = k.take<char>(z.eb * G);
+    c->slice_scratch = k.take<char>(z.scr);
   }
   if (c->deriv) {
-    c->Tt2 = k.take<char>(n.Tt);
-    c->dX1[0] = k.take<char>(n.X);
-    c->dX1[1] = k.take<char>(n.X);
-    c->dX2 = k.take<char>(n.X);
-    c->dO = k.take<char>(n.O);
-    c->dR1 = k.take<char>(n.R1 ? n.R1 : 256);
-    c->dR2 = k.take<char>(n.R2 ? n.R2 : 256);
+    c->Tt2 = k.take<char>(z.Tt);
+    c->dX1[0] = k.take<char>(z.X1);
+    c->dX1[1] = k.take<char>(z.X1);
+    c->dX2 = k.take<char>(z.X2);
+    c->dO = k.take<char>(z.O);
+    c->dR1 = k.take<char>(z.R1);
+    c->dR2 = k.take<char>(z.R2);
   }
   return k.off;
 }
@@ -546,63 +605,21 @@ Contraction plan_contraction(const std::vector<Ax>& axes, int b, int chi_b, cons
 template <class Tin, class Tout>
 void contract_axes_z2(std::vector<Ax>& axes, const Tin* O, long long ldO, Tout* out, int b, int chi_b,
                       const double* Ub, const long long* final_out_stride, long long out_base,
-                      const Z2Layout* L, const int* pi, cudaStream_t s) {
+                      const Z2Layout* L, const int* pi, const SlotStrides& st, cudaStream_t s) {
   Contraction r = plan_contraction(axes, b, chi_b, final_out_stride);
-  launch_epi_z2<Tin, Tout>(O, ldO, out, r.rest, r.sk, out_base, b, axes[r.im].dim, Ub, chi_b, L, pi, s);
+  launch_epi_z2<Tin, Tout>(O, ldO, out, r.rest, r.sk, out_base, b, axes[r.im].dim, Ub, chi_b, L, pi, st, s);
   axes = r.out_axes;
 }
 
 // With in2 (laid out like in), the same contraction of in2 with U2 is added.
 template <class Tin, class Tout>
 void contract_axes(std::vector<Ax>& axes, const Tin* in, Tout* out, int b, int chi_b, const double* Ub,
-                   const long long* final_out_stride, long long out_base, cudaStream_t s,
+                   const long long* final_out_stride, long long out_base, const SlotStrides& st, cudaStream_t s,
                    const Tin* in2 = nullptr, const double* U2 = nullptr) {
-  int im = -1, in_ = -1;
-  for (int i = 0; i < (int)axes.size(); ++i) {
-    if (axes[i].kind == 0 && axes[i].slot == b) im = i;
-    if (axes[i].kind == 2 && axes[i].slot == b) in_ = i;
-  }
-  std::vector<Ax> out_axes;
-  View v{};
-  int kaxis = -1;
-  for (int i = 0; i < (int)axes.size(); ++i) {
-    if (i == im) continue;
-    Ax ax = axes[i];
-    if (i == in_) {
-      kaxis = v.ndim;
-      ax.dim = chi_b;
-      ax.stride = 0;
-    }
-    v.shape[v.ndim] = ax.dim;
-    v.in_stride[v.ndim] = ax.stride;
-    out_axes.push_back(ax);
-    ++v.ndim;
-  }
-  // output strides
-  long long st = 1;
-  for (int i = v.ndim - 1; i >= 0; --i) {
-    v.out_stride[i] = final_out_stride ? final_out_stride[i] : st;
-    st *= v.shape[i];
-  }
-  // rest view: the output axes without k'
-  View rest;
-  rest.ndim = 0;
-  for (int i = 0; i < v.ndim; ++i) {
-    if (i == kaxis) continue;
-    rest.shape[rest.ndim] = v.shape[i];
-    rest.in_stride[rest.ndim] = v.in_stride[i];
-    rest.out_stride[rest.ndim] = v.out_stride[i];
-    ++rest.ndim;
-  }
-  launch_pair_contract_all<Tin, Tout>(in, out, rest, axes[im].dim, axes[in_].dim, axes[im].stride,
-                                      axes[in_].stride, v.out_stride[kaxis], Ub, chi_b, 0, out_base, s, in2, U2);
-  // new axes describe the dense output (only meaningful when not final)
-  st = 1;
-  for (int i = v.ndim - 1; i >= 0; --i) {
-    out_axes[i].stride = st;
-    st *= out_axes[i].dim;
-  }
-  axes = out_axes;
+  Contraction r = plan_contraction(axes, b, chi_b, final_out_stride);
+  launch_pair_contract_all<Tin, Tout>(in, out, r.rest, axes[r.im].dim, axes[r.in_].dim, axes[r.im].stride,
+                                      axes[r.in_].stride, r.sk, Ub, chi_b, out_base, st, s, in2, U2);
+  axes = r.out_axes;
 }
 
 // Strides of the final output (Tnext in the new geometry) for an axes list.
@@ -657,85 +674,46 @@ struct Tangents {
   const double* dU[2] = {nullptr, nullptr};
 };
 
-// Per-step scratch of one instance of a squeeze group: slot j of every per-step buffer (the plan
-// holds opts.group slots of each).
-struct Slot {
-  void *Tt, *Bt, *X1, *X2, *Y, *O, *R1, *R2;
-  double *Tnext, *yt;
-  int *ey, *eb;
-  unsigned* amax;  // [0] bound of the B operand's source, [1] of the A operand's (fp16 planes)
-  int *z2rank, *z2kcol, *z2colpos, *z2pi;
-  GemmBlocks* z2blk;
-};
-
-Slot slot(const hotrg_ctx* c, int j) {
-  auto at = [j](void* base, size_t stride) -> void* {
-    return base ? static_cast<void*>(static_cast<char*>(base) + stride * (size_t)j) : nullptr;
-  };
-  Slot q;
-  q.Tt = at(c->Tt, c->st_Tt);
-  q.Bt = at(c->Bt, c->st_Bt);
-  q.X1 = at(c->X1, c->st_X);
-  q.X2 = at(c->X2, c->st_X);
-  q.Y = at(c->Y, c->st_Y);
-  q.O = at(c->O, c->st_O);
-  q.R1 = at(c->R1, c->st_R1);
-  q.R2 = at(c->R2, c->st_R2);
-  q.Tnext = static_cast<double*>(at(c->Tnext, c->st_Tnext));
-  q.yt = static_cast<double*>(at(c->yt, c->st_yt));
-  q.ey = static_cast<int*>(at(c->ey, c->st_ey));
-  q.eb = static_cast<int*>(at(c->eb, c->st_eb));
-  q.amax = c->amax + 2 * j;
-  q.z2rank = c->z2rank ? c->z2rank + c->Pmax * j : nullptr;
-  q.z2kcol = c->z2kcol ? c->z2kcol + c->Pmax * j : nullptr;
-  q.z2colpos = c->z2colpos ? c->z2colpos + c->Pmax * kMaxBond * j : nullptr;
-  q.z2pi = c->z2pi ? c->z2pi + j : nullptr;
-  q.z2blk = c->z2blk ? c->z2blk + j : nullptr;
-  return q;
-}
-
-// The instances squeezed together: instance j reads T1[j] (lower site, A operand) and T2[j] (upper
-// site, B operand) with isometries U[j], writes out[j] and works in per-step slot j; inst[j] is its
-// index in the context (zero-field layouts). One GEMM launch per chunk covers all of them.
+// Per-step scratch regions. Per instance j of a squeeze group (strides st_*): Tt, Bt, X1, Tnext, the row exponents of
+// Bt, the zero-field tables. Per slot z = j * (chunks in flight) + chunk, at strides chosen by each step (slot_bytes):
+// X2, Y, O, R1, R2, yt, ey, and the chunk's parity and GEMM blocks.
+// The instances squeezed together: instance j reads T1 + j t_inst (lower site, A operand) and T2 + j t_inst (upper site,
+// B operand) with isometries U + j u_inst and writes out + j out_inst; inst0 + j is its index in the context (zero-field
+// layouts).
 struct Group {
-  int n = 0;
-  std::vector<const double*> T1, T2, U;
-  std::vector<double*> out;
-  std::vector<int> inst;
-  void add(const double* t1, const double* t2, const double* u, double* o, int i) {
-    T1.push_back(t1);
-    T2.push_back(t2);
-    U.push_back(u);
-    out.push_back(o);
-    inst.push_back(i);
-    ++n;
-  }
+  int n = 0, inst0 = 0;
+  const double *T1 = nullptr, *T2 = nullptr, *U = nullptr;
+  double* out = nullptr;
+  long long t_inst = 0, u_inst = 0, out_inst = 0;
 };
-
-bool slices_fit(const hotrg_ctx* c, const StepNeeds& need, int nblk) {
-  return need.yt <= c->sz_yt && need.ey * nblk <= c->sz_ey && need.eb * nblk <= c->sz_eb && need.scr <= c->sz_scr;
-}
 
 // An operand on digit slices: column block `blk` (of ldk columns) of the planes at `base`, its row exponents the
 // blk-th run of `rows` entries of `exps`.
-SliceOperand slice_operand(void* base, long long plane, long long ld, long long ldk, int blk, int* exps, long long rows,
+SliceOperand slice_operand(void* base, long long plane, long long ld, long long ldk, int blk, void* exps, long long rows,
                            size_t inst_bytes, size_t exp_inst_bytes) {
   SliceOperand o;
   o.p = static_cast<__half*>(base) + blk * ldk;
   o.ld = ld;
   o.plane = plane;
   o.inst = (long long)(inst_bytes / sizeof(__half));
-  o.exps = exps + blk * rows;
+  o.exps = static_cast<int*>(exps) + blk * rows;
   o.exp_inst = (long long)(exp_inst_bytes / sizeof(int));
   return o;
 }
 
-// planes: 0 = FP64 path (TC = double), 2 / 3 = tensor-core path (TC = float) with 3 / 6 passes.
-template <class TC>
-// Coarse-grained tensor of the pair (T1 lower site, T2 upper site along a) into `out` (new
-// geometry gn) for every instance of the group: T1 feeds the A operand, T2 the B operand. The
-// small operand and epilogue kernels run instance by instance; the squeeze GEMM of a chunk is one
-// batched launch over the group. With tangents (a group of one, T1 = T2 = T), also
+// Coarse-grained tensor of the pair (T1 lower site, T2 upper site along a) into `out` (new geometry gn) for every
+// instance of the group: T1 feeds the A operand, T2 the B operand. planes: 0 = FP64 path (TC = double), 2 / 3 =
+// tensor-core path (TC = float) with 3 / 6 passes.
+//
+// A chunk fixes the new indices of the transverse axes but the last. The chunks of the inner fixed axis run `nb` at a
+// time (chunk_batch): every kernel launch covers them for all instances of the group, with the GEMM's B operand shared
+// by the chunks of an instance. A step of 25 to 100 small chunks is bound by its launches and by kernels that fill a
+// fraction of the chip (4D, bond dimension 5: 75 GEMM tiles on 152 SMs, 7 launches a chunk).
+//
+// z2: zero-field squeeze of T with itself (z2.cu): parity-blocked operands, two dense GEMM blocks per chunk, the first
+// epilogue contraction reading the blocked output. Same output up to the order of summation.
+//
+// With tangents (a group of one, T1 = T2 = T), also
 //   dT' = S(dT, T) + S(T, dT) + sum over the six places of an isometry of S with dU there,
 // computed as a dual-number pass: every producer and epilogue stage propagates (x, dx), and the
 // O(D^15) contraction of a tangent is one GEMM over the concatenated k range,
@@ -743,462 +721,329 @@ template <class TC>
 // with the operand blocks laid out side by side in one row: Y' = [dY_0 | Y | dY_1] and
 // Bt' = [dBt_1 | Bt | dBt_0] (row stride 3 ldk), so that [dY_0 | Y] pairs with [Bt | dBt_0] and
 // [Y | dY_1] with [dBt_1 | Bt].
+template <class TC>
 int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, const int* chi, const int* trans,
-            int nt, int planes, int npass, const Tangents& tg = Tangents()) {
+            int nt, int planes, int npass, bool z2, const Tangents& tg = Tangents()) {
   using Op = typename Ops<TC>::Op;
   constexpr bool mixed = std::is_same<TC, float>::value;
   cudaStream_t s = c->stream;
   const int ng = G.n;
-  if (ng < 1 || ng > c->group || (tg.n && ng != 1)) return HOTRG_ESTATE;
+  if (ng < 1 || ng > c->group || (tg.n && (ng != 1 || z2)) || (z2 && nt < 1)) return HOTRG_ESTATE;
   const long long P = g.P;
-  const int nblk = tg.n ? 3 : 1;
-  const int fwd_blk = tg.n ? 1 : 0;
   const int c3 = nt ? trans[nt - 1] : -1;
   const int chi3 = c3 >= 0 ? chi[c3] : 1;
   auto Ub = [&](const double* base, int b) { return base + (long long)b * kMaxBond * kMaxGram; };
   // bounds of this step's buffers against the plan
-  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes, c->slices, c->group);
-  if (need.Tt > c->sz_Tt || need.Bt * nblk > c->sz_Bt || need.X > c->sz_X || need.Y * nblk > c->sz_Y ||
-      need.O > c->sz_O || need.R1 > c->sz_R1 || need.R2 > c->sz_R2 || !slices_fit(c, need, nblk))
+  StepNeeds need;
+  if (!step_needs(c, g.D, a, planes, &need) || P > c->Pmax || (tg.n && (!c->Tt2 || !c->dO || tg.n > 2)))
     return HOTRG_ENOMEM;
   const bool sl = need.scr > 0;  // FP64 products on digit slices
-  if (tg.n && (!c->Tt2 || !c->dO || tg.n > 2)) return HOTRG_ESTATE;
-  const long long ldk = mixed || sl ? round_up(P, 64) : P;
-  const long long ld = nblk * ldk;
+  const int blks = tg.n ? 3 : 1;
+  const int fwd_blk = tg.n ? 1 : 0;
+  const long long ldk = z2 ? round_up(P, 64) + 64 : (mixed || sl ? round_up(P, 64) : P);
+  const long long ld = blks * ldk;
   const int nparts = mixed ? planes : 1;
   const long long bt_plane = (long long)chi3 * P * ld, y_plane = P * ld;
+  // slot strides of this step (bytes)
+  const size_t cX = slot_bytes(need.X2), cY = slot_bytes(need.Y), cO = slot_bytes(need.O), cR1 = slot_bytes(need.R1),
+               cR2 = slot_bytes(need.R2), cyt = slot_bytes(need.yt), cey = slot_bytes(need.ey);
+  unsigned* const amaxB = c->amax;
+  unsigned* const amaxA = c->amax + c->group;
   // fp16 planes (FP16 modes; the forward squeeze only, tangents keep bf16): each operand's scale
   // comes from the largest entry of its source, measured on the device. |Bt| <= sqrt(D_c3) max|Tt|
   // (each Bt entry contracts a fibre of D_c3 entries with part of a unit isometry vector); Y's
   // entries are the source's own.
   const bool f16 = mixed && tg.n == 0 && f16_planes(c->precision, planes);
   const float bt_mult = c3 >= 0 ? (float)std::sqrt((double)g.D[c3]) : 1.f;
-  // which: 0 = B operand, 1 = A operand (fp16 scale bound amax[which])
-  auto blocks = [&](void* base, long long plane_elems, int blk, int which = -1, const unsigned* amax = nullptr) {
+  // which: 0 = B operand, 1 = A operand, -1 = a tangent block (no fp16 scale)
+  auto blocks = [&](void* base, long long plane_elems, int blk, int which) {
     Planes<Op> pl;
     pl.nparts = nparts;
     for (int k = 0; k < 3; ++k)
       pl.p[k] = static_cast<Op*>(base) + (size_t)(k < nparts ? k : 0) * plane_elems + blk * ldk;
     if (f16 && which >= 0) {
       pl.fmt = 1;
-      pl.amax = amax + which;
+      pl.amax = which ? amaxA : amaxB;
       pl.amax_mult = which == 0 ? bt_mult : 1.f;
     }
     return pl;
   };
-  // tangent p: A operand block, B operand block written by its build, and the GEMM's first blocks
-  auto dy_blk = [](int p) { return p == 0 ? 0 : 2; };
-  auto dbt_blk = [](int p) { return p == 0 ? 2 : 0; };
-  auto gemm_a_blk = [](int p) { return p == 0 ? 0 : 1; };
-  auto gemm_b_blk = [](int p) { return p == 0 ? 1 : 0; };
-  const Slot S0 = slot(c, 0);
-  auto slice_y = [&](const Slot& S, int blk) {
-    return slice_operand(S.Y, y_plane, ld, ldk, blk, S.ey, P, c->st_Y, c->st_ey);
+  auto slice_y = [&](int blk) { return slice_operand(c->Y, y_plane, ld, ldk, blk, c->ey, P, cY, cey); };
+  auto slice_bt = [&](int blk) {
+    return slice_operand(c->Bt, bt_plane, ld, ldk, blk, c->eb, (long long)chi3 * P, c->sz.Bt, c->sz.eb);
   };
-  auto slice_bt = [&](const Slot& S, int blk) {
-    return slice_operand(S.Bt, bt_plane, ld, ldk, blk, S.eb, (long long)chi3 * P, c->st_Bt, c->st_eb);
-  };
-  // the operands in double before slicing: B in O (free until the first chunk's GEMM), A in yt, rows of P entries
-  auto dense_plane = [&](void* base) {
+  // operands in double before slicing: B in O (free until the first chunk's GEMM), A in yt
+  auto plain = [&](void* base) {
     Planes<Op> q;
     q.nparts = 1;
     for (int k = 0; k < 3; ++k) q.p[k] = static_cast<Op*>(base);
     return q;
   };
-  auto build_bt = [&](const Slot& S, const TC* src, int blk, int which, const double* U, const TC* src2,
-                      const double* U2) {
-    if constexpr (!mixed) {
-      if (sl) {
-        launch_build_bt<TC, Op>(src, dense_plane(S.O), P, g, c3, U, chi3, s, src2, U2);
-        launch_slice_rows(static_cast<double*>(S.O), P, (long long)chi3 * P, P, slice_bt(S, blk), 1, 0, s);
-        return;
-      }
-    }
-    launch_build_bt<TC, Op>(src, blocks(S.Bt, bt_plane, blk, which, S.amax), ld, g, c3, U, chi3, s, src2, U2);
-  };
-  auto build_y = [&](const Slot& S, auto* src, int blk, int which) {
-    using Tin = typename std::remove_const<typename std::remove_pointer<decltype(src)>::type>::type;
-    if constexpr (!mixed) {
-      if (sl) {
-        launch_build_y<Tin, Op>(src, dense_plane(S.yt), P, g, a, s);
-        launch_slice_rows(S.yt, P, P, P, slice_y(S, blk), 1, 0, s);
-        return;
-      }
-    }
-    launch_build_y<Tin, Op>(src, blocks(S.Y, y_plane, blk, which, S.amax), ld, g, a, s);
-  };
+  const long long ldt = z2 ? ldk : P;  // row length of those
+  const Z2Layout* L = z2 ? c->z2L + G.inst0 : nullptr;
+  const Z2Tables tab{c->z2rank, c->z2kcol, c->z2colpos, c->Pmax, c->Pmax * kMaxBond};
+  // tangent p: A operand block, B operand block written by its build, and the GEMM's first blocks
+  auto dy_blk = [](int p) { return p == 0 ? 0 : 2; };
+  auto dbt_blk = [](int p) { return p == 0 ? 2 : 0; };
+  auto gemm_a_blk = [](int p) { return p == 0 ? 0 : 1; };
+  auto gemm_b_blk = [](int p) { return p == 0 ? 1 : 0; };
   // B operand(s), one per instance
   PhaseScope* ops_scope = new PhaseScope(c, PH_OPERANDS);
-  if (tg.n && mixed && ldk != P) {
-    // the concatenated k range runs over the zero padding between blocks
-    cudaMemsetAsync(S0.Bt, 0, sizeof(Op) * nparts * bt_plane, s);
-    cudaMemsetAsync(S0.Y, 0, sizeof(Op) * nparts * y_plane, s);
+  if (z2) {
+    launch_z2_layout(c->z2ev + G.inst0 * kMaxD, c->z2ev_new + G.inst0 * kMaxD, ng, g, c3, chi3, c->z2L + G.inst0, s);
+    launch_z2_tables(L, P, chi3, tab, ng, s);
   }
-  for (int j = 0; j < ng; ++j) {
-    const Slot S = slot(c, j);
-    TC* Tt = static_cast<TC*>(S.Tt);
-    launch_transpose<TC>(G.T2[j], Tt, P, s);
-    if (f16) launch_absmax<TC>(Tt, P, P, P, S.amax + 0, s);
-    build_bt(S, Tt, fwd_blk, 0, c3 >= 0 ? Ub(G.U[j], c3) : nullptr, nullptr, nullptr);
+  // zeros where the GEMM's k-blocks run over columns that hold no entries: between and after the k classes, and the
+  // padding between the blocks of a concatenated k range (slicing writes its own)
+  if ((z2 || (tg.n && mixed && ldk != P)) && !sl) {
+    cudaMemsetAsync(c->Bt, 0, c->sz.Bt * (ng - 1) + sizeof(Op) * nparts * bt_plane, s);
+    cudaMemsetAsync(c->Y, 0, cY * (ng * need.nb - 1) + sizeof(Op) * nparts * y_plane, s);
+  }
+  auto build_bt = [&](const TC* src, int blk, int which, const double* U, const TC* src2, const double* U2) {
+    const long long src_inst = (long long)(c->sz.Tt / sizeof(TC)), bt_inst = (long long)(c->sz.Bt / sizeof(Op));
+    const long long o_inst = sl ? (long long)chi3 * P * ldt : bt_inst;  // sliced: the instances one after the other in O
+    const int at_once = sl ? std::max(1, std::min<int>(ng, (int)(c->sz.O * (size_t)c->group / (sizeof(double) * o_inst)))) : ng;
+    for (int j0 = 0; j0 < ng; j0 += at_once) {
+      const int n = std::min(at_once, ng - j0);
+      Planes<Op> dst = sl ? plain(c->O) : blocks(c->Bt, bt_plane, blk, which);
+      const TC* sj = src + j0 * src_inst;
+      const double* uj = U ? U + j0 * G.u_inst : nullptr;
+      if (z2)
+        launch_build_bt_z2<TC, Op>(sj, src_inst, dst, o_inst, ldk, g, c3, uj, G.u_inst, chi3, tab.from(j0), L + j0, n, s);
+      else
+        launch_build_bt<TC, Op>(sj, src_inst, dst, o_inst, sl ? ldt : ld, g, c3, uj, G.u_inst, chi3, n, s, src2, U2);
+      if constexpr (!mixed) {
+        if (sl) {
+          SliceOperand o = slice_bt(blk);
+          o.p += j0 * o.inst;
+          o.exps += j0 * o.exp_inst;
+          launch_slice_rows(static_cast<double*>(c->O), ldt, (long long)chi3 * P, ldt, o, n, o_inst, s,
+                            z2 ? L + j0 : nullptr, nullptr, 0, 1);
+        }
+      }
+    }
+  };
+  {
+    TC* Tt = static_cast<TC*>(c->Tt);
+    const long long tt_inst = (long long)(c->sz.Tt / sizeof(TC));
+    launch_transpose<TC>(G.T2, G.t_inst, Tt, tt_inst, P, ng, s);
+    if (f16) launch_absmax<TC>(Tt, P, P, P, amaxB, s, ng, tt_inst);
+    build_bt(Tt, fwd_blk, 0, c3 >= 0 ? Ub(G.U, c3) : nullptr, nullptr, nullptr);
   }
   for (int p = 0; p < tg.n; ++p) {
     TC* dTt = static_cast<TC*>(c->Tt2);
-    launch_transpose<TC>(tg.dT[p], dTt, P, s);
+    launch_transpose<TC>(tg.dT[p], 0, dTt, 0, P, 1, s);
     const bool two = tg.dU[p] && c3 >= 0;
-    build_bt(S0, dTt, dbt_blk(p), -1, c3 >= 0 ? Ub(G.U[0], c3) : nullptr, two ? static_cast<TC*>(S0.Tt) : nullptr,
+    build_bt(dTt, dbt_blk(p), -1, c3 >= 0 ? Ub(G.U, c3) : nullptr, two ? static_cast<TC*>(c->Tt) : nullptr,
              two ? Ub(tg.dU[p], c3) : nullptr);
   }
   delete ops_scope;
-  TC* O = static_cast<TC*>(S0.O);
+  TC* O = static_cast<TC*>(c->O);
   TC* dO = static_cast<TC*>(c->dO);
   const long long N = (long long)chi3 * P, ldO = output_ld(N, sl);
-  // chunks over the other transverse axes
+  const long long o_slot = (long long)(cO / sizeof(TC)), x_slot = (long long)(cX / sizeof(TC));
+  // chunks: outer fixed axis (4D only) one at a time, inner fixed axis nb at a time
   const int no = nt > 0 ? nt - 1 : 0;
-  int kcnt[kMaxD] = {0, 0, 0, 0};
-  long long nchunks = 1;
-  for (int i = 0; i < no; ++i) nchunks *= chi[trans[i]];
-  int prev_k0 = -1;
-  // instance j's operand planes and output are slot j's: one launch for the group
-  GemmBatch bat;
-  bat.batch = ng;
-  bat.a_inst = (long long)(c->st_Y / sizeof(Op));
-  bat.b_inst = (long long)(c->st_Bt / sizeof(Op));
-  bat.c_inst = (long long)(c->st_O / sizeof(TC));
-  bat.amax_inst = 2;
-  const GemmBatch* batp = ng > 1 ? &bat : nullptr;
-  auto gemm = [&](int ablk, int bblk, TC* C, long long K) -> int {
-    PhaseScope gemm_scope(c, PH_GEMM);
-    if constexpr (mixed) {
-      const int rc = launch_gemm_split(blocks(S0.Y, y_plane, ablk, 1, S0.amax), ld,
-                                       blocks(S0.Bt, bt_plane, bblk, 0, S0.amax), ld, reinterpret_cast<float*>(C),
-                                       ldO, P, N, K, npass, c->status, c->timeout_s, s, c->kblock, c->group_m,
-                                       fold_group_for(c, npass), nullptr, batp, false, c->cta_group);
-      if (rc) return rc;
-      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * npass * ng;
-    } else if (sl) {
-      // the concatenated k range of a tangent runs as two products: the row exponents belong to one block each
-      for (int h = 0; h < (K > P ? 2 : 1); ++h) {
-        const int rc = launch_gemm_slices(slice_y(S0, ablk + h), slice_bt(S0, bblk + h), reinterpret_cast<double*>(C),
-                                          ldO, P, N, P, static_cast<int*>(c->slice_scratch), c->status, c->timeout_s, s,
-                                          nullptr, batp, h == 1);
-        if (rc) return rc;
-      }
-      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * kSliceProducts * ng;
-    } else {
-      launch_gemm_f64(blocks(S0.Y, y_plane, ablk).p[0], ld, blocks(S0.Bt, bt_plane, bblk).p[0], ld, C, ldO, P, N,
-                      K, s, nullptr, batp);
-      if (c->timing) c->t_gemm_tflops += 2.0 * P * (double)N * K * ng;
-    }
-    if (c->timing) {
-      c->t_gemm_flops += 2.0 * P * (double)N * K * ng;
-      ++c->t_gemm_launches;
-    }
-    return HOTRG_OK;
-  };
-  for (long long ch = 0; ch < nchunks; ++ch) {
-    long long r = ch;
-    for (int i = no - 1; i >= 0; --i) {
-      kcnt[i] = (int)(r % chi[trans[i]]);
-      r /= chi[trans[i]];
-    }
-    // producer: mode products on the unprimed legs of the other transverse axes
-    ops_scope = new PhaseScope(c, PH_OPERANDS);
-    for (int j = 0; j < ng; ++j) {
-      const Slot S = slot(c, j);
-      const double* T1 = G.T1[j];
-      const double* U = G.U[j];
+  const int outer = no == 2 ? chi[trans[0]] : 1;
+  const int inner_axis = no ? trans[no - 1] : -1;
+  const int inner = no ? chi[inner_axis] : 1;
+  const long long x1_inst = (long long)(c->sz.X1 / sizeof(TC));
+  for (int k0 = 0; k0 < outer; ++k0)
+    for (int kb = 0; kb < inner; kb += need.nb) {
+      const int nb = std::min(need.nb, inner - kb), nz = ng * nb;
+      // producer: mode products on the unprimed legs of the other transverse axes, then the A operand
+      ops_scope = new PhaseScope(c, PH_OPERANDS);
+      if (z2)
+        launch_z2_chunk(L, c->z2ev_new + G.inst0 * kMaxD, ng, nb, no, no > 0 ? trans[0] : 0, no == 2 ? k0 : kb,
+                        no > 1 ? trans[1] : 0, kb, N, c->z2blk, c->z2pi, c->z2flops,
+                        mixed ? npass : (sl ? kSliceProducts : 1), s);
+      // A operand column block blk of every slot from src (slots src_slot apart)
+      auto build_y = [&](auto* src, long long src_slot, int blk, int which) {
+        using Tin = typename std::remove_const<typename std::remove_pointer<decltype(src)>::type>::type;
+        const Planes<Op> dst = sl ? plain(c->yt) : blocks(c->Y, y_plane, blk, which);
+        const long long dst_slot = (long long)((sl ? cyt : cY) / sizeof(Op));
+        if (z2)
+          launch_build_y_z2<Tin, Op>(src, src_slot, dst, dst_slot, ldk, g, a, tab, L, c->z2pi, ng, nb, s);
+        else
+          launch_build_y<Tin, Op>(src, src_slot, dst, dst_slot, sl ? ldt : ld, g, a, nz, s);
+        if constexpr (!mixed) {
+          if (sl)
+            launch_slice_rows(static_cast<double*>(c->yt), ldt, P, ldt, slice_y(blk), nz, dst_slot, s, L, c->z2pi, 1, nb);
+        }
+      };
       if (no == 0) {
-        if (f16) launch_absmax<double>(T1, P, P, P, S.amax + 1, s);
-        build_y(S, T1, fwd_blk, 1);
-        for (int p = 0; p < tg.n; ++p) build_y(S, tg.dT[p], dy_blk(p), -1);
+        if (f16) launch_absmax<double>(G.T1, P, P, P, amaxA, s, ng, G.t_inst);
+        build_y(G.T1, G.t_inst, fwd_blk, 1);
+        for (int p = 0; p < tg.n; ++p) build_y(tg.dT[p], 0, dy_blk(p), -1);
       } else {
-        TC* X1 = static_cast<TC*>(S.X1);
-        TC* X2 = static_cast<TC*>(S.X2);
-        const int b0 = trans[0];
         // the mode product that writes X also measures max |X|, the fp16 scale bound of Y
-        if (kcnt[0] != prev_k0) {
-          launch_mode_unprimed<double, TC>(T1, X1, g, b0, Ub(U, b0), kcnt[0], s, nullptr, nullptr,
-                                           (f16 && no == 1) ? S.amax + 1 : nullptr);
-          for (int p = 0; p < tg.n; ++p)
-            launch_mode_unprimed<double, TC>(tg.dT[p], static_cast<TC*>(c->dX1[p]), g, b0, Ub(U, b0), kcnt[0], s,
-                                             tg.dU[p] ? T1 : nullptr, tg.dU[p] ? Ub(tg.dU[p], b0) : nullptr);
+        TC *X1 = static_cast<TC*>(c->X1), *X2 = static_cast<TC*>(c->X2);
+        unsigned* bound = f16 ? amaxA : nullptr;
+        const double* Ui = Ub(G.U, inner_axis);
+        if (no == 2) {
+          if (kb == 0)
+            launch_mode_unprimed<double, TC>(G.T1, G.t_inst, X1, x1_inst, g, trans[0], Ub(G.U, trans[0]), G.u_inst, k0,
+                                             ng, 1, s);
+          launch_mode_unprimed<TC, TC>(X1, x1_inst, X2, x_slot, g, inner_axis, Ui, G.u_inst, kb, ng, nb, s, nullptr,
+                                       nullptr, bound);
+        } else {
+          launch_mode_unprimed<double, TC>(G.T1, G.t_inst, X2, x_slot, g, inner_axis, Ui, G.u_inst, kb, ng, nb, s,
+                                           nullptr, nullptr, bound);
         }
-        const TC* X = X1;
-        if (no >= 2) {
-          launch_mode_unprimed<TC, TC>(X1, X2, g, trans[1], Ub(U, trans[1]), kcnt[1], s, nullptr, nullptr,
-                                       f16 ? S.amax + 1 : nullptr);
-          X = X2;
-        }
-        build_y(S, X, fwd_blk, 1);
+        build_y(X2, x_slot, fwd_blk, 1);
         for (int p = 0; p < tg.n; ++p) {
-          const TC* dX = static_cast<TC*>(c->dX1[p]);
-          if (no >= 2) {
-            TC* dX2 = static_cast<TC*>(c->dX2);
-            launch_mode_unprimed<TC, TC>(dX, dX2, g, trans[1], Ub(U, trans[1]), kcnt[1], s,
-                                         tg.dU[p] ? X1 : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[1]) : nullptr);
-            dX = dX2;
+          TC *dX1 = static_cast<TC*>(c->dX1[p]), *dX2 = static_cast<TC*>(c->dX2);
+          const double* dUi = tg.dU[p] ? Ub(tg.dU[p], inner_axis) : nullptr;
+          if (no == 2) {
+            if (kb == 0)
+              launch_mode_unprimed<double, TC>(tg.dT[p], 0, dX1, 0, g, trans[0], Ub(G.U, trans[0]), 0, k0, 1, 1, s,
+                                               tg.dU[p] ? G.T1 : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[0]) : nullptr);
+            launch_mode_unprimed<TC, TC>(dX1, 0, dX2, x_slot, g, inner_axis, Ui, 0, kb, 1, nb, s, dUi ? X1 : nullptr,
+                                         dUi);
+          } else {
+            launch_mode_unprimed<double, TC>(tg.dT[p], 0, dX2, x_slot, g, inner_axis, Ui, 0, kb, 1, nb, s,
+                                             dUi ? G.T1 : nullptr, dUi);
           }
-          build_y(S, dX, dy_blk(p), -1);
+          build_y(dX2, x_slot, dy_blk(p), -1);
         }
       }
-    }
-    if (no > 0) prev_k0 = kcnt[0];
-    delete ops_scope;
-    // the O(D^15) GEMM, all instances of the group in one launch
-    {
-      const int rc = gemm(fwd_blk, fwd_blk, O, P);
-      if (rc) return rc;
-      c->last_gemm.M = P;
-      c->last_gemm.N = N;
-      c->last_gemm.K = P;
-      c->last_gemm.ldk = ld;
-      c->last_gemm.npass = npass;
-      c->last_gemm.nparts = planes;
-      c->last_gemm.fmt = f16 ? 1 : 0;
-      c->last_gemm.mult_b = bt_mult;
-      c->last_gemm.blk = nullptr;
-    }
-    // epilogue: O axes [m_0..m_{d-1}, j, n_0..n_{d-1}]
-    std::vector<Ax> hist[kMaxD];  // axes of the input of each contraction of the chain
-    TC* dbufs[2] = {static_cast<TC*>(c->dR1), static_cast<TC*>(c->dR2)};
-    long long out_base = 0;
-    for (int i = 0; i < no; ++i) out_base += (long long)kcnt[i] * gn.Sn[trans[i]] * gn.P;
-    {
-      PhaseScope epi_scope(c, PH_EPILOGUE);
-      for (int j = 0; j < ng; ++j) {
-        const Slot S = slot(c, j);
-        TC* bufs[2] = {static_cast<TC*>(S.R1), static_cast<TC*>(S.R2)};
+      delete ops_scope;
+      // the O(D^15) GEMM, all slots in one launch
+      GemmBatch bat;
+      bat.batch = nz;
+      bat.b_div = nb;
+      bat.a_inst = (long long)(cY / sizeof(Op));
+      bat.b_inst = (long long)(c->sz.Bt / sizeof(Op));
+      bat.c_inst = o_slot;
+      const GemmBatch* batp = nz > 1 ? &bat : nullptr;
+      const GemmBlocks* blk = z2 ? c->z2blk : nullptr;
+      auto gemm = [&](int ablk, int bblk, TC* C, long long K) -> int {
+        PhaseScope gemm_scope(c, PH_GEMM);
+        double tensor = 1.0;
+        if constexpr (mixed) {
+          const int rc = launch_gemm_split(blocks(c->Y, y_plane, ablk, 1), ld, blocks(c->Bt, bt_plane, bblk, 0), ld,
+                                           reinterpret_cast<float*>(C), ldO, P, N, K, npass, c->status, c->timeout_s, s,
+                                           c->kblock, c->group_m, fold_group_for(c, npass), blk, batp, false,
+                                           c->cta_group);
+          if (rc) return rc;
+          tensor = npass;
+        } else if (sl) {
+          // the concatenated k range of a tangent runs as two products: the row exponents belong to one block each
+          for (int h = 0; h < (K > ldk ? 2 : 1); ++h) {
+            const int rc = launch_gemm_slices(slice_y(ablk + h), slice_bt(bblk + h), reinterpret_cast<double*>(C), ldO, P,
+                                              N, z2 ? ldk : P, static_cast<int*>(c->slice_scratch), c->status,
+                                              c->timeout_s, s, blk, batp, h == 1);
+            if (rc) return rc;
+          }
+          tensor = kSliceProducts;
+        } else {
+          launch_gemm_f64(blocks(c->Y, y_plane, ablk, 1).p[0], ld, blocks(c->Bt, bt_plane, bblk, 0).p[0], ld,
+                          reinterpret_cast<double*>(C), ldO, P, N, K, s, blk, batp);
+        }
+        if (c->timing) {
+          ++c->t_gemm_launches;
+          if (z2) {
+            c->t_z2 = true;  // the blocks' flops are counted on the device (k_z2_chunk)
+          } else {
+            const double f = 2.0 * P * (double)N * K * nz;
+            c->t_gemm_flops += f;
+            c->t_gemm_tflops += f * tensor;
+          }
+        }
+        return HOTRG_OK;
+      };
+      {
+        const int rc = gemm(fwd_blk, fwd_blk, O, z2 ? ldk : P);
+        if (rc) return rc;
+        if (mixed) {  // what the autotuner replays: slot 0's operands (and block descriptor)
+          c->last_gemm.M = P;
+          c->last_gemm.N = N;
+          c->last_gemm.K = z2 ? ldk : P;
+          c->last_gemm.ldk = ld;
+          c->last_gemm.npass = npass;
+          c->last_gemm.nparts = planes;
+          c->last_gemm.fmt = f16 ? 1 : 0;
+          c->last_gemm.mult_b = bt_mult;
+          c->last_gemm.blk = blk;
+        } else if (!z2) {
+          c->last_gemm.npass = 0;
+        }
+      }
+      // epilogue: O axes [m_0..m_{d-1}, j, n_0..n_{d-1}]
+      long long out_base = 0;
+      if (no == 2) out_base += (long long)k0 * gn.Sn[trans[0]] * gn.P;
+      if (no >= 1) out_base += (long long)kb * gn.Sn[inner_axis] * gn.P;
+      const long long out_chunk = no ? gn.Sn[inner_axis] * gn.P : 0;
+      std::vector<Ax> hist[kMaxD];  // axes of the input of each contraction of the chain
+      const long long r_slot[2] = {(long long)(cR1 / sizeof(TC)), (long long)(cR2 / sizeof(TC))};
+      TC* bufs[2] = {static_cast<TC*>(c->R1), static_cast<TC*>(c->R2)};
+      {
+        PhaseScope epi_scope(c, PH_EPILOGUE);
         std::vector<Ax> axes;
         for (int b = 0; b < c->d; ++b) axes.push_back({g.D[b], g.Sn[b] * ldO, 0, b});
         axes.push_back({chi3, P, 1, -1});
         for (int b = 0; b < c->d; ++b) axes.push_back({g.D[b], g.Sn[b], 2, b});
-        const TC* cur = static_cast<TC*>(S.O);
+        const TC* cur = O;
+        SlotStrides st{ng, nb, o_slot, 0, 0, G.u_inst};
+        long long fs[kMaxAxes];
         for (int i = 0; i < no; ++i) {
           hist[i] = axes;
-          contract_axes<TC, TC>(axes, cur, bufs[i], trans[i], chi[trans[i]], Ub(G.U[j], trans[i]), nullptr, 0, s);
+          st.out_inst = r_slot[i] * nb;
+          st.out_chunk = r_slot[i];
+          if (z2 && i == 0)
+            contract_axes_z2<TC, TC>(axes, cur, ldO, bufs[i], trans[i], chi[trans[i]], Ub(G.U, trans[i]), nullptr, 0, L,
+                                     c->z2pi, st, s);
+          else
+            contract_axes<TC, TC>(axes, cur, bufs[i], trans[i], chi[trans[i]], Ub(G.U, trans[i]), nullptr, 0, st, s);
           cur = bufs[i];
+          st.in_slot = r_slot[i];
         }
         hist[no] = axes;
-        long long fs[kMaxAxes];
+        st.out_inst = G.out_inst;
+        st.out_chunk = out_chunk;
         if (c3 >= 0) {
           // final axes after contracting c3 (m_c3 removed, n_c3 -> k'_c3)
           final_strides(axes, c3, c3, gn, c3, fs);
-          contract_axes<TC, double>(axes, cur, G.out[j], c3, chi3, Ub(G.U[j], c3), fs, out_base, s);
+          if (z2 && no == 0)
+            contract_axes_z2<TC, double>(axes, cur, ldO, G.out, c3, chi3, Ub(G.U, c3), fs, out_base, L, c->z2pi, st, s);
+          else
+            contract_axes<TC, double>(axes, cur, G.out, c3, chi3, Ub(G.U, c3), fs, out_base, st, s);
         } else {
-          copy_final<TC>(axes, cur, G.out[j], gn, s);
+          for (int j = 0; j < ng; ++j)
+            copy_final<TC>(axes, cur + j * o_slot, G.out + j * G.out_inst, gn, s);
+        }
+      }
+      // tangents (a group of one): dO by one GEMM over the concatenated k range, then the epilogue
+      // chain in dual numbers (dR' = C_U(dR) + C_dU(R))
+      TC* dbufs[2] = {static_cast<TC*>(c->dR1), static_cast<TC*>(c->dR2)};
+      for (int p = 0; p < tg.n; ++p) {
+        const int rc = gemm(gemm_a_blk(p), gemm_b_blk(p), dO, ldk + P);
+        if (rc) return rc;
+        PhaseScope epi_scope(c, PH_EPILOGUE);
+        const TC* cur = dO;
+        const TC* curF = O;
+        SlotStrides st{1, nb, o_slot, 0, 0, 0};
+        for (int i = 0; i < no; ++i) {
+          std::vector<Ax> ax = hist[i];
+          st.out_chunk = r_slot[i];
+          contract_axes<TC, TC>(ax, cur, dbufs[i], trans[i], chi[trans[i]], Ub(G.U, trans[i]), nullptr, 0, st, s,
+                                tg.dU[p] ? curF : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[i]) : nullptr);
+          cur = dbufs[i];
+          curF = bufs[i];
+          st.in_slot = r_slot[i];
+        }
+        std::vector<Ax> ax = hist[no];
+        long long fs[kMaxAxes];
+        st.out_chunk = out_chunk;
+        if (c3 >= 0) {
+          final_strides(ax, c3, c3, gn, c3, fs);
+          contract_axes<TC, double>(ax, cur, tg.dout[p], c3, chi3, Ub(G.U, c3), fs, out_base, st, s,
+                                    tg.dU[p] ? curF : nullptr, tg.dU[p] ? Ub(tg.dU[p], c3) : nullptr);
+        } else {
+          copy_final<TC>(ax, cur, tg.dout[p], gn, s);
         }
       }
     }
-    // tangents (a group of one): dO by one GEMM over the concatenated k range, then the epilogue
-    // chain in dual numbers (dR' = C_U(dR) + C_dU(R))
-    for (int p = 0; p < tg.n; ++p) {
-      const int rc = gemm(gemm_a_blk(p), gemm_b_blk(p), dO, ldk + P);
-      if (rc) return rc;
-      PhaseScope epi_scope(c, PH_EPILOGUE);
-      const double* U = G.U[0];
-      TC* bufs[2] = {static_cast<TC*>(S0.R1), static_cast<TC*>(S0.R2)};
-      const TC* cur = dO;
-      const TC* curF = O;
-      for (int i = 0; i < no; ++i) {
-        std::vector<Ax> ax = hist[i];
-        contract_axes<TC, TC>(ax, cur, dbufs[i], trans[i], chi[trans[i]], Ub(U, trans[i]), nullptr, 0, s,
-                              tg.dU[p] ? curF : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[i]) : nullptr);
-        cur = dbufs[i];
-        curF = bufs[i];
-      }
-      std::vector<Ax> ax = hist[no];
-      long long fs[kMaxAxes];
-      if (c3 >= 0) {
-        final_strides(ax, c3, c3, gn, c3, fs);
-        contract_axes<TC, double>(ax, cur, tg.dout[p], c3, chi3, Ub(U, c3), fs, out_base, s,
-                                  tg.dU[p] ? curF : nullptr, tg.dU[p] ? Ub(tg.dU[p], c3) : nullptr);
-      } else {
-        copy_final<TC>(ax, cur, tg.dout[p], gn, s);
-      }
-    }
-  }
-  return HOTRG_OK;
-}
-
-// The zero-field squeeze of T with itself (z2.cu) for every instance of the group: parity-blocked
-// operands, two dense GEMM blocks per chunk and instance (one batched launch over the group, each
-// instance with its own block descriptor), the first epilogue contraction reading the blocked
-// output. TC = float: the tensor-core path (bf16 or fp16 planes, npass split products); TC = double:
-// the FP64 path. Same output as squeeze<TC> up to the order of summation.
-template <class TC>
-int squeeze_z2(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, const int* chi, const int* trans,
-               int nt, int planes, int npass) {
-  using Op = typename Ops<TC>::Op;
-  constexpr bool mixed = std::is_same<TC, float>::value;
-  cudaStream_t s = c->stream;
-  const int ng = G.n;
-  if (ng < 1 || ng > c->group) return HOTRG_ESTATE;
-  const long long P = g.P;
-  const long long ldz = round_up(P, 64) + 64;
-  const int c3 = trans[nt - 1];
-  const int chi3 = chi[c3];
-  auto Ub = [&](int j, int b) { return G.U[j] + (long long)b * kMaxBond * kMaxGram; };
-  StepNeeds need = needs_for(c->d, g.D, a, c->Dcut, planes, c->slices, c->group);
-  if (need.Tt > c->sz_Tt || need.Bt > c->sz_Bt || need.X > c->sz_X || need.Y > c->sz_Y || need.O > c->sz_O ||
-      need.R1 > c->sz_R1 || need.R2 > c->sz_R2 || P > c->Pmax || !slices_fit(c, need, 1))
-    return HOTRG_ENOMEM;
-  const bool sl = need.scr > 0;  // FP64 products on digit slices
-  const int nparts = mixed ? planes : 1;
-  const long long bt_plane = (long long)chi3 * P * ldz, y_plane = P * ldz;
-  // fp16 planes in the FP16 modes, with the scale bounds of squeeze<TC> (B: sqrt(D_c3) max|Tt|)
-  const bool f16 = mixed && f16_planes(c->precision, planes);
-  const float bt_mult = (float)std::sqrt((double)g.D[c3]);
-  auto pl = [&](void* base, long long plane_elems, int which, const unsigned* amax) {  // which: 0 = B, 1 = A
-    Planes<Op> q;
-    q.nparts = nparts;
-    for (int k = 0; k < 3; ++k) q.p[k] = static_cast<Op*>(base) + (size_t)(k < nparts ? k : 0) * plane_elems;
-    if (f16) {
-      q.fmt = 1;
-      q.amax = amax + which;
-      q.amax_mult = which == 0 ? bt_mult : 1.f;
-    }
-    return q;
-  };
-  const long long N = (long long)chi3 * P, ldO = output_ld(N, sl);
-  const Slot S0 = slot(c, 0);
-  auto slice_y = [&](const Slot& S) {
-    return slice_operand(S.Y, y_plane, ldz, ldz, 0, S.ey, P, c->st_Y, c->st_ey);
-  };
-  auto slice_bt = [&](const Slot& S) {
-    return slice_operand(S.Bt, bt_plane, ldz, ldz, 0, S.eb, (long long)chi3 * P, c->st_Bt, c->st_eb);
-  };
-  PhaseScope* ops_scope = new PhaseScope(c, PH_OPERANDS);
-  for (int j = 0; j < ng; ++j) {
-    const Slot S = slot(c, j);
-    const int inst = G.inst[j];
-    Z2Layout* L = c->z2L + inst;
-    launch_z2_layout(c->z2ev + inst * kMaxD, c->z2ev_new + inst * kMaxD, 1, g, c3, chi3, L, s);
-    launch_z2_tables(L, P, chi3, S.z2rank, S.z2kcol, S.z2colpos, s);
-    // zeros between and after the k classes (the GEMM's k-blocks run over them; slicing writes its own)
-    if (!sl) {
-      cudaMemsetAsync(S.Bt, 0, sizeof(Op) * nparts * bt_plane, s);
-      cudaMemsetAsync(S.Y, 0, sizeof(Op) * nparts * y_plane, s);
-    }
-    TC* Tt = static_cast<TC*>(S.Tt);
-    launch_transpose<TC>(G.T2[j], Tt, P, s);
-    if (f16) launch_absmax<TC>(Tt, P, P, P, S.amax + 0, s);
-    launch_build_bt_z2<TC, Op>(Tt, pl(sl ? S.O : S.Bt, bt_plane, 0, S.amax), ldz, g, c3, Ub(j, c3), chi3, S.z2rank,
-                               S.z2kcol, S.z2colpos, L, s);
-    if (sl)
-      launch_slice_rows(static_cast<double*>(S.O), ldz, (long long)chi3 * P, ldz, slice_bt(S), 1, 0, s, L, S.z2pi, 0);
-  }
-  delete ops_scope;
-  const int no = nt - 1;
-  int kcnt[kMaxD] = {0, 0, 0, 0};
-  long long nchunks = 1;
-  for (int i = 0; i < no; ++i) nchunks *= chi[trans[i]];
-  int prev_k0 = -1;
-  GemmBatch bat;
-  bat.batch = ng;
-  bat.a_inst = (long long)(c->st_Y / sizeof(Op));
-  bat.b_inst = (long long)(c->st_Bt / sizeof(Op));
-  bat.c_inst = (long long)(c->st_O / sizeof(TC));
-  bat.amax_inst = 2;
-  const GemmBatch* batp = ng > 1 ? &bat : nullptr;
-  for (long long ch = 0; ch < nchunks; ++ch) {
-    long long r = ch;
-    for (int i = no - 1; i >= 0; --i) {
-      kcnt[i] = (int)(r % chi[trans[i]]);
-      r /= chi[trans[i]];
-    }
-    ops_scope = new PhaseScope(c, PH_OPERANDS);
-    for (int j = 0; j < ng; ++j) {
-      const Slot S = slot(c, j);
-      const int inst = G.inst[j];
-      const Z2Layout* L = c->z2L + inst;
-      launch_z2_chunk(L, c->z2ev_new + inst * kMaxD, no, no > 0 ? trans[0] : 0, kcnt[0], no > 1 ? trans[1] : 0,
-                      kcnt[1], N, S.z2blk, S.z2pi, c->z2flops, mixed ? npass : (sl ? kSliceProducts : 1), s);
-      if (no == 0) {
-        if (f16) launch_absmax<double>(G.T1[j], P, P, P, S.amax + 1, s);
-        launch_build_y_z2<double, Op>(G.T1[j], pl(sl ? S.yt : S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol,
-                                      L, S.z2pi, s);
-      } else {
-        TC* X1 = static_cast<TC*>(S.X1);
-        TC* X2 = static_cast<TC*>(S.X2);
-        // the mode product that writes X also measures max |X|, the fp16 scale bound of Y
-        if (kcnt[0] != prev_k0)
-          launch_mode_unprimed<double, TC>(G.T1[j], X1, g, trans[0], Ub(j, trans[0]), kcnt[0], s, nullptr, nullptr,
-                                           (f16 && no == 1) ? S.amax + 1 : nullptr);
-        const TC* X = X1;
-        if (no >= 2) {
-          launch_mode_unprimed<TC, TC>(X1, X2, g, trans[1], Ub(j, trans[1]), kcnt[1], s, nullptr, nullptr,
-                                       f16 ? S.amax + 1 : nullptr);
-          X = X2;
-        }
-        launch_build_y_z2<TC, Op>(X, pl(sl ? S.yt : S.Y, y_plane, 1, S.amax), ldz, g, a, S.z2rank, S.z2kcol, L, S.z2pi,
-                                  s);
-      }
-      if (sl) launch_slice_rows(S.yt, ldz, P, ldz, slice_y(S), 1, 0, s, L, S.z2pi, 1);
-    }
-    if (no > 0) prev_k0 = kcnt[0];
-    delete ops_scope;
-    {
-      PhaseScope gemm_scope(c, PH_GEMM);
-      if constexpr (mixed) {
-        const int rc = launch_gemm_split(pl(S0.Y, y_plane, 1, S0.amax), ldz, pl(S0.Bt, bt_plane, 0, S0.amax), ldz,
-                                         static_cast<float*>(S0.O), ldO, P, N, ldz, npass, c->status, c->timeout_s,
-                                         s, c->kblock, c->group_m, fold_group_for(c, npass), S0.z2blk, batp, false,
-                                         c->cta_group);
-        if (rc) return rc;
-        // what the autotuner replays: slot 0's operands and block descriptor of this chunk
-        c->last_gemm.M = P;
-        c->last_gemm.N = N;
-        c->last_gemm.K = ldz;
-        c->last_gemm.ldk = ldz;
-        c->last_gemm.npass = npass;
-        c->last_gemm.nparts = planes;
-        c->last_gemm.fmt = f16 ? 1 : 0;
-        c->last_gemm.mult_b = bt_mult;
-        c->last_gemm.blk = S0.z2blk;
-      } else if (sl) {
-        const int rc = launch_gemm_slices(slice_y(S0), slice_bt(S0), static_cast<double*>(S0.O), ldO, P, N, ldz,
-                                          static_cast<int*>(c->slice_scratch), c->status, c->timeout_s, s, S0.z2blk,
-                                          batp);
-        if (rc) return rc;
-      } else {
-        launch_gemm_f64(pl(S0.Y, y_plane, 1, S0.amax).p[0], ldz, pl(S0.Bt, bt_plane, 0, S0.amax).p[0], ldz,
-                        static_cast<double*>(S0.O), ldO, P, N, ldz, s, S0.z2blk, batp);
-      }
-      // the blocks' flops are counted on the device (k_z2_chunk)
-      if (c->timing) {
-        ++c->t_gemm_launches;
-        c->t_z2 = true;
-      }
-    }
-    PhaseScope epi_scope(c, PH_EPILOGUE);
-    long long out_base = 0;
-    for (int i = 0; i < no; ++i) out_base += (long long)kcnt[i] * gn.Sn[trans[i]] * gn.P;
-    for (int j = 0; j < ng; ++j) {
-      const Slot S = slot(c, j);
-      const Z2Layout* L = c->z2L + G.inst[j];
-      const TC* O = static_cast<TC*>(S.O);
-      std::vector<Ax> axes;
-      for (int b = 0; b < c->d; ++b) axes.push_back({g.D[b], g.Sn[b] * ldO, 0, b});
-      axes.push_back({chi3, P, 1, -1});
-      for (int b = 0; b < c->d; ++b) axes.push_back({g.D[b], g.Sn[b], 2, b});
-      TC* bufs[2] = {static_cast<TC*>(S.R1), static_cast<TC*>(S.R2)};
-      long long fs[kMaxAxes];
-      if (no == 0) {
-        final_strides(axes, c3, c3, gn, c3, fs);
-        contract_axes_z2<TC, double>(axes, O, ldO, G.out[j], c3, chi3, Ub(j, c3), fs, out_base, L, S.z2pi, s);
-        continue;
-      }
-      contract_axes_z2<TC, TC>(axes, O, ldO, bufs[0], trans[0], chi[trans[0]], Ub(j, trans[0]), nullptr, 0, L,
-                               S.z2pi, s);
-      const TC* cur = bufs[0];
-      for (int i = 1; i < no; ++i) {
-        contract_axes<TC, TC>(axes, cur, bufs[i], trans[i], chi[trans[i]], Ub(j, trans[i]), nullptr, 0, s);
-        cur = bufs[i];
-      }
-      final_strides(axes, c3, c3, gn, c3, fs);
-      contract_axes<TC, double>(axes, cur, G.out[j], c3, chi3, Ub(j, c3), fs, out_base, s);
-    }
-  }
   return HOTRG_OK;
 }
 
@@ -1339,7 +1184,7 @@ int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const ho
   }
   for (int i = 0; i < c->batch; ++i) {
     double* Ti = c->T + i * P2;
-    launch_norm_log(Ti, n0, c->norm_partial, c->cval + i, c->lnc_log + (long long)i * (c->max_steps + 1),
+    launch_norm_log(Ti, 0, 1, n0, c->norm_partial, c->cval + i, c->lnc_log + (long long)i * (c->max_steps + 1), 0,
                     c->L + i, c->dstep, c->status, s);
     if (c->deriv)
       for (int w = 0; w < 2; ++w) {
@@ -1347,10 +1192,10 @@ int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const ho
         launch_tangent_norm(Ti, dTi, nullptr, dTi, n0, c->cval + i, c->norm_partial, c->dlnc + w * c->batch + i,
                             c->dL + w * c->batch + i, c->dstep, s);
       }
-    launch_scale(Ti, Ti, n0, c->cval + i, s);
+    launch_scale(Ti, 0, Ti, 0, 1, n0, c->cval + i, s);
     for (int w = 0; c->impure && w < 2; ++w) {
       double* Si = c->SI + (w * c->batch + i) * P2;
-      launch_scale(Si, Si, n0, c->cval + i, s);
+      launch_scale(Si, 0, Si, 0, 1, n0, c->cval + i, s);
     }
   }
   launch_trace_x(c->T, P2, c->batch, g, d - 1, c->L, c->dstep, c->out3, s);
@@ -1442,10 +1287,14 @@ static int enqueue_step(hotrg_ctx* c, int a, int step) {
   for (int i0 = 0; i0 < c->batch; i0 += c->group) {
     const int ng = std::min(c->group, c->batch - i0);
     Group grp;
-    for (int j = 0; j < ng; ++j) {
-      const double* Ti = c->T + (i0 + j) * P2max;
-      grp.add(Ti, Ti, c->U + (i0 + j) * c->u_stride, slot(c, j).Tnext, i0 + j);
-    }
+    grp.n = ng;
+    grp.inst0 = i0;
+    grp.T1 = grp.T2 = c->T + i0 * P2max;
+    grp.t_inst = P2max;
+    grp.U = c->U + i0 * c->u_stride;
+    grp.u_inst = c->u_stride;
+    grp.out = c->Tnext;
+    grp.out_inst = (long long)(c->st_Tnext / sizeof(double));
     Tangents tg;  // the group is a single instance when there are tangents (group_for)
     if (c->deriv) {
       tg.n = 2;
@@ -1455,43 +1304,36 @@ static int enqueue_step(hotrg_ctx* c, int a, int step) {
         tg.dU[w] = c->deriv_mode == 2 ? c->dU + (w * c->batch + i0) * c->u_stride : nullptr;
       }
     }
-    int rc = (c->z2 && nt > 0)
-                 ? (planes ? squeeze_z2<float>(c, grp, g, gn, a, chi, trans, nt, planes, npass)
-                           : squeeze_z2<double>(c, grp, g, gn, a, chi, trans, nt, 0, 0))
-             : planes ? squeeze<float>(c, grp, g, gn, a, chi, trans, nt, planes, npass, tg)
-                      : squeeze<double>(c, grp, g, gn, a, chi, trans, nt, 0, 0, tg);
+    int rc = planes ? squeeze<float>(c, grp, g, gn, a, chi, trans, nt, planes, npass, c->z2 && nt > 0, tg)
+                    : squeeze<double>(c, grp, g, gn, a, chi, trans, nt, 0, 0, c->z2 && nt > 0, tg);
     if (rc) return rc;
     // impure tensors with the pure flow's isometries (a group of one): the pair merges with itself
     // at step 1 (Eq. (SS)) and with a pure site after (Eq. (ST)); the single spin always with a pure
     // site
     for (int w = 0; c->impure && w < 2; ++w) {
       const double* Si = c->SI + (w * c->batch + i0) * P2max;
-      const double* partner = (w == 0 && step == 1) ? Si : grp.T1[0];
-      Group imp;
-      imp.add(Si, partner, grp.U[0], c->Stmp + w * P2max, i0);
-      rc = planes ? squeeze<float>(c, imp, g, gn, a, chi, trans, nt, planes, npass)
-                  : squeeze<double>(c, imp, g, gn, a, chi, trans, nt, 0, 0);
+      Group imp = grp;
+      imp.T1 = Si;
+      imp.T2 = (w == 0 && step == 1) ? Si : grp.T1;
+      imp.out = c->Stmp + w * P2max;
+      rc = planes ? squeeze<float>(c, imp, g, gn, a, chi, trans, nt, planes, npass, false)
+                  : squeeze<double>(c, imp, g, gn, a, chi, trans, nt, 0, 0, false);
       if (rc) return rc;
     }
-    for (int j = 0; j < ng; ++j) {
-      const int i = i0 + j;
-      const double* Tn = grp.out[j];
-      double* Tw = c->T + i * P2max;
-      {
-        PhaseScope norm_scope(c, PH_NORM);
-        launch_norm_log(Tn, gn.P * gn.P, c->norm_partial, c->cval + i, c->lnc_log + (long long)i * (c->max_steps + 1),
-                        c->L + i, c->dstep, c->status, s);
-      }
-      // tangent of T' / ||T'||
-      for (int w = 0; w < tg.n; ++w) {
-        double* dTi = c->dT + (w * c->batch + i) * P2max;
-        launch_tangent_norm(Tn, tg.dout[w], nullptr, dTi, gn.P * gn.P, c->cval + i, c->norm_partial,
-                            c->dlnc + w * c->batch + i, c->dL + w * c->batch + i, c->dstep, s);
-      }
-      launch_scale(Tn, Tw, gn.P * gn.P, c->cval + i, s);
-      for (int w = 0; c->impure && w < 2; ++w)
-        launch_scale(c->Stmp + w * P2max, c->SI + (w * c->batch + i) * P2max, gn.P * gn.P, c->cval + i, s);
+    {
+      PhaseScope norm_scope(c, PH_NORM);
+      launch_norm_log(grp.out, grp.out_inst, ng, gn.P * gn.P, c->norm_partial, c->cval + i0,
+                      c->lnc_log + (long long)i0 * (c->max_steps + 1), c->max_steps + 1, c->L + i0, c->dstep, c->status, s);
     }
+    // tangent of T' / ||T'|| (a group of one)
+    for (int w = 0; w < tg.n; ++w) {
+      const int j = w * c->batch + i0;
+      launch_tangent_norm(grp.out, tg.dout[w], nullptr, c->dT + j * P2max, gn.P * gn.P, c->cval + i0, c->norm_partial,
+                          c->dlnc + j, c->dL + j, c->dstep, s);
+    }
+    launch_scale(grp.out, grp.out_inst, c->T + i0 * P2max, P2max, ng, gn.P * gn.P, c->cval + i0, s);
+    for (int w = 0; c->impure && w < 2; ++w)
+      launch_scale(c->Stmp + w * P2max, 0, c->SI + (w * c->batch + i0) * P2max, 0, 1, gn.P * gn.P, c->cval + i0, s);
   }
   launch_trace_x(c->T, P2max, c->batch, gn, a, c->L, c->dstep, c->out3, s);
   for (int w = 0; c->impure && w < 2; ++w)
@@ -1981,8 +1823,8 @@ int hotrg_autotune(hotrg_ctx* c, hotrg_tuning* out) {
   Y.nparts = Bt.nparts = lg.nparts;
   if (lg.fmt == 1) {  // the fp16 planes and scale bounds the last step's GEMM used
     Y.fmt = Bt.fmt = 1;
-    Y.amax = c->amax + 1;
-    Bt.amax = c->amax + 0;
+    Y.amax = c->amax + c->group;
+    Bt.amax = c->amax;
     Bt.amax_mult = lg.mult_b;
   }
   for (int k = 0; k < 3; ++k) {

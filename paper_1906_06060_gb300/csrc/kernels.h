@@ -18,10 +18,10 @@ void launch_init_tensor(double* T, long long inst_stride, int batch, int d, cons
 // *dstep += 1 (device-side step counter read by the kernels below, so that a captured step
 // can be replayed for any step number).
 void launch_step_advance(int* dstep, cudaStream_t s);
-// c = ||x||_F (deterministic), lnc_log[n] = ln c, L += 2^-n ln c with n = *dstep; status on a bad
-// norm.
-void launch_norm_log(const double* x, long long n, double* partial, double* c_out,
-                     double* lnc_log, double* L, const int* dstep, int* status, cudaStream_t s);
+// For `batch` tensors x + i x_inst: c = ||x||_F (deterministic) into c_out[i], lnc_log[i log_inst + n] = ln c, L[i] +=
+// 2^-n ln c with n = *dstep; status on a bad norm. partial: 1024 doubles per tensor.
+void launch_norm_log(const double* x, long long x_inst, int batch, long long n, double* partial, double* c_out,
+                     double* lnc_log, long long log_inst, double* L, const int* dstep, int* status, cudaStream_t s);
 // Tangents of the flow (fixed isometries). dT = d T^(0) / d beta (which = 0) or d / d h (which = 1).
 void launch_init_tangent(double* dT, long long inst_stride, int batch, int d, const double* beta, const double* h,
                          int which, cudaStream_t s);
@@ -38,47 +38,60 @@ void launch_trace_ratio(const double* S, const double* T, long long t_stride, in
                         cudaStream_t s);
 // *out = max |x| over a rows x cols array with row stride ld (upper bound as a float; the bits
 // of that non-negative float are written, after zeroing *out on the stream).
+// `batch` arrays x + i x_inst, out[i].
 template <class T>
-void launch_absmax(const T* x, long long rows, long long cols, long long ld, unsigned* out, cudaStream_t s);
-// dst = src / *c
-void launch_scale(const double* src, double* dst, long long n, const double* c, cudaStream_t s);
+void launch_absmax(const T* x, long long rows, long long cols, long long ld, unsigned* out, cudaStream_t s,
+                   int batch = 1, long long x_inst = 0);
+// dst + i dst_inst = (src + i src_inst) / c[i], i < batch
+void launch_scale(const double* src, long long src_inst, double* dst, long long dst_inst, int batch, long long n,
+                  const double* c, cudaStream_t s);
 // Tr T (Eq. (tTr)) and ln Z/N = L + 2^-n ln Tr (n = *dstep); X^(n) along `axis` (Eq. (x)).
 // One CTA per instance: T + i*t_stride, L + i, out3 + 3 i.
 void launch_trace_x(const double* T, long long t_stride, int batch, Geom g, int axis, const double* L,
                     const int* dstep, double* out3, cudaStream_t s);
-// out[..u_b=j..] = sum_i U[kk][i][j] in[..u_b=i..] on unprimed leg b (U: [chi][Db][Db] fp64);
-// with in2, plus the same product of in2 with U2. With amax, *amax = max |out| (the bits of a
+// The launchers below cover ng instances (and, per instance, nb chunks of a squeeze) in one launch: instance j reads at
+// j x its instance stride, slot z = j nb + chunk at z x its slot stride (elements). See squeeze() in hotrg.cu.
+
+// For chunk c of instance j: out_z[..u_b=j..] = sum_i U_j[kk + c][i][j] in_j[..u_b=i..] on unprimed leg b (U: [chi][Db][Db]
+// fp64); with in2 (one instance), plus the same product of in2 with U2. With amax, amax[z] = max |out_z| (the bits of a
 // non-negative float, as launch_absmax writes them).
 template <class Tin, class Tout>
-void launch_mode_unprimed(const Tin* in, Tout* out, Geom g, int b, const double* U, int kk,
-                          cudaStream_t s, const Tin* in2 = nullptr, const double* U2 = nullptr,
-                          unsigned* amax = nullptr);
-// Tt[p][u] = T[u][p] (P x P), converted to Tout.
+void launch_mode_unprimed(const Tin* in, long long in_inst, Tout* out, long long out_slot, Geom g, int b, const double* U,
+                          long long u_inst, int kk, int ng, int nb, cudaStream_t s, const Tin* in2 = nullptr,
+                          const double* U2 = nullptr, unsigned* amax = nullptr);
+// Tt_j[p][u] = T_j[u][p] (P x P), converted to Tout.
 template <class Tout>
-void launch_transpose(const double* T, Tout* Tt, long long P, cudaStream_t s);
+void launch_transpose(const double* T, long long t_inst, Tout* Tt, long long tt_inst, long long P, int ng, cudaStream_t s);
 // B operand, K-major: Bt[(j*P + n)][k] = sum_x U3[j][k_c3][x] Tt[n][k | c3 := x], j < chi3.
-// c3 < 0: Bt = Tt. Mixed: 2 or 3 bf16 planes; FP64: one double plane. With Tt2 (c3 >= 0), plus
-// the same sum over Tt2 with U3b.
+// c3 < 0: Bt = Tt. Mixed: 2 or 3 16-bit planes (instance i's scale bound at amax + i); FP64: one double plane. With Tt2
+// (c3 >= 0, one instance), plus the same sum over Tt2 with U3b.
 template <class Tin, class Tout>
-void launch_build_bt(const Tin* Tt, const Planes<Tout>& out, long long ld, Geom g, int c3,
-                     const double* U3, int chi3, cudaStream_t s, const Tin* Tt2 = nullptr,
-                     const double* U3b = nullptr);
-// A operand, K-major: Y[m][k] = X[u = (k_b, m_a)][p = (m_b, k_a)] for a step along `a`.
+void launch_build_bt(const Tin* Tt, long long tt_inst, const Planes<Tout>& out, long long out_inst, long long ld, Geom g,
+                     int c3, const double* U3, long long u_inst, int chi3, int ng, cudaStream_t s,
+                     const Tin* Tt2 = nullptr, const double* U3b = nullptr);
+// A operand of slot z, K-major: Y[m][k] = X[u = (k_b, m_a)][p = (m_b, k_a)] for a step along `a` (scale bound at
+// amax + z).
 template <class Tin, class Tout>
-void launch_build_y(const Tin* X, const Planes<Tout>& out, long long ld, Geom g, int a,
-                    cudaStream_t s);
-// Generic pair contraction / strided copy (see View): out[o] = sum_{i,j} U[k'][i][j] in[...].
+void launch_build_y(const Tin* X, long long x_slot, const Planes<Tout>& out, long long out_slot, long long ld, Geom g,
+                    int a, int nz, cudaStream_t s);
+// Strided copy (see View).
 template <class Tin, class Tout>
 void launch_pair_contract(const Tin* in, Tout* out, const View& v, int kaxis, int Di, int Dj,
                           long long si, long long sj, const double* U, int chi, long long in_base,
                           long long out_base, cudaStream_t s);
-// Same contraction with one thread per index of `rest` (the output axes without k'), computing
-// all chi outputs out[o + k' sk]; every input element is read once. With in2 (same layout), plus
-// the same contraction of in2 with U2.
+// The slots of an epilogue contraction: slot z = j nb + c reads at z in_slot and writes at j out_inst + c out_chunk with
+// the isometry at j u_inst.
+struct SlotStrides {
+  int ng, nb;
+  long long in_slot, out_inst, out_chunk, u_inst;
+};
+// Pair contraction out[o] = sum_{i,j} U[k'][i][j] in[...], one thread per index of `rest` (the output axes without k'),
+// computing all chi outputs out[o + k' sk]; every input element is read once. With in2 (same layout), plus the same
+// contraction of in2 with U2.
 template <class Tin, class Tout>
 void launch_pair_contract_all(const Tin* in, Tout* out, const View& rest, int Di, int Dj, long long si,
-                              long long sj, long long sk, const double* U, int chi, long long in_base,
-                              long long out_base, cudaStream_t s, const Tin* in2 = nullptr,
+                              long long sj, long long sk, const double* U, int chi, long long out_base,
+                              const SlotStrides& st, cudaStream_t s, const Tin* in2 = nullptr,
                               const double* U2 = nullptr);
 // Raise the dynamic shared-memory limit of the two-input kernels (call once, before any capture).
 void prepare_kernel_attributes();
@@ -167,7 +180,7 @@ void launch_gemm_f64(const double* A, long long lda, const double* Bt, long long
 // ---- gemm_f64tc.cu --------------------------------------------------------------------------
 // FP64 products on the tensor cores from exact integer slices. An operand: kSliceCount planes of fp16 digits (`plane`
 // elements apart, rows of `ld`, instances `inst` apart) and the exponent of every row (instances exp_inst apart).
-constexpr int kSliceCount = 7;
+constexpr int kSliceCount = 8;
 constexpr int kSliceProducts = kSliceCount * (kSliceCount + 1) / 2;  // digit pairs a product runs
 constexpr int kSliceCtas = 152;  // CTAs of a launch at most (one per SM): the scratch area is sized for them
 struct SliceOperand {
@@ -181,11 +194,11 @@ bool slices_take(long long M, long long N, long long K);
 // Bytes of the level-sum scratch of a launch over `batch` products of at most M x N.
 size_t slice_scratch_bytes(long long M, long long N, int batch);
 // Digits and row exponents of `rows` x K doubles (row stride ldx; `batch` instances x_inst apart). With L (zero-field
-// operands, one instance) only the columns of each row's parity class, see k_slice_rows.
+// operands: instance z / nb's layout, slot z's chunk parity) only the columns of each row's parity class, see k_slice_rows.
 struct Z2Layout;
 void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
                        long long x_inst, cudaStream_t s, const Z2Layout* L = nullptr, const int* pi = nullptr,
-                       int which = 0);
+                       int which = 0, int nb = 1);
 // C[m][n] (+)= sum_k A[m][k] Bt[n][k]; blk and bat as for launch_gemm_f64. Returns 0 or a hotrg_status.
 int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,
                        long long K, int* scratch, int* status, double timeout_s, cudaStream_t s,
@@ -213,12 +226,12 @@ struct GemmBlocks {
 constexpr int kMaxGemmBatch = 256;
 // Batched launch (up to kMaxGemmBatch instances): `batch` independent products of the same shape in one
 // persistent launch; plane k of instance i starts at A.p[k] + i a_inst (elements, multiple of 8,
-// at least M lda), likewise B (b_inst) and C (c_inst); with blk, instance i's blocks are blk[i];
-// fp16 scale bounds at A.amax + i amax_inst and B.amax + i amax_inst.
+// at least M lda), likewise C (c_inst) and, by b_div, B (b_inst); with blk, instance i's blocks are blk[i];
+// fp16 scale bounds at A.amax + i and B.amax + i / b_div. Products i / b_div with the same value share one B operand (the
+// chunks of an instance): B of product i is at (i / b_div) b_inst.
 struct GemmBatch {
-  int batch = 1;
+  int batch = 1, b_div = 1;
   long long a_inst = 0, b_inst = 0, c_inst = 0;
-  int amax_inst = 0;
 };
 int launch_gemm_split(const Planes<__nv_bfloat16>& A, long long lda, const Planes<__nv_bfloat16>& B,
                       long long ldb, float* C, long long ldc, long long M, long long N, long long K,
@@ -251,26 +264,32 @@ struct Z2Layout {
 // Layouts of every instance (ev, ev_new: [batch][kMaxD] even counts before / after the step).
 void launch_z2_layout(const int* ev, const int* ev_new, int batch, Geom g, int c3, int chi3, Z2Layout* out,
                       cudaStream_t s);
-// rank_tab[P], kcol_tab[P], colpos_tab[chi3 * P] of one instance's layout.
-void launch_z2_tables(const Z2Layout* L, long long P, int chi3, int* rank_tab, int* kcol_tab, int* colpos_tab,
-                      cudaStream_t s);
-// The chunk's parity (fixed new indices k0 of axis b0, k1 of b1; nfix of them) and its two GEMM
-// blocks; flops[0] += their 2 M N K, flops[1] += that times npass.
-void launch_z2_chunk(const Z2Layout* L, const int* ev_new, int nfix, int b0, int k0, int b1, int k1, long long ldO,
-                     GemmBlocks* blk, int* pi, double* flops, int npass, cudaStream_t s);
+// Index tables of ng instances: rank[P], kcol[P] (instance stride p_inst) and colpos[chi3 * P] (stride c_inst).
+struct Z2Tables {
+  int *rank, *kcol, *colpos;
+  long long p_inst, c_inst;
+  Z2Tables from(int j) const { return {rank + j * p_inst, kcol + j * p_inst, colpos + j * c_inst, p_inst, c_inst}; }
+};
+void launch_z2_tables(const Z2Layout* L, long long P, int chi3, const Z2Tables& t, int ng, cudaStream_t s);
+// For every slot z = j nb + c: the chunk's parity pi[z] (new indices k0 of axis b0 and k1 of b1 fixed, nfix of them, the
+// last of them advanced by c; ev_new: [ng][kMaxD]) and its two GEMM blocks blk[z]; flops[0] += their 2 M N K, flops[1] +=
+// that times npass.
+void launch_z2_chunk(const Z2Layout* L, const int* ev_new, int ng, int nb, int nfix, int b0, int k0, int b1, int k1,
+                     long long N, GemmBlocks* blk, int* pi, double* flops, int npass, cudaStream_t s);
 // ev[i][b] = ev_new[i][b] for the axes b in trans_mask (end of a step).
 void launch_z2_advance(int* ev, const int* ev_new, int batch, unsigned trans_mask, cudaStream_t s);
 template <class Tin, class Tout>
-void launch_build_y_z2(const Tin* X, const Planes<Tout>& out, long long ld, Geom g, int a,
-                       const int* rank_tab, const int* kcol_tab, const Z2Layout* L, const int* pi, cudaStream_t s);
+void launch_build_y_z2(const Tin* X, long long x_slot, const Planes<Tout>& out, long long out_slot, long long ld, Geom g,
+                       int a, const Z2Tables& t, const Z2Layout* L, const int* pi, int ng, int nb, cudaStream_t s);
 template <class Tin, class Tout>
-void launch_build_bt_z2(const Tin* Tt, const Planes<Tout>& out, long long ld, Geom g, int c3, const double* U3,
-                        int chi3, const int* rank_tab, const int* kcol_tab, const int* colpos_tab, const Z2Layout* L,
+void launch_build_bt_z2(const Tin* Tt, long long tt_inst, const Planes<Tout>& out, long long out_inst, long long ld, Geom g,
+                        int c3, const double* U3, long long u_inst, int chi3, const Z2Tables& t, const Z2Layout* L, int ng,
                         cudaStream_t s);
 // First epilogue contraction (over slot t0, Dt x Dt -> chi) from the parity-blocked GEMM output;
-// rest / sk / out_base as for launch_pair_contract_all.
+// rest / sk / out_base / st as for launch_pair_contract_all (instance j's layout L + j, slot z's parity pi + z).
 template <class Tin, class Tout>
-void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, long long sk, long long out_base,
-                   int t0, int Dt, const double* U, int chi, const Z2Layout* L, const int* pi, cudaStream_t s);
+void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, long long sk, long long out_base, int t0,
+                   int Dt, const double* U, int chi, const Z2Layout* L, const int* pi, const SlotStrides& st,
+                   cudaStream_t s);
 
 }  // namespace hotrg

@@ -35,7 +35,9 @@ __device__ __forceinline__ float abs_up(float x) { return fabsf(x); }
 // non-negative float (their unsigned order is the order of the values). NaN entries are skipped.
 template <class T>
 __global__ void __launch_bounds__(256) k_absmax(const T* __restrict__ x, long long rows, long long cols,
-                                                long long ld, unsigned* out) {
+                                                long long ld, unsigned* out, long long x_inst) {
+  x += (long long)blockIdx.y * x_inst;
+  out += blockIdx.y;
   float m = 0.f;
   const long long total = rows * cols;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -116,9 +118,11 @@ __device__ double block_sum(double v, double* sh) {
   return r;
 }
 
-__global__ void __launch_bounds__(256) k_sumsq_partial(const double* __restrict__ x, long long n,
+__global__ void __launch_bounds__(256) k_sumsq_partial(const double* __restrict__ x, long long x_inst, long long n,
                                                        double* __restrict__ partial) {
   __shared__ double sh[256];
+  x += (long long)blockIdx.y * x_inst;
+  partial += (long long)blockIdx.y * kNormBlocks;
   double s = 0.0;
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)kNormBlocks * 256) {
     const double v = x[i];
@@ -131,8 +135,13 @@ __global__ void __launch_bounds__(256) k_sumsq_partial(const double* __restrict_
 __global__ void k_step_advance(int* dstep) { *dstep += 1; }
 
 __global__ void __launch_bounds__(256) k_norm_finish(const double* __restrict__ partial, double* c_out,
-                                                     double* lnc_log, double* L, const int* dstep, int* status) {
+                                                     double* lnc_log, long long log_inst, double* L, const int* dstep,
+                                                     int* status) {
   const int step = *dstep;
+  partial += (long long)blockIdx.x * kNormBlocks;
+  c_out += blockIdx.x;
+  lnc_log += (long long)blockIdx.x * log_inst;
+  L += blockIdx.x;
   __shared__ double sh[256];
   double s = 0.0;
   for (int i = threadIdx.x; i < kNormBlocks; i += 256) s += partial[i];
@@ -222,9 +231,11 @@ __global__ void __launch_bounds__(256) k_trace_ratio(const double* __restrict__ 
   if (threadIdx.x == 0) out[blockIdx.x] = ta / tb;
 }
 
-__global__ void k_scale(const double* __restrict__ src, double* __restrict__ dst, long long n,
-                        const double* __restrict__ c) {
-  const double cv = *c;
+__global__ void k_scale(const double* __restrict__ src, long long src_inst, double* __restrict__ dst, long long dst_inst,
+                        long long n, const double* __restrict__ c) {
+  src += (long long)blockIdx.y * src_inst;
+  dst += (long long)blockIdx.y * dst_inst;
+  const double cv = c[blockIdx.y];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     dst[i] = src[i] / cv;
@@ -282,8 +293,17 @@ __global__ void __launch_bounds__(256) k_mode_unprimed(const Tin* __restrict__ i
                                                        long long total, long long stride_b, int Db,
                                                        const double* __restrict__ U, int kk,
                                                        const Tin* __restrict__ in2, const double* __restrict__ U2,
-                                                       unsigned* amax) {
+                                                       unsigned* amax, long long in_inst, long long out_slot,
+                                                       long long u_inst) {
   using Acc = AccT<Tout>;
+  // chunk blockIdx.y of instance blockIdx.z (the input comes from L2 for every chunk but the first)
+  const int slot = blockIdx.z * gridDim.y + blockIdx.y;
+  in += blockIdx.z * in_inst;
+  if (TWO) in2 += blockIdx.z * in_inst;
+  out += slot * out_slot;
+  U += blockIdx.z * u_inst;
+  kk += blockIdx.y;
+  if (amax) amax += slot;
   __shared__ Acc W[kMaxGram];
   __shared__ Acc W2[TWO ? kMaxGram : 1];
   for (int t = threadIdx.x; t < Db * Db; t += blockDim.x) {
@@ -324,8 +344,10 @@ __global__ void __launch_bounds__(256) k_mode_unprimed(const Tin* __restrict__ i
 // ---------------------------------------------------------------------------- transpose
 template <class Tout>
 __global__ void __launch_bounds__(256) k_transpose(const double* __restrict__ T, Tout* __restrict__ Tt,
-                                                   long long P) {
+                                                   long long P, long long t_inst, long long tt_inst) {
   __shared__ double tile[32][33];
+  T += blockIdx.z * t_inst;
+  Tt += blockIdx.z * tt_inst;
   const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32;
   for (int k = threadIdx.y; k < 32; k += 8) {
     const long long r = r0 + k, c = c0 + threadIdx.x;
@@ -347,8 +369,13 @@ __global__ void __launch_bounds__(256) k_build_bt(const Tin* __restrict__ Tt, Pl
                                                   long long ld, long long P,
                                                   long long Sc, int Dc, const double* __restrict__ U3,
                                                   int chi3, const Tin* __restrict__ Tt2,
-                                                  const double* __restrict__ U3b) {
+                                                  const double* __restrict__ U3b, long long tt_inst, long long out_inst,
+                                                  long long u_inst) {
   using Acc = AccT<Tout>;
+  Tt += blockIdx.y * tt_inst;
+  if (TWO) Tt2 += blockIdx.y * tt_inst;
+  if (U3) U3 += blockIdx.y * u_inst;
+  out.advance(blockIdx.y, out_inst);
   extern __shared__ unsigned char smraw[];
   Acc* W = reinterpret_cast<Acc*>(smraw);  // [chi3][Dc][Dc], then the same for U3b
   const int nW = chi3 * Dc * Dc;
@@ -392,8 +419,10 @@ __global__ void __launch_bounds__(256) k_build_bt(const Tin* __restrict__ Tt, Pl
 constexpr int kYMT = 4;
 template <class Tin, class Tout>
 __global__ void __launch_bounds__(256) k_build_y(const Tin* __restrict__ X, Planes<Tout> out, long long ld,
-                                                 Geom g, int a) {
+                                                 Geom g, int a, long long x_slot, long long out_slot) {
   using Acc = AccT<Tout>;
+  X += blockIdx.z * x_slot;
+  out.advance(blockIdx.z, out_slot);
   __shared__ Acc tile[32][33];
   __shared__ long long Rk[32], Cm[32 * kYMT];
   const int P = (int)g.P;
@@ -488,68 +517,71 @@ __global__ void __launch_bounds__(256) k_pair_contract(const Tin* __restrict__ i
 
 // All chi outputs of one "rest" index per thread: out[o + k' sk] = sum_{i,j} U[k'][i][j] in[r + i si + j sj]
 // (r, o: offsets of the rest index in the input and output views). Every input element is read
-// once; W is held in shared memory as [i][j][k'] so a warp reads it by broadcast.
+// once; W is held in shared memory as [i][j][k'], rows padded to 16 bytes, so a warp reads it by broadcast.
 // TWO: out also accumulates the same contraction of in2 with U2 (the tangent of an epilogue
 // contraction: dR' = C_U(dR) + C_dU(R)).
-// N > 0: chi = Dj = N at compile time (the steady-state shape: no predicated-off loads or FMAs,
-// W rows padded to 16-byte shared-memory loads); N = 0: any chi <= 16 and Dj <= 16.
-template <class Tin, class Tout, bool TWO, int N>
+// CHI = chi at compile time (exact accumulators, no predicated-off FMAs). NJ = Dj at compile time for the FP32
+// steady-state shape (chi = Dj; a row of loads is issued before its FMAs), 0: any Dj, four loads at a time. The FP64
+// instances are bound by the FP64 units (chi FMAs per input entry at two a clock and SM).
+template <class Tin, class Tout, bool TWO, int CHI, int NJ>
 __global__ void __launch_bounds__(256) k_pair_contract_all(const Tin* __restrict__ in, Tout* __restrict__ out,
                                                            View v, long long total, int Di, int Dj,
                                                            long long si, long long sj, long long sk,
-                                                           const double* __restrict__ U, int chi,
-                                                           long long in_base, long long out_base,
+                                                           const double* __restrict__ U, long long out_base,
                                                            const Tin* __restrict__ in2,
-                                                           const double* __restrict__ U2) {
+                                                           const double* __restrict__ U2, SlotStrides st) {
   using Acc = AccT<Tout>;
-  constexpr int kMaxChi = N > 0 ? N : kMaxBond;
-  constexpr int kMaxJ = N > 0 ? N : kMaxBond;
+  constexpr int PAD = 16 / (int)sizeof(Acc);
+  constexpr int WS = (CHI + PAD - 1) / PAD * PAD;
+  constexpr int U4 = NJ > 0 ? NJ : 4;  // loads issued together
   extern __shared__ __align__(16) unsigned char smraw[];
-  // W row stride: chi, or N padded to a multiple of 4
-  const int ws = N > 0 ? (N + 3) / 4 * 4 : chi;
-  Acc* W = reinterpret_cast<Acc*>(smraw);  // [Di*Dj][ws], then the same for U2
+  Acc* W = reinterpret_cast<Acc*>(smraw);  // [Di*Dj][WS], then the same for U2
+  const long long in_off = (blockIdx.z * gridDim.y + blockIdx.y) * st.in_slot;
+  out_base += blockIdx.z * st.out_inst + blockIdx.y * st.out_chunk;
+  in += in_off;
+  if (TWO) in2 += in_off;
+  U += blockIdx.z * st.u_inst;
   const int nij = Di * Dj;
-  Acc* W2 = W + (long long)ws * nij;
-  for (int t = threadIdx.x; t < ws * nij; t += blockDim.x) {
+  Acc* W2 = W + (long long)WS * nij;
+  for (int t = threadIdx.x; t < WS * nij; t += blockDim.x) {
     const int k = t / nij, ij = t % nij;
-    W[ij * ws + k] = k < chi ? (U ? (Acc)U[t] : (Acc)1) : (Acc)0;
-    if (TWO) W2[ij * ws + k] = k < chi ? (Acc)U2[t] : (Acc)0;
+    W[ij * WS + k] = k < CHI ? (Acc)U[t] : (Acc)0;
+    if (TWO) W2[ij * WS + k] = k < CHI ? (Acc)U2[t] : (Acc)0;
   }
   __syncthreads();
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    long long rem = idx, ioff = in_base, ooff = out_base;
+    long long rem = idx, ioff = 0, ooff = out_base;
     for (int ax = v.ndim - 1; ax >= 0; --ax) {
       const long long c = rem % v.shape[ax];
       rem /= v.shape[ax];
       ioff += c * v.in_stride[ax];
       ooff += c * v.out_stride[ax];
     }
-    Acc acc[kMaxChi];
+    Acc acc[CHI];
 #pragma unroll
-    for (int k = 0; k < kMaxChi; ++k) acc[k] = 0;
-    // one row of Dj loads issued before its FMAs (bytes in flight to stream HBM)
+    for (int k = 0; k < CHI; ++k) acc[k] = 0;
     for (int pass = 0; pass < (TWO ? 2 : 1); ++pass) {
       const Tin* base_in = pass ? in2 : in;
       const Acc* Wp = pass ? W2 : W;
       for (int i = 0; i < Di; ++i) {
         const Tin* src = base_in + ioff + i * si;
-        Acc x[kMaxJ];
+        for (int j0 = 0; j0 < (NJ > 0 ? NJ : Dj); j0 += U4) {
+          Acc x[U4];
 #pragma unroll
-        for (int j = 0; j < kMaxJ; ++j) x[j] = (N > 0 || j < Dj) ? (Acc)src[j * sj] : (Acc)0;
+          for (int u = 0; u < U4; ++u) x[u] = (NJ > 0 || j0 + u < Dj) ? (Acc)src[(j0 + u) * sj] : (Acc)0;
 #pragma unroll
-        for (int j = 0; j < kMaxJ; ++j) {
-          if (N == 0 && j >= Dj) break;
-          const Acc* w = Wp + (i * Dj + j) * ws;
+          for (int u = 0; u < U4; ++u) {
+            if (NJ == 0 && j0 + u >= Dj) break;
+            const Acc* w = Wp + (i * Dj + j0 + u) * WS;
 #pragma unroll
-          for (int k = 0; k < kMaxChi; ++k)
-            if (N > 0 || k < chi) acc[k] += w[k] * x[j];
+            for (int k = 0; k < CHI; ++k) acc[k] += w[k] * x[u];
+          }
         }
       }
     }
 #pragma unroll
-    for (int k = 0; k < kMaxChi; ++k)
-      if (N > 0 || k < chi) out[ooff + k * sk] = (Tout)acc[k];
+    for (int k = 0; k < CHI; ++k) out[ooff + k * sk] = (Tout)acc[k];
   }
 }
 
@@ -569,11 +601,11 @@ void launch_step_advance(int* dstep, cudaStream_t s) {
   count_launches(1);
 }
 
-void launch_norm_log(const double* x, long long n, double* partial, double* c_out, double* lnc_log,
-                     double* L, const int* dstep, int* status, cudaStream_t s) {
-  k_sumsq_partial<<<kNormBlocks, 256, 0, s>>>(x, n, partial);
+void launch_norm_log(const double* x, long long x_inst, int batch, long long n, double* partial, double* c_out,
+                     double* lnc_log, long long log_inst, double* L, const int* dstep, int* status, cudaStream_t s) {
+  k_sumsq_partial<<<dim3(kNormBlocks, batch), 256, 0, s>>>(x, x_inst, n, partial);
   count_launches(1);
-  k_norm_finish<<<1, 256, 0, s>>>(partial, c_out, lnc_log, L, dstep, status);
+  k_norm_finish<<<batch, 256, 0, s>>>(partial, c_out, lnc_log, log_inst, L, dstep, status);
   count_launches(1);
 }
 
@@ -607,8 +639,9 @@ void launch_trace_ratio(const double* S, const double* T, long long t_stride, in
   count_launches(1);
 }
 
-void launch_scale(const double* src, double* dst, long long n, const double* c, cudaStream_t s) {
-  k_scale<<<grid_for(n, 256), 256, 0, s>>>(src, dst, n, c);
+void launch_scale(const double* src, long long src_inst, double* dst, long long dst_inst, int batch, long long n,
+                  const double* c, cudaStream_t s) {
+  k_scale<<<dim3(grid_for(n, 256), batch), 256, 0, s>>>(src, src_inst, dst, dst_inst, n, c);
   count_launches(1);
 }
 
@@ -619,39 +652,45 @@ void launch_trace_x(const double* T, long long t_stride, int batch, Geom g, int 
 }
 
 template <class Tin, class Tout>
-void launch_mode_unprimed(const Tin* in, Tout* out, Geom g, int b, const double* U, int kk,
-                          cudaStream_t s, const Tin* in2, const double* U2, unsigned* amax) {
+void launch_mode_unprimed(const Tin* in, long long in_inst, Tout* out, long long out_slot, Geom g, int b, const double* U,
+                          long long u_inst, int kk, int ng, int nb, cudaStream_t s, const Tin* in2, const double* U2,
+                          unsigned* amax) {
   const long long total = g.P * g.P;
   const long long nbase = total / g.D[b];
-  if (amax) cudaMemsetAsync(amax, 0, sizeof(unsigned), s);
+  if (amax) cudaMemsetAsync(amax, 0, sizeof(unsigned) * ng * nb, s);
+  const dim3 grid(grid_for(nbase, 256), nb, ng);
   if (in2)
-    k_mode_unprimed<Tin, Tout, true><<<grid_for(nbase, 256), 256, 0, s>>>(in, out, total, g.Sn[b] * g.P,
-                                                                           g.D[b], U, kk, in2, U2, amax);
+    k_mode_unprimed<Tin, Tout, true><<<grid, 256, 0, s>>>(in, out, total, g.Sn[b] * g.P, g.D[b], U, kk, in2, U2, amax,
+                                                          in_inst, out_slot, u_inst);
   else
-    k_mode_unprimed<Tin, Tout, false><<<grid_for(nbase, 256), 256, 0, s>>>(in, out, total, g.Sn[b] * g.P,
-                                                                            g.D[b], U, kk, nullptr, nullptr, amax);
+    k_mode_unprimed<Tin, Tout, false><<<grid, 256, 0, s>>>(in, out, total, g.Sn[b] * g.P, g.D[b], U, kk, nullptr, nullptr,
+                                                           amax, in_inst, out_slot, u_inst);
   count_launches(1);
 }
 
 template <class T>
-void launch_absmax(const T* x, long long rows, long long cols, long long ld, unsigned* out, cudaStream_t s) {
-  cudaMemsetAsync(out, 0, sizeof(unsigned), s);
-  k_absmax<T><<<grid_for(rows * cols, 256), 256, 0, s>>>(x, rows, cols, ld, out);
+void launch_absmax(const T* x, long long rows, long long cols, long long ld, unsigned* out, cudaStream_t s, int batch,
+                   long long x_inst) {
+  cudaMemsetAsync(out, 0, sizeof(unsigned) * batch, s);
+  k_absmax<T><<<dim3(grid_for(rows * cols, 256), batch), 256, 0, s>>>(x, rows, cols, ld, out, x_inst);
   count_launches(1);
 }
-template void launch_absmax<float>(const float*, long long, long long, long long, unsigned*, cudaStream_t);
-template void launch_absmax<double>(const double*, long long, long long, long long, unsigned*, cudaStream_t);
+template void launch_absmax<float>(const float*, long long, long long, long long, unsigned*, cudaStream_t, int, long long);
+template void launch_absmax<double>(const double*, long long, long long, long long, unsigned*, cudaStream_t, int,
+                                    long long);
 
 template <class Tout>
-void launch_transpose(const double* T, Tout* Tt, long long P, cudaStream_t s) {
-  dim3 grid((unsigned)((P + 31) / 32), (unsigned)((P + 31) / 32));
-  k_transpose<Tout><<<grid, dim3(32, 8), 0, s>>>(T, Tt, P);
+void launch_transpose(const double* T, long long t_inst, Tout* Tt, long long tt_inst, long long P, int ng,
+                      cudaStream_t s) {
+  dim3 grid((unsigned)((P + 31) / 32), (unsigned)((P + 31) / 32), (unsigned)ng);
+  k_transpose<Tout><<<grid, dim3(32, 8), 0, s>>>(T, Tt, P, t_inst, tt_inst);
   count_launches(1);
 }
 
 template <class Tin, class Tout>
-void launch_build_bt(const Tin* Tt, const Planes<Tout>& out, long long ld, Geom g, int c3,
-                     const double* U3, int chi3, cudaStream_t s, const Tin* Tt2, const double* U3b) {
+void launch_build_bt(const Tin* Tt, long long tt_inst, const Planes<Tout>& out, long long out_inst, long long ld, Geom g,
+                     int c3, const double* U3, long long u_inst, int chi3, int ng, cudaStream_t s, const Tin* Tt2,
+                     const double* U3b) {
   using Acc = AccT<Tout>;
   const long long Sc = c3 >= 0 ? g.Sn[c3] : 0;
   const int Dc = c3 >= 0 ? g.D[c3] : 1;
@@ -659,21 +698,21 @@ void launch_build_bt(const Tin* Tt, const Planes<Tout>& out, long long ld, Geom 
   const bool two = Tt2 && c3 >= 0;
   const size_t smem = sizeof(Acc) * (size_t)nchi * Dc * Dc * (two ? 2 : 1);
   const long long total = (long long)nchi * g.P * g.P;
+  const dim3 grid(grid_for(total, 256), ng);
   if (two)
-    k_build_bt<Tin, Tout, true><<<grid_for(total, 256), 256, smem, s>>>(Tt, out, ld, g.P, Sc, Dc, U3, nchi,
-                                                                         Tt2, U3b);
+    k_build_bt<Tin, Tout, true><<<grid, 256, smem, s>>>(Tt, out, ld, g.P, Sc, Dc, U3, nchi, Tt2, U3b, tt_inst, out_inst,
+                                                        u_inst);
   else
-    k_build_bt<Tin, Tout, false><<<grid_for(total, 256), 256, smem, s>>>(Tt, out, ld, g.P, Sc, Dc,
-                                                                          c3 >= 0 ? U3 : nullptr, nchi,
-                                                                          nullptr, nullptr);
+    k_build_bt<Tin, Tout, false><<<grid, 256, smem, s>>>(Tt, out, ld, g.P, Sc, Dc, c3 >= 0 ? U3 : nullptr, nchi, nullptr,
+                                                         nullptr, tt_inst, out_inst, u_inst);
   count_launches(1);
 }
 
 template <class Tin, class Tout>
-void launch_build_y(const Tin* X, const Planes<Tout>& out, long long ld, Geom g, int a,
-                    cudaStream_t s) {
-  dim3 grid((unsigned)((g.P + 31) / 32), (unsigned)((g.P + 32 * kYMT - 1) / (32 * kYMT)));
-  k_build_y<Tin, Tout><<<grid, dim3(32, 8), 0, s>>>(X, out, ld, g, a);
+void launch_build_y(const Tin* X, long long x_slot, const Planes<Tout>& out, long long out_slot, long long ld, Geom g,
+                    int a, int nz, cudaStream_t s) {
+  dim3 grid((unsigned)((g.P + 31) / 32), (unsigned)((g.P + 32 * kYMT - 1) / (32 * kYMT)), (unsigned)nz);
+  k_build_y<Tin, Tout><<<grid, dim3(32, 8), 0, s>>>(X, out, ld, g, a, x_slot, out_slot);
   count_launches(1);
 }
 
@@ -691,84 +730,97 @@ void launch_pair_contract(const Tin* in, Tout* out, const View& v, int kaxis, in
   count_launches(1);
 }
 
-template <class Tin, class Tout>
-void launch_pair_contract_all(const Tin* in, Tout* out, const View& rest, int Di, int Dj, long long si,
-                              long long sj, long long sk, const double* U, int chi, long long in_base,
-                              long long out_base, cudaStream_t s, const Tin* in2, const double* U2) {
+template <class Tin, class Tout, bool TWO, int CHI, int NJ>
+static void pair_contract_all(const Tin* in, Tout* out, const View& rest, int Di, int Dj, long long si, long long sj,
+                              long long sk, const double* U, long long out_base, const SlotStrides& st, cudaStream_t s,
+                              const Tin* in2, const double* U2) {
   using Acc = AccT<Tout>;
+  constexpr int PAD = 16 / (int)sizeof(Acc);
   long long total = 1;
   for (int i = 0; i < rest.ndim; ++i) total *= rest.shape[i];
-  const size_t smem = sizeof(Acc) * (size_t)chi * Di * Dj * (in2 ? 2 : 1);
-  const size_t smem_pad = sizeof(Acc) * (size_t)((chi + 3) / 4 * 4) * Di * Dj;
-  const int grid = grid_for(total, 256);
-  if (in2) {
-    k_pair_contract_all<Tin, Tout, true, 0><<<grid, 256, smem, s>>>(in, out, rest, total, Di, Dj, si, sj, sk, U,
-                                                                     chi, in_base, out_base, in2, U2);
-    count_launches(1);
-    return;
-  }
-  // the steady-state FP32 shape (chi = Dj) with compile-time extents
-  if constexpr (std::is_same<Tin, float>::value) {
-    if (U && chi == Dj && chi >= 6) switch (chi) {
-#define HOTRG_PCA(NN)                                                                                      \
-  case NN:                                                                                                 \
-    k_pair_contract_all<Tin, Tout, false, NN><<<grid, 256, smem_pad, s>>>(in, out, rest, total, Di, Dj, si, sj, \
-                                                                          sk, U, chi, in_base, out_base,      \
-                                                                          nullptr, nullptr);                  \
-    count_launches(1);                                                                                     \
-    return;
-      HOTRG_PCA(6) HOTRG_PCA(7) HOTRG_PCA(8) HOTRG_PCA(9) HOTRG_PCA(10) HOTRG_PCA(11)
-      HOTRG_PCA(12) HOTRG_PCA(13) HOTRG_PCA(14) HOTRG_PCA(15) HOTRG_PCA(16)
-#undef HOTRG_PCA
-        default:
-          break;
-      }
-  }
-  k_pair_contract_all<Tin, Tout, false, 0><<<grid, 256, smem, s>>>(in, out, rest, total, Di, Dj, si, sj, sk, U,
-                                                                    chi, in_base, out_base, nullptr, nullptr);
+  const size_t smem = sizeof(Acc) * (size_t)((CHI + PAD - 1) / PAD * PAD) * Di * Dj * (TWO ? 2 : 1);
+  k_pair_contract_all<Tin, Tout, TWO, CHI, NJ><<<dim3(grid_for(total, 256), st.nb, st.ng), 256, smem, s>>>(
+      in, out, rest, total, Di, Dj, si, sj, sk, U, out_base, in2, U2, st);
   count_launches(1);
+}
+
+template <class Tin, class Tout>
+void launch_pair_contract_all(const Tin* in, Tout* out, const View& rest, int Di, int Dj, long long si,
+                              long long sj, long long sk, const double* U, int chi, long long out_base,
+                              const SlotStrides& st, cudaStream_t s, const Tin* in2, const double* U2) {
+  switch (chi) {
+#define HOTRG_PCA(C)                                                                                               \
+  case C:                                                                                                          \
+    if (in2)                                                                                                       \
+      pair_contract_all<Tin, Tout, true, C, 0>(in, out, rest, Di, Dj, si, sj, sk, U, out_base, st, s, in2, U2);      \
+    else if (std::is_same<Tin, float>::value && C >= 6 && Dj == C)                                                 \
+      pair_contract_all<Tin, Tout, false, C, std::is_same<Tin, float>::value && C >= 6 ? C : 0>(                   \
+          in, out, rest, Di, Dj, si, sj, sk, U, out_base, st, s, nullptr, nullptr);                                \
+    else                                                                                                           \
+      pair_contract_all<Tin, Tout, false, C, 0>(in, out, rest, Di, Dj, si, sj, sk, U, out_base, st, s, nullptr,      \
+                                                nullptr);                                                          \
+    return;
+    HOTRG_PCA(1) HOTRG_PCA(2) HOTRG_PCA(3) HOTRG_PCA(4) HOTRG_PCA(5) HOTRG_PCA(6) HOTRG_PCA(7) HOTRG_PCA(8)
+    HOTRG_PCA(9) HOTRG_PCA(10) HOTRG_PCA(11) HOTRG_PCA(12) HOTRG_PCA(13) HOTRG_PCA(14) HOTRG_PCA(15) HOTRG_PCA(16)
+#undef HOTRG_PCA
+    default:
+      return;
+  }
 }
 
 // The two-input contractions and B-operand builds in FP64 can need more than the default 48 KB
 // of dynamic shared memory (2 x 16 x 256 doubles): raise the limit once, outside any capture.
+template <class Tin, class Tout>
+static void raise_two_input_limit(int big) {
+#define HOTRG_PCA_ATTR(C) \
+  cudaFuncSetAttribute(k_pair_contract_all<Tin, Tout, true, C, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  HOTRG_PCA_ATTR(12) HOTRG_PCA_ATTR(13) HOTRG_PCA_ATTR(14) HOTRG_PCA_ATTR(15) HOTRG_PCA_ATTR(16)
+#undef HOTRG_PCA_ATTR
+}
+
 void prepare_kernel_attributes() {
+  // 2 x round_up(chi, 2) x Di Dj doubles: above 48 KB from chi = 12 on (12 x 256 x 2 x 8 bytes = 48 KB)
   const int big = (int)(2 * sizeof(double) * kMaxBond * kMaxGram);
-  cudaFuncSetAttribute(k_pair_contract_all<double, double, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       big);
-  cudaFuncSetAttribute(k_pair_contract_all<float, float, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  cudaFuncSetAttribute(k_pair_contract_all<float, double, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       big);
+  raise_two_input_limit<double, double>(big);
+  raise_two_input_limit<float, float>(big);
+  raise_two_input_limit<float, double>(big);
   cudaFuncSetAttribute(k_build_bt<double, double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   cudaFuncSetAttribute(k_build_bt<float, __nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 // explicit instantiations: FP64 path (double everywhere) and BF16X3 path (float intermediates)
-template void launch_mode_unprimed<double, double>(const double*, double*, Geom, int, const double*, int, cudaStream_t,
-                                                   const double*, const double*, unsigned*);
-template void launch_mode_unprimed<double, float>(const double*, float*, Geom, int, const double*, int, cudaStream_t,
-                                                  const double*, const double*, unsigned*);
-template void launch_mode_unprimed<float, float>(const float*, float*, Geom, int, const double*, int, cudaStream_t,
-                                                 const float*, const double*, unsigned*);
-template void launch_transpose<double>(const double*, double*, long long, cudaStream_t);
-template void launch_transpose<float>(const double*, float*, long long, cudaStream_t);
-template void launch_build_bt<double, double>(const double*, const Planes<double>&, long long, Geom, int, const double*, int,
-                                              cudaStream_t, const double*, const double*);
-template void launch_build_bt<float, __nv_bfloat16>(const float*, const Planes<__nv_bfloat16>&, long long, Geom, int,
-                                                    const double*, int, cudaStream_t, const float*, const double*);
-template void launch_build_y<double, double>(const double*, const Planes<double>&, long long, Geom, int, cudaStream_t);
-template void launch_build_y<float, __nv_bfloat16>(const float*, const Planes<__nv_bfloat16>&, long long, Geom, int, cudaStream_t);
-template void launch_build_y<double, __nv_bfloat16>(const double*, const Planes<__nv_bfloat16>&, long long, Geom, int, cudaStream_t);
+#define HOTRG_MODE(TI, TO)                                                                                            \
+  template void launch_mode_unprimed<TI, TO>(const TI*, long long, TO*, long long, Geom, int, const double*, long long, \
+                                             int, int, int, cudaStream_t, const TI*, const double*, unsigned*);
+HOTRG_MODE(double, double)
+HOTRG_MODE(double, float)
+HOTRG_MODE(float, float)
+#undef HOTRG_MODE
+template void launch_transpose<double>(const double*, long long, double*, long long, long long, int, cudaStream_t);
+template void launch_transpose<float>(const double*, long long, float*, long long, long long, int, cudaStream_t);
+#define HOTRG_BT(TI, TO)                                                                                          \
+  template void launch_build_bt<TI, TO>(const TI*, long long, const Planes<TO>&, long long, long long, Geom, int,   \
+                                        const double*, long long, int, int, cudaStream_t, const TI*, const double*);
+HOTRG_BT(double, double)
+HOTRG_BT(float, __nv_bfloat16)
+#undef HOTRG_BT
+#define HOTRG_Y(TI, TO)                                                                                               \
+  template void launch_build_y<TI, TO>(const TI*, long long, const Planes<TO>&, long long, long long, Geom, int, int, \
+                                       cudaStream_t);
+HOTRG_Y(double, double)
+HOTRG_Y(float, __nv_bfloat16)
+HOTRG_Y(double, __nv_bfloat16)
+#undef HOTRG_Y
 template void launch_pair_contract<double, double>(const double*, double*, const View&, int, int, int, long long, long long, const double*, int, long long, long long, cudaStream_t);
 template void launch_pair_contract<float, float>(const float*, float*, const View&, int, int, int, long long, long long, const double*, int, long long, long long, cudaStream_t);
 template void launch_pair_contract<float, double>(const float*, double*, const View&, int, int, int, long long, long long, const double*, int, long long, long long, cudaStream_t);
-template void launch_pair_contract_all<double, double>(const double*, double*, const View&, int, int, long long, long long,
-                                                       long long, const double*, int, long long, long long, cudaStream_t,
-                                                       const double*, const double*);
-template void launch_pair_contract_all<float, float>(const float*, float*, const View&, int, int, long long, long long,
-                                                     long long, const double*, int, long long, long long, cudaStream_t,
-                                                     const float*, const double*);
-template void launch_pair_contract_all<float, double>(const float*, double*, const View&, int, int, long long, long long,
-                                                      long long, const double*, int, long long, long long, cudaStream_t,
-                                                      const float*, const double*);
+#define HOTRG_PCA(TI, TO)                                                                                              \
+  template void launch_pair_contract_all<TI, TO>(const TI*, TO*, const View&, int, int, long long, long long, long long, \
+                                                 const double*, int, long long, const SlotStrides&, cudaStream_t,       \
+                                                 const TI*, const double*);
+HOTRG_PCA(double, double)
+HOTRG_PCA(float, float)
+HOTRG_PCA(float, double)
+#undef HOTRG_PCA
 
 }  // namespace hotrg

@@ -95,8 +95,11 @@ __global__ void k_z2_layout(const int* ev, const int* ev_new, Geom g, int c3, in
 
 // rank_tab[i] = rank of natural index i (even class first); kcol_tab[i] = its operand column;
 // colpos_tab[j * P + n] = GEMM-output column of (j, n).
-__global__ void k_z2_tables(const Z2Layout* Lp, int P, int chi3, int* rank_tab, int* kcol_tab, int* colpos_tab) {
-  const Z2Layout L = *Lp;
+__global__ void k_z2_tables(const Z2Layout* Lp, int P, int chi3, Z2Tables t0) {
+  const Z2Layout L = Lp[blockIdx.y];
+  int* const rank_tab = t0.rank + blockIdx.y * t0.p_inst;
+  int* const kcol_tab = t0.kcol + blockIdx.y * t0.p_inst;
+  int* const colpos_tab = t0.colpos + blockIdx.y * t0.c_inst;
   const long long total = (long long)chi3 * P;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -115,33 +118,47 @@ __global__ void k_z2_tables(const Z2Layout* Lp, int P, int chi3, int* rank_tab, 
   }
 }
 
-// pi = parity of the chunk's fixed new indices; the GEMM's two blocks (row class cm, k class
-// and column group cm ^ pi).
-__global__ void k_z2_chunk(const Z2Layout* Lp, const int* ev_new, int nfix, int b0, int k0, int b1, int k1,
-                           long long ldO, GemmBlocks* blk, int* pi_out, double* flops, int npass) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const Z2Layout& L = *Lp;
-  int pi = 0;
-  if (nfix > 0) pi ^= k0 >= ev_new[b0] ? 1 : 0;
-  if (nfix > 1) pi ^= k1 >= ev_new[b1] ? 1 : 0;
-  GemmBlocks g;
-  g.nb = 2;
-  for (int cm = 0; cm < 2; ++cm) {
-    const int ck = cm ^ pi;
-    g.m0[cm] = cm ? L.ncls[0] : 0;
-    g.mc[cm] = L.ncls[cm];
-    g.k0[cm] = L.kstart[ck];
-    g.kc[cm] = L.ncls[ck];
-    g.n0[cm] = L.goff[ck];
-    g.nc[cm] = ck ? (int)(ldO - L.goff[1]) : L.goff[1];
+// Per slot: pi = parity of the chunk's fixed new indices; the GEMM's two blocks (row class cm, k class
+// and column group cm ^ pi). One block for all slots (at most kMaxGemmBatch).
+__global__ void __launch_bounds__(kMaxGemmBatch) k_z2_chunk(const Z2Layout* Lp, const int* ev_new, int nz, int nb, int nfix,
+                                                            int b0, int k0, int b1, int k1, long long N, GemmBlocks* blk,
+                                                            int* pi_out, double* flops, int npass) {
+  __shared__ double part[kMaxGemmBatch];
+  const int z = threadIdx.x;
+  if (z < nz) {
+    const int j = z / nb, c = z % nb;
+    const Z2Layout& L = Lp[j];
+    ev_new += j * kMaxD;
+    if (nfix > 1) k1 += c;
+    else k0 += c;
+    int pi = 0;
+    if (nfix > 0) pi ^= k0 >= ev_new[b0] ? 1 : 0;
+    if (nfix > 1) pi ^= k1 >= ev_new[b1] ? 1 : 0;
+    GemmBlocks g;
+    g.nb = 2;
+    for (int cm = 0; cm < 2; ++cm) {
+      const int ck = cm ^ pi;
+      g.m0[cm] = cm ? L.ncls[0] : 0;
+      g.mc[cm] = L.ncls[cm];
+      g.k0[cm] = L.kstart[ck];
+      g.kc[cm] = L.ncls[ck];
+      g.n0[cm] = L.goff[ck];
+      g.nc[cm] = ck ? (int)(N - L.goff[1]) : L.goff[1];
+    }
+    blk[z] = g;
+    pi_out[z] = pi;
+    double f = 0.0;
+    for (int b = 0; b < 2; ++b) f += 2.0 * g.mc[b] * (double)g.nc[b] * g.kc[b];
+    part[z] = f;
   }
-  *blk = g;
-  *pi_out = pi;
-  // algorithmic flops of the two blocks: [0] 2 M N K, [1] times the split passes
-  double f = 0.0;
-  for (int b = 0; b < 2; ++b) f += 2.0 * g.mc[b] * (double)g.nc[b] * g.kc[b];
-  flops[0] += f;
-  flops[1] += f * npass;
+  __syncthreads();
+  if (z == 0) {
+    // algorithmic flops of the blocks: [0] 2 M N K, [1] times the split passes
+    double f = 0.0;
+    for (int i = 0; i < nz; ++i) f += part[i];
+    flops[0] += f;
+    flops[1] += f * npass;
+  }
 }
 
 __global__ void k_z2_advance(int* ev, const int* ev_new, int batch, unsigned trans_mask) {
@@ -159,9 +176,15 @@ __global__ void k_z2_advance(int* ev, const int* ev_new, int batch, unsigned tra
 constexpr int Y_MT = 4;
 template <class Tin, class Tout>
 __global__ void __launch_bounds__(256) k_build_y_z2(const Tin* __restrict__ X, Planes<Tout> out,
-                                                    long long ld, Geom g, int a, const int* __restrict__ rank_tab,
-                                                    const int* __restrict__ kcol_tab, const Z2Layout* Lp,
-                                                    const int* pi_ptr) {
+                                                    long long ld, Geom g, int a, Z2Tables tab, const Z2Layout* Lp,
+                                                    const int* pi_ptr, int nb, long long x_slot, long long out_slot) {
+  const int inst = blockIdx.z / nb;  // slot blockIdx.z
+  X += blockIdx.z * x_slot;
+  out.advance(blockIdx.z, out_slot);
+  const int* __restrict__ rank_tab = tab.rank + inst * tab.p_inst;
+  const int* __restrict__ kcol_tab = tab.kcol + inst * tab.p_inst;
+  Lp += inst;
+  pi_ptr += blockIdx.z;
   __shared__ long long Rk[32], Cm[32 * Y_MT];
   __shared__ int rowr[32 * Y_MT], colk[32], parm[32 * Y_MT], park[32];
   const int P = (int)g.P;
@@ -216,10 +239,17 @@ __global__ void __launch_bounds__(256) k_build_y_z2(const Tin* __restrict__ X, P
 template <class Tin, class Tout>
 __global__ void __launch_bounds__(256) k_build_bt_z2(const Tin* __restrict__ Tt, Planes<Tout> out,
                                                      long long ld, long long P, long long Sc, int Dc,
-                                                     const double* __restrict__ U3, int chi3,
-                                                     const int* __restrict__ rank_tab, const int* __restrict__ kcol_tab,
-                                                     const int* __restrict__ colpos_tab, const Z2Layout* Lp) {
+                                                     const double* __restrict__ U3, int chi3, Z2Tables tab,
+                                                     const Z2Layout* Lp, long long tt_inst, long long out_inst,
+                                                     long long u_inst) {
   using Acc = ZAcc<Tout>;
+  Tt += blockIdx.y * tt_inst;
+  out.advance(blockIdx.y, out_inst);
+  U3 += blockIdx.y * u_inst;
+  Lp += blockIdx.y;
+  const int* __restrict__ rank_tab = tab.rank + blockIdx.y * tab.p_inst;
+  const int* __restrict__ kcol_tab = tab.kcol + blockIdx.y * tab.p_inst;
+  const int* __restrict__ colpos_tab = tab.colpos + blockIdx.y * tab.c_inst;
   extern __shared__ unsigned char smraw_bt[];
   Acc* W = reinterpret_cast<Acc*>(smraw_bt);  // [chi3][Dc][Dc]
   const int nW = chi3 * Dc * Dc;
@@ -334,8 +364,14 @@ template <class Tin, class Tout, int CHI>
 __global__ void __launch_bounds__(256, epi_min_blocks<Tin>()) k_epi_z2(const Tin* __restrict__ O, long long ldO, Tout* __restrict__ out,
                                                 View rest, int total, long long sk, long long out_base,
                                                 int t0, const double* __restrict__ U,
-                                                const Z2Layout* Lp, const int* pi_ptr) {
+                                                const Z2Layout* Lp, const int* pi_ptr, SlotStrides st) {
   using Acc = ZAcc<Tin>;
+  const int slot = blockIdx.z * gridDim.y + blockIdx.y;
+  O += slot * st.in_slot;
+  out_base += blockIdx.z * st.out_inst + blockIdx.y * st.out_chunk;
+  U += blockIdx.z * st.u_inst;
+  Lp += blockIdx.z;
+  pi_ptr += slot;
   constexpr int CHIP = chi_pad<CHI>();
   extern __shared__ __align__(16) unsigned char smraw_epi[];
   Acc* W = reinterpret_cast<Acc*>(smraw_epi);  // [D*D][CHIP]
@@ -456,15 +492,14 @@ void launch_z2_layout(const int* ev, const int* ev_new, int batch, Geom g, int c
   count_launches(1);
 }
 
-void launch_z2_tables(const Z2Layout* L, long long P, int chi3, int* rank_tab, int* kcol_tab, int* colpos_tab,
-                      cudaStream_t s) {
-  k_z2_tables<<<grid_cap((long long)chi3 * P), 256, 0, s>>>(L, (int)P, chi3, rank_tab, kcol_tab, colpos_tab);
+void launch_z2_tables(const Z2Layout* L, long long P, int chi3, const Z2Tables& t, int ng, cudaStream_t s) {
+  k_z2_tables<<<dim3(grid_cap((long long)chi3 * P), ng), 256, 0, s>>>(L, (int)P, chi3, t);
   count_launches(1);
 }
 
-void launch_z2_chunk(const Z2Layout* L, const int* ev_new, int nfix, int b0, int k0, int b1, int k1, long long ldO,
-                     GemmBlocks* blk, int* pi, double* flops, int npass, cudaStream_t s) {
-  k_z2_chunk<<<1, 32, 0, s>>>(L, ev_new, nfix, b0, k0, b1, k1, ldO, blk, pi, flops, npass);
+void launch_z2_chunk(const Z2Layout* L, const int* ev_new, int ng, int nb, int nfix, int b0, int k0, int b1, int k1,
+                     long long N, GemmBlocks* blk, int* pi, double* flops, int npass, cudaStream_t s) {
+  k_z2_chunk<<<1, kMaxGemmBatch, 0, s>>>(L, ev_new, ng * nb, nb, nfix, b0, k0, b1, k1, N, blk, pi, flops, npass);
   count_launches(1);
 }
 
@@ -474,35 +509,37 @@ void launch_z2_advance(int* ev, const int* ev_new, int batch, unsigned trans_mas
 }
 
 template <class Tin, class Tout>
-void launch_build_y_z2(const Tin* X, const Planes<Tout>& out, long long ld, Geom g, int a,
-                       const int* rank_tab, const int* kcol_tab, const Z2Layout* L, const int* pi, cudaStream_t s) {
-  dim3 grid((unsigned)((g.P + 31) / 32), (unsigned)((g.P + 32 * Y_MT - 1) / (32 * Y_MT)));
-  k_build_y_z2<Tin, Tout><<<grid, dim3(32, 8), 0, s>>>(X, out, ld, g, a, rank_tab, kcol_tab, L, pi);
+void launch_build_y_z2(const Tin* X, long long x_slot, const Planes<Tout>& out, long long out_slot, long long ld, Geom g,
+                       int a, const Z2Tables& t, const Z2Layout* L, const int* pi, int ng, int nb, cudaStream_t s) {
+  dim3 grid((unsigned)((g.P + 31) / 32), (unsigned)((g.P + 32 * Y_MT - 1) / (32 * Y_MT)), (unsigned)(ng * nb));
+  k_build_y_z2<Tin, Tout><<<grid, dim3(32, 8), 0, s>>>(X, out, ld, g, a, t, L, pi, nb, x_slot, out_slot);
   count_launches(1);
 }
 
 template <class Tin, class Tout>
-void launch_build_bt_z2(const Tin* Tt, const Planes<Tout>& out, long long ld, Geom g, int c3, const double* U3,
-                        int chi3, const int* rank_tab, const int* kcol_tab, const int* colpos_tab, const Z2Layout* L,
+void launch_build_bt_z2(const Tin* Tt, long long tt_inst, const Planes<Tout>& out, long long out_inst, long long ld, Geom g,
+                        int c3, const double* U3, long long u_inst, int chi3, const Z2Tables& t, const Z2Layout* L, int ng,
                         cudaStream_t s) {
   const size_t smem = sizeof(ZAcc<Tout>) * (size_t)chi3 * g.D[c3] * g.D[c3];
   const long long total = (long long)chi3 * g.P * g.P;
-  k_build_bt_z2<Tin, Tout><<<grid_cap(total), 256, smem, s>>>(Tt, out, ld, g.P, g.Sn[c3], g.D[c3], U3, chi3, rank_tab,
-                                                               kcol_tab, colpos_tab, L);
+  k_build_bt_z2<Tin, Tout><<<dim3(grid_cap(total), ng), 256, smem, s>>>(Tt, out, ld, g.P, g.Sn[c3], g.D[c3], U3, chi3, t,
+                                                                        L, tt_inst, out_inst, u_inst);
   count_launches(1);
 }
 
 template <class Tin, class Tout>
-void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, long long sk, long long out_base,
-                   int t0, int Dt, const double* U, int chi, const Z2Layout* L, const int* pi, cudaStream_t s) {
+void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, long long sk, long long out_base, int t0,
+                   int Dt, const double* U, int chi, const Z2Layout* L, const int* pi, const SlotStrides& st,
+                   cudaStream_t s) {
   long long total = 1;
   for (int i = 0; i < rest.ndim; ++i) total *= rest.shape[i];
   const size_t smem = sizeof(ZAcc<Tin>) * (size_t)((chi + 3) / 4 * 4) * Dt * Dt;
   const int n = (int)total;  // rest < 2^31 entries (P^2 chi3 / Dt^2 <= 2.3e9 / 4 for Dcut <= 14)
+  const dim3 grid(grid_cap(total), st.nb, st.ng);
   switch (chi) {
-#define HOTRG_EPI_Z2(C)                                                                                        \
-  case C:                                                                                                      \
-    k_epi_z2<Tin, Tout, C><<<grid_cap(total), 256, smem, s>>>(O, ldO, out, rest, n, sk, out_base, t0, U, L, pi); \
+#define HOTRG_EPI_Z2(C)                                                                                      \
+  case C:                                                                                                    \
+    k_epi_z2<Tin, Tout, C><<<grid, 256, smem, s>>>(O, ldO, out, rest, n, sk, out_base, t0, U, L, pi, st);      \
     break;
     HOTRG_EPI_Z2(1) HOTRG_EPI_Z2(2) HOTRG_EPI_Z2(3) HOTRG_EPI_Z2(4) HOTRG_EPI_Z2(5) HOTRG_EPI_Z2(6)
     HOTRG_EPI_Z2(7) HOTRG_EPI_Z2(8) HOTRG_EPI_Z2(9) HOTRG_EPI_Z2(10) HOTRG_EPI_Z2(11) HOTRG_EPI_Z2(12)
@@ -515,22 +552,26 @@ void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, lon
 }
 
 using bf16 = __nv_bfloat16;
-template void launch_build_y_z2<float, bf16>(const float*, const Planes<bf16>&, long long, Geom, int, const int*,
-                                             const int*, const Z2Layout*, const int*, cudaStream_t);
-template void launch_build_y_z2<double, bf16>(const double*, const Planes<bf16>&, long long, Geom, int, const int*,
-                                              const int*, const Z2Layout*, const int*, cudaStream_t);
-template void launch_build_y_z2<double, double>(const double*, const Planes<double>&, long long, Geom, int,
-                                                const int*, const int*, const Z2Layout*, const int*, cudaStream_t);
-template void launch_build_bt_z2<float, bf16>(const float*, const Planes<bf16>&, long long, Geom, int, const double*,
-                                              int, const int*, const int*, const int*, const Z2Layout*, cudaStream_t);
-template void launch_build_bt_z2<double, double>(const double*, const Planes<double>&, long long, Geom, int,
-                                                 const double*, int, const int*, const int*, const int*,
-                                                 const Z2Layout*, cudaStream_t);
-template void launch_epi_z2<float, float>(const float*, long long, float*, const View&, long long, long long, int,
-                                          int, const double*, int, const Z2Layout*, const int*, cudaStream_t);
-template void launch_epi_z2<float, double>(const float*, long long, double*, const View&, long long, long long, int,
-                                           int, const double*, int, const Z2Layout*, const int*, cudaStream_t);
-template void launch_epi_z2<double, double>(const double*, long long, double*, const View&, long long, long long,
-                                            int, int, const double*, int, const Z2Layout*, const int*, cudaStream_t);
+#define HOTRG_YZ(TI, TO)                                                                                                  \
+  template void launch_build_y_z2<TI, TO>(const TI*, long long, const Planes<TO>&, long long, long long, Geom, int,         \
+                                          const Z2Tables&, const Z2Layout*, const int*, int, int, cudaStream_t);
+HOTRG_YZ(float, bf16)
+HOTRG_YZ(double, bf16)
+HOTRG_YZ(double, double)
+#undef HOTRG_YZ
+#define HOTRG_BTZ(TI, TO)                                                                                                 \
+  template void launch_build_bt_z2<TI, TO>(const TI*, long long, const Planes<TO>&, long long, long long, Geom, int,        \
+                                           const double*, long long, int, const Z2Tables&, const Z2Layout*, int,          \
+                                           cudaStream_t);
+HOTRG_BTZ(float, bf16)
+HOTRG_BTZ(double, double)
+#undef HOTRG_BTZ
+#define HOTRG_EPIZ(TI, TO)                                                                                               \
+  template void launch_epi_z2<TI, TO>(const TI*, long long, TO*, const View&, long long, long long, int, int,             \
+                                      const double*, int, const Z2Layout*, const int*, const SlotStrides&, cudaStream_t);
+HOTRG_EPIZ(float, float)
+HOTRG_EPIZ(float, double)
+HOTRG_EPIZ(double, double)
+#undef HOTRG_EPIZ
 
 }  // namespace hotrg

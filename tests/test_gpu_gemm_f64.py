@@ -1,0 +1,115 @@
+"""The FP64 product from exact integer slices (csrc/gemm_f64tc.cu) at the edges of its tiles, its ring and its sums."""
+import math
+from ctypes import c_void_p
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def gemm_f64(A, B, cta_group=1, pad=0):
+    import torch
+    from paper_1906_06060_gb300 import _lib
+    lib = _lib.load()
+    M, K = A.shape
+    N = B.shape[0]
+    a, b = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = torch.full((M, N + pad), -7.0, dtype=torch.float64, device="cuda")
+    n = lib.hotrg_gemm_f64_scratch_bytes(M, N, K)
+    scratch = torch.empty(n, dtype=torch.uint8, device="cuda")
+    s = c_void_p(torch.cuda.current_stream().cuda_stream)
+    _lib.check(lib.hotrg_gemm_f64(c_void_p(a.data_ptr()), K, c_void_p(b.data_ptr()), K, c_void_p(C.data_ptr()), N + pad,
+                                  M, N, K, cta_group, c_void_p(scratch.data_ptr()), n, s), "hotrg_gemm_f64")
+    _lib.check(lib.hotrg_gemm_status(c_void_p(scratch.data_ptr()), s), "status")
+    out = C.cpu().numpy()
+    assert np.all(out[:, N:] == -7.0)  # nothing beyond the columns is written
+    return out[:, :N]
+
+
+SHAPES = [(128, 256, 64), (129, 257, 65), (257, 511, 128), (256, 512, 1000), (300, 1030, 1023), (625, 260, 2049)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("cta_group", [1, 2])
+def test_integers_are_exact(M, N, K, cta_group):
+    """Entries of at most 20 bits fit the rows' fixed-point numbers whatever their power-of-two scale, and their
+    sums fit 53 bits: the product has no rounding at all."""
+    rng = np.random.default_rng(M + N + K)
+    a = rng.integers(-(2 ** 20) + 1, 2 ** 20, (M, K))
+    b = rng.integers(-(2 ** 20) + 1, 2 ** 20, (N, K))
+    a[3] = 0
+    b[:, 0] = 2 ** 20 - 1
+    ea, eb = rng.integers(-300, 300, M), rng.integers(-300, 300, N)
+    ref = np.ldexp((a @ b.T).astype(np.float64), ea[:, None] + eb[None, :])
+    got = gemm_f64(np.ldexp(a.astype(np.float64), ea[:, None]), np.ldexp(b.astype(np.float64), eb[:, None]), cta_group,
+                   pad=(-N) % 4 + (4 if N % 2 else 0))
+    assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("signs", [False, True])
+def test_largest_digits_fill_the_accumulators_exactly(signs):
+    """Every digit at +-128, a whole number of accumulator chains: the sums reach their bounds. The exact value of an
+    entry is an integer times (sum_i 2^(-8 i))^2, rounded once (and once more by the level-6 carry)."""
+    from fractions import Fraction
+    rng = np.random.default_rng(5)
+    x = sum(2.0 ** (-8 * i) for i in range(7))  # the eighth digit does not fit a double beside the first
+    M, N, K = 128, 256, 2048
+    sa = np.where(rng.random((M, K)) < 0.5, -1.0, 1.0) if signs else np.ones((M, K))
+    sb = np.where(rng.random((N, K)) < 0.5, -1.0, 1.0) if signs else np.ones((N, K))
+    ref = (sa @ sb.T) * float(Fraction(x) ** 2)
+    # fixed-point rows hold x exactly; far below one digit pair of the levels that are kept
+    assert np.abs(gemm_f64(x * sa, x * sb) - ref).max() <= K * 2.0 ** -52
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 400, 777), (128, 300, 4100)])
+@pytest.mark.parametrize("decay", [0.0, 0.01])
+def test_error_is_below_the_fp64_chains(M, N, K, decay):
+    """Gaussian rows, flat and decaying over many orders: against exactly summed products, within one rounding of the
+    result plus K 2^-55 of the rows' largest entries (2^-56 from each operand's fixed point, entries of the other below
+    its row's largest, and the dropped digit pairs), and in the 2-norm no further off than NumPy's FP64 product."""
+    rng = np.random.default_rng(K)
+    w = np.exp(-decay * np.arange(K))
+    A, B = rng.standard_normal((M, K)) * w, rng.standard_normal((N, K)) * w
+    got = gemm_f64(A, B)
+    host = A @ B.T
+    rows, cols = rng.integers(0, M, 300), rng.integers(0, N, 300)
+    e, e_host = [], []
+    for m, n in zip(rows, cols):
+        p = A[m] * B[n]
+        split = 134217729.0  # Dekker's exact product: p + err == A B
+        ah, bh = A[m] * split, B[n] * split
+        ah, bh = ah - (ah - A[m]), bh - (bh - B[n])
+        al, bl = A[m] - ah, B[n] - bh
+        err = ((ah * bh - p) + ah * bl + al * bh) + al * bl
+        ref = math.fsum(np.concatenate([p, err]))
+        tol = 2.0 ** -52 * abs(ref) + 2 * K * 2.0 ** -55 * np.abs(A[m]).max() * np.abs(B[n]).max()
+        assert abs(got[m, n] - ref) <= tol
+        e.append(got[m, n] - ref)
+        e_host.append(host[m, n] - ref)
+    assert np.linalg.norm(e) <= np.linalg.norm(e_host)
+
+
+def test_non_finite_rows_and_zero_rows():
+    rng = np.random.default_rng(0)
+    A, B = rng.standard_normal((130, 100)), rng.standard_normal((300, 100))
+    A[3, 5], A[7, 1], B[11, 99] = np.nan, np.inf, -np.inf
+    A[20] = 0.0
+    A[21] *= 1e-310  # subnormal entries
+    C = gemm_f64(A, B)
+    bad = np.zeros(C.shape, dtype=bool)
+    bad[[3, 7]] = True
+    bad[:, 11] = True
+    assert np.array_equal(np.isnan(C), bad)
+    assert np.all(C[20][~bad[20]] == 0.0)
+    ref = A[21] @ np.where(np.isfinite(B), B, 0.0).T
+    assert np.abs(C[21] - ref)[~bad[21]].max() <= 1e-320
+
+
+@pytest.mark.parametrize("M,N,K", [(127, 256, 64), (128, 255, 64), (128, 256, 63), (128, 256, 16321)])
+def test_shapes_it_does_not_take(M, N, K):
+    from paper_1906_06060_gb300 import _lib
+    lib = _lib.load()
+    assert lib.hotrg_gemm_f64_scratch_bytes(M, N, K) == 0
+    p = c_void_p(256)
+    assert lib.hotrg_gemm_f64(p, K, p, K, p, N, M, N, K, 1, p, 1 << 40, None) == _lib.HOTRG_EINVAL
