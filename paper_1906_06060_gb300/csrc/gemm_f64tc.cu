@@ -73,7 +73,7 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
       : "memory");
 }
-// issued by the first CTA of a pair for either CTA (see tma_load_3d_pair)
+// the same from either CTA of a pair: `dst` in its own shared memory, the bytes count on the first CTA's barrier `bar`
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
                                                  int z, int w) {
   asm volatile(
@@ -186,7 +186,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int total = s_total;
 
   if (warp == 0) {
-    if (lane == 0 && leader) {
+    // every CTA copies its own tiles (128 rows of A, its share of the B rows); a pair's bytes all count on the first
+    // CTA's barriers, and a stage is freed in both CTAs by the commit of the MMAs that read it
+    if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
       long long issued = 0;
@@ -195,8 +197,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         int inst, mt, nt;
         Blk bk;
         locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
-        const int arow = bk.m0 + mt * TC_BM * CG;
-        const int brow = bk.n0 + nt * TC_BN;
+        const int arow = bk.m0 + mt * TC_BM * CG + (int)rank * TC_BM;
+        const int brow = bk.n0 + nt * TC_BN + (int)rank * B_ROWS;
         const int binst = inst / p.b_div;
         for (int s = NSL - 1; s >= 0 && ok; --s)
           for (int kb = 0; kb < bk.num_kb && ok; ++kb) {
@@ -205,25 +207,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.timeout_ns)) { ok = false; break; }
               const uint32_t fb = full0 + 8 * stage;
               const uint32_t sa = smem_u32(smem + stage * STAGE_BYTES), sb = sa + A_TILE;
-              mbar_expect_tx(fb, CG * STAGE_BYTES);
+              if (leader) mbar_expect_tx(fb, CG * STAGE_BYTES);
               if constexpr (CG == 1) {
                 tma_load_4d(sa, &maps.a, fb, kx, arow, i, inst);
                 tma_load_4d(sb, &maps.b, fb, kx, brow, s - i, binst);
               } else {
-                tma_load_4d_pair(sa, &maps.a, fb, kx, arow, i, inst);
-                tma_load_4d_pair(sb, &maps.b, fb, kx, brow, s - i, binst);
-                tma_load_4d_pair(mapa_rank(sa, 1), &maps.a, fb, kx, arow + TC_BM, i, inst);
-                tma_load_4d_pair(mapa_rank(sb, 1), &maps.b, fb, kx, brow + B_ROWS, s - i, binst);
+                const uint32_t fb0 = mapa_rank(fb, 0);
+                tma_load_4d_pair(sa, &maps.a, fb0, kx, arow, i, inst);
+                tma_load_4d_pair(sb, &maps.b, fb0, kx, brow, s - i, binst);
               }
               ++issued;
               if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
           }
       }
-      // drain the copies in flight on every exit path (see k_gemm_split)
-      for (long long i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i)
-        mbar_wait(full0 + 8 * (int)(i % STAGES), (uint32_t)((i / STAGES) & 1), abort_flag, drain_ns(p.timeout_ns),
-                  false);
+      // drain the copies in flight on every exit path (see k_gemm_split); the second CTA of a pair waits for the first at
+      // the final cluster barrier
+      if (leader) {
+        for (long long i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i)
+          mbar_wait(full0 + 8 * (int)(i % STAGES), (uint32_t)((i / STAGES) & 1), abort_flag, drain_ns(p.timeout_ns),
+                    false);
+        // a given-up pair may have copies of the second CTA in flight for a stage this CTA never announced: they
+        // always land, within microseconds
+        if (CG == 2 && !ok)
+          for (const unsigned long long t0 = globaltimer_ns(); globaltimer_ns() - t0 < 2000000ull;) {}
+      }
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {
@@ -250,7 +258,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
               for (int k = 0; k < SBK / 16; ++k)
                 mma_f16<CG>(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), p.idesc, (t | k) ? 1u : 0u);
-              mma_commit_local<CG>(empty0 + 8 * stage);
+              mma_commit<CG>(empty0 + 8 * stage);
               if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
             if (!ok) break;
@@ -336,34 +344,41 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int* eb = p.eb + (long long)(inst / p.b_div) * p.eb_inst + col0;
         double* dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
         const bool v4 = p.vec == 4 && (bk.n0 & 3) == 0 && col0 + 128 <= col_end;
-        // every level comes back from the scratch area (this thread's own stores): a rolled loop over four columns,
-        // since 128 unrolled assemblies from registers (300 KB of code) ran from the instruction cache's misses
-        auto value = [&](const int4* l, int u, int ebj) -> double {
-          auto at = [&](int k) { return (long long)reinterpret_cast<const int*>(l + k)[u]; };
-          if (ea == kExpNaN || ebj == kExpNaN) return nan("");
-          return assemble((at(5) << 16) + (at(4) << 8) + at(3), (at(2) << 16) + (at(1) << 8) + at(0), ea + ebj - 54);
-        };
-#pragma unroll 2
-        for (int j = 0; j < 128; j += 4) {
-          if (col0 + j >= col_end) break;
-          int4 l[SC_PLANES];
+        // every level comes back from the scratch area (this thread's own stores) in a rolled loop: 128 unrolled
+        // assemblies from registers (300 KB of code) ran from the instruction cache's misses. All loads of 16 columns
+        // are in flight together: the loop is bound by their latency
+        constexpr int JG = 4;
+        for (int j0 = 0; j0 < 128; j0 += 4 * JG) {
+          if (col0 + j0 >= col_end) break;
+          int4 l[JG][SC_PLANES];
 #pragma unroll
-          for (int k = 0; k < SC_PLANES; ++k) l[k] = park[(k * 32 + j / 4) * TC_FOLD_THREADS];
-          double v[4];
+          for (int g = 0; g < JG; ++g)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) v[u] = col0 + j + u < col_end ? value(l, u, eb[j + u]) : 0.0;
-          if (v4) {
-            if (p.accumulate) {
+            for (int k = 0; k < SC_PLANES; ++k) l[g][k] = park[(k * 32 + j0 / 4 + g) * TC_FOLD_THREADS];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) v[u] += dst[j + u];
+          for (int g = 0; g < JG; ++g) {
+            const int j = j0 + 4 * g;
+            auto value = [&](int u) -> double {
+              if (col0 + j + u >= col_end) return 0.0;
+              auto at = [&](int k) { return (long long)(u == 0 ? l[g][k].x : u == 1 ? l[g][k].y : u == 2 ? l[g][k].z : l[g][k].w); };
+              const int ebj = eb[j + u];
+              if (ea == kExpNaN || ebj == kExpNaN) return nan("");
+              return assemble((at(5) << 16) + (at(4) << 8) + at(3), (at(2) << 16) + (at(1) << 8) + at(0), ea + ebj - 54);
+            };
+            double v[4] = {value(0), value(1), value(2), value(3)};
+            if (v4) {
+              if (p.accumulate) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] += dst[j + u];
+              }
+              asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + j), "d"(v[0]), "d"(v[1]), "d"(v[2]),
+                           "d"(v[3])
+                           : "memory");
+            } else {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (col0 + j + u < col_end) dst[j + u] = p.accumulate ? dst[j + u] + v[u] : v[u];
             }
-            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + j), "d"(v[0]), "d"(v[1]), "d"(v[2]),
-                         "d"(v[3])
-                         : "memory");
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              if (col0 + j + u < col_end) dst[j + u] = p.accumulate ? dst[j + u] + v[u] : v[u];
           }
         }
       }
@@ -548,6 +563,12 @@ int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, 
                        long long K, int* scratch, int* status, double timeout_s, cudaStream_t s, const GemmBlocks* blk,
                        const GemmBatch* bat, bool accumulate, int cta_group) {
   if (!slices_take(M, N, K)) return HOTRG_EINVAL;
+  if (cta_group == 0) {
+    // pairs (half the B copies per SM: 789 against 831 us at 1000 x 10000 x 1000) where their 256-row tiles pad no more
+    // rows than 128-row ones (else slower by what they pad: 768 against 640 rows at M = 625)
+    const long long m = blk ? (M + 1) / 2 : M;
+    cta_group = (m + 255) / 256 * 2 == (m + 127) / 128 ? 2 : 1;
+  }
   const int batch = bat ? bat->batch : 1;
   if (batch < 1 || batch > kMaxGemmBatch || (A.ld % 8) || (B.ld % 8) || A.ld < K || B.ld < K || ldc < N)
     return HOTRG_EINVAL;

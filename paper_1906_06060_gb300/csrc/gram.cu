@@ -126,7 +126,21 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
     rowoffA[q] = ra < nr ? (long long)(ra / Da) * S1 + (long long)(ra % Da) * S2 : -1;
     rowoffB[q] = rb < nr ? (long long)(rb / Da) * S1 + (long long)(rb % Da) * S2 : -1;
   }
-  const int tx = tid % (GT / 4), ty = tid / (GT / 4);
+  // 4 x 4 outputs per thread. A diagonal tile of a symmetric product needs the blocks on and above its diagonal only: the
+  // first T (T + 1) / 2 threads take them, row by row, the other warps sit out the FP64 work, which is what bounds the
+  // kernel (13 blocks an edge: 91 of 169; steady block-sparse step at bond dimension 10, all on diagonal tiles: 67.7 ms
+  // with all blocks)
+  constexpr int EB = GT / 4;
+  int tx = tid % EB, ty = tid / EB;
+  bool mine = true;
+  const bool diag = sym && tr == tc;  // (rows and columns of the tile are the same entries)
+  if (diag) {
+    mine = tid < EB * (EB + 1) / 2;
+    ty = 0;
+    for (int left = tid; mine && left >= EB - ty; ++ty) left -= EB - ty;
+    tx = mine ? ty + (tid - (ty * EB - ty * (ty - 1) / 2)) : 0;
+    if (!mine) ty = 0;
+  }
   double acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -135,32 +149,32 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
 
   for (long long kc = kb; kc < ke; kc += GK) {
     if (tid < GK) {
-      long long col = kc + tid;
       long long off = -1;
-      if (col < ke) {
+      if (kc + tid < ke) {
+        unsigned col = (unsigned)(kc + tid);  // K = P^2 / nr < 2^31
         off = 0;
         if (colcls < 0) {
           for (int l = li.nrest - 1; l >= 0; --l) {
-            const long long c = col % li.dim[l];
-            col /= li.dim[l];
+            const unsigned c = col % (unsigned)li.dim[l];
+            col /= (unsigned)li.dim[l];
             off += c * li.stride[l];
           }
         } else {
           // blocked order inside the class: patterns of that parity in increasing order, then
           // row-major inside the pattern's box
-          long long local = col - (colcls ? K0 : 0);
+          unsigned local = col - (unsigned)(colcls ? K0 : 0);
           int pat = 0;
           for (; pat < (1 << li.nrest); ++pat) {
             if ((__popc(pat) & 1) != colcls) continue;
-            if (local < patsz[pat]) break;
-            local -= patsz[pat];
+            if (local < (unsigned)patsz[pat]) break;
+            local -= (unsigned)patsz[pat];
           }
           for (int l = li.nrest - 1; l >= 0; --l) {
             const int bit = (pat >> l) & 1;
-            const int dl = bit ? li.dim[l] - e_rest[l] : e_rest[l];
-            const long long c = local % dl;
+            const unsigned dl = bit ? li.dim[l] - e_rest[l] : e_rest[l];
+            const unsigned c = local % dl;
             local /= dl;
-            off += (c + (bit ? e_rest[l] : 0)) * li.stride[l];
+            off += (long long)(c + (bit ? e_rest[l] : 0)) * li.stride[l];
           }
         }
       }
@@ -172,16 +186,17 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
       const long long co = coloff[kk];
       const long long ra = rowoffA[rr], rb = rowoffB[rr];
       As[kk][rr] = (co >= 0 && ra >= 0) ? TA[ra + co] : 0.0;
-      Bs[kk][rr] = (co >= 0 && rb >= 0) ? TB[rb + co] : 0.0;
+      if (!diag) Bs[kk][rr] = (co >= 0 && rb >= 0) ? TB[rb + co] : 0.0;
     }
     __syncthreads();
+    if (mine)
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
       double a[4], b[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+      for (int j = 0; j < 4; ++j) b[j] = (diag ? As : Bs)[kk][tx * 4 + j];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -191,6 +206,7 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
   }
   // partial sums at the rows' positions in parity order (base + class-local index)
   double* out = partial + (long long)split * nr * nr;
+  if (!mine) return;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty * 4 + i;
@@ -203,41 +219,50 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
   }
 }
 
-// Q[e] = sum over the splits in a fixed order; with sym, entries below the diagonal tiles read
-// their mirror; with ev, the partial sums are in parity row order.
-__global__ void k_reduce_splits(const double* __restrict__ partial, int nsplit, int nr, int gt, int sym,
-                                double* __restrict__ Q, long long q_stride, const int* __restrict__ ev,
-                                int ax1, int ax2, int Da) {
+// Q[e] = sum over the splits in a fixed order; with sym, entries below the diagonal's 4 x 4 blocks read
+// their mirror; with ev, the partial sums are in parity row order. A block covers 32 entries, each split over REDUCE_Y
+// threads (a small Gram matrix has over a thousand splits: one thread an entry took 100 us).
+constexpr int REDUCE_Y = 16;
+__global__ void __launch_bounds__(32 * REDUCE_Y) k_reduce_splits(const double* __restrict__ partial, int nsplit, int nr,
+                                                                 int sym, double* __restrict__ Q, long long q_stride,
+                                                                 const int* __restrict__ ev, int ax1, int ax2, int Da) {
+  __shared__ double part[REDUCE_Y][32];
   const int nn = nr * nr;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nn) return;
+  const int e = blockIdx.x * 32 + threadIdx.x;
   partial += (long long)blockIdx.y * nsplit * nn;
   Q += (long long)blockIdx.y * q_stride;
-  int r = e / nr, c = e % nr;
-  int base = 0;
-  if (ev) {
-    // rows of different parity: zero; otherwise the class-local positions in parity order
-    const int e1 = ev[blockIdx.y * kMaxD + ax1], e2 = ev[blockIdx.y * kMaxD + ax2];
-    int neven = 0, br = 0, bc = 0;
-    const int pr = gram_row_par(r, Da, e1, e2), pc = gram_row_par(c, Da, e1, e2);
-    if (pr != pc) {
-      Q[e] = 0.0;
-      return;
+  int src = -1;  // position of the entry's partial sums, -1: zero
+  if (e < nn) {
+    int r = e / nr, c = e % nr, base = 0;
+    bool zero = false;
+    if (ev) {
+      // rows of different parity: zero; otherwise the class-local positions in parity order
+      const int e1 = ev[blockIdx.y * kMaxD + ax1], e2 = ev[blockIdx.y * kMaxD + ax2];
+      int neven = 0, br = 0, bc = 0;
+      const int pr = gram_row_par(r, Da, e1, e2), pc = gram_row_par(c, Da, e1, e2);
+      zero = pr != pc;
+      for (int q = 0; q < nr && !zero; ++q) {
+        const int pq = gram_row_par(q, Da, e1, e2);
+        neven += pq == 0;
+        if (q < r && pq == pr) ++br;
+        if (q < c && pq == pc) ++bc;
+      }
+      base = pr ? neven : 0;
+      r = br;
+      c = bc;
     }
-    for (int q = 0; q < nr; ++q) {
-      const int pq = gram_row_par(q, Da, e1, e2);
-      neven += pq == 0;
-      if (q < r && pq == pr) ++br;
-      if (q < c && pq == pc) ++bc;
-    }
-    base = pr ? neven : 0;
-    r = br;
-    c = bc;
+    if (!zero) src = (sym && r / 4 > c / 4) ? (base + c) * nr + base + r : (base + r) * nr + base + c;
   }
-  const int src = (sym && r / gt > c / gt) ? (base + c) * nr + base + r : (base + r) * nr + base + c;
   double s = 0.0;
-  for (int k = 0; k < nsplit; ++k) s += partial[(long long)k * nn + src];
-  Q[e] = s;
+  if (src >= 0)
+    for (int k = threadIdx.y; k < nsplit; k += REDUCE_Y) s += partial[(long long)k * nn + src];
+  part[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && e < nn) {
+    s = 0.0;
+    for (int y = 0; y < REDUCE_Y; ++y) s += part[y][threadIdx.x];
+    Q[e] = s;
+  }
 }
 
 __global__ void k_gram_combine(const double* __restrict__ Q1, const double* __restrict__ Q2, long long q_stride,
@@ -288,15 +313,17 @@ __global__ void k_gram_combine_tangent(const double* __restrict__ Q1, const doub
 
 }  // namespace
 
-// Tile edge for nr x nr outputs: the candidate that computes the fewest padded entries.
+// Tile edge for nr x nr outputs: the candidate whose warps issue the fewest FP64 operations (whole warps of 4 x 4 blocks:
+// all of a tile off the diagonal, the upper triangle of one on it).
 static int gram_tile(int nr, bool sym) {
-  const int cand[5] = {36, 44, 52, 60, 64};
+  const int cand[7] = {20, 28, 36, 44, 52, 60, 64};
   int best = 64;
-  long long best_area = -1;
+  long long best_warps = -1;
   for (int gt : cand) {
-    const long long n = (nr + gt - 1) / gt;
-    const long long area = (sym ? n * (n + 1) / 2 : n * n) * gt * gt;
-    if (best_area < 0 || area < best_area) { best_area = area; best = gt; }
+    const long long n = (nr + gt - 1) / gt, t = gt / 4;
+    const long long full = (t * t + 31) / 32, tri = (t * (t + 1) / 2 + 31) / 32;
+    const long long warps = sym ? n * tri + n * (n - 1) / 2 * full : n * n * full;
+    if (best_warps < 0 || warps < best_warps) { best_warps = warps; best = gt; }
   }
   return best;
 }
@@ -364,13 +391,13 @@ void launch_half_gram(const double* T, long long t_stride, int batch, Geom g, in
                                                             Da, nr, K, ntile, sym ? 1 : 0, nsplit, partial,      \
                                                             z2ev);                                               \
     break;
-    HOTRG_GRAM(36) HOTRG_GRAM(44) HOTRG_GRAM(52) HOTRG_GRAM(60) HOTRG_GRAM(64)
+    HOTRG_GRAM(20) HOTRG_GRAM(28) HOTRG_GRAM(36) HOTRG_GRAM(44) HOTRG_GRAM(52) HOTRG_GRAM(60) HOTRG_GRAM(64)
 #undef HOTRG_GRAM
   }
   count_launches(1);
   const int nn = nr * nr;
-  k_reduce_splits<<<dim3((nn + 255) / 256, batch), 256, 0, s>>>(partial, nsplit, nr, gt, sym ? 1 : 0, Q, q_stride,
-                                                                 z2ev, li.ax1, li.ax2, Da);
+  k_reduce_splits<<<dim3((nn + 31) / 32, batch), dim3(32, REDUCE_Y), 0, s>>>(partial, nsplit, nr, sym ? 1 : 0, Q, q_stride,
+                                                                             z2ev, li.ax1, li.ax2, Da);
   count_launches(1);
 }
 
