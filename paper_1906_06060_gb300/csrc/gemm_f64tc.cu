@@ -19,7 +19,7 @@
 //
 // Work: 36 tensor products of 2 M N K flops against one on the FP64 units at 1/2000 of the rate.
 // Kernel structure, ring and bounded waits as k_gemm_split (gemm_tc.cu): warp 0 copies, warp 1 issues MMAs, warps
-// 2-9 fold. Per output tile the levels run one after the other, least significant first, each over all k-blocks; a
+// 4-11 fold. Per output tile the levels run one after the other, least significant first, each over all k-blocks; a
 // ring stage holds one digit tile of A and one of B. A finished level sum goes to a per-CTA scratch area in global
 // memory (L2), one 16-byte access per thread and four columns, coalesced; the last level combines them in registers.
 #include "tc_ptx.cuh"
@@ -185,6 +185,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   const int total = s_total;
 
+  if (warp < TC_FOLD_WARP0) {
+  regs_give<TC_ROLE_REGS>();
   if (warp == 0) {
     // every CTA copies its own tiles (128 rows of A, its share of the B rows); a pair's bytes all count on the first
     // CTA's barriers, and a stage is freed in both CTAs by the commit of the MMAs that read it
@@ -270,9 +272,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       mma_commit_local<CG>(final_bar);
       mbar_wait(final_bar, 0, abort_flag, drain_ns(p.timeout_ns), false);
     }
+  }
   } else {
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const int ftid = (int)threadIdx.x - 64;
+    regs_take<TC_FOLD_REGS>();
+    const int q = warp & 3, half = (warp - TC_FOLD_WARP0) >> 2;
+    const int ftid = (int)threadIdx.x - 32 * TC_FOLD_WARP0;
     int4* const park = p.scratch + (size_t)blockIdx.x * (SC_PLANES * 32 * TC_FOLD_THREADS) + ftid;
     const uint32_t tempty_dst = CG == 2 && !leader ? mapa_rank(tempty0, 0) : tempty0;
     int buf = 0;
@@ -299,13 +303,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           tc_fence_after();
           const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * TC_BN + half * 128);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            // one 32-column load at a time: two would not fit beside the 128 sums
-            uint32_t r[32];
-            tmem_ld32(taddr + c * 32, r);
+          for (int c = 0; c < 4; c += 2) {
+            uint32_t r0[32], r1[32];
+            tmem_ld32(taddr + c * 32, r0);
+            tmem_ld32(taddr + (c + 1) * 32, r1);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) acc[c * 32 + j] += __float2int_rn(__uint_as_float(r[j]));
+            for (int j = 0; j < 32; ++j) {
+              acc[c * 32 + j] += __float2int_rn(__uint_as_float(r0[j]));
+              acc[(c + 1) * 32 + j] += __float2int_rn(__uint_as_float(r1[j]));
+            }
           }
           tc_fence_before();
           __syncwarp();
@@ -524,6 +531,9 @@ int launch_slices_variant(long long tiles, const SliceOperand& A, const SliceOpe
         return HOTRG_EDEVICE;
       }
     }
+    // the register shares need what they were planned with
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs < TC_LAUNCH_REGS) return HOTRG_EDEVICE;
     resident[dev].store(n);
   }
   // the scratch area holds kSliceCtas CTAs

@@ -25,15 +25,15 @@
 // small cross terms first so the large hi*hi products meet a small accumulator) and each
 // k-block's partial sum is folded into an FP32 register accumulator with round-to-nearest adds.
 //
-// Kernel structure (one CTA per SM, persistent over output tiles, 320 threads):
+// Kernel structure (one CTA per SM, persistent over output tiles, 384 threads):
 //   warp 0      TMA producer: per k-block loads every 16-bit plane of the 128 x BK A tile and
 //               of the 256 x BK B tile (BK*2-byte swizzle) into one stage of a shared-memory
 //               ring, so the passes of a k-block reuse the same stage (BK = 64 or 32).
 //   warp 1      MMA issuer: one thread issues tcgen05.mma.cta_group::1.kind::f16 (M=128,
 //               N=256, K=16) for all passes of one k-block into one of two TMEM buffers (2 x 256
 //               FP32 columns), releases the stage and hands the buffer over with tcgen05.commit.
-//   warps 2-9   fold/epilogue: warp w reads TMEM lanes 32*(w%4).. (its hardware quadrant),
-//               columns 128*((w-2)/4).. of the buffer, adds them into 128 FP32 registers per
+//   warps 4-11  fold/epilogue: warp w reads TMEM lanes 32*(w%4).. (its hardware quadrant),
+//               columns 128*((w-4)/4).. of the buffer, adds them into 128 FP32 registers per
 //               thread and frees the buffer; after the last k-block it stores its 128 columns.
 //
 // CTA pairs (CG = 2, a thread-block cluster of two CTAs on two SMs, one 256 x 256 output tile):
@@ -48,7 +48,8 @@
 // fold warps of both report freed TMEM buffers to the first CTA. Measured reasons: a single CTA's
 // 128 x 256 MMA chain, with operands resident and nothing else running, kept the tensor pipe busy
 // about 2/3 of the time (pairs: about 3/4); and a pair whose second CTA issued its own copies,
-// counted remotely on the first CTA's barrier, lost a quarter of its rate to the cross-SM hand-over.
+// counted remotely on the first CTA's barrier, lost a quarter of its rate to the cross-SM hand-over (again with the
+// stage freed in both CTAs by a multicast commit: 906 -> 1166 ms of GEMM in a steady step at bond dimension 10).
 // Every mbarrier wait is bounded by a timeout; on expiry the CTA records ST_TIMEOUT, drains
 // the copies and MMAs it issued (waits bounded by max(timeout, 1 s): issued work always
 // completes, so a short caller limit never lets the CTA exit before it), frees TMEM and returns.
@@ -74,7 +75,13 @@ struct Cfg {
   static constexpr uint32_t B_TILE = (TC_BN / CG) * BK * 2;
   static constexpr uint32_t STAGE_BYTES = NPL * (A_TILE + B_TILE);
   static constexpr int STAGES = (int)((216u * 1024u) / STAGE_BYTES) > 6 ? 6 : (int)((216u * 1024u) / STAGE_BYTES);
-  static constexpr size_t SMEM = 1024 + STAGES * STAGE_BYTES + 256;
+  // ring, barriers, and STORE_COLS columns of 32 rows (padded by one) per fold warp for ragged stores; the tile prefix is
+  // static shared memory
+  static constexpr size_t BASE = 1024 + STAGES * STAGE_BYTES + 256;
+  static constexpr size_t LEFT = 227 * 1024 - sizeof(int) * (kMaxGemmBatch + 4) - BASE;
+  static constexpr int STORE_COLS = LEFT >= (TC_FOLD_THREADS / 32) * 32 * 9 * sizeof(float) ? 8 : 4;
+  static constexpr size_t SMEM = BASE + (TC_FOLD_THREADS / 32) * 32 * (STORE_COLS + 1) * sizeof(float);
+  static_assert(SMEM - BASE <= LEFT, "a CTA's shared memory");
 };
 
 struct TmapSet {
@@ -110,7 +117,7 @@ struct TcParams {
   long long ldc;
   int* status;
   unsigned long long timeout_ns;
-  int vec4;
+  int vec8;  // rows of C start on 32-byte boundaries
   const GemmBlocks* blk;  // null: one dense product over M x N x K
   uint32_t idesc;         // idesc_for(fp16 operands, CTA group)
   // fp16 operands carry power-of-two scales 2^eA, 2^eB (see Planes): the epilogue multiplies by
@@ -226,6 +233,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   const int total = s_total;
 
+  if (warp < TC_FOLD_WARP0) {
+  regs_give<TC_ROLE_REGS>();
   if (warp == 0) {
     if (lane == 0 && leader) {
       int stage = 0;
@@ -340,9 +349,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       mma_commit_local<CG>(final_bar);
       mbar_wait(final_bar, 0, abort_flag, drain_ns(p.timeout_ns), false);
     }
+  }
   } else {
+    regs_take<TC_FOLD_REGS>();
     const int q = warp & 3;          // TMEM lane quadrant this warp may access
-    const int half = (warp - 2) >> 2;  // which 128 of the 256 columns
+    const int half = (warp - TC_FOLD_WARP0) >> 2;  // which 128 of the 256 columns
     // where this warp reports a freed TMEM buffer: the MMA-issuing CTA's barriers (contiguous in
     // its shared memory, so buffer b's barrier is 8 b bytes further in either address window)
     const uint32_t tempty_dst = CG == 2 && !leader ? mapa_rank(tempty0, 0) : tempty0;
@@ -407,16 +418,41 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const long long row = (long long)bk.m0 + (long long)mt * TC_BM * CG + (long long)rank * TC_BM + q * 32 + lane;
       const long long col0 = (long long)bk.n0 + (long long)nt * TC_BN + half * 128;
       const long long row_end = (long long)bk.m0 + bk.mc, col_end = (long long)bk.n0 + bk.nc;
-      if (row < row_end && col0 < col_end) {
-        float* dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
-        if (p.vec4 && (bk.n0 & 3) == 0 && col0 + 128 <= col_end) {
+      float* const cbase = p.C + (long long)inst * p.c_inst;
+      // Whole rows of 128 columns at 32-byte aligned addresses: each thread stores its row, 32 bytes a time (whole
+      // sectors). Otherwise (ragged columns, an odd row stride, a block that starts off the boundary) the warp passes a few
+      // columns at a time through shared memory and stores 32 bytes of four rows at once: one thread per row would store
+      // single floats, 32 sectors an instruction (2401 x 16807 x 2401, FP16X3: 632 us).
+      if (p.vec8 && (bk.n0 & 7) == 0 && col0 + 128 <= col_end) {
+        if (row < row_end) {
+          float* dst = cbase + row * p.ldc + col0;
 #pragma unroll
-          for (int j = 0; j < 128; j += 4)
-            *reinterpret_cast<float4*>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
-        } else {
+          for (int j = 0; j < 128; j += 8)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + j), "f"(acc[j]),
+                         "f"(acc[j + 1]), "f"(acc[j + 2]), "f"(acc[j + 3]), "f"(acc[j + 4]), "f"(acc[j + 5]),
+                         "f"(acc[j + 6]), "f"(acc[j + 7])
+                         : "memory");
+        }
+      } else if (row - lane < row_end && col0 < col_end) {
+        const int nrow = (int)min(32LL, row_end - (row - lane));
+        constexpr int SC = C::STORE_COLS;  // columns at a time; rows padded by one (no bank conflicts)
+        float* const stg = reinterpret_cast<float*>(smem + TC_STAGES * STAGE_BYTES + 256) + (warp - TC_FOLD_WARP0) * (32 * (SC + 1));
+        float* const put = stg + lane * (SC + 1);
+        const float* const get = stg + lane / SC * (SC + 1) + lane % SC;
+        float* dst = cbase + (row - lane + lane / SC) * p.ldc + col0 + lane % SC;
+        const int left = (int)min(128LL, col_end - col0) - lane % SC;
 #pragma unroll
-          for (int j = 0; j < 128; ++j)
-            if (col0 + j < col_end) dst[j] = acc[j];
+        for (int c = 0; c < 128; c += SC) {
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < SC; ++u) put[u] = acc[c + u];
+          __syncwarp();
+          if (c < left) {
+            float* d = dst + c;
+#pragma unroll 2
+            for (int r = 0; r < 32; r += 32 / SC, d += 32 / SC * p.ldc)
+              if (r + lane / SC < nrow) *d = get[r * (SC + 1)];
+          }
         }
       }
     }
@@ -518,6 +554,9 @@ int launch_variant(long long tiles, const Planes<__nv_bfloat16>& A, long long ld
         return HOTRG_EDEVICE;
       }
     }
+    // the register shares need what they were planned with
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs < TC_LAUNCH_REGS) return HOTRG_EDEVICE;
     resident[dev].store(n);
   }
   const long long units = tiles >= 0 && tiles < n ? (tiles > 0 ? tiles : 1) : n;
@@ -573,7 +612,7 @@ int launch_gemm_split(const Planes<__nv_bfloat16>& A, long long lda, const Plane
   p.ldc = ldc;
   p.status = status;
   p.timeout_ns = (unsigned long long)(timeout_s * 1e9);
-  p.vec4 = ((ldc % 4) == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0);
+  p.vec8 = (ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(C) & 31) == 0 && (!bat || bat->c_inst % 8 == 0);
   p.blk = blk;
   p.idesc = idesc_for(A.fmt == 1, cta_group);
   p.amaxA = A.fmt == 1 ? A.amax : nullptr;

@@ -43,18 +43,23 @@ __device__ int gram_row_sorted(int s, int nr, int Da, int e1, int e2, int neven)
   return 0;
 }
 
-// Output tiles of edge GT ((GT/4)^2 threads, 4 x 4 outputs each). With sym (TA = TB: Q is
-// symmetric) only the tiles on and above the diagonal are computed; the reduction mirrors the
-// rest. Rows of a tile come from TA, columns from TB (both T for the Gram itself; the tangent dT
+// Output tiles of edge GT in 4 x 4 blocks. With sym (TA = TB: Q is symmetric) only the tiles on and above the diagonal are
+// computed, and of a diagonal tile only the blocks on and above its diagonal; the reduction mirrors the rest. A CTA has
+// one thread per block of a diagonal tile; off the diagonal a thread takes two blocks. Every warp has FP64 work: with one
+// thread per block of the full tile, a diagonal tile's working warps were the first ones of every CTA and shared a part
+// of the SM's FP64 units. Rows of a tile come from TA, columns from TB (both T for the Gram itself; the tangent dT
 // and T for its derivative).
+constexpr int gram_threads(int gt) { return (gt / 4 * (gt / 4 + 1) / 2 + 31) / 32 * 32; }
+constexpr int gram_blocks(int gt) { return (gt / 4 * (gt / 4) + gram_threads(gt) - 1) / gram_threads(gt); }
+
 template <int GT>
-__global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double* __restrict__ TA,
+__global__ void __launch_bounds__(gram_threads(GT)) k_half_gram(const double* __restrict__ TA,
                                                                    const double* __restrict__ TB, long long t_stride,
                                                                    LegInfo li, long long S1, long long S2, int Da,
                                                                    int nr, long long K, int ntile, int sym,
                                                                    int nsplit, double* __restrict__ partial,
                                                                    const int* __restrict__ ev) {
-  constexpr int NT = (GT / 4) * (GT / 4);
+  constexpr int NT = gram_threads(GT), NB = gram_blocks(GT);
   TA += (long long)blockIdx.z * t_stride;
   TB += (long long)blockIdx.z * t_stride;
   partial += (long long)blockIdx.z * nsplit * nr * nr;
@@ -126,26 +131,35 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
     rowoffA[q] = ra < nr ? (long long)(ra / Da) * S1 + (long long)(ra % Da) * S2 : -1;
     rowoffB[q] = rb < nr ? (long long)(rb / Da) * S1 + (long long)(rb % Da) * S2 : -1;
   }
-  // 4 x 4 outputs per thread. A diagonal tile of a symmetric product needs the blocks on and above its diagonal only: the
-  // first T (T + 1) / 2 threads take them, row by row, the other warps sit out the FP64 work, which is what bounds the
-  // kernel (13 blocks an edge: 91 of 169; steady block-sparse step at bond dimension 10, all on diagonal tiles: 67.7 ms
-  // with all blocks)
   constexpr int EB = GT / 4;
-  int tx = tid % EB, ty = tid / EB;
-  bool mine = true;
   const bool diag = sym && tr == tc;  // (rows and columns of the tile are the same entries)
-  if (diag) {
-    mine = tid < EB * (EB + 1) / 2;
-    ty = 0;
-    for (int left = tid; mine && left >= EB - ty; ++ty) left -= EB - ty;
-    tx = mine ? ty + (tid - (ty * EB - ty * (ty - 1) / 2)) : 0;
-    if (!mine) ty = 0;
+  int tx[NB], ty[NB];
+  bool mine[NB];
+  // blocks that hold outputs (a class a little larger than the tile leaves most of the next tile empty: 58 rows of a bond
+  // with 7 + 3 values cost four times a class of 50)
+  const int vr = min(EB, (ncls - r0 + 3) / 4), vc = min(EB, (ncls - c0 + 3) / 4);
+#pragma unroll
+  for (int u = 0; u < NB; ++u) {
+    const int blk = tid + u * NT;
+    mine[u] = blk < (diag ? vr * (vr + 1) / 2 : vr * vc);
+    if (diag) {
+      // blocks on and above the diagonal, row by row
+      int row = 0, left = mine[u] ? blk : 0;
+      while (left >= vr - row) left -= vr - row++;
+      ty[u] = row;
+      tx[u] = row + left;
+    } else {
+      ty[u] = mine[u] ? blk / vc : 0;
+      tx[u] = mine[u] ? blk % vc : 0;
+    }
   }
-  double acc[4][4];
+  double acc[NB][4][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int u = 0; u < NB; ++u)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[u][i][j] = 0.0;
 
   for (long long kc = kb; kc < ke; kc += GK) {
     if (tid < GK) {
@@ -189,32 +203,39 @@ __global__ void __launch_bounds__((GT / 4) * (GT / 4)) k_half_gram(const double*
       if (!diag) Bs[kk][rr] = (co >= 0 && rb >= 0) ? TB[rb + co] : 0.0;
     }
     __syncthreads();
-    if (mine)
 #pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
+    for (int u = 0; u < NB; ++u) {
+      if (u > 0 && diag) break;
+      if (!mine[u]) continue;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+      for (int kk = 0; kk < GK; ++kk) {
+        double a[4], b[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = (diag ? As : Bs)[kk][tx * 4 + j];
+        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty[u] * 4 + i];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < 4; ++j) b[j] = (diag ? As : Bs)[kk][tx[u] * 4 + j];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[u][i][j] = fma(a[i], b[j], acc[u][i][j]);
+      }
     }
     __syncthreads();
   }
   // partial sums at the rows' positions in parity order (base + class-local index)
   double* out = partial + (long long)split * nr * nr;
-  if (!mine) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = r0 + ty * 4 + i;
-    if (r >= ncls) continue;
+  for (int u = 0; u < NB; ++u) {
+    if (!mine[u]) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = c0 + tx * 4 + j;
-      if (c < ncls) out[(long long)(base + r) * nr + base + c] = acc[i][j];
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + ty[u] * 4 + i;
+      if (r >= ncls) continue;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = c0 + tx[u] * 4 + j;
+        if (c < ncls) out[(long long)(base + r) * nr + base + c] = acc[u][i][j];
+      }
     }
   }
 }
@@ -313,15 +334,14 @@ __global__ void k_gram_combine_tangent(const double* __restrict__ Q1, const doub
 
 }  // namespace
 
-// Tile edge for nr x nr outputs: the candidate whose warps issue the fewest FP64 operations (whole warps of 4 x 4 blocks:
-// all of a tile off the diagonal, the upper triangle of one on it).
+// Tile edge for nr x nr outputs: the candidate whose warps issue the fewest FP64 operations (whole warps of 4 x 4 blocks).
 static int gram_tile(int nr, bool sym) {
   const int cand[7] = {20, 28, 36, 44, 52, 60, 64};
   int best = 64;
   long long best_warps = -1;
   for (int gt : cand) {
-    const long long n = (nr + gt - 1) / gt, t = gt / 4;
-    const long long full = (t * t + 31) / 32, tri = (t * (t + 1) / 2 + 31) / 32;
+    const long long n = (nr + gt - 1) / gt;
+    const long long full = gram_blocks(gt) * gram_threads(gt) / 32, tri = gram_threads(gt) / 32;
     const long long warps = sym ? n * tri + n * (n - 1) / 2 * full : n * n * full;
     if (best_warps < 0 || warps < best_warps) { best_warps = warps; best = gt; }
   }
@@ -336,7 +356,7 @@ static int gram_tiles(int nr, bool sym, int gt) {
 // split-K factor for nr x nr outputs over `batch` instances (about kGramWarps warps in total)
 static int nsplit_for(int nr, long long K, int batch, bool sym) {
   const int gt = gram_tile(nr, sym);
-  const int wpc = ((gt / 4) * (gt / 4) + 31) / 32;
+  const int wpc = gram_threads(gt) / 32;
   int nsplit = kGramWarps / (gram_tiles(nr, sym, gt) * wpc * batch);
   if (nsplit < 1) nsplit = 1;
   if (nsplit > K) nsplit = (int)K;
@@ -387,7 +407,7 @@ void launch_half_gram(const double* T, long long t_stride, int batch, Geom g, in
   switch (gt) {
 #define HOTRG_GRAM(GT_)                                                                                        \
   case GT_:                                                                                                    \
-    k_half_gram<GT_><<<grid, (GT_ / 4) * (GT_ / 4), 0, s>>>(A, T, t_stride, li, leg_stride(l1), leg_stride(l2), \
+    k_half_gram<GT_><<<grid, gram_threads(GT_), 0, s>>>(A, T, t_stride, li, leg_stride(l1), leg_stride(l2), \
                                                             Da, nr, K, ntile, sym ? 1 : 0, nsplit, partial,      \
                                                             z2ev);                                               \
     break;

@@ -35,8 +35,8 @@ constexpr int kSpecCap = kMaxGram;  // eigenvalues stored per (step, axis)
 
 long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
 
-// Row stride of a chunk's GEMM output: the slice GEMM stores 32 bytes (four doubles) at a time.
-long long output_ld(long long n, bool slices) { return slices ? round_up(n, 4) : n; }
+// Row stride of a chunk's GEMM output: the tensor-core GEMMs store 32 bytes (eight floats, four doubles) at a time.
+long long output_ld(long long n, bool mixed, bool slices) { return mixed ? round_up(n, 8) : slices ? round_up(n, 4) : n; }
 
 // Bytes a slot of a per-step buffer takes (256-byte aligned: TMA plane starts).
 size_t slot_bytes(size_t n) { return (size_t)round_up((long long)(n ? n : 1), kAlign); }
@@ -134,7 +134,7 @@ StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool sl
   n.X1 = no == 2 ? (size_t)(P * P) * es : 0;
   n.X2 = no >= 1 ? (size_t)(P * P) * es : 0;
   n.Y = (size_t)(P * ldk) * op * nblk;
-  n.O = (size_t)(P * output_ld(chi3 * P, sl)) * es;
+  n.O = (size_t)(P * output_ld(chi3 * P, mixed, sl)) * es;
   if (sl) {
     n.O = std::max(n.O, (size_t)(chi3 * P * ldk) * 8);
     n.yt = (size_t)(P * ldk) * 8;
@@ -171,7 +171,7 @@ struct hotrg_ctx {
   int fold_group = 0;  // k-blocks per accumulator fold (0: one)
   // shape of the last split-precision GEMM launched (what the autotuner times)
   struct LastGemm {
-    long long M = 0, N = 0, K = 0, ldk = 0;
+    long long M = 0, N = 0, K = 0, ldk = 0, ldo = 0;
     int npass = 0, nparts = 0, fmt = 0;
     float mult_b = 1.f;
     const GemmBlocks* blk = nullptr;  // block-sparse: the descriptor of the last chunk (slot 0)
@@ -840,7 +840,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
   delete ops_scope;
   TC* O = static_cast<TC*>(c->O);
   TC* dO = static_cast<TC*>(c->dO);
-  const long long N = (long long)chi3 * P, ldO = output_ld(N, sl);
+  const long long N = (long long)chi3 * P, ldO = output_ld(N, mixed, sl);
   const long long o_slot = (long long)(cO / sizeof(TC)), x_slot = (long long)(cX / sizeof(TC));
   // chunks: outer fixed axis (4D only) one at a time, inner fixed axis nb at a time
   const int no = nt > 0 ? nt - 1 : 0;
@@ -960,6 +960,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
           c->last_gemm.N = N;
           c->last_gemm.K = z2 ? ldk : P;
           c->last_gemm.ldk = ld;
+          c->last_gemm.ldo = ldO;
           c->last_gemm.npass = npass;
           c->last_gemm.nparts = planes;
           c->last_gemm.fmt = f16 ? 1 : 0;
@@ -1858,7 +1859,7 @@ int hotrg_autotune(hotrg_ctx* c, hotrg_tuning* out) {
     double t_min = 1e300;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, c->stream);
-      const int r = launch_gemm_split(Y, lg.ldk, Bt, lg.ldk, static_cast<float*>(c->O), lg.N, lg.M, lg.N, lg.K,
+      const int r = launch_gemm_split(Y, lg.ldk, Bt, lg.ldk, static_cast<float*>(c->O), lg.ldo, lg.M, lg.N, lg.K,
                                       lg.npass, c->status, c->timeout_s, c->stream, cd.kb, cd.gm, cd.fg, lg.blk,
                                       nullptr, false, cd.cg);
       cudaEventRecord(e1, c->stream);

@@ -16,8 +16,15 @@ namespace {
 
 constexpr int TC_BM = 128, TC_BN = 256;
 constexpr int kMaxDevices = 64;
-constexpr int TC_THREADS = 320;
-constexpr int TC_FOLD_THREADS = 256;  // warps 2-9
+// Warpgroup 0: warp 0 copies, warp 1 issues MMAs (warps 2 and 3 idle); warpgroups 1 and 2 (warps 4-11): fold. The fold
+// warps hold 128 sums a thread beside the tensor-memory loads in flight: they take registers over from warpgroup 0
+// (setmaxnreg; the shares add up to what the launch allocates, 168 x 384).
+constexpr int TC_THREADS = 384;
+constexpr int TC_FOLD_WARP0 = 4;
+constexpr int TC_FOLD_THREADS = 256;
+constexpr int TC_LAUNCH_REGS = 168;
+constexpr int TC_ROLE_REGS = 56, TC_FOLD_REGS = 224;
+static_assert(128 * TC_ROLE_REGS + TC_FOLD_THREADS * TC_FOLD_REGS <= TC_LAUNCH_REGS * TC_THREADS, "register shares");
 constexpr uint32_t TMEM_COLS = 2 * TC_BN;
 
 // kind::f16 instruction descriptor: D = F32 (bits 4-5 = 1), A and B format (bits 7-9, 10-12:
@@ -89,7 +96,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 // Bounded wait. Returns false if another role aborted or this wait exceeded timeout_ns.
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                        unsigned long long timeout_ns, bool honour_abort = true) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = globaltimer_ns();
@@ -120,8 +127,8 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
       : "memory");
 }
-// The same load for a CTA pair, issued by the pair's first CTA: `dst` is a shared::cluster address in
-// either CTA (mapa for the second), the bytes count on the first CTA's barrier `bar`.
+// The same load for a CTA pair: `dst` is a shared::cluster address in either CTA (mapa for the other one), the bytes count
+// on the first CTA's barrier `bar` (a shared::cluster address).
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
                                                  int z) {
   asm volatile(
@@ -222,6 +229,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
+}
+template <int N>
+__device__ __forceinline__ void regs_give() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_take() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
