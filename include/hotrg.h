@@ -118,8 +118,8 @@ typedef struct hotrg_opts {
                              thread-block cluster of two SMs) per 256 x 256 tile, whose tcgen05
                              MMAs read A rows from both CTAs and half of the B rows from each;
                              1 = one CTA per 128 x 256 tile. Both give identical results. 0 =
-                             default: 2 with opts.z2, else 1 (the faster at the Dcut = 10
-                             shapes); the autotuner may change it. 1 or 2 fix it; EINVAL
+                             default: 2 (the faster at every measured squeeze shape); the
+                             autotuner may change it. 1 or 2 fix it; EINVAL
                              otherwise */
 } hotrg_opts;
 
@@ -282,8 +282,8 @@ const char *hotrg_strerror(int code);
  * width of a pipeline stage (0 = 64; the 6-pass GEMM always uses 32). fold_group: stages whose
  * products share one tensor-core accumulator before it is folded into FP32 registers with
  * round-to-nearest adds (0 = 1; larger values are clamped to what the kernel variant's ring
- * allows, at most 2). The launch uses one CTA per 128 x 256 output tile (the flow contexts can
- * also run CTA pairs: opts.cta_group).
+ * allows, at most 2). The launch uses a CTA pair per 256 x 256 output tile (M <= 128: one CTA per
+ * 128 x 256 tile); both give identical results.
  * Enqueued on `stream`; not synchronised. Errors: EINVAL (sizes, npass, kblock, alignment),
  * EDEVICE. */
 size_t hotrg_gemm_scratch_bytes(long long M, long long N, long long K);

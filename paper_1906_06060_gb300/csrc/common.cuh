@@ -131,23 +131,27 @@ __device__ __forceinline__ float plane_scale(const Planes<__nv_bfloat16>& o) {
   return o.fmt ? pow2f(f16_scale_exponent(plane_bound(o.amax, o.amax_mult))) : 1.f;
 }
 __device__ __forceinline__ float plane_scale(const Planes<double>&) { return 1.f; }
-__device__ __forceinline__ void store_planes_sc(const Planes<__nv_bfloat16>& o, long long i, float x, float sc) {
+// The (up to three) 16-bit parts of x, as raw patterns
+__device__ __forceinline__ void split_planes(const Planes<__nv_bfloat16>& o, float x, float sc, __nv_bfloat16 (&q)[3]) {
   if (o.fmt) {
     const float xs = x * sc;
     const __half hi = __float2half_rn(xs);
-    const __half lo = __float2half_rn(xs - __half2float(hi));
-    o.p[0][i] = __ushort_as_bfloat16(__half_as_ushort(hi));
-    if (o.nparts > 1) o.p[1][i] = __ushort_as_bfloat16(__half_as_ushort(lo));
+    q[0] = __ushort_as_bfloat16(__half_as_ushort(hi));
+    q[1] = __ushort_as_bfloat16(__half_as_ushort(__float2half_rn(xs - __half2float(hi))));
+    q[2] = q[1];
     return;
   }
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  o.p[0][i] = h;
-  if (o.nparts > 1) {
-    const float r1 = x - __bfloat162float(h);
-    const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-    o.p[1][i] = mid;
-    if (o.nparts > 2) o.p[2][i] = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-  }
+  q[0] = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(q[0]);
+  q[1] = __float2bfloat16_rn(r1);
+  q[2] = __float2bfloat16_rn(r1 - __bfloat162float(q[1]));
+}
+__device__ __forceinline__ void store_planes_sc(const Planes<__nv_bfloat16>& o, long long i, float x, float sc) {
+  __nv_bfloat16 q[3];
+  split_planes(o, x, sc, q);
+  o.p[0][i] = q[0];
+  if (o.nparts > 1) o.p[1][i] = q[1];
+  if (o.nparts > 2) o.p[2][i] = q[2];
 }
 __device__ __forceinline__ void store_planes_sc(const Planes<double>& o, long long i, double x, float) {
   o.p[0][i] = x;

@@ -165,7 +165,7 @@ struct hotrg_ctx {
   int d = 0, Dcut = 0, batch = 1, precision = HOTRG_FP64, fp64_steps = 2, x6_steps = 0, max_steps = 64;
   int kblock = 64;
   bool kblock_fixed = false;  // the caller fixed the k-block (else the autotuner may change it)
-  int cta_group = 1;          // CTAs per squeeze-GEMM output tile (1 or 2)
+  int cta_group = 2;          // CTAs per squeeze-GEMM output tile (1 or 2)
   bool cta_group_fixed = false;
   int group_m = 16;
   int fold_group = 0;  // k-blocks per accumulator fold (0: one)
@@ -1143,9 +1143,7 @@ int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const ho
   c->group = group_for(opt);
   c->timeout_s = opt->wait_timeout_s > 0 ? opt->wait_timeout_s : 4.0;
   c->max_sweeps = opt->max_sweeps > 0 ? opt->max_sweeps : 40;
-  // the faster of the two at the Dcut = 10 shapes: pairs for the two-block squeeze (A rows of a block
-  // fit L2), single CTAs for the dense one
-  c->cta_group = opt->cta_group ? opt->cta_group : (c->z2 ? 2 : 1);
+  c->cta_group = opt->cta_group ? opt->cta_group : 2;  // pairs: the faster form at every measured squeeze shape
   c->cta_group_fixed = opt->cta_group != 0;
   c->stream = static_cast<cudaStream_t>(opt->stream);
   c->beta = vb;

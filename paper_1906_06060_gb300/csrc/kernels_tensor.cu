@@ -39,11 +39,14 @@ __global__ void __launch_bounds__(256) k_absmax(const T* __restrict__ x, long lo
   x += (long long)blockIdx.y * x_inst;
   out += blockIdx.y;
   float m = 0.f;
-  const long long total = rows * cols;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long r = i / cols, c = i - r * cols;
-    m = fmaxf(m, abs_up(x[r * ld + c]));
+  // contiguous rows as one, else a row per block at a time (no index division: 110 us at 16807 x 2401 with one)
+  const bool flat = ld == cols;
+  const long long n = flat ? rows * cols : cols, nr = flat ? 1 : rows;
+  const long long i0 = threadIdx.x + (flat ? (long long)blockIdx.x * 256 : 0), step = flat ? (long long)gridDim.x * 256 : 256;
+  for (long long r = flat ? 0 : blockIdx.x; r < nr; r += gridDim.x) {
+    const T* xr = x + r * ld;
+#pragma unroll 8
+    for (long long i = i0; i < n; i += step) m = fmaxf(m, abs_up(xr[i]));
   }
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
