@@ -282,89 +282,97 @@ __global__ void __launch_bounds__(256) k_build_bt_z2(const Tin* __restrict__ Tt,
 // with O stored as O[rank(m)][colpos(j, n)]. rest = (m_b for b != t0, j, n_b for b != t0) in that
 // order, shaped and strided by `rest` (out_stride) and sk (stride of k'). Only the (i, jj)
 // parity combinations of the chunk's two computed blocks are read; the rest of O is zero.
-//
-// One thread computes all chi outputs of up to JB values j of one parity class: they share their parities and with them
-// the isometry weights, which come from shared memory (rows padded to 16 bytes) once for JB entries of O. One j a thread
-// was bound by those loads (three 16-byte loads an entry, two sets of rows in a warp: 78 % of the L1 pipe, 0.82 ms for the
-// 2 GB of a chunk at bond dimension 10, 0.3 ms of DRAM traffic). The last two n digits are enumerated pattern by pattern,
-// so that a warp reads runs of a whole box row of columns (25 entries at 10 = 5 + 5 values, not 5) and has one parity.
+// CHI = chi (compile-time: exact accumulator count, no predicated FMAs).
+// W rows padded to a multiple of 4 entries (16-byte shared-memory loads)
 template <int CHI>
 constexpr int chi_pad() {
   return (CHI + 3) / 4 * 4;
 }
-// values j per thread: as many accumulators as leave two CTAs per SM; the FP64 instances are bound by the FP64 units
-template <class Tin>
-constexpr int epi_jb(int chi) {
-  return std::is_same<Tin, float>::value ? (chi <= 10 ? 5 : chi <= 13 ? 4 : 3) : 1;
-}
-// j groups of a class split e + (chi3 - e), at most
-constexpr int epi_groups(int chi3, int jb) { return jb == 1 ? chi3 : (chi3 + jb - 1) / jb + 1; }
 
-// Rows of one parity class with a compile-time column count NC: acc[q][k] += sum over the nrow
-// rows r and the NC columns u of w[r * wrow + u * CHIP + k] * src[joff[q] + r * rstep + u * cs], a row's loads issued before
-// its FMAs.
-template <class Tin, class Acc, int CHI, int JB, int NC>
-__device__ __forceinline__ void epi_class_rows(const Tin* __restrict__ src, const int (&joff)[JB], long long rstep,
-                                               int cs, int nrow, const Acc* __restrict__ w, int wrow,
-                                               Acc (&acc)[JB][CHI]) {
+// Rows of one parity class with a compile-time column count NC: acc[k] += sum over the nrow
+// rows r and the NC columns u of w[r * wrow + u * CHIP + k] * src[r * rstep + u * cs]. The
+// loads of max(1, 8 / NC) rows are issued before their FMAs (few registers: the kernel is
+// latency-bound and gains more from resident warps than from loads in flight per thread).
+template <class Tin, class Acc, int CHI, int NC>
+__device__ __forceinline__ void epi_class_rows(const Tin* __restrict__ src, long long rstep, long long cs,
+                                               int nrow, const Acc* __restrict__ w, int wrow, Acc* acc) {
   constexpr int CHIP = chi_pad<CHI>();
-  for (int r = 0; r < nrow; ++r, src += rstep, w += wrow) {
-    Acc x[JB][NC];
+  constexpr int R = NC >= 8 ? 1 : 8 / NC;
+  for (int r0 = 0; r0 < nrow; r0 += R) {
+    Acc x[R][NC];
 #pragma unroll
-    for (int q = 0; q < JB; ++q)
+    for (int r = 0; r < R; ++r) {
+      const bool ok = r0 + r < nrow;
+      const Tin* p = src + (long long)(r0 + r) * rstep;
 #pragma unroll
-      for (int u = 0; u < NC; ++u) x[q][u] = (Acc)src[joff[q] + u * cs];
+      for (int u = 0; u < NC; ++u) x[r][u] = ok ? (Acc)p[u * cs] : (Acc)0;
+    }
 #pragma unroll
-    for (int u = 0; u < NC; ++u)
+    for (int r = 0; r < R; ++r) {
+      if (r0 + r >= nrow) break;
+      const Acc* wr = w + (r0 + r) * wrow;
 #pragma unroll
-      for (int k = 0; k < CHI; ++k) {
-        const Acc wk = w[u * CHIP + k];
+      for (int u = 0; u < NC; ++u)
 #pragma unroll
-        for (int q = 0; q < JB; ++q) acc[q][k] += wk * x[q][u];
-      }
+        for (int k = 0; k < CHI; ++k) acc[k] += wr[u * CHIP + k] * x[r][u];
+    }
   }
 }
 
-// Same for any column count (runtime ncol).
-template <class Tin, class Acc, int CHI, int JB>
-__device__ __forceinline__ void epi_class_rows_any(const Tin* __restrict__ src, const int (&joff)[JB], long long rstep,
-                                                   int cs, int nrow, int ncol, const Acc* __restrict__ w, int wrow,
-                                                   Acc (&acc)[JB][CHI]) {
+// Same for any column count (runtime ncol), two rows' loads (up to 8 each) before the FMAs.
+template <class Tin, class Acc, int CHI>
+__device__ __forceinline__ void epi_class_rows_any(const Tin* __restrict__ src, long long rstep, long long cs,
+                                                   int nrow, int ncol, const Acc* __restrict__ w, int wrow,
+                                                   Acc* acc) {
   constexpr int CHIP = chi_pad<CHI>();
-  for (int r = 0; r < nrow; ++r, src += rstep, w += wrow)
-    for (int u0 = 0; u0 < ncol; u0 += 4) {
-      Acc x[JB][4];
+  for (int i = 0; i < nrow; i += 2) {
+    const bool two = i + 1 < nrow;
+    const Tin* src0 = src + (long long)i * rstep;
+    const Tin* src1 = src0 + rstep;
+    for (int u0 = 0; u0 < ncol; u0 += 8) {
+      Acc x0[8], x1[8];
 #pragma unroll
-      for (int q = 0; q < JB; ++q)
+      for (int u = 0; u < 8; ++u) {
+        const bool ok = u0 + u < ncol;
+        x0[u] = ok ? (Acc)src0[(long long)(u0 + u) * cs] : (Acc)0;
+        x1[u] = (ok && two) ? (Acc)src1[(long long)(u0 + u) * cs] : (Acc)0;
+      }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[q][u] = u0 + u < ncol ? (Acc)src[joff[q] + (u0 + u) * cs] : (Acc)0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         if (u0 + u >= ncol) break;
+        const Acc* w0 = w + i * wrow + (u0 + u) * CHIP;
+        const Acc* w1 = w0 + wrow;
 #pragma unroll
-        for (int k = 0; k < CHI; ++k) {
-          const Acc wk = w[(u0 + u) * CHIP + k];
+        for (int k = 0; k < CHI; ++k) acc[k] += w0[k] * x0[u];
+        if (two) {
 #pragma unroll
-          for (int q = 0; q < JB; ++q) acc[q][k] += wk * x[q][u];
+          for (int k = 0; k < CHI; ++k) acc[k] += w1[k] * x1[u];
         }
       }
     }
+  }
+}
+
+// CTAs per SM the register budget targets: four for the FP32 path; two for FP64 (its
+// accumulators take twice the registers)
+template <class Tin>
+constexpr int epi_min_blocks() {
+  return std::is_same<Tin, float>::value ? 4 : 2;
 }
 
 template <class Tin, class Tout, int CHI>
-__global__ void __launch_bounds__(256, 2) k_epi_z2(const Tin* __restrict__ O, long long ldO, Tout* __restrict__ out,
-                                                   View rest, int total, long long sk, long long out_base, int t0,
-                                                   const double* __restrict__ U, const Z2Layout* Lp, const int* pi_ptr,
-                                                   SlotStrides st) {
+__global__ void __launch_bounds__(256, epi_min_blocks<Tin>()) k_epi_z2(const Tin* __restrict__ O, long long ldO, Tout* __restrict__ out,
+                                                View rest, int total, long long sk, long long out_base,
+                                                int t0, const double* __restrict__ U,
+                                                const Z2Layout* Lp, const int* pi_ptr, SlotStrides st) {
   using Acc = ZAcc<Tin>;
-  constexpr int CHIP = chi_pad<CHI>();
-  constexpr int JB = epi_jb<Tin>(CHI);
   const int slot = blockIdx.z * gridDim.y + blockIdx.y;
   O += slot * st.in_slot;
   out_base += blockIdx.z * st.out_inst + blockIdx.y * st.out_chunk;
   U += blockIdx.z * st.u_inst;
   Lp += blockIdx.z;
   pi_ptr += slot;
+  constexpr int CHIP = chi_pad<CHI>();
   extern __shared__ __align__(16) unsigned char smraw_epi[];
   Acc* W = reinterpret_cast<Acc*>(smraw_epi);  // [D*D][CHIP]
   __shared__ Z2Layout L;
@@ -384,63 +392,33 @@ __global__ void __launch_bounds__(256, 2) k_epi_z2(const Tin* __restrict__ O, lo
   __syncthreads();
   const int pi = *pi_ptr;
   const int d = L.d, et = L.e[t0], nd = rest.ndim;
-  const int ngroups = epi_groups(L.chi3, JB), g0 = (L.e3 + JB - 1) / JB, g1 = (L.chi3 - L.e3 + JB - 1) / JB;
-  // the last two n slots other than t0 (hi, lo; hi < 0: a single one)
-  const int lo = d - 1 == t0 ? d - 2 : d - 1;
-  const int hi = lo - 1 == t0 ? lo - 2 : lo - 1;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-    // decode rest coordinates, last axis first: the d-1 n digits (the last two in pattern order), the group of j, the d-1
-    // m digits (32-bit: rest has < 2^31 entries); unrolled over the slots so that the digits stay in registers
+    // decode rest coordinates, last axis first: the d-1 n digits, j, the d-1 m digits (32-bit:
+    // rest has < 2^31 entries); unrolled over the slots so that the digits stay in registers
     int rem = idx;
     long long ooff = out_base;
     int ax = nd - 1;
     int dm[kMaxD], dn[kMaxD];
     int pm = 0, pn = 0;
-    int dlo, dhi = 0;
-    if (hi >= 0) {
-      const int nlo = L.D[lo], nhi = L.D[hi], elo = L.e[lo], ehi = L.e[hi];
-      const int qq = rem / (nlo * nhi);
-      int q = rem - qq * (nlo * nhi);
-      rem = qq;
-      const bool oddhi = q >= ehi * nlo;
-      if (oddhi) q -= ehi * nlo;
-      const int rows = oddhi ? nhi - ehi : ehi;
-      const bool oddlo = q >= rows * elo;
-      if (oddlo) q -= rows * elo;
-      const int w = oddlo ? nlo - elo : elo;
-      const int r = q / w;
-      dhi = r + (oddhi ? ehi : 0);
-      dlo = q - r * w + (oddlo ? elo : 0);
-    } else {
-      const int qq = rem / L.D[lo];
-      dlo = rem - qq * L.D[lo];
-      rem = qq;
-    }
 #pragma unroll
     for (int b = kMaxD - 1; b >= 0; --b) {
       dn[b] = 0;
       if (b >= d || b == t0) continue;
-      if (b == lo) dn[b] = dlo;
-      else if (b == hi) dn[b] = dhi;
-      else {
-        const int sh = shape[ax];
-        const int qq = rem / sh;
-        dn[b] = rem - qq * sh;
-        rem = qq;
-      }
+      const int sh = shape[ax];
+      const int qq = rem / sh;
+      dn[b] = rem - qq * sh;
+      rem = qq;
       ooff += (long long)dn[b] * ostr[ax--];
       if (dn[b] >= L.e[b]) pn |= 1 << b;
     }
-    const int qg = rem / ngroups;
-    int jg = rem - qg * ngroups;
-    rem = qg;
-    if (jg >= g0 + g1) continue;
-    const long long ostr_j = ostr[ax--];
-    const int pj = jg >= g0 ? 1 : 0;
-    if (pj) jg -= g0;
-    const int jfirst = (pj ? L.e3 : 0) + jg * JB;
-    const int jn = min(JB, (pj ? L.chi3 : L.e3) - jfirst);
-    ooff += (long long)jfirst * ostr_j;
+    int j;
+    {
+      const int sh = shape[ax];
+      const int qq = rem / sh;
+      j = rem - qq * sh;
+      rem = qq;
+      ooff += (long long)j * ostr[ax--];
+    }
 #pragma unroll
     for (int b = kMaxD - 1; b >= 0; --b) {
       dm[b] = 0;
@@ -452,12 +430,11 @@ __global__ void __launch_bounds__(256, 2) k_epi_z2(const Tin* __restrict__ O, lo
       ooff += (long long)dm[b] * ostr[ax--];
       if (dm[b] >= L.e[b]) pm |= 1 << b;
     }
+    const int pj = j >= L.e3 ? 1 : 0;
     const int tau = pi ^ pj ^ (popc4(pm) & 1) ^ (popc4(pn) & 1);
-    Acc acc[JB][CHI];
+    Acc acc[CHI];
 #pragma unroll
-    for (int q = 0; q < JB; ++q)
-#pragma unroll
-      for (int k = 0; k < CHI; ++k) acc[q][k] = 0;
+    for (int k = 0; k < CHI; ++k) acc[k] = 0;
     // loop over the column class: its width is the same in every lane of a warp (the row class
     // ci = cj ^ tau varies with the lane's parities, only as a row count)
     for (int cj = 0; cj < 2; ++cj) {
@@ -465,46 +442,39 @@ __global__ void __launch_bounds__(256, 2) k_epi_z2(const Tin* __restrict__ O, lo
       const int patm = pm | (ci << t0), patn = pn | (cj << t0);
       const int parn = popc4(patn) & 1;
       long long rb = L.patoff[patm];
-      int cb = L.patoff[patn] - (parn ? L.ncls[0] : 0);
+      long long cb = L.patoff[patn] - (parn ? L.ncls[0] : 0);
 #pragma unroll
       for (int b = 0; b < kMaxD; ++b) {
         if (b >= d || b == t0) continue;
         rb += (long long)(dm[b] - (((patm >> b) & 1) ? L.e[b] : 0)) * L.bs[patm][b];
-        cb += (dn[b] - (((patn >> b) & 1) ? L.e[b] : 0)) * L.bs[patn][b];
+        cb += (long long)(dn[b] - (((patn >> b) & 1) ? L.e[b] : 0)) * L.bs[patn][b];
       }
       const int grp = parn ^ pj;
-      cb += L.goff[grp];
-      int joff[JB];  // (values beyond the class repeat the first one and are not stored)
-#pragma unroll
-      for (int q = 0; q < JB; ++q) joff[q] = cb + L.jstart[grp][jfirst + (q < jn ? q : 0)];
-      const long long rstep = L.bs[patm][t0] * ldO;
-      const int cs = L.bs[patn][t0];
+      cb += L.goff[grp] + L.jstart[grp][j];
+      const long long rstep = L.bs[patm][t0] * ldO, cs = L.bs[patn][t0];
       const int i0 = ci ? et : 0, nrow = ci ? Dt - et : et;
       const int j0 = cj ? et : 0, ncol = cj ? Dt - et : et;
-      const Tin* src = O + rb * ldO;
+      const Tin* src = O + rb * ldO + cb;
       const Acc* w = W + (i0 * Dt + j0) * CHIP;
       const int wrow = Dt * CHIP;
-      if constexpr (std::is_same<Tin, float>::value && std::is_same<Tout, float>::value && CHI >= 6) {
+      if constexpr (std::is_same<Tin, float>::value && CHI >= 6) {
         switch (ncol) {
-#define HOTRG_EPI_NC(NC)                                                                \
-  case NC:                                                                              \
-    epi_class_rows<Tin, Acc, CHI, JB, NC>(src, joff, rstep, cs, nrow, w, wrow, acc);    \
+#define HOTRG_EPI_NC(NC) \
+  case NC:               \
+    epi_class_rows<Tin, Acc, CHI, NC>(src, rstep, cs, nrow, w, wrow, acc); \
     break;
-          HOTRG_EPI_NC(2) HOTRG_EPI_NC(3) HOTRG_EPI_NC(4) HOTRG_EPI_NC(5) HOTRG_EPI_NC(6) HOTRG_EPI_NC(7)
+          HOTRG_EPI_NC(1) HOTRG_EPI_NC(2) HOTRG_EPI_NC(3) HOTRG_EPI_NC(4)
+          HOTRG_EPI_NC(5) HOTRG_EPI_NC(6) HOTRG_EPI_NC(7) HOTRG_EPI_NC(8)
 #undef HOTRG_EPI_NC
           default:
-            epi_class_rows_any<Tin, Acc, CHI, JB>(src, joff, rstep, cs, nrow, ncol, w, wrow, acc);
+            epi_class_rows_any<Tin, Acc, CHI>(src, rstep, cs, nrow, ncol, w, wrow, acc);
         }
       } else {
-        epi_class_rows_any<Tin, Acc, CHI, JB>(src, joff, rstep, cs, nrow, ncol, w, wrow, acc);
+        epi_class_rows_any<Tin, Acc, CHI>(src, rstep, cs, nrow, ncol, w, wrow, acc);
       }
     }
 #pragma unroll
-    for (int q = 0; q < JB; ++q)
-      if (q < jn) {
-#pragma unroll
-        for (int k = 0; k < CHI; ++k) out[ooff + q * ostr_j + k * sk] = (Tout)acc[q][k];
-      }
+    for (int k = 0; k < CHI; ++k) out[ooff + k * sk] = (Tout)acc[k];
   }
 }
 
@@ -561,11 +531,8 @@ template <class Tin, class Tout>
 void launch_epi_z2(const Tin* O, long long ldO, Tout* out, const View& rest, long long sk, long long out_base, int t0,
                    int Dt, const double* U, int chi, const Z2Layout* L, const int* pi, const SlotStrides& st,
                    cudaStream_t s) {
-  // rest indices with the j axis (after the m slots) in groups
-  const int jaxis = (rest.ndim - 1) / 2, chi3 = rest.shape[jaxis];
-  long long total = epi_groups(chi3, epi_jb<Tin>(chi));
-  for (int i = 0; i < rest.ndim; ++i)
-    if (i != jaxis) total *= rest.shape[i];
+  long long total = 1;
+  for (int i = 0; i < rest.ndim; ++i) total *= rest.shape[i];
   const size_t smem = sizeof(ZAcc<Tin>) * (size_t)((chi + 3) / 4 * 4) * Dt * Dt;
   const int n = (int)total;  // rest < 2^31 entries (P^2 chi3 / Dt^2 <= 2.3e9 / 4 for Dcut <= 14)
   const dim3 grid(grid_cap(total), st.nb, st.ng);
