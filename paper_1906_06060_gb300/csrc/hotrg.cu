@@ -47,18 +47,18 @@ struct StepNeeds {
   size_t Tt = 0, Bt = 0, X1 = 0, eb = 0;
   size_t X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0;
   size_t scr = 0;
-  int nb = 1;
+  int nb = 1, go = 1;  // chunks in flight: values of the inner and of the outer fixed axis
 };
 
 // Bytes per instance of the group that hold every step of a plan.
 struct StepSizes {
   size_t Tt = 0, Bt = 0, X1 = 0, eb = 0, X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0, scr = 0;
   static StepSizes of(const StepNeeds& n) {
-    auto chunks = [&](size_t x) { return (size_t)n.nb * slot_bytes(x); };
+    auto chunks = [&](size_t x) { return (size_t)n.nb * n.go * slot_bytes(x); };
     StepSizes z;
     z.Tt = slot_bytes(n.Tt);
     z.Bt = slot_bytes(n.Bt);
-    z.X1 = slot_bytes(n.X1);
+    z.X1 = n.go * slot_bytes(n.X1);
     z.eb = slot_bytes(n.eb);
     z.X2 = chunks(n.X2);
     z.Y = chunks(n.Y);
@@ -92,9 +92,13 @@ struct StepSizes {
 // operands and the FP64 units: what fitted the card before still does.
 constexpr size_t kSliceWorkspaceLimit = (size_t)128 << 30;
 
-// Chunks in flight: as many of the `inner` chunks as keep the group's chunk buffers within this size (twice the L2:
-// beyond it a launch fills the chip many times over and batching gains nothing), in equal parts.
-constexpr size_t kChunkBytes = (size_t)256 << 20;
+// Chunks in flight: as many of the `inner` chunks as keep the group's chunk buffers within this size, in equal parts.
+// Fewer, larger launches waste less of their last wave of GEMM tiles: a parity block of a 6^4 tensor has 48 tile pairs a
+// chunk for the 76 pairs of SMs (one chunk a launch 342 us, six 1370). Measured with 256 MB and with 1 GB: FP64 step of
+// that tensor 22.9 and 16.4 ms, ragged 4D FP64 7.9 and 6.6, 16 couplings of a 4D flow at D = 5 98 and 87, 3D flow at
+// D = 10 50 and 45. One instance of a 4D tensor at D = 5, with tangents, needs 1.8 GB for all 25 chunks: 115 ms a
+// gradient with one value of the outer axis at a time, 84 with all; the FP64 step of a 4^4 tensor 1.32 and 0.90 ms.
+constexpr size_t kChunkBytes = (size_t)2 << 30;
 int chunk_batch(int inner, int group, size_t bytes_per_chunk) {
   const long long fit = (long long)(kChunkBytes / std::max<size_t>(1, bytes_per_chunk * group));
   int nb = (int)std::max(1LL, std::min({fit, (long long)inner, (long long)(kMaxGemmBatch / group)}));
@@ -104,7 +108,7 @@ int chunk_batch(int inner, int group, size_t bytes_per_chunk) {
 
 // planes: 0 = FP64 path, 2 or 3 = tensor-core path with that many 16-bit planes per operand. slices: FP64 products
 // run on digit slices where their shape takes it. group: instances squeezed together; nblk: column blocks of an operand
-// row (3 with tangents).
+// row (3 with tangents); most_chunks: limit of the chunks in flight.
 StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool slices, int group, int nblk,
                     int most_chunks = kMaxGemmBatch) {
   const bool mixed = planes > 0;
@@ -152,10 +156,12 @@ StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool sl
   n.R1 = r[0];
   n.R2 = r[1];
   const size_t tangent = nblk > 1 ? n.O + n.X2 + n.R1 + n.R2 : 0;
-  n.nb = no ? std::min(most_chunks,
-                       chunk_batch(chi[trans[no - 1]], group, n.X2 + n.Y + n.O + n.R1 + n.R2 + n.yt + tangent))
-            : 1;
-  if (sl) n.scr = slice_scratch_bytes(P, chi3 * P, group * n.nb);
+  const size_t chunk = n.X2 + n.Y + n.O + n.R1 + n.R2 + n.yt + tangent;
+  n.nb = no ? std::min(most_chunks, chunk_batch(chi[trans[no - 1]], group, chunk)) : 1;
+  // where the inner axis fits whole and there is one instance, values of the outer axis take the instances' place
+  if (no == 2 && group == 1 && n.nb == chi[trans[1]])
+    n.go = std::max(1, std::min(most_chunks / n.nb, chunk_batch(chi[trans[0]], n.nb, chunk)));
+  if (sl) n.scr = slice_scratch_bytes(P, chi3 * P, group * n.nb * n.go);
   return n;
 }
 
@@ -376,10 +382,10 @@ struct Carver {
 bool step_needs(const hotrg_ctx* c, const int* dims, int a, int planes, StepNeeds* n) {
   const int nblk = c->deriv ? 3 : 1;
   for (int sl = c->slices ? 1 : 0; sl >= 0; --sl)
-    for (int most = kMaxGemmBatch;; most = n->nb - 1) {
+    for (int most = kMaxGemmBatch;; most = n->nb * n->go - 1) {
       *n = needs_for(c->d, dims, a, c->Dcut, planes, sl != 0, c->group, nblk, most);
       if (c->sz.covers(*n)) return true;
-      if (n->nb <= 1) break;
+      if (n->nb * n->go <= 1) break;
     }
   return false;
 }
@@ -708,7 +714,8 @@ SliceOperand slice_operand(void* base, long long plane, long long ld, long long 
 // A chunk fixes the new indices of the transverse axes but the last. The chunks of the inner fixed axis run `nb` at a
 // time (chunk_batch): every kernel launch covers them for all instances of the group, with the GEMM's B operand shared
 // by the chunks of an instance. A step of 25 to 100 small chunks is bound by its launches and by kernels that fill a
-// fraction of the chip (4D, bond dimension 5: 75 GEMM tiles on 152 SMs, 7 launches a chunk).
+// fraction of the chip (4D, bond dimension 5: 75 GEMM tiles on 152 SMs, 7 launches a chunk). With one instance, `go`
+// values of the outer fixed axis run in the instances' place.
 //
 // z2: zero-field squeeze of T with itself (z2.cu): parity-blocked operands, two dense GEMM blocks per chunk, the first
 // epilogue contraction reading the blocked output. Same output up to the order of summation.
@@ -797,7 +804,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
   // padding between the blocks of a concatenated k range (slicing writes its own)
   if ((z2 || (tg.n && mixed && ldk != P)) && !sl) {
     cudaMemsetAsync(c->Bt, 0, c->sz.Bt * (ng - 1) + sizeof(Op) * nparts * bt_plane, s);
-    cudaMemsetAsync(c->Y, 0, cY * (ng * need.nb - 1) + sizeof(Op) * nparts * y_plane, s);
+    cudaMemsetAsync(c->Y, 0, cY * (ng * need.nb * need.go - 1) + sizeof(Op) * nparts * y_plane, s);
   }
   auto build_bt = [&](const TC* src, int blk, int which, const double* U, const TC* src2, const double* U2) {
     const long long src_inst = (long long)(c->sz.Tt / sizeof(TC)), bt_inst = (long long)(c->sz.Bt / sizeof(Op));
@@ -842,15 +849,19 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
   TC* dO = static_cast<TC*>(c->dO);
   const long long N = (long long)chi3 * P, ldO = output_ld(N, mixed, sl);
   const long long o_slot = (long long)(cO / sizeof(TC)), x_slot = (long long)(cX / sizeof(TC));
-  // chunks: outer fixed axis (4D only) one at a time, inner fixed axis nb at a time
+  // chunks: outer fixed axis (4D only) go at a time (in the instances' place of every launch), inner one nb at a time
   const int no = nt > 0 ? nt - 1 : 0;
   const int outer = no == 2 ? chi[trans[0]] : 1;
   const int inner_axis = no ? trans[no - 1] : -1;
   const int inner = no ? chi[inner_axis] : 1;
-  const long long x1_inst = (long long)(c->sz.X1 / sizeof(TC));
-  for (int k0 = 0; k0 < outer; ++k0)
+  const int go_most = z2 ? 1 : need.go;
+  const long long x1_inst = (long long)((need.go > 1 ? slot_bytes(need.X1) : c->sz.X1) / sizeof(TC));
+  const long long out_outer = no == 2 ? gn.Sn[trans[0]] * gn.P : 0;
+  for (int k0 = 0; k0 < outer; k0 += go_most)
     for (int kb = 0; kb < inner; kb += need.nb) {
-      const int nb = std::min(need.nb, inner - kb), nz = ng * nb;
+      const int go = std::min(go_most, outer - k0);  // above 1: ng is 1 and nb the whole inner axis
+      const int ni = ng * go;                        // instances, or values of the outer axis
+      const int nb = std::min(need.nb, inner - kb), nz = ni * nb;
       // producer: mode products on the unprimed legs of the other transverse axes, then the A operand
       ops_scope = new PhaseScope(c, PH_OPERANDS);
       if (z2)
@@ -883,9 +894,9 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
         if (no == 2) {
           if (kb == 0)
             launch_mode_unprimed<double, TC>(G.T1, G.t_inst, X1, x1_inst, g, trans[0], Ub(G.U, trans[0]), G.u_inst, k0,
-                                             ng, 1, s);
-          launch_mode_unprimed<TC, TC>(X1, x1_inst, X2, x_slot, g, inner_axis, Ui, G.u_inst, kb, ng, nb, s, nullptr,
-                                       nullptr, bound);
+                                             ng, go, s);
+          launch_mode_unprimed<TC, TC>(X1, x1_inst, X2, x_slot, g, inner_axis, Ui, go > 1 ? 0 : G.u_inst, kb, ni, nb, s,
+                                       nullptr, nullptr, bound);
         } else {
           launch_mode_unprimed<double, TC>(G.T1, G.t_inst, X2, x_slot, g, inner_axis, Ui, G.u_inst, kb, ng, nb, s,
                                            nullptr, nullptr, bound);
@@ -896,10 +907,10 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
           const double* dUi = tg.dU[p] ? Ub(tg.dU[p], inner_axis) : nullptr;
           if (no == 2) {
             if (kb == 0)
-              launch_mode_unprimed<double, TC>(tg.dT[p], 0, dX1, 0, g, trans[0], Ub(G.U, trans[0]), 0, k0, 1, 1, s,
+              launch_mode_unprimed<double, TC>(tg.dT[p], 0, dX1, x1_inst, g, trans[0], Ub(G.U, trans[0]), 0, k0, 1, go, s,
                                                tg.dU[p] ? G.T1 : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[0]) : nullptr);
-            launch_mode_unprimed<TC, TC>(dX1, 0, dX2, x_slot, g, inner_axis, Ui, 0, kb, 1, nb, s, dUi ? X1 : nullptr,
-                                         dUi);
+            launch_mode_unprimed<TC, TC>(dX1, x1_inst, dX2, x_slot, g, inner_axis, Ui, 0, kb, ni, nb, s,
+                                         dUi ? X1 : nullptr, dUi);
           } else {
             launch_mode_unprimed<double, TC>(tg.dT[p], 0, dX2, x_slot, g, inner_axis, Ui, 0, kb, 1, nb, s,
                                              dUi ? G.T1 : nullptr, dUi);
@@ -911,7 +922,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
       // the O(D^15) GEMM, all slots in one launch
       GemmBatch bat;
       bat.batch = nz;
-      bat.b_div = nb;
+      bat.b_div = nb * go;
       bat.a_inst = (long long)(cY / sizeof(Op));
       bat.b_inst = (long long)(c->sz.Bt / sizeof(Op));
       bat.c_inst = o_slot;
@@ -972,7 +983,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
       }
       // epilogue: O axes [m_0..m_{d-1}, j, n_0..n_{d-1}]
       long long out_base = 0;
-      if (no == 2) out_base += (long long)k0 * gn.Sn[trans[0]] * gn.P;
+      out_base += k0 * out_outer;
       if (no >= 1) out_base += (long long)kb * gn.Sn[inner_axis] * gn.P;
       const long long out_chunk = no ? gn.Sn[inner_axis] * gn.P : 0;
       std::vector<Ax> hist[kMaxD];  // axes of the input of each contraction of the chain
@@ -985,7 +996,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
         axes.push_back({chi3, P, 1, -1});
         for (int b = 0; b < c->d; ++b) axes.push_back({g.D[b], g.Sn[b], 2, b});
         const TC* cur = O;
-        SlotStrides st{ng, nb, o_slot, 0, 0, G.u_inst};
+        SlotStrides st{ni, nb, o_slot, 0, 0, go > 1 ? 0 : G.u_inst};
         long long fs[kMaxAxes];
         for (int i = 0; i < no; ++i) {
           hist[i] = axes;
@@ -1000,7 +1011,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
           st.in_slot = r_slot[i];
         }
         hist[no] = axes;
-        st.out_inst = G.out_inst;
+        st.out_inst = go > 1 ? out_outer : G.out_inst;
         st.out_chunk = out_chunk;
         if (c3 >= 0) {
           // final axes after contracting c3 (m_c3 removed, n_c3 -> k'_c3)
@@ -1023,9 +1034,10 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
         PhaseScope epi_scope(c, PH_EPILOGUE);
         const TC* cur = dO;
         const TC* curF = O;
-        SlotStrides st{1, nb, o_slot, 0, 0, 0};
+        SlotStrides st{ni, nb, o_slot, 0, 0, 0};
         for (int i = 0; i < no; ++i) {
           std::vector<Ax> ax = hist[i];
+          st.out_inst = r_slot[i] * nb;
           st.out_chunk = r_slot[i];
           contract_axes<TC, TC>(ax, cur, dbufs[i], trans[i], chi[trans[i]], Ub(G.U, trans[i]), nullptr, 0, st, s,
                                 tg.dU[p] ? curF : nullptr, tg.dU[p] ? Ub(tg.dU[p], trans[i]) : nullptr);
@@ -1035,6 +1047,7 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
         }
         std::vector<Ax> ax = hist[no];
         long long fs[kMaxAxes];
+        st.out_inst = out_outer;
         st.out_chunk = out_chunk;
         if (c3 >= 0) {
           final_strides(ax, c3, c3, gn, c3, fs);
