@@ -5,6 +5,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/hotrg.h"
 
 namespace hotrg {
@@ -155,6 +157,22 @@ __device__ __forceinline__ void store_planes_sc(const Planes<__nv_bfloat16>& o, 
 }
 __device__ __forceinline__ void store_planes_sc(const Planes<double>& o, long long i, double x, float) {
   o.p[0][i] = x;
+}
+
+// Accumulator of an output type.
+template <class Tout>
+using AccT = typename std::conditional<std::is_same<Tout, double>::value, double, float>::type;
+
+// Upper bound of |x| as a float (rounded up from double).
+__device__ __forceinline__ float abs_up(double x) { return __double2float_ru(fabs(x)); }
+__device__ __forceinline__ float abs_up(float x) { return fabsf(x); }
+
+// Blocks of a grid-stride kernel over n items.
+inline int grid_for(long long n, int block, int cap = 152 * 16) {
+  long long g = (n + block - 1) / block;
+  if (g > cap) g = cap;
+  if (g < 1) g = 1;
+  return (int)g;
 }
 
 }  // namespace hotrg

@@ -13,24 +13,9 @@ long long launches_total() { return g_launches.load(std::memory_order_relaxed); 
 
 namespace {
 
-template <class Tout>
-using AccT = typename std::conditional<std::is_same<Tout, double>::value, double, float>::type;
-
-
-inline int grid_for(long long n, int block, int cap = 152 * 16) {
-  long long g = (n + block - 1) / block;
-  if (g > cap) g = cap;
-  if (g < 1) g = 1;
-  return (int)g;
-}
-
 constexpr int kNormBlocks = 1024;
 
 // ---------------------------------------------------------------------------- max |x|
-// Upper bound of |x| as a float (rounded up from double).
-__device__ __forceinline__ float abs_up(double x) { return __double2float_ru(fabs(x)); }
-__device__ __forceinline__ float abs_up(float x) { return fabsf(x); }
-
 // *out = max(*out, max |x|) over rows x cols entries with row stride ld, as the bits of a
 // non-negative float (their unsigned order is the order of the values). NaN entries are skipped.
 template <class T>
@@ -283,64 +268,6 @@ __global__ void __launch_bounds__(256) k_trace_x(const double* __restrict__ T, l
     out3[0] = tr;
     out3[1] = tr > 0.0 ? *L + ldexp(log(tr), -step) : nan("");
     out3[2] = trA * trA / trA2;
-  }
-}
-
-// ---------------------------------------------------------------------------- mode product
-// One thread per "base" (an input index with digit b = 0): it reads the Db inputs along leg b
-// once and writes all Db outputs, so every input element is read from memory once.
-// TWO: out also accumulates the same product of a second input with a second matrix (the
-// tangent of a mode product: dX = M_U(dT) + M_dU(T)).
-template <class Tin, class Tout, bool TWO>
-__global__ void __launch_bounds__(256) k_mode_unprimed(const Tin* __restrict__ in, Tout* __restrict__ out,
-                                                       long long total, long long stride_b, int Db,
-                                                       const double* __restrict__ U, int kk,
-                                                       const Tin* __restrict__ in2, const double* __restrict__ U2,
-                                                       unsigned* amax, long long in_inst, long long out_slot,
-                                                       long long u_inst) {
-  using Acc = AccT<Tout>;
-  // chunk blockIdx.y of instance blockIdx.z (the input comes from L2 for every chunk but the first)
-  const int slot = blockIdx.z * gridDim.y + blockIdx.y;
-  in += blockIdx.z * in_inst;
-  if (TWO) in2 += blockIdx.z * in_inst;
-  out += slot * out_slot;
-  U += blockIdx.z * u_inst;
-  kk += blockIdx.y;
-  if (amax) amax += slot;
-  __shared__ Acc W[kMaxGram];
-  __shared__ Acc W2[TWO ? kMaxGram : 1];
-  for (int t = threadIdx.x; t < Db * Db; t += blockDim.x) {
-    W[t] = (Acc)U[(long long)kk * Db * Db + t];
-    if (TWO) W2[t] = (Acc)U2[(long long)kk * Db * Db + t];
-  }
-  __syncthreads();
-  const long long nbase = total / Db;
-  float m = 0.f;  // max |out| of this thread (with amax: the bound of an fp16 operand's source)
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < nbase;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long base = (t / stride_b) * stride_b * Db + t % stride_b;
-    Acc x[kMaxBond], x2[TWO ? kMaxBond : 1];
-#pragma unroll
-    for (int i = 0; i < kMaxBond; ++i)
-      if (i < Db) {
-        x[i] = (Acc)in[base + i * stride_b];
-        if (TWO) x2[i] = (Acc)in2[base + i * stride_b];
-      }
-    for (int j = 0; j < Db; ++j) {
-      Acc acc = 0;
-#pragma unroll
-      for (int i = 0; i < kMaxBond; ++i)
-        if (i < Db) {
-          acc += W[i * Db + j] * x[i];
-          if (TWO) acc += W2[i * Db + j] * x2[i];
-        }
-      out[base + j * stride_b] = (Tout)acc;
-      if (amax) m = fmaxf(m, abs_up((Tout)acc));
-    }
-  }
-  if (amax) {
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(amax, __float_as_uint(m));
   }
 }
 
@@ -654,23 +581,6 @@ void launch_trace_x(const double* T, long long t_stride, int batch, Geom g, int 
   count_launches(1);
 }
 
-template <class Tin, class Tout>
-void launch_mode_unprimed(const Tin* in, long long in_inst, Tout* out, long long out_slot, Geom g, int b, const double* U,
-                          long long u_inst, int kk, int ng, int nb, cudaStream_t s, const Tin* in2, const double* U2,
-                          unsigned* amax) {
-  const long long total = g.P * g.P;
-  const long long nbase = total / g.D[b];
-  if (amax) cudaMemsetAsync(amax, 0, sizeof(unsigned) * ng * nb, s);
-  const dim3 grid(grid_for(nbase, 256), nb, ng);
-  if (in2)
-    k_mode_unprimed<Tin, Tout, true><<<grid, 256, 0, s>>>(in, out, total, g.Sn[b] * g.P, g.D[b], U, kk, in2, U2, amax,
-                                                          in_inst, out_slot, u_inst);
-  else
-    k_mode_unprimed<Tin, Tout, false><<<grid, 256, 0, s>>>(in, out, total, g.Sn[b] * g.P, g.D[b], U, kk, nullptr, nullptr,
-                                                           amax, in_inst, out_slot, u_inst);
-  count_launches(1);
-}
-
 template <class T>
 void launch_absmax(const T* x, long long rows, long long cols, long long ld, unsigned* out, cudaStream_t s, int batch,
                    long long x_inst) {
@@ -792,13 +702,6 @@ void prepare_kernel_attributes() {
 }
 
 // explicit instantiations: FP64 path (double everywhere) and BF16X3 path (float intermediates)
-#define HOTRG_MODE(TI, TO)                                                                                            \
-  template void launch_mode_unprimed<TI, TO>(const TI*, long long, TO*, long long, Geom, int, const double*, long long, \
-                                             int, int, int, cudaStream_t, const TI*, const double*, unsigned*);
-HOTRG_MODE(double, double)
-HOTRG_MODE(double, float)
-HOTRG_MODE(float, float)
-#undef HOTRG_MODE
 template void launch_transpose<double>(const double*, long long, double*, long long, long long, int, cudaStream_t);
 template void launch_transpose<float>(const double*, long long, float*, long long, long long, int, cudaStream_t);
 #define HOTRG_BT(TI, TO)                                                                                          \
