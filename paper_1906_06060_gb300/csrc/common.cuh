@@ -167,6 +167,16 @@ using AccT = typename std::conditional<std::is_same<Tout, double>::value, double
 __device__ __forceinline__ float abs_up(double x) { return __double2float_ru(fabs(x)); }
 __device__ __forceinline__ float abs_up(float x) { return fabsf(x); }
 
+// Entry idx of a B operand of chi3 P rows and P columns (row = j P + n < 2^31): 32-bit divisions where the entries can
+// be counted in 32 bits. (Five 64-bit divisions an entry were most of the zero-field operand's 10.3 ms at D = 10.)
+struct BtIndex {
+  unsigned row, k;
+  __device__ __forceinline__ BtIndex(long long idx, long long P, long long total) {
+    row = total <= 0xffffffffLL ? (unsigned)idx / (unsigned)P : (unsigned)(idx / P);
+    k = (unsigned)(idx - (long long)row * P);
+  }
+};
+
 // Blocks of a grid-stride kernel over n items.
 inline int grid_for(long long n, int block, int cap = 152 * 16) {
   long long g = (n + block - 1) / block;

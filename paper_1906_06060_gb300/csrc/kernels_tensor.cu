@@ -318,13 +318,12 @@ __global__ void __launch_bounds__(256) k_build_bt(const Tin* __restrict__ Tt, Pl
   const long long total = (long long)chi3 * P * P;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    const long long k = idx % P;
-    const long long row = idx / P;  // j*P + n
-    const long long n = row % P;
-    const int j = (int)(row / P);
+    const BtIndex e(idx, P, total);
+    const unsigned k = e.k, row = e.row, j = row / (unsigned)P;
+    const long long n = row - j * (unsigned)P;
     Acc acc;
     if (Sc > 0) {
-      const int kc = (int)((k / Sc) % Dc);
+      const unsigned kc = (k / (unsigned)Sc) % (unsigned)Dc;
       const long long base = n * P + k - (long long)kc * Sc;
       const Acc* w = W + ((long long)j * Dc + kc) * Dc;
       acc = 0;
@@ -336,7 +335,7 @@ __global__ void __launch_bounds__(256) k_build_bt(const Tin* __restrict__ Tt, Pl
     } else {
       acc = (Acc)Tt[n * P + k];
     }
-    store_planes(out, row * ld + k, acc);
+    store_planes(out, (long long)row * ld + k, acc);
   }
 }
 
@@ -481,12 +480,23 @@ __global__ void __launch_bounds__(256) k_pair_contract_all(const Tin* __restrict
   __syncthreads();
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    long long rem = idx, ioff = 0, ooff = out_base;
-    for (int ax = v.ndim - 1; ax >= 0; --ax) {
-      const long long c = rem % v.shape[ax];
-      rem /= v.shape[ax];
-      ioff += c * v.in_stride[ax];
-      ooff += c * v.out_stride[ax];
+    long long ioff = 0, ooff = out_base;
+    if (total <= 0xffffffffLL) {
+      unsigned rem = (unsigned)idx;
+      for (int ax = v.ndim - 1; ax >= 0; --ax) {
+        const unsigned n = (unsigned)v.shape[ax], q = rem / n, c = rem - q * n;
+        rem = q;
+        ioff += c * v.in_stride[ax];
+        ooff += c * v.out_stride[ax];
+      }
+    } else {
+      long long rem = idx;
+      for (int ax = v.ndim - 1; ax >= 0; --ax) {
+        const long long c = rem % v.shape[ax];
+        rem /= v.shape[ax];
+        ioff += c * v.in_stride[ax];
+        ooff += c * v.out_stride[ax];
+      }
     }
     Acc acc[CHI];
 #pragma unroll
@@ -649,11 +659,27 @@ static void pair_contract_all(const Tin* in, Tout* out, const View& rest, int Di
                               const Tin* in2, const double* U2) {
   using Acc = AccT<Tout>;
   constexpr int PAD = 16 / (int)sizeof(Acc);
+  // axes that run on from one another in both tensors become one: the index of an output costs a division an axis
+  View v;
+  v.ndim = 0;
   long long total = 1;
-  for (int i = 0; i < rest.ndim; ++i) total *= rest.shape[i];
+  for (int i = 0; i < rest.ndim; ++i) {
+    total *= rest.shape[i];
+    if (rest.shape[i] == 1) continue;
+    const int l = v.ndim - 1;
+    if (l >= 0 && v.in_stride[l] == rest.in_stride[i] * rest.shape[i] &&
+        v.out_stride[l] == rest.out_stride[i] * rest.shape[i] && (long long)v.shape[l] * rest.shape[i] < (1LL << 31)) {
+      v.shape[l] *= rest.shape[i];
+    } else {
+      ++v.ndim;
+      v.shape[l + 1] = rest.shape[i];
+    }
+    v.in_stride[v.ndim - 1] = rest.in_stride[i];
+    v.out_stride[v.ndim - 1] = rest.out_stride[i];
+  }
   const size_t smem = sizeof(Acc) * (size_t)((CHI + PAD - 1) / PAD * PAD) * Di * Dj * (TWO ? 2 : 1);
   k_pair_contract_all<Tin, Tout, TWO, CHI, NJ><<<dim3(grid_for(total, 256), st.nb, st.ng), 256, smem, s>>>(
-      in, out, rest, total, Di, Dj, si, sj, sk, U, out_base, in2, U2, st);
+      in, out, v, total, Di, Dj, si, sj, sk, U, out_base, in2, U2, st);
   count_launches(1);
 }
 

@@ -260,15 +260,14 @@ __global__ void __launch_bounds__(256) k_build_bt_z2(const Tin* __restrict__ Tt,
   const long long total = (long long)chi3 * P * P;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    const long long k = idx % P;
-    const long long row = idx / P;  // j*P + n
+    const BtIndex e(idx, P, total);
+    const unsigned k = e.k, row = e.row;
     const int cp = colpos_tab[row];
     const int grp = cp >= goff1 ? 1 : 0;
     const int park = rank_tab[k] >= ncls0 ? 1 : 0;
     if (grp != park) continue;
-    const long long n = row % P;
-    const int j = (int)(row / P);
-    const int kc = (int)((k / Sc) % Dc);
+    const unsigned j = row / (unsigned)P, kc = (k / (unsigned)Sc) % (unsigned)Dc;
+    const long long n = row - j * (unsigned)P;
     const long long base = n * P + k - (long long)kc * Sc;
     const Acc* w = W + ((long long)j * Dc + kc) * Dc;
     Acc acc = 0;
