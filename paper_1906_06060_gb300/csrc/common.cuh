@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "../../include/hotrg.h"
@@ -167,8 +168,7 @@ using AccT = typename std::conditional<std::is_same<Tout, double>::value, double
 __device__ __forceinline__ float abs_up(double x) { return __double2float_ru(fabs(x)); }
 __device__ __forceinline__ float abs_up(float x) { return fabsf(x); }
 
-// Entry idx of a B operand of chi3 P rows and P columns (row = j P + n < 2^31): 32-bit divisions where the entries can
-// be counted in 32 bits. (Five 64-bit divisions an entry were most of the zero-field operand's 10.3 ms at D = 10.)
+// Entry idx of a P x P matrix: a 32-bit division where the entries can be counted in 32 bits.
 struct BtIndex {
   unsigned row, k;
   __device__ __forceinline__ BtIndex(long long idx, long long P, long long total) {
@@ -176,6 +176,40 @@ struct BtIndex {
     k = (unsigned)(idx - (long long)row * P);
   }
 };
+
+// B operands: weights U3[j][kc][x] in shared memory, rows of x padded to 16 bytes (one 16-byte read for 4 or 2 of them).
+template <class Acc>
+__host__ __device__ constexpr int bt_row(int Dc) {
+  constexpr int PAD = 16 / (int)sizeof(Acc);
+  return (Dc + PAD - 1) / PAD * PAD;
+}
+template <class Acc>
+__device__ __forceinline__ void load_bt_weights(Acc* W, const double* U, int chi3, int Dc) {
+  const int ws = bt_row<Acc>(Dc);
+  for (int t = threadIdx.x; t < chi3 * Dc * Dc; t += blockDim.x) W[t / Dc * ws + t % Dc] = U ? (Acc)U[t] : (Acc)1;
+}
+// acc + sum_x w[x] x[x], in the order of x
+template <class Acc>
+__device__ __forceinline__ Acc bt_dot(Acc acc, const Acc* w, const Acc* x, int Dc) {
+  constexpr int PAD = 16 / (int)sizeof(Acc);
+  struct alignas(16) Run {
+    Acc v[PAD];
+  };
+#pragma unroll
+  for (int i = 0; i < kMaxBond; i += PAD)
+    if (i < Dc) {
+      const Run r = *reinterpret_cast<const Run*>(w + i);
+#pragma unroll
+      for (int u = 0; u < PAD; ++u)
+        if (i + u < Dc) acc += r.v[u] * x[i + u];
+    }
+  return acc;
+}
+// rows j of one thread: all of them, or fewer where P^2 threads an instance would leave SMs idle
+inline int bt_rows_per_thread(long long threads, int chi3) {
+  const long long parts = std::max(1LL, std::min<long long>(chi3, 152LL * 2048 / std::max(1LL, threads)));
+  return (int)((chi3 + parts - 1) / parts);
+}
 
 // Blocks of a grid-stride kernel over n items.
 inline int grid_for(long long n, int block, int cap = 152 * 16) {

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(256) k_build_bt_z2(const Tin* __restrict__ Tt,
                                                      long long ld, long long P, long long Sc, int Dc,
                                                      const double* __restrict__ U3, int chi3, Z2Tables tab,
                                                      const Z2Layout* Lp, long long tt_inst, long long out_inst,
-                                                     long long u_inst) {
+                                                     long long u_inst, int jper) {
   using Acc = ZAcc<Tout>;
   Tt += blockIdx.y * tt_inst;
   out.advance(blockIdx.y, out_inst);
@@ -250,29 +250,31 @@ __global__ void __launch_bounds__(256) k_build_bt_z2(const Tin* __restrict__ Tt,
   const int* __restrict__ rank_tab = tab.rank + blockIdx.y * tab.p_inst;
   const int* __restrict__ kcol_tab = tab.kcol + blockIdx.y * tab.p_inst;
   const int* __restrict__ colpos_tab = tab.colpos + blockIdx.y * tab.c_inst;
-  extern __shared__ unsigned char smraw_bt[];
-  Acc* W = reinterpret_cast<Acc*>(smraw_bt);  // [chi3][Dc][Dc]
-  const int nW = chi3 * Dc * Dc;
-  for (int t = threadIdx.x; t < nW; t += blockDim.x) W[t] = (Acc)U3[t];
+  extern __shared__ __align__(16) unsigned char smraw_bt[];
+  Acc* W = reinterpret_cast<Acc*>(smraw_bt);  // [chi3][Dc][bt_row(Dc)]
+  const int ws = bt_row<Acc>(Dc);
+  load_bt_weights(W, U3, chi3, Dc);
   __syncthreads();
   const int ncls0 = Lp->ncls[0];
   const int goff1 = Lp->goff[1];
-  const long long total = (long long)chi3 * P * P;
+  const long long total = P * P;
+  const int j0 = blockIdx.z * jper, j1 = min(chi3, j0 + jper);
+  // (n, k) of a thread, all its j (as k_build_bt)
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
     const BtIndex e(idx, P, total);
-    const unsigned k = e.k, row = e.row;
-    const int cp = colpos_tab[row];
-    const int grp = cp >= goff1 ? 1 : 0;
-    const int park = rank_tab[k] >= ncls0 ? 1 : 0;
-    if (grp != park) continue;
-    const unsigned j = row / (unsigned)P, kc = (k / (unsigned)Sc) % (unsigned)Dc;
-    const long long n = row - j * (unsigned)P;
-    const long long base = n * P + k - (long long)kc * Sc;
-    const Acc* w = W + ((long long)j * Dc + kc) * Dc;
-    Acc acc = 0;
-    for (int x = 0; x < Dc; ++x) acc += w[x] * (Acc)Tt[base + x * Sc];
-    store_planes(out, (long long)cp * ld + kcol_tab[k], acc);
+    const unsigned k = e.k, kc = (k / (unsigned)Sc) % (unsigned)Dc;
+    const long long n = e.row, base = idx - (long long)kc * Sc;
+    const int park = rank_tab[k] >= ncls0 ? 1 : 0, col = kcol_tab[k];
+    Acc x[kMaxBond];
+#pragma unroll
+    for (int i = 0; i < kMaxBond; ++i)
+      if (i < Dc) x[i] = (Acc)Tt[base + i * Sc];
+    for (int j = j0; j < j1; ++j) {
+      const int cp = colpos_tab[j * P + n];
+      if ((cp >= goff1 ? 1 : 0) != park) continue;
+      store_planes(out, (long long)cp * ld + col, bt_dot((Acc)0, W + (j * Dc + (int)kc) * ws, x, Dc));
+    }
   }
 }
 
@@ -519,10 +521,11 @@ template <class Tin, class Tout>
 void launch_build_bt_z2(const Tin* Tt, long long tt_inst, const Planes<Tout>& out, long long out_inst, long long ld, Geom g,
                         int c3, const double* U3, long long u_inst, int chi3, const Z2Tables& t, const Z2Layout* L, int ng,
                         cudaStream_t s) {
-  const size_t smem = sizeof(ZAcc<Tout>) * (size_t)chi3 * g.D[c3] * g.D[c3];
-  const long long total = (long long)chi3 * g.P * g.P;
-  k_build_bt_z2<Tin, Tout><<<dim3(grid_cap(total), ng), 256, smem, s>>>(Tt, out, ld, g.P, g.Sn[c3], g.D[c3], U3, chi3, t,
-                                                                        L, tt_inst, out_inst, u_inst);
+  const size_t smem = sizeof(ZAcc<Tout>) * (size_t)chi3 * g.D[c3] * bt_row<ZAcc<Tout>>(g.D[c3]);
+  const int jper = bt_rows_per_thread(g.P * g.P * ng, chi3);
+  const dim3 grid(grid_cap(g.P * g.P), ng, (chi3 + jper - 1) / jper);
+  k_build_bt_z2<Tin, Tout><<<grid, 256, smem, s>>>(Tt, out, ld, g.P, g.Sn[c3], g.D[c3], U3, chi3, t, L, tt_inst, out_inst,
+                                                   u_inst, jper);
   count_launches(1);
 }
 
