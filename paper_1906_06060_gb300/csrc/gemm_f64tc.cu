@@ -101,6 +101,49 @@ __device__ __forceinline__ double assemble(long long hi, long long lo, int e) {
   return __longlong_as_double((long long)(u ? bits | ((unsigned long long)v & 0x8000000000000000ULL) : 0ULL));
 }
 
+// Where a fold thread's 128 entries of a finished tile (its row, columns col0 ...) go.
+struct TileOut {
+  double* dst = nullptr;  // null: nothing to do
+  const int* eb;
+  int ea, ncol;  // ncol: columns of the 128 inside the block
+  bool v4;
+};
+
+// Results of columns [j0, j0 + 4 JG) from the level sums in the scratch area (this thread's own stores). All loads are in
+// flight together: the loop is bound by their latency.
+template <int JG>
+__device__ __forceinline__ void finish_columns(const SliceParams& p, const TileOut& o, const int4* park, int j0) {
+  int4 l[JG][SC_PLANES];
+#pragma unroll
+  for (int g = 0; g < JG; ++g)
+#pragma unroll
+    for (int k = 0; k < SC_PLANES; ++k) l[g][k] = park[(k * 32 + j0 / 4 + g) * TC_FOLD_THREADS];
+#pragma unroll
+  for (int g = 0; g < JG; ++g) {
+    const int j = j0 + 4 * g;
+    auto value = [&](int u) -> double {
+      if (j + u >= o.ncol) return 0.0;
+      auto at = [&](int k) { return (long long)(u == 0 ? l[g][k].x : u == 1 ? l[g][k].y : u == 2 ? l[g][k].z : l[g][k].w); };
+      const int ebj = o.eb[j + u];
+      if (o.ea == kExpNaN || ebj == kExpNaN) return nan("");
+      return assemble((at(5) << 16) + (at(4) << 8) + at(3), (at(2) << 16) + (at(1) << 8) + at(0), o.ea + ebj - 54);
+    };
+    double v[4] = {value(0), value(1), value(2), value(3)};
+    if (o.v4) {
+      if (p.accumulate) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] += o.dst[j + u];
+      }
+      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o.dst + j), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+                   : "memory");
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (j + u < o.ncol) o.dst[j + u] = p.accumulate ? o.dst[j + u] + v[u] : v[u];
+    }
+  }
+}
+
 template <int CG>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_gemm_slices(const __grid_constant__ SliceMaps maps, SliceParams p) {
@@ -282,6 +325,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     int buf = 0;
     uint32_t bphase = 0;
     bool ok = true;
+    // a finished tile's results are formed four columns at a time between the chains of the next tile, up to its first
+    // parked level: formed at once, they held the MMAs up (683 -> 647 us at 1000 x 10000 x 1000, 2812 -> 2711 at 2048 x
+    // 16384 x 2048, pairs)
+    TileOut done;
+    int next = 0;  // columns of `done` formed so far
     for (int tile = cta0; tile < total && ok; tile += ncta) {
       int num_kb;
       {
@@ -290,6 +338,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         locate<SBK, CG>(p, s_prefix, tile, inst, bk, mt, nt);
         num_kb = bk.num_kb;
       }
+      int per = 0;  // column groups to form per chain
+      if (done.dst) {
+        int before = 0;
+        for (int s = NSL - 1; s >= 5; --s) before += (num_kb * (s + 1) + CHAIN - 1) / CHAIN;
+        per = (32 + before - 1) / max(1, before);
+      }
+      auto finish_some = [&](int groups) {
+        if (done.dst)
+          for (int g = 0; g < groups && next < done.ncol; ++g, next += 4) finish_columns<1>(p, done, park, next);
+        __syncwarp();
+      };
       int acc[128];
 #pragma unroll
       for (int j = 0; j < 128; ++j) acc[j] = 0;
@@ -323,8 +382,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             else mbar_arrive_remote(bar);
           }
           if (++buf == 2) { buf = 0; bphase ^= 1; }
+          if (s >= 5) finish_some(per);
         }
         if (!ok) break;
+        if (s == 5) finish_some(32);  // (the scratch area is written from here on)
         if (s > 5) {
           // carry into the next level's unit, rounded
 #pragma unroll
@@ -346,50 +407,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const long long row = (long long)bk.m0 + (long long)mt * TC_BM * CG + (long long)rank * TC_BM + q * 32 + lane;
       const long long col0 = (long long)bk.n0 + (long long)nt * TC_BN + half * 128;
       const long long row_end = (long long)bk.m0 + bk.mc, col_end = (long long)bk.n0 + bk.nc;
+      done.dst = nullptr;
+      next = 0;
       if (row < row_end && col0 < col_end) {
-        const int ea = p.ea[(long long)inst * p.ea_inst + row];
-        const int* eb = p.eb + (long long)(inst / p.b_div) * p.eb_inst + col0;
-        double* dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
-        const bool v4 = p.vec == 4 && (bk.n0 & 3) == 0 && col0 + 128 <= col_end;
-        // every level comes back from the scratch area (this thread's own stores) in a rolled loop: 128 unrolled
-        // assemblies from registers (300 KB of code) ran from the instruction cache's misses. All loads of 16 columns
-        // are in flight together: the loop is bound by their latency
-        constexpr int JG = 4;
-        for (int j0 = 0; j0 < 128; j0 += 4 * JG) {
-          if (col0 + j0 >= col_end) break;
-          int4 l[JG][SC_PLANES];
-#pragma unroll
-          for (int g = 0; g < JG; ++g)
-#pragma unroll
-            for (int k = 0; k < SC_PLANES; ++k) l[g][k] = park[(k * 32 + j0 / 4 + g) * TC_FOLD_THREADS];
-#pragma unroll
-          for (int g = 0; g < JG; ++g) {
-            const int j = j0 + 4 * g;
-            auto value = [&](int u) -> double {
-              if (col0 + j + u >= col_end) return 0.0;
-              auto at = [&](int k) { return (long long)(u == 0 ? l[g][k].x : u == 1 ? l[g][k].y : u == 2 ? l[g][k].z : l[g][k].w); };
-              const int ebj = eb[j + u];
-              if (ea == kExpNaN || ebj == kExpNaN) return nan("");
-              return assemble((at(5) << 16) + (at(4) << 8) + at(3), (at(2) << 16) + (at(1) << 8) + at(0), ea + ebj - 54);
-            };
-            double v[4] = {value(0), value(1), value(2), value(3)};
-            if (v4) {
-              if (p.accumulate) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] += dst[j + u];
-              }
-              asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + j), "d"(v[0]), "d"(v[1]), "d"(v[2]),
-                           "d"(v[3])
-                           : "memory");
-            } else {
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                if (col0 + j + u < col_end) dst[j + u] = p.accumulate ? dst[j + u] + v[u] : v[u];
-            }
-          }
-        }
+        done.ea = p.ea[(long long)inst * p.ea_inst + row];
+        done.eb = p.eb + (long long)(inst / p.b_div) * p.eb_inst + col0;
+        done.dst = p.C + (long long)inst * p.c_inst + row * p.ldc + col0;
+        done.ncol = (int)min(128LL, col_end - col0);
+        done.v4 = p.vec == 4 && (bk.n0 & 3) == 0 && done.ncol == 128;
       }
     }
+    // the last tile (a given-up kernel leaves no result worth storing)
+    if (ok && done.dst)
+      for (int j0 = 0; j0 < done.ncol; j0 += 16) finish_columns<4>(p, done, park, j0);
   }
   if constexpr (CG == 1) {
     __syncthreads();
@@ -574,7 +604,7 @@ int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, 
                        const GemmBatch* bat, bool accumulate, int cta_group) {
   if (!slices_take(M, N, K)) return HOTRG_EINVAL;
   if (cta_group == 0) {
-    // pairs (half the B copies per SM: 789 against 831 us at 1000 x 10000 x 1000) where their 256-row tiles pad no more
+    // pairs (half the B copies per SM: 647 against 708 us at 1000 x 10000 x 1000) where their 256-row tiles pad no more
     // rows than 128-row ones (else slower by what they pad: 768 against 640 rows at M = 625)
     const long long m = blk ? (M + 1) / 2 : M;
     cta_group = (m + 255) / 256 * 2 == (m + 127) / 128 ? 2 : 1;

@@ -47,6 +47,17 @@ def test_integers_are_exact(M, N, K, cta_group):
     assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("M,N,K", [(700, 20003, 64), (650, 16384, 200), (1100, 12289, 1090)])
+@pytest.mark.parametrize("cta_group", [1, 2])
+def test_several_tiles_of_a_cta_are_exact(M, N, K, cta_group):
+    """More tiles than CTAs: a tile's results are formed between the next one's accumulator chains (few of them at one
+    k-block), ragged tiles among them. Integers of 18 bits: no rounding."""
+    rng = np.random.default_rng(K)
+    a = rng.integers(-(2 ** 18), 2 ** 18, (M, K)).astype(np.float64)
+    b = rng.integers(-(2 ** 18), 2 ** 18, (N, K)).astype(np.float64)
+    assert np.array_equal(gemm_f64(a, b, cta_group, pad=(-N) % 4), a @ b.T)  # (sums below 2^53: exact in any order)
+
+
 @pytest.mark.parametrize("signs", [False, True])
 def test_largest_digits_fill_the_accumulators_exactly(signs):
     """Every digit at +-128, a whole number of accumulator chains: the sums reach their bounds. The exact value of an
