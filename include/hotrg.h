@@ -49,9 +49,13 @@ typedef enum hotrg_status {
 
 typedef enum hotrg_precision {
   HOTRG_FP64 = 0,   /* every contraction in FP64. The squeeze products run on the tensor cores from exact integer
-                       slices (each operand row as a 63-bit fixed-point number, 36 digit products, exact sums, one
-                       rounding) where the shape takes them (P >= 128, chi P >= 256, row length at most 16320, and a
-                       workspace up to 128 GiB), on the CUDA cores elsewhere; the rest on the CUDA cores */
+                       slices (the columns of both operands balanced by powers of two, each operand row as a 63-bit
+                       fixed-point number, 36 digit products, exact sums, one rounding) where the shape takes them
+                       (P >= 128, chi P >= 256, row length at most 16320, and a workspace up to 128 GiB), on the CUDA
+                       cores elsewhere; the rest on the CUDA cores. The error of a slice product beside its rounding
+                       is absolute, at most (2^-53 + K 2^-58) and typically 2^-55 of the product of the two rows'
+                       largest balanced entries, where that of an FP64 sum follows the sum's own terms. A row with
+                       a NaN or an infinity gives NaN */
   HOTRG_BF16X3 = 1, /* squeeze GEMM on tcgen05 tensor cores with split operands x = hi + lo
                        (bf16 each); products hi*hi + hi*lo + lo*hi accumulate in FP32 (TMEM):
                        O(2^-16) relative error per product. Gram matrices, eigensolver, norms

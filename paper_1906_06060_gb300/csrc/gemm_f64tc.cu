@@ -2,8 +2,10 @@
 // from exact integer slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
 //
 // GB300 has no fast FP64 unit (1.25 TFLOP/s nominal, 4 flop per clock and SM), its fp16 tensor cores run at
-// 8192 flop per clock and SM. Every row of an operand is scaled by a power of two 2^-e that brings its largest entry
-// below 1 and rounded to a 63-bit fixed-point number, which is cut into 8 balanced digits of 8 bits,
+// 8192 flop per clock and SM. Column k of A is scaled by a power of two c(k), the size of the largest entry of Bt's
+// column k, and column k of Bt by 1 / c(k): the product is the same. Then every row of an operand is scaled by a power of
+// two 2^-e that brings its largest entry below 1 and rounded to a 63-bit fixed-point number, which is cut into 8 balanced
+// digits of 8 bits,
 //   x 2^-e = sum_i q_i 2^-(7 + 8 i),  -128 <= q_i <= 128,
 // each stored as an fp16 integer (exact). The product is the sum over the digit pairs with i + j <= 7 (36 products),
 // grouped by level s = i + j:
@@ -11,11 +13,16 @@
 // Exactness: |qA qB| <= 2^14, so a chain of 16 x 64 products stays within 2^24 and the tensor cores' FP32 accumulator
 // holds it exactly; every chain is added into an int32 register accumulator (|L_s| <= (s + 1) K 2^14 < 2^31 for
 // K <= 16320). Levels 7 and 6 are folded into level 5 with a rounding shift each, and the six level sums are combined
-// exactly and rounded once. Entries within 2^-10 of their row's largest are held exactly; the dropped digit pairs are
-// worth about sqrt(7 K) 2^-65 of the two rows' largest entries. (Seven digits and 28 products, 13 - 22 % faster, drop
-// sqrt(6 K) 2^-57: at K = 4100 on rows that decay, further off than an FP64 product, so they are not taken.) Measured
-// relative error 5e-17 to 7e-17, one rounding, where FP64 products have 3e-16 to 1.1e-15. Rows holding NaN or infinity
-// give NaN.
+// exactly and rounded once.
+// Error of C[m][n]: one rounding of the result, and what the carries, the rows' last bits and the dropped digit pairs are
+// worth, at most (2^-53 + K 2^-58) R and typically 2^-55 R with R = max_k |A[m][k] c(k)| max_k |Bt[n][k] / c(k)|. It is an
+// error relative to R, where that of an FP64 sum (up to K 2^-53) is relative to sum_k |A[m][k] Bt[n][k]|. The two are of
+// one size within a factor of K for rows that share their decay, and, by the column scales, where A's columns grow as
+// Bt's decay (a tensor in an unbalanced gauge of its bonds); an output whose rows are large in different columns from
+// those of their neighbours can be far below R and keeps fewer bits than an FP64 sum would give it. (Seven digits and 28
+// products, 13 - 22 % faster, drop sqrt(6 K) 2^-57: at K = 4100 on rows that decay, further off than an FP64 product, so
+// they are not taken.) Measured over random rows, flat and decaying, in the 2-norm:
+// 5e-17 to 7e-17, one rounding, where FP64 products have 3e-16 to 1.1e-15. Rows holding NaN or infinity give NaN.
 //
 // Work: 36 tensor products of 2 M N K flops against one on the FP64 units at 1/2000 of the rate.
 // Kernel structure, ring and bounded waits as k_gemm_split (gemm_tc.cu): warp 0 copies, warp 1 issues MMAs, warps
@@ -442,16 +449,49 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------- slicing
+// Column fields: fields[k] = max over the rows of X (`rows` x K, row stride ldx, instances x_inst apart) of the exponent
+// field of X[.][k], an integer >= 1 for a non-zero finite entry, so 0 for a column without one; `fields` starts at zero.
+// A thread per column, the rows over blockIdx.y. Bound by reading X once; the column scales cost 0.4 % of a 4D FP64 step
+// (bond dimensions 5 x 6 x 4 x 5: 5.71 -> 5.73 ms), 1.5 % of a gradient (4D, bond dimension 5: 75.0 -> 76.1, where the
+// tangents' operands are built twice). Zero-field operands (L != null, instance blockIdx.z): a
+// column holds entries only in the rows of its class' column group.
+__device__ __forceinline__ int exponent_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+constexpr int FIELD_COLS = 128;
+__global__ void __launch_bounds__(FIELD_COLS) k_column_fields(const double* __restrict__ X, long long ldx, long long rows,
+                                                              int K, int* fields, const Z2Layout* __restrict__ L,
+                                                              long long x_inst, long long f_inst) {
+  X += (long long)blockIdx.z * x_inst;
+  fields += (long long)blockIdx.z * f_inst;
+  const int k = blockIdx.x * FIELD_COLS + threadIdx.x;
+  long long r = 0, end = k < K ? rows : 0;
+  if (L && k < K) {
+    L += blockIdx.z;
+    const int ck = k >= L->kstart[1] ? 1 : 0;
+    r = ck ? L->goff[1] : 0;
+    end = k - L->kstart[ck] >= L->ncls[ck] ? r : ck ? rows : L->goff[1];
+  }
+  int top = 0;
+#pragma unroll 4
+  for (r += blockIdx.y; r < end; r += gridDim.y) {
+    const double x = X[r * ldx + k];
+    const int f = exponent_field(x);
+    if (!is_zero(x) && f < 0x7FF) top = max(top, max(f, 1));
+  }
+  if (top) atomicMax(fields + k, top);
+}
+
 // One warp per row: the row's largest exponent field gives its scale, then every entry becomes NSL fp16 digits, all in
 // integer arithmetic (in FP64 operations, ten an entry at two a clock and SM, a 10^4 x 10^3 operand took 160 us; its
 // traffic is worth 32). Rows are read twice (the second time from L1 / L2), two columns a lane; digits are stored four
 // bytes a lane, coalesced.
+// Column scales: entry k counts as x 2^s(k) in Bt's rows and x 2^-s(k) in A's, s from the column fields of Bt (s cancels in
+// every product of the two; it exists only as an integer added to exponent fields). `side` = -1: a row of Bt, 1: of A. In
+// a column of zeros of Bt, A's entries count as zeros.
 // Zero-field operands (L != null): row r of slot blockIdx.y (instance blockIdx.y / nb) belongs to a parity class that
 // holds entries only in the columns [kstart, kstart + ncls) of its k class; the columns up to the next multiple of 64 get
-// zeros (the GEMM's k-blocks run over them). which = 0: row r of Bt, k class = its column group; which = 1: row r of A, k
-// class = its row class ^ pi[slot].
+// zeros (the GEMM's k-blocks run over them). k class of a row of Bt: its column group; of A: its row class ^ pi[slot].
 constexpr int SLICE_WARPS = 4;
-__device__ __forceinline__ int exponent_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 __device__ __forceinline__ long long fixed_point(double x, int top) {
   // x 2^(kSliceBits - e) with e = top - 1022, rounded half away from zero: the mantissa moved by the fields' difference
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
@@ -461,37 +501,62 @@ __device__ __forceinline__ long long fixed_point(double x, int top) {
   const unsigned long long v = sh <= 0 ? m << -sh : (sh > 54 ? 0ULL : (m + (1ULL << (sh - 1))) >> sh);
   return (long long)b < 0 ? -(long long)v : (long long)v;
 }
+// what column k's field adds to the exponent field of its entries; `dropped`: the entry counts as zero
+__device__ __forceinline__ int column_shift(int field, int side, bool& dropped) {
+  dropped = side > 0 && field == 0;
+  return side * (max(field, 1) - 1023);
+}
 __global__ void __launch_bounds__(32 * SLICE_WARPS) k_slice_rows(const double* __restrict__ X, long long ldx,
                                                                  long long rows, int K, __half* out, long long ld,
                                                                  long long plane, int* __restrict__ exps,
                                                                  const Z2Layout* __restrict__ L,
-                                                                 const int* __restrict__ pi, int which, long long x_inst,
-                                                                 long long o_inst, long long e_inst, int nb) {
+                                                                 const int* __restrict__ pi, int side, long long x_inst,
+                                                                 long long o_inst, long long e_inst, int nb,
+                                                                 const int* __restrict__ fields, long long f_inst) {
   const int lane = threadIdx.x % 32;
   const long long row = (long long)blockIdx.x * SLICE_WARPS + threadIdx.x / 32;
   if (row >= rows) return;
   X += (long long)blockIdx.y * x_inst + row * ldx;
   out += (long long)blockIdx.y * o_inst + row * ld;
+  fields += (blockIdx.y / nb) * f_inst;
   int kc = K, kpad = K;
   if (L) {
     L += blockIdx.y / nb;
-    const int ck = which == 0 ? (row >= L->goff[1] ? 1 : 0) : ((row >= L->ncls[0] ? 1 : 0) ^ pi[blockIdx.y]);
+    const int ck = side < 0 ? (row >= L->goff[1] ? 1 : 0) : ((row >= L->ncls[0] ? 1 : 0) ^ pi[blockIdx.y]);
     X += L->kstart[ck];
     out += L->kstart[ck];
+    fields += L->kstart[ck];
     kc = L->ncls[ck];
     kpad = (kc + 63) / 64 * 64;
   }
-  int top = 1;  // (all subnormal: their unit's field)
+  constexpr int kNone = -(1 << 20);  // no entry but zeros
+  int top = kNone;
+  bool finite = true;
 #pragma unroll 4
-  for (int k = lane; k < kc; k += 32) top = max(top, exponent_field(X[k]));
+  for (int k = lane; k < kc; k += 32) {
+    const double x = X[k];
+    const int f = exponent_field(x);
+    bool dropped;
+    const int shift = column_shift(fields[k], side, dropped);
+    finite = finite && f < 0x7FF;
+    if (!dropped && !is_zero(x)) top = max(top, max(f, 1) + shift);
+  }
   for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-  const bool finite = top < 0x7FF;
+  finite = __all_sync(0xffffffffu, finite);
+  if (top == kNone) top = 1022;
   if (lane == 0) exps[(long long)blockIdx.y * e_inst + row] = finite ? top - 1022 : kExpNaN;
 #pragma unroll 2
   for (int k = 2 * lane; k < kpad; k += 64) {
     long long v[2];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) v[u] = (finite && k + u < kc) ? fixed_point(X[k + u], top) : 0;
+    for (int u = 0; u < 2; ++u) {
+      v[u] = 0;
+      if (finite && k + u < kc) {
+        bool dropped;
+        const int shift = column_shift(fields[k + u], side, dropped);
+        if (!dropped) v[u] = fixed_point(X[k + u], top - shift);
+      }
+    }
     const bool both = k + 1 < kpad;
 #pragma unroll
     for (int i = NSL - 1; i >= 0; --i) {
@@ -592,10 +657,22 @@ size_t slice_scratch_bytes(long long M, long long N, int batch) {
   return (size_t)t * SC_PLANES * 128 * TC_FOLD_THREADS * sizeof(int);
 }
 
+void launch_column_fields(const double* X, long long ldx, long long rows, long long K, int* fields, long long f_inst,
+                          int batch, long long x_inst, cudaStream_t s, const Z2Layout* L) {
+  const int gx = (int)((K + FIELD_COLS - 1) / FIELD_COLS);
+  // about 16 blocks an SM, at least 8 rows a block
+  const long long gy = std::max(1LL, std::min((rows + 7) / 8, 152LL * 16 / ((long long)gx * batch)));
+  k_column_fields<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)batch), FIELD_COLS, 0, s>>>(X, ldx, rows, (int)K, fields, L,
+                                                                                          x_inst, f_inst);
+  count_launches(1);
+}
+
 void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
-                       long long x_inst, cudaStream_t s, const Z2Layout* L, const int* pi, int which, int nb) {
+                       long long x_inst, const int* fields, long long f_inst, int side, cudaStream_t s, int nb,
+                       const Z2Layout* L, const int* pi) {
   k_slice_rows<<<dim3((unsigned)((rows + SLICE_WARPS - 1) / SLICE_WARPS), (unsigned)batch), 32 * SLICE_WARPS, 0, s>>>(
-      X, ldx, rows, (int)K, out.p, out.ld, out.plane, out.exps, L, pi, which, x_inst, out.inst, out.exp_inst, nb);
+      X, ldx, rows, (int)K, out.p, out.ld, out.plane, out.exps, L, pi, side, x_inst, out.inst, out.exp_inst, nb, fields,
+      f_inst);
   count_launches(1);
 }
 

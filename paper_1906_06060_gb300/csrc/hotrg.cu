@@ -41,18 +41,19 @@ long long output_ld(long long n, bool mixed, bool slices) { return mixed ? round
 // Bytes a slot of a per-step buffer takes (256-byte aligned: TMA plane starts).
 size_t slot_bytes(size_t n) { return (size_t)round_up((long long)(n ? n : 1), kAlign); }
 
-// Sizes (bytes) of the per-step buffers for one configuration: Tt, Bt, X1, eb per instance of a group, the others per
-// chunk in flight; nb: chunks in flight; yt, ey, eb, scr: FP64 products on digit slices.
+// Sizes (bytes) of the per-step buffers for one configuration: Tt, Bt, X1, eb, kf per instance of a group, the others per
+// chunk in flight; nb: chunks in flight; yt, ey, eb, kf, scr: FP64 products on digit slices.
 struct StepNeeds {
   size_t Tt = 0, Bt = 0, X1 = 0, eb = 0;
   size_t X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0;
+  size_t kf = 0;
   size_t scr = 0;
   int nb = 1, go = 1;  // chunks in flight: values of the inner and of the outer fixed axis
 };
 
 // Bytes per instance of the group that hold every step of a plan.
 struct StepSizes {
-  size_t Tt = 0, Bt = 0, X1 = 0, eb = 0, X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0, scr = 0;
+  size_t Tt = 0, Bt = 0, X1 = 0, eb = 0, kf = 0, X2 = 0, Y = 0, O = 0, R1 = 0, R2 = 0, yt = 0, ey = 0, scr = 0;
   static StepSizes of(const StepNeeds& n) {
     auto chunks = [&](size_t x) { return (size_t)n.nb * n.go * slot_bytes(x); };
     StepSizes z;
@@ -60,6 +61,7 @@ struct StepSizes {
     z.Bt = slot_bytes(n.Bt);
     z.X1 = n.go * slot_bytes(n.X1);
     z.eb = slot_bytes(n.eb);
+    z.kf = slot_bytes(n.kf);
     z.X2 = chunks(n.X2);
     z.Y = chunks(n.Y);
     z.O = chunks(n.O);
@@ -72,7 +74,7 @@ struct StepSizes {
   }
   template <class F>
   static void each(F f) {
-    for (size_t StepSizes::*m : {&StepSizes::Tt, &StepSizes::Bt, &StepSizes::X1, &StepSizes::eb, &StepSizes::X2,
+    for (size_t StepSizes::*m : {&StepSizes::Tt, &StepSizes::Bt, &StepSizes::X1, &StepSizes::eb, &StepSizes::kf, &StepSizes::X2,
                                  &StepSizes::Y, &StepSizes::O, &StepSizes::R1, &StepSizes::R2, &StepSizes::yt,
                                  &StepSizes::ey, &StepSizes::scr})
       f(m);
@@ -144,6 +146,7 @@ StepNeeds needs_for(int d, const int* dims, int a, int Dcut, int planes, bool sl
     n.yt = (size_t)(P * ldk) * 8;
     n.ey = (size_t)P * sizeof(int) * nblk;
     n.eb = (size_t)(chi3 * P) * sizeof(int) * nblk;
+    n.kf = (size_t)ldk * sizeof(int);
   }
   // epilogue intermediates: contract the other transverse axes in order
   long long cur = P * chi3 * P;
@@ -235,8 +238,9 @@ struct hotrg_ctx {
   void *R1 = nullptr, *R2 = nullptr;
   // FP64 products on the tensor cores (gemm_f64tc.cu): the Y and Bt buffers then hold digit planes. yt: the A operand
   // in double before slicing (the B operand is built in O, free until the first chunk), ey / eb: row exponents,
-  // slice_scratch: level sums of the running launch
+  // kf: column fields, slice_scratch: level sums of the running launch
   bool slices = true;
+  int* kf = nullptr;
   void *yt = nullptr, *ey = nullptr, *eb = nullptr, *slice_scratch = nullptr;
   // instances squeezed together (one GEMM launch per chunk batch for all of them): every per-step buffer holds `group`
   // times the bytes sz lists
@@ -475,6 +479,7 @@ size_t carve(hotrg_ctx* c, char* base) {
     c->yt = k.take<char>(z.yt * G);
     c->ey = k.take<char>(z.ey * G);
     c->eb = k.take<char>(z.eb * G);
+    c->kf = k.take<int>(z.kf * G);
     c->slice_scratch = k.take<char>(z.scr);
   }
   if (c->deriv) {
@@ -680,8 +685,8 @@ struct Tangents {
   const double* dU[2] = {nullptr, nullptr};
 };
 
-// Per-step scratch regions. Per instance j of a squeeze group (strides st_*): Tt, Bt, X1, Tnext, the row exponents of
-// Bt, the zero-field tables. Per slot z = j * (chunks in flight) + chunk, at strides chosen by each step (slot_bytes):
+// Per-step scratch regions. Per instance j of a squeeze group (strides st_*): Tt, Bt, X1, Tnext, the row exponents and
+// column fields of Bt, the zero-field tables. Per slot z = j * (chunks in flight) + chunk, at strides chosen by each step (slot_bytes):
 // X2, Y, O, R1, R2, yt, ey, and the chunk's parity and GEMM blocks.
 // The instances squeezed together: instance j reads T1 + j t_inst (lower site, A operand) and T2 + j t_inst (upper site,
 // B operand) with isometries U + j u_inst and writes out + j out_inst; inst0 + j is its index in the context (zero-field
@@ -806,7 +811,13 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
     cudaMemsetAsync(c->Bt, 0, c->sz.Bt * (ng - 1) + sizeof(Op) * nparts * bt_plane, s);
     cudaMemsetAsync(c->Y, 0, cY * (ng * need.nb * need.go - 1) + sizeof(Op) * nparts * y_plane, s);
   }
-  auto build_bt = [&](const TC* src, int blk, int which, const double* U, const TC* src2, const double* U2) {
+  // On digit slices the column scales come first: those of all blocks, as the tangents' products share A operands. The
+  // tangents' blocks are built to gather theirs, then again to be cut; the forward block, between, does both at once.
+  enum { kGather, kCut, kBoth };
+  const long long kf_inst = (long long)(c->sz.kf / sizeof(int));
+  if (sl) cudaMemsetAsync(c->kf, 0, c->sz.kf * (ng - 1) + sizeof(int) * ldt, s);
+  auto build_bt = [&](const TC* src, int blk, int which, const double* U, const TC* src2, const double* U2,
+                      int part = kBoth) {
     const long long src_inst = (long long)(c->sz.Tt / sizeof(TC)), bt_inst = (long long)(c->sz.Bt / sizeof(Op));
     const long long o_inst = sl ? (long long)chi3 * P * ldt : bt_inst;  // sliced: the instances one after the other in O
     const int at_once = sl ? std::max(1, std::min<int>(ng, (int)(c->sz.O * (size_t)c->group / (sizeof(double) * o_inst)))) : ng;
@@ -821,29 +832,33 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
         launch_build_bt<TC, Op>(sj, src_inst, dst, o_inst, sl ? ldt : ld, g, c3, uj, G.u_inst, chi3, n, s, src2, U2);
       if constexpr (!mixed) {
         if (sl) {
+          const double* built = static_cast<double*>(c->O);
+          int* const kf = c->kf + j0 * kf_inst;
+          const Z2Layout* Lj = z2 ? L + j0 : nullptr;
+          if (part != kCut) launch_column_fields(built, ldt, (long long)chi3 * P, ldt, kf, kf_inst, n, o_inst, s, Lj);
+          if (part == kGather) continue;
           SliceOperand o = slice_bt(blk);
           o.p += j0 * o.inst;
           o.exps += j0 * o.exp_inst;
-          launch_slice_rows(static_cast<double*>(c->O), ldt, (long long)chi3 * P, ldt, o, n, o_inst, s,
-                            z2 ? L + j0 : nullptr, nullptr, 0, 1);
+          launch_slice_rows(built, ldt, (long long)chi3 * P, ldt, o, n, o_inst, kf, kf_inst, -1, s, 1, Lj);
         }
       }
     }
   };
-  {
-    TC* Tt = static_cast<TC*>(c->Tt);
-    const long long tt_inst = (long long)(c->sz.Tt / sizeof(TC));
-    launch_transpose<TC>(G.T2, G.t_inst, Tt, tt_inst, P, ng, s);
-    if (f16) launch_absmax<TC>(Tt, P, P, P, amaxB, s, ng, tt_inst);
-    build_bt(Tt, fwd_blk, 0, c3 >= 0 ? Ub(G.U, c3) : nullptr, nullptr, nullptr);
-  }
-  for (int p = 0; p < tg.n; ++p) {
+  TC* const Tt = static_cast<TC*>(c->Tt);
+  const long long tt_inst = (long long)(c->sz.Tt / sizeof(TC));
+  launch_transpose<TC>(G.T2, G.t_inst, Tt, tt_inst, P, ng, s);
+  if (f16) launch_absmax<TC>(Tt, P, P, P, amaxB, s, ng, tt_inst);
+  auto tangent_bt = [&](int p, int part) {
     TC* dTt = static_cast<TC*>(c->Tt2);
     launch_transpose<TC>(tg.dT[p], 0, dTt, 0, P, 1, s);
     const bool two = tg.dU[p] && c3 >= 0;
-    build_bt(dTt, dbt_blk(p), -1, c3 >= 0 ? Ub(G.U, c3) : nullptr, two ? static_cast<TC*>(c->Tt) : nullptr,
-             two ? Ub(tg.dU[p], c3) : nullptr);
-  }
+    build_bt(dTt, dbt_blk(p), -1, c3 >= 0 ? Ub(G.U, c3) : nullptr, two ? Tt : nullptr, two ? Ub(tg.dU[p], c3) : nullptr,
+             part);
+  };
+  for (int p = 0; p < tg.n && sl; ++p) tangent_bt(p, kGather);
+  build_bt(Tt, fwd_blk, 0, c3 >= 0 ? Ub(G.U, c3) : nullptr, nullptr, nullptr);
+  for (int p = 0; p < tg.n; ++p) tangent_bt(p, kCut);
   delete ops_scope;
   TC* O = static_cast<TC*>(c->O);
   TC* dO = static_cast<TC*>(c->dO);
@@ -879,7 +894,8 @@ int squeeze(hotrg_ctx* c, const Group& G, const Geom& g, const Geom& gn, int a, 
           launch_build_y<Tin, Op>(src, src_slot, dst, dst_slot, sl ? ldt : ld, g, a, nz, s);
         if constexpr (!mixed) {
           if (sl)
-            launch_slice_rows(static_cast<double*>(c->yt), ldt, P, ldt, slice_y(blk), nz, dst_slot, s, L, c->z2pi, 1, nb);
+            launch_slice_rows(static_cast<double*>(c->yt), ldt, P, ldt, slice_y(blk), nz, dst_slot, c->kf, kf_inst, 1, s,
+                              nb * go, L, c->z2pi);
         }
       };
       if (no == 0) {
@@ -2025,11 +2041,11 @@ int hotrg_gemm_split_f16(const float* A, long long lda, const float* Bt, long lo
   return cudaGetLastError() == cudaSuccess ? HOTRG_OK : HOTRG_EDEVICE;
 }
 
-// scratch: status word (256 bytes), row exponents, digit planes and level sums of the launch
+// scratch: status word (256 bytes), row exponents, column fields, digit planes and level sums of the launch
 size_t hotrg_gemm_f64_scratch_bytes(long long M, long long N, long long K) {
   if (!slices_take(M, N, K)) return 0;
   const long long ld = round_up(K, 64);
-  return (size_t)(kAlign + round_up((M + N) * (long long)sizeof(int), kAlign) + round_up(2 * kSliceCount * M * ld, kAlign) +
+  return (size_t)(kAlign + round_up((M + N + K) * (long long)sizeof(int), kAlign) + round_up(2 * kSliceCount * M * ld, kAlign) +
                   round_up(2 * kSliceCount * N * ld, kAlign)) +
          slice_scratch_bytes(M, N, 1);
 }
@@ -2047,14 +2063,18 @@ int hotrg_gemm_f64(const double* A, long long lda, const double* Bt, long long l
   int* status = reinterpret_cast<int*>(p);
   p += kAlign;
   int* exps = reinterpret_cast<int*>(p);
-  p += round_up((M + N) * (long long)sizeof(int), kAlign);
+  int* const kf = exps + M + N;
+  p += round_up((M + N + K) * (long long)sizeof(int), kAlign);
   const SliceOperand a = slice_operand(p, M * ld, ld, ld, 0, exps, M, 0, 0);
   p += round_up(2 * kSliceCount * M * ld, kAlign);
   const SliceOperand b = slice_operand(p, N * ld, ld, ld, 0, exps + M, N, 0, 0);
   p += round_up(2 * kSliceCount * N * ld, kAlign);
-  if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return HOTRG_EDEVICE;
-  launch_slice_rows(A, lda, M, K, a, 1, 0, s);
-  launch_slice_rows(Bt, ldb, N, K, b, 1, 0, s);
+  if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess ||
+      cudaMemsetAsync(kf, 0, sizeof(int) * K, s) != cudaSuccess)
+    return HOTRG_EDEVICE;
+  launch_column_fields(Bt, ldb, N, K, kf, 0, 1, 0, s);
+  launch_slice_rows(A, lda, M, K, a, 1, 0, kf, 0, 1, s);
+  launch_slice_rows(Bt, ldb, N, K, b, 1, 0, kf, 0, -1, s);
   const int rc = launch_gemm_slices(a, b, C, ldc, M, N, K, reinterpret_cast<int*>(p), status, 4.0, s, nullptr, nullptr,
                                     false, cta_group);
   if (rc) return rc;

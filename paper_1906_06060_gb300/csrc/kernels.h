@@ -193,12 +193,18 @@ struct SliceOperand {
 bool slices_take(long long M, long long N, long long K);
 // Bytes of the level-sum scratch of a launch over `batch` products of at most M x N.
 size_t slice_scratch_bytes(long long M, long long N, int batch);
-// Digits and row exponents of `rows` x K doubles (row stride ldx; `batch` instances x_inst apart). With L (zero-field
-// operands: instance z / nb's layout, slot z's chunk parity) only the columns of each row's parity class, see k_slice_rows.
 struct Z2Layout;
+// Column scales of a product, from its Bt (`rows` x K doubles, row stride ldx; `batch` instances x_inst apart):
+// fields[k] = max(fields[k], largest exponent field in column k), instances f_inst apart, zeroed by the caller. With L
+// (zero-field operands) only the entries of the parity classes.
+void launch_column_fields(const double* X, long long ldx, long long rows, long long K, int* fields, long long f_inst,
+                          int batch, long long x_inst, cudaStream_t s, const Z2Layout* L = nullptr);
+// Digits and row exponents of `rows` x K doubles (row stride ldx; `batch` slots x_inst apart) with the column scales of
+// slot z's instance z / nb. side: -1 for Bt, 1 for A. With L (zero-field operands: instance z / nb's layout, slot z's
+// chunk parity) only the columns of each row's parity class, see k_slice_rows.
 void launch_slice_rows(const double* X, long long ldx, long long rows, long long K, const SliceOperand& out, int batch,
-                       long long x_inst, cudaStream_t s, const Z2Layout* L = nullptr, const int* pi = nullptr,
-                       int which = 0, int nb = 1);
+                       long long x_inst, const int* fields, long long f_inst, int side, cudaStream_t s, int nb = 1,
+                       const Z2Layout* L = nullptr, const int* pi = nullptr);
 // C[m][n] (+)= sum_k A[m][k] Bt[n][k]; blk and bat as for launch_gemm_f64. cta_group: 1 or 2 CTAs per tile (the same
 // results), 0: by shape. Returns 0 or a hotrg_status.
 int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,

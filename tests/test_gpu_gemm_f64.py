@@ -124,3 +124,91 @@ def test_shapes_it_does_not_take(M, N, K):
     assert lib.hotrg_gemm_f64_scratch_bytes(M, N, K) == 0
     p = c_void_p(256)
     assert lib.hotrg_gemm_f64(p, K, p, K, p, N, M, N, K, 1, p, 1 << 40, None) == _lib.HOTRG_EINVAL
+
+
+def _exact_dot(a, b):
+    """Sum of a b, rounded once (Dekker's exact products)."""
+    p, split = a * b, 134217729.0
+    ah, bh = a * split, b * split
+    ah, bh = ah - (ah - a), bh - (bh - b)
+    al, bl = a - ah, b - bh
+    return math.fsum(np.concatenate([p, ((ah * bh - p) + ah * bl + al * bh) + al * bl]))
+
+
+@pytest.mark.parametrize("M,N,K,decay", [(300, 400, 600, 0.04), (130, 300, 128, 0.5), (257, 260, 2049, 0.02),
+                                         (128, 256, 64, -0.9)])
+@pytest.mark.parametrize("cta_group", [1, 2])
+def test_columns_that_grow_where_the_others_decay(M, N, K, decay, cta_group):
+    """A decays along k as Bt grows, by up to 28 orders: the products are of one size, and what counts are each row's
+    small entries. Error: a rounding and (2^-53 + K 2^-58) of the product of the rows' largest entries after the
+    power-of-two column scales (the sizes of Bt's columns); in the 2-norm no further off than NumPy's FP64 product."""
+    rng = np.random.default_rng(K)
+    A = rng.standard_normal((M, K)) * np.exp(-decay * np.arange(K))
+    B = rng.standard_normal((N, K)) * np.exp(decay * np.arange(K))
+    got = gemm_f64(A, B, cta_group)
+    host = A @ B.T
+    c = np.ldexp(1.0, np.frexp(np.abs(B).max(0))[1] - 1)
+    ra, rb = np.abs(A * c).max(1), np.abs(B / c).max(1)
+    e, e_host = [], []
+    for m, n in zip(rng.integers(0, M, 300), rng.integers(0, N, 300)):
+        ref = _exact_dot(A[m], B[n])
+        assert abs(got[m, n] - ref) <= 2.0 ** -53 * abs(ref) + (2.0 ** -53 + K * 2.0 ** -58) * ra[m] * rb[n]
+        e.append(got[m, n] - ref)
+        e_host.append(host[m, n] - ref)
+    assert np.linalg.norm(e) <= np.linalg.norm(e_host)
+
+
+def test_columns_of_zeros_and_extreme_columns():
+    """A column of zeros of Bt leaves no trace of A's entries there, however large, unless they are not finite; columns at
+    the ends of the exponent range, subnormal ones included, cancel in the scales. Integers: no rounding."""
+    rng = np.random.default_rng(1)
+    M, N, K = 130, 300, 100
+    a = rng.integers(-(2 ** 20) + 1, 2 ** 20, (M, K))
+    b = rng.integers(-(2 ** 20) + 1, 2 ** 20, (N, K))
+    b[:, 7] = 0
+    ref = (a @ b.T).astype(np.float64)
+    g = rng.integers(-900, 900, K)
+    g[[3, 4]] = 1000, -1000
+    A, B = np.ldexp(a.astype(np.float64), -g), np.ldexp(b.astype(np.float64), g)
+    A[:, 7] = 1e300
+    B[:, 11] = np.ldexp(b[:, 11].astype(np.float64), -1074)
+    A[:, 11] = np.ldexp(a[:, 11].astype(np.float64), 1000)
+    ref = (ref - np.outer(a[:, 11], b[:, 11])) + np.ldexp(np.outer(a[:, 11], b[:, 11]).astype(np.float64), -74)
+    A[9, 7] = np.nan
+    got = gemm_f64(A, B)
+    assert np.all(np.isnan(got[9]))
+    keep = np.arange(M) != 9
+    # (column 11 is 2^-74 of the others: the sum of the two rounds once)
+    assert np.abs(got - ref)[keep].max() <= 2.0 ** -52 * np.abs(ref).max()
+
+
+def test_step_of_a_tensor_in_an_unbalanced_gauge():
+    """The bond along the merged axis scaled by 2^-12 i on its lower leg and 2^12 i on its upper one: the same contraction,
+    from operands whose rows spread over 36 bits in opposite directions. Every block of the new tensor (a pair of values of
+    the outer legs of that axis) against the oracle, to the rounding that the isometries allow: 8 n eps lambda_0 / gap for
+    each of six, as a step from a balanced tensor, and 1e-13."""
+    from oracle import hotrg_ref as R
+    from paper_1906_06060_gb300 import HOTRG
+    from tests.inputs import random_site_tensor
+    n = 4
+    T = random_site_tensor((n,) * 4, seed=3)
+    for axis in range(8):
+        shape = [1] * 8
+        shape[axis] = n
+        T = T * (0.8 ** np.arange(n)).reshape(shape)
+    g = np.ldexp(1.0, 12 * np.arange(n))
+    T = T / g.reshape((1, 1, 1, n, 1, 1, 1, 1)) * g
+    ref, info = R.coarse_grain(T, 3, n)
+    ref /= R.frobenius(ref)
+    tol = 1e-13
+    for iso in info.isometries.values():
+        lam = iso.eigenvalues
+        tol += 8 * lam.size * 2.0 ** -52 * lam[0] / np.min(lam[:n] - lam[1:n + 1])
+    with HOTRG(4, 0.3, 0.0, n, precision="fp64") as f:
+        f.set_tensor(T)
+        f.step(3)
+        got = f.get_tensor()
+    for u in range(n):
+        for p in range(n):
+            x, y = got[:, :, :, u, :, :, :, p], ref[:, :, :, u, :, :, :, p]
+            assert np.linalg.norm(x - y) <= tol * np.linalg.norm(y), (u, p)
