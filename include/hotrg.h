@@ -340,11 +340,12 @@ int hotrg_gemm_f64(const double *A, long long lda, const double *Bt, long long l
 /* Failure-detection probe of the bounded device-side waits (the paper has no counterpart): two
  * launches of the tensor-core GEMM (BF16X3, one output tile: first on one CTA, then on a CTA pair)
  * whose copy-issuing thread issues no copies, so that the first wait for operand data can never
- * be satisfied. The waits give up after timeout_s (0 < timeout_s <= 10), each kernel records the
- * timeout, frees its tensor memory and returns; nothing is left in flight. `scratch` (device,
- * 256-B aligned) holds at least hotrg_gemm_wait_probe_bytes() bytes. Synchronises `stream`;
- * returns HOTRG_ETIMEOUT when both launches timed out as intended, else the first other status.
- * Other errors: EINVAL, EDEVICE. */
+ * be satisfied, and four of the FP64 product on slices (one CTA; a pair of which both CTAs, only the
+ * second or only the first issue no copies). The waits give up after timeout_s (0 < timeout_s <= 10),
+ * each kernel records the timeout, frees its tensor memory and returns; nothing is left in flight.
+ * `scratch` (device, 256-B aligned) holds at least hotrg_gemm_wait_probe_bytes() bytes. Synchronises
+ * `stream`; returns HOTRG_ETIMEOUT when every launch timed out as intended, else the first other
+ * status. Other errors: EINVAL, EDEVICE. */
 size_t hotrg_gemm_wait_probe_bytes(void);
 int hotrg_gemm_wait_probe(double timeout_s, void *scratch, size_t scratch_bytes, void *stream);
 

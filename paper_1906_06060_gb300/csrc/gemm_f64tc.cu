@@ -70,6 +70,7 @@ struct SliceParams {
   uint32_t idesc;
   int accumulate;  // C += instead of C =
   int vec;         // entries per store: 4 (32-byte aligned rows) or 1
+  int stall;       // wait probe: bit r: CTA r of the pair (or the CTA) issues no copies
 };
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (warp == 0) {
     // every CTA copies its own tiles (128 rows of A, its share of the B rows); a pair's bytes all count on the first
     // CTA's barriers, and a stage is freed in both CTAs by the commit of the MMAs that read it
-    if (lane == 0) {
+    if (lane == 0 && !(p.stall >> rank & 1)) {
       int stage = 0;
       uint32_t phase = 0;
       long long issued = 0;
@@ -273,16 +274,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
           }
       }
-      // drain the copies in flight on every exit path (see k_gemm_split); the second CTA of a pair waits for the first at
-      // the final cluster barrier
+      // drain the copies in flight (see k_gemm_split; of a given-up pair: below)
       if (leader) {
         for (long long i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i)
           mbar_wait(full0 + 8 * (int)(i % STAGES), (uint32_t)((i / STAGES) & 1), abort_flag, drain_ns(p.timeout_ns),
-                    false);
-        // a given-up pair may have copies of the second CTA in flight for a stage this CTA never announced: they
-        // always land, within microseconds
-        if (CG == 2 && !ok)
-          for (const unsigned long long t0 = globaltimer_ns(); globaltimer_ns() - t0 < 2000000ull;) {}
+                    CG == 2);
       }
     }
   } else if (warp == 1) {
@@ -437,9 +433,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                    : "memory");
     }
   } else {
+    // A warp that gave up, or saw that its CTA did, tells the other CTA: after the barrier both know, and neither issues
+    // copies any more.
+    if (lane == 0 && *abort_flag) store_remote(mapa_rank(smem_u32(tmem_slot + 1), rank ^ 1u), 1);
     __syncwarp();
     cluster_sync();
-    if (threadIdx.x == 0 && *abort_flag) atomic_status(p.status, ST_TIMEOUT);
+    if (*abort_flag) {
+      // Copies of a stage that only one of the CTAs filled complete no phase of its barrier, so nothing signals that the
+      // last ones have landed: 2 ms, a thousand times what a copy takes, before either CTA may leave.
+      for (const unsigned long long t0 = globaltimer_ns(); globaltimer_ns() - t0 < 2000000ull;) {}
+      __syncwarp();
+      cluster_sync();
+      if (threadIdx.x == 0) atomic_status(p.status, ST_TIMEOUT);
+    }
     if (warp == 1) {
       tc_fence_after();
       asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
@@ -678,7 +684,7 @@ void launch_slice_rows(const double* X, long long ldx, long long rows, long long
 
 int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,
                        long long K, int* scratch, int* status, double timeout_s, cudaStream_t s, const GemmBlocks* blk,
-                       const GemmBatch* bat, bool accumulate, int cta_group) {
+                       const GemmBatch* bat, bool accumulate, int cta_group, int stall) {
   if (!slices_take(M, N, K)) return HOTRG_EINVAL;
   if (cta_group == 0) {
     // pairs (half the B copies per SM: 647 against 708 us at 1000 x 10000 x 1000) where their 256-row tiles pad no more
@@ -712,6 +718,7 @@ int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, 
   p.timeout_ns = (unsigned long long)(timeout_s * 1e9);
   p.blk = blk;
   p.accumulate = accumulate ? 1 : 0;
+  p.stall = stall;
   p.vec = (ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(C) & 31) == 0 && (p.c_inst % 4) == 0 ? 4 : 1;
   p.idesc = idesc_for(true, cta_group);
   long long t = slice_tiles(M, N, cta_group) * batch;

@@ -2050,6 +2050,33 @@ size_t hotrg_gemm_f64_scratch_bytes(long long M, long long N, long long K) {
          slice_scratch_bytes(M, N, 1);
 }
 
+}  // extern "C"
+
+namespace {
+struct SliceScratch {
+  int* status;
+  int* kf;
+  SliceOperand a, b;
+  int* sums;
+  SliceScratch(void* scratch, long long M, long long N, long long K) {
+    const long long ld = round_up(K, 64);
+    char* p = static_cast<char*>(scratch);
+    status = reinterpret_cast<int*>(p);
+    p += kAlign;
+    int* exps = reinterpret_cast<int*>(p);
+    kf = exps + M + N;
+    p += round_up((M + N + K) * (long long)sizeof(int), kAlign);
+    a = slice_operand(p, M * ld, ld, ld, 0, exps, M, 0, 0);
+    p += round_up(2 * kSliceCount * M * ld, kAlign);
+    b = slice_operand(p, N * ld, ld, ld, 0, exps + M, N, 0, 0);
+    p += round_up(2 * kSliceCount * N * ld, kAlign);
+    sums = reinterpret_cast<int*>(p);
+  }
+};
+}  // namespace
+
+extern "C" {
+
 int hotrg_gemm_f64(const double* A, long long lda, const double* Bt, long long ldb, double* C, long long ldc, long long M,
                    long long N, long long K, int cta_group, void* scratch, size_t scratch_bytes, void* stream) {
   if (!A || !Bt || !C || !scratch || lda < K || ldb < K || ldc < N || (cta_group != 1 && cta_group != 2))
@@ -2058,31 +2085,23 @@ int hotrg_gemm_f64(const double* A, long long lda, const double* Bt, long long l
       (reinterpret_cast<uintptr_t>(scratch) % kAlign))
     return HOTRG_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const long long ld = round_up(K, 64);
-  char* p = static_cast<char*>(scratch);
-  int* status = reinterpret_cast<int*>(p);
-  p += kAlign;
-  int* exps = reinterpret_cast<int*>(p);
-  int* const kf = exps + M + N;
-  p += round_up((M + N + K) * (long long)sizeof(int), kAlign);
-  const SliceOperand a = slice_operand(p, M * ld, ld, ld, 0, exps, M, 0, 0);
-  p += round_up(2 * kSliceCount * M * ld, kAlign);
-  const SliceOperand b = slice_operand(p, N * ld, ld, ld, 0, exps + M, N, 0, 0);
-  p += round_up(2 * kSliceCount * N * ld, kAlign);
-  if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess ||
-      cudaMemsetAsync(kf, 0, sizeof(int) * K, s) != cudaSuccess)
+  const SliceScratch q(scratch, M, N, K);
+  if (cudaMemsetAsync(q.status, 0, sizeof(int), s) != cudaSuccess ||
+      cudaMemsetAsync(q.kf, 0, sizeof(int) * K, s) != cudaSuccess)
     return HOTRG_EDEVICE;
-  launch_column_fields(Bt, ldb, N, K, kf, 0, 1, 0, s);
-  launch_slice_rows(A, lda, M, K, a, 1, 0, kf, 0, 1, s);
-  launch_slice_rows(Bt, ldb, N, K, b, 1, 0, kf, 0, -1, s);
-  const int rc = launch_gemm_slices(a, b, C, ldc, M, N, K, reinterpret_cast<int*>(p), status, 4.0, s, nullptr, nullptr,
-                                    false, cta_group);
+  launch_column_fields(Bt, ldb, N, K, q.kf, 0, 1, 0, s);
+  launch_slice_rows(A, lda, M, K, q.a, 1, 0, q.kf, 0, 1, s);
+  launch_slice_rows(Bt, ldb, N, K, q.b, 1, 0, q.kf, 0, -1, s);
+  const int rc = launch_gemm_slices(q.a, q.b, C, ldc, M, N, K, q.sums, q.status, 4.0, s, nullptr, nullptr, false,
+                                    cta_group);
   if (rc) return rc;
   return cudaGetLastError() == cudaSuccess ? HOTRG_OK : HOTRG_EDEVICE;
 }
 
 size_t hotrg_gemm_wait_probe_bytes(void) {
-  return hotrg_gemm_scratch_bytes(TC_PROBE_M, TC_PROBE_N, TC_PROBE_K) + sizeof(float) * TC_PROBE_M * TC_PROBE_N;
+  const size_t out = TC_PROBE_M * TC_PROBE_N;
+  return std::max(hotrg_gemm_scratch_bytes(TC_PROBE_M, TC_PROBE_N, TC_PROBE_K) + sizeof(float) * out,
+                  hotrg_gemm_f64_scratch_bytes(TC_PROBE_M, TC_PROBE_N, TC_PROBE_K) + sizeof(double) * out);
 }
 
 int hotrg_gemm_wait_probe(double timeout_s, void* scratch, size_t scratch_bytes, void* stream) {
@@ -2110,6 +2129,19 @@ int hotrg_gemm_wait_probe(double timeout_s, void* scratch, size_t scratch_bytes,
     if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return HOTRG_EDEVICE;
     const int rc = launch_gemm_split(Ap, K, Bp, K, C, N, M, N, K, 3, status, timeout_s, s, 64, 16, 1, nullptr,
                                      nullptr, true, cg);
+    if (rc) return rc;
+    const int st = hotrg_gemm_status(scratch, stream);
+    if (st != HOTRG_ETIMEOUT) return st;
+  }
+  // FP64 slices: one CTA, then a pair with no copies, with the second CTA's missing (the first one's copies land in stages
+  // that never fill) and with the first one's
+  const SliceScratch q(scratch, M, N, K);
+  double* const D = reinterpret_cast<double*>(reinterpret_cast<char*>(q.sums) + slice_scratch_bytes(M, N, 1));
+  for (int stall : {0, 3, 2, 1}) {
+    const int cg = stall ? 2 : 1;
+    if (cudaMemsetAsync(q.status, 0, sizeof(int), s) != cudaSuccess) return HOTRG_EDEVICE;
+    const int rc = launch_gemm_slices(q.a, q.b, D, N, M, N, K, q.sums, q.status, timeout_s, s, nullptr, nullptr, false, cg,
+                                      cg == 1 ? 1 : stall);
     if (rc) return rc;
     const int st = hotrg_gemm_status(scratch, stream);
     if (st != HOTRG_ETIMEOUT) return st;

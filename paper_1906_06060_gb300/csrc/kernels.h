@@ -206,11 +206,12 @@ void launch_slice_rows(const double* X, long long ldx, long long rows, long long
                        long long x_inst, const int* fields, long long f_inst, int side, cudaStream_t s, int nb = 1,
                        const Z2Layout* L = nullptr, const int* pi = nullptr);
 // C[m][n] (+)= sum_k A[m][k] Bt[n][k]; blk and bat as for launch_gemm_f64. cta_group: 1 or 2 CTAs per tile (the same
-// results), 0: by shape. Returns 0 or a hotrg_status.
+// results), 0: by shape. stall (test of the bounded waits): bit r: CTA r of a pair (or the CTA of a tile) issues no copies.
+// Returns 0 or a hotrg_status.
 int launch_gemm_slices(const SliceOperand& A, const SliceOperand& B, double* C, long long ldc, long long M, long long N,
                        long long K, int* scratch, int* status, double timeout_s, cudaStream_t s,
                        const GemmBlocks* blk = nullptr, const GemmBatch* bat = nullptr, bool accumulate = false,
-                       int cta_group = 0);
+                       int cta_group = 0, int stall = 0);
 
 // ---- gemm_tc.cu ----------------------------------------------------------------------------
 // C[m][n] = sum over passes p of sum_k A_{a(p)}[m][k] Bt_{b(p)}[n][k], bf16 operand planes on

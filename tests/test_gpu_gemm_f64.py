@@ -212,3 +212,24 @@ def test_step_of_a_tensor_in_an_unbalanced_gauge():
         for p in range(n):
             x, y = got[:, :, :, u, :, :, :, p], ref[:, :, :, u, :, :, :, p]
             assert np.linalg.norm(x - y) <= tol * np.linalg.norm(y), (u, p)
+
+
+def test_waits_that_run_out_leave_the_device_usable():
+    """The wait probe's FP64 launches (one CTA; pairs whose CTAs issue no copies, or only one of them does) give up within
+    their limit, and exact products follow on the same device."""
+    import time
+
+    import torch
+    from paper_1906_06060_gb300 import _lib
+    lib = _lib.load()
+    n = lib.hotrg_gemm_wait_probe_bytes()
+    scratch = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    s = c_void_p(torch.cuda.current_stream().cuda_stream)
+    t0 = time.time()
+    for _ in range(3):
+        assert lib.hotrg_gemm_wait_probe(0.05, c_void_p(scratch.data_ptr()), n, s) == _lib.HOTRG_ETIMEOUT
+    assert time.time() - t0 < 10.0  # six launches of one limit each, a drain of a second at most in each
+    rng = np.random.default_rng(2)
+    a, b = rng.integers(-1000, 1000, (300, 200)).astype(np.float64), rng.integers(-1000, 1000, (520, 200)).astype(np.float64)
+    for cta_group in (1, 2):
+        assert np.array_equal(gemm_f64(a, b, cta_group), a @ b.T)
