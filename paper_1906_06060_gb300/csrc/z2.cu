@@ -459,6 +459,8 @@ __global__ void __launch_bounds__(256, epi_min_blocks<Tin>()) k_epi_z2(const Tin
       const Acc* w = W + (i0 * Dt + j0) * CHIP;
       const int wrow = Dt * CHIP;
       if constexpr (std::is_same<Tin, float>::value && CHI >= 6) {
+        // widths up to 12: deep in a phase a bond of ten has classes of one and nine (a 10^4 step's 100 launches, classes of
+        // two and eight: 83 ms; of one and nine: 90, through epi_class_rows_any 187)
         switch (ncol) {
 #define HOTRG_EPI_NC(NC) \
   case NC:               \
@@ -466,6 +468,7 @@ __global__ void __launch_bounds__(256, epi_min_blocks<Tin>()) k_epi_z2(const Tin
     break;
           HOTRG_EPI_NC(1) HOTRG_EPI_NC(2) HOTRG_EPI_NC(3) HOTRG_EPI_NC(4)
           HOTRG_EPI_NC(5) HOTRG_EPI_NC(6) HOTRG_EPI_NC(7) HOTRG_EPI_NC(8)
+          HOTRG_EPI_NC(9) HOTRG_EPI_NC(10) HOTRG_EPI_NC(11) HOTRG_EPI_NC(12)
 #undef HOTRG_EPI_NC
           default:
             epi_class_rows_any<Tin, Acc, CHI>(src, rstep, cs, nrow, ncol, w, wrow, acc);

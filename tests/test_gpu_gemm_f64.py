@@ -233,3 +233,52 @@ def test_waits_that_run_out_leave_the_device_usable():
     a, b = rng.integers(-1000, 1000, (300, 200)).astype(np.float64), rng.integers(-1000, 1000, (520, 200)).astype(np.float64)
     for cta_group in (1, 2):
         assert np.array_equal(gemm_f64(a, b, cta_group), a @ b.T)
+
+
+def _cut(x, column_exponents):
+    """The kernel's digits of one row (entry k scaled by 2^column_exponents[k] first) and the row's exponent."""
+    man, ex = np.frexp(x)
+    man = np.ldexp(man, 53).astype(np.int64)
+    ex = ex + column_exponents
+    e = int(ex[x != 0].max())
+    shift = ex - e + 10  # x 2^(63 - e) = man 2^shift
+    v = np.where(shift >= 0, man << np.clip(shift, 0, 10),
+                 np.sign(man) * ((np.abs(man) + (np.int64(1) << np.clip(-shift - 1, 0, 60))) >> np.clip(-shift, 0, 61)))
+    digits = np.zeros((8, x.size), dtype=np.int64)
+    for i in range(7, 0, -1):
+        digits[i] = ((v & 255) ^ 128) - 128
+        v = (v - digits[i]) >> 8
+    digits[0] = v
+    return digits, e
+
+
+@pytest.mark.parametrize("M,N,K,cta_group", [(128, 256, 1024, 1), (128, 256, 16320, 1), (300, 256, 16320, 2),
+                                             (130, 257, 16319, 2)])
+def test_extreme_digits_are_summed_exactly(M, N, K, cta_group):
+    """Rows whose digits are all at the ends of their range: accumulator chains up to 15/16 of 2^24, level sums up to 7/8
+    of 2^31, carries between levels of that size. The kernel's arithmetic in Python's integers, rounded once, gives the
+    same bits."""
+    from fractions import Fraction
+    rng = np.random.default_rng(K)
+    low = np.ldexp(float(-0x7F80808080808000), -63)    # digits -127, -128 (six times), 0
+    high = np.ldexp(float(0x7F7F7F7F7F7F7C00), -63)    # 127 (six times), 124, 0
+    tail = np.ldexp(float(-0x80808080808080), -63)     # 0, -128 (seven times)
+    rows = np.array([np.full(K, low), np.full(K, high), np.where(np.arange(K) % 2, low, -low),
+                     np.concatenate([[high], np.full(K - 1, tail)]), rng.choice([low, -low, high, -high, tail, -tail], K)])
+    c = np.frexp(np.abs(rows).max(0))[1] - 1
+    a = [_cut(x, c) for x in rows]
+    b = [_cut(x, -c) for x in rows]
+    assert a[0][0][:, 5].tolist() == [-127] + [-128] * 6 + [0] and a[1][0][:, 5].tolist() == [127] * 6 + [124, 0]
+    assert a[3][0][:, 5].tolist() == [0] + [-128] * 7
+    ref, largest = np.zeros((5, 5)), 0
+    for i, (qa, ea) in enumerate(a):
+        for j, (qb, eb) in enumerate(b):
+            level = [sum(int(qa[u] @ qb[s - u]) for u in range(s + 1)) for s in range(8)]
+            largest = max(largest, max(abs(x) for x in level))
+            level[6] += (level[7] + 128) >> 8
+            level[5] += (level[6] + 128) >> 8
+            assert max(abs(x) for x in level) < 2 ** 31 - 128
+            ref[i, j] = float(sum(Fraction(level[s], 2 ** (14 + 8 * s)) for s in range(6)) * Fraction(2) ** (ea + eb))
+    assert largest > 6.9 * 2 ** 14 * K  # seven pairs of (nearly) extreme digits
+    got = gemm_f64(rows[np.arange(M) % 5], rows[np.arange(N) % 5], cta_group)
+    assert np.array_equal(got, ref[np.arange(M) % 5][:, np.arange(N) % 5])

@@ -112,3 +112,23 @@ def test_uneven_parity_classes(dims, evens, axis):
     assert abs(out[0][0] - out[1][0]) < 1e-12
     for a, b in zip(out[0][1], out[1][1]):
         np.testing.assert_allclose(b, a, rtol=0, atol=8 * a.size * EPS * a[0])
+
+
+@pytest.mark.parametrize("precision", ["fp16x3", "bf16x6"])
+@pytest.mark.parametrize("even", [0, 1, 2, 3, 4, 5, 8, 13])
+def test_wide_parity_classes_in_split_precision(even, precision):
+    """Classes of 0 to 13 values on the bond that the first zero-field contraction takes: the block-sparse against the dense
+    squeeze of one tensor by what does not depend on the bonds' order, the norm and the next step's Gram spectra (FP32
+    rounding, 6e-6, and the split's own 2^-16)."""
+    dims, evens = (13, 5, 4), (even, 3, 2)
+    T = random_z2_site_tensor(dims, evens, seed=even + 1)
+    out = []
+    for z2 in (False, True):
+        with _flow(3, 13, z2=True, precision=precision, fp64_steps=0) as f:
+            f.set_tensor(T, evens=evens if z2 else None)
+            f.step(2)
+            f.step(2)
+            out.append((f.ln_norms()[1], [f.spectra(2, b) for b in (0, 1)]))
+    assert abs(out[0][0] - out[1][0]) < 2.2e-5
+    for a, b in zip(out[0][1], out[1][1]):
+        np.testing.assert_allclose(b, a, rtol=0, atol=4.4e-5 * a[0])
