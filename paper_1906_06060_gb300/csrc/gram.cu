@@ -359,12 +359,11 @@ static int nsplit_for(int nr, long long K, int batch, bool sym) {
   const int wpc = gram_threads(gt) / 32;
   int nsplit = kGramWarps / (gram_tiles(nr, sym, gt) * wpc * batch);
   if (nsplit < 1) nsplit = 1;
-  // short rows (up to a 4^4 tensor): at least four columns a split. With one each, a 16 x 16 Gram matrix of a 4^4 tensor
-  // (4096 columns) took 37 us of products and 48 us of reduction over 3648 splits; 19 and 15 with 1024. (512 splits: 13
-  // and 9, but the order of these sums picks the basis inside degenerate eigenvalues, and with it the dense and the
-  // block-sparse three-product flows of a 5^4 tensor differed by 2.1e-6 in their spectra instead of 1.0e-6.)
-  const long long most = K <= 4096 ? (K + 3) / 4 : K;
-  if (nsplit > most) nsplit = (int)most;
+  // at least four columns a split, and no split without any: every split costs a partial sum to write and to reduce. (A
+  // 16 x 16 Gram matrix over 4096 columns: 37 us of products and 48 of reduction in 3648 splits, 19 and 15 in 1024; the six
+  // 16 to 25 row ones of a 4 x 5 x 4 x 5 tensor over 6400 to 10000: 240 us of reduction with two or three columns, 129 now.)
+  const long long least = std::max((K + nsplit - 1) / nsplit, 4LL);
+  nsplit = (int)std::max(1LL, std::min((long long)nsplit, (K + least - 1) / least));
   return nsplit;
 }
 

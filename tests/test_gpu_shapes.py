@@ -132,3 +132,10 @@ def test_wide_parity_classes_in_split_precision(even, precision):
     assert abs(out[0][0] - out[1][0]) < 2.2e-5
     for a, b in zip(out[0][1], out[1][1]):
         np.testing.assert_allclose(b, a, rtol=0, atol=4.4e-5 * a[0])
+
+
+@pytest.mark.parametrize("dims,axis,dcut", [((5, 4, 4, 4), 3, 5), ((4, 5, 4, 5), 3, 5), ((5, 5, 5, 4), 1, 5), ((2, 1), 1, 2),
+                                            ((11, 11, 2), 2, 11)])
+def test_gram_sums_over_a_few_columns_a_split(dims, axis, dcut):
+    """Gram matrices over 2 to 12500 columns: four columns a split where there are not enough for the whole grid."""
+    _check_step(dims, axis, dcut, precision="fp64")
