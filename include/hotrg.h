@@ -21,8 +21,8 @@
  *  - A context's first error is sticky: later calls on it return the same code.
  *  - Calls are ordered on the context's CUDA stream. hotrg_step only enqueues work; query
  *    functions (free energy, observables, spectra, get_tensor) synchronise that stream.
- *  - The library never allocates device memory: the caller passes one device workspace of at
- *    least hotrg_workspace_size() bytes (256-byte aligned) and keeps it alive until
+ *  - The library never allocates device memory: the caller passes one device workspace of
+ *    hotrg_workspace_size() bytes, or of less down to hotrg_workspace_min() (256-byte aligned), and keeps it alive until
  *    hotrg_destroy. Host pointers passed in are only accessed during the call.
  *  - One context must not be used from two host threads at once.
  */
@@ -38,7 +38,7 @@ extern "C" {
 typedef enum hotrg_status {
   HOTRG_OK = 0,
   HOTRG_EINVAL = -1,   /* bad argument: d, beta, Dcut, axis, sizes, null pointer */
-  HOTRG_ENOMEM = -2,   /* workspace smaller than hotrg_workspace_size() */
+  HOTRG_ENOMEM = -2,   /* workspace smaller than hotrg_workspace_min() */
   HOTRG_ENUMERIC = -3, /* NaN/Inf or zero norm, or Tr T <= 0 */
   HOTRG_ENOCONV = -4,  /* eigensolver did not converge within its sweep limit */
   HOTRG_ETIMEOUT = -5, /* a bounded device-side wait gave up */
@@ -85,7 +85,7 @@ typedef struct hotrg_opts {
   const double *beta;     /* [batch] host array; NULL: all instances use the beta argument */
   const double *h;        /* [batch] host array; NULL: all instances use the h argument */
   void *stream;           /* cudaStream_t for all work; NULL = legacy default stream */
-  void *workspace;        /* device pointer, >= hotrg_workspace_size() bytes, 256-B aligned */
+  void *workspace;        /* device pointer, >= hotrg_workspace_min() bytes, 256-B aligned */
   size_t workspace_bytes;
   int max_steps;          /* capacity of the per-step logs, 1..64 (default 64) */
   int kblock;             /* split modes: K width of a pipeline stage, 32 or 64 (0 = 64) */
@@ -117,7 +117,8 @@ typedef struct hotrg_opts {
   int group;              /* instances squeezed together: the squeeze GEMM of a chunk is one persistent
                              launch over a group (its tile list spans the group's instances), and the
                              workspace holds that many copies of the per-step buffers. 1..256, capped
-                             at batch; 0 (default) = 8; with derivatives or impurities always 1 */
+                             at batch; 0 (default) = 8; with derivatives or impurities always 1; fewer
+                             where the workspace does not hold that many (identical results) */
   int cta_group;          /* split modes: CTAs per squeeze-GEMM output tile. 2 = a pair of CTAs (a
                              thread-block cluster of two SMs) per 256 x 256 tile, whose tcgen05
                              MMAs read A rows from both CTAs and half of the B rows from each;
@@ -154,9 +155,13 @@ typedef struct hotrg_ctx hotrg_ctx;
 void hotrg_opts_default(hotrg_opts *o);
 
 /* Bytes of device workspace for a context of dimension d (1..4) and bond cut Dcut (2..16) with
- * the given options (precision, batch and max_steps are read; NULL means defaults).
+ * the given options (precision, batch and max_steps are read; NULL means defaults): what the fastest
+ * form of its steps takes. hotrg_init accepts less, down to hotrg_workspace_min(), and then runs fewer
+ * chunks of a squeeze at a time and squeezes fewer instances together (identical results), and near the
+ * minimum runs the FP64 products on the FP64 units (much slower, other rounding).
  * Errors: EINVAL for d or Dcut out of range, batch < 1, or bytes == NULL. */
 int hotrg_workspace_size(int d, int Dcut, const hotrg_opts *opt, size_t *bytes);
+int hotrg_workspace_min(int d, int Dcut, const hotrg_opts *opt, size_t *bytes);
 
 /* Create a context (Sec. 2): builds T^(0) = sum_s V_s prod W[s, leg] for every instance on the
  * device, normalises it (c_0) and starts the ln Z accumulator at ln c_0.

@@ -86,13 +86,15 @@ class HOTRG:
     workspace holds that many copies of the per-step buffers).
     cta_group: CTAs per squeeze-GEMM output tile, 2 (a CTA pair, 256 x 256 tiles) or 1 (128 x 256);
     0: pairs, and the autotuner may change it.
+    workspace: bytes of device memory to work in, down to hotrg_workspace_min (0: hotrg_workspace_size, or as much
+    of it as the device has free, halved until it fits; see include/hotrg.h for what a smaller one costs).
     """
 
     def __init__(self, d: int, beta, h, Dcut: int, precision: str = "fp64", fp64_steps: int = 2,
                  max_steps: int = 64, stream=None, wait_timeout_s: float = 4.0, x6_steps: int = 0,
                  kblock: int = 0, graphs: bool = True, fold_group: int = 0, derivatives=False,
                  impurities: bool = False, z2: bool = False, max_sweeps: int = 0, group: int = 0,
-                 cta_group: int = 0):
+                 cta_group: int = 0, workspace: int = 0):
         torch = _torch()
         lib = _lib.load()
         betas = np.atleast_1d(np.asarray(beta, dtype=np.float64))
@@ -109,10 +111,20 @@ class HOTRG:
         self.h = hs
         o = _opts(precision, batch, fp64_steps, max_steps, wait_timeout_s, x6_steps, kblock, graphs, fold_group,
                   derivatives, impurities, z2, max_sweeps, group, cta_group)
-        n = c_size_t(0)
-        check(lib.hotrg_workspace_size(d, Dcut, byref(o), byref(n)), "hotrg_workspace_size")
+        n = c_size_t(workspace)
+        if not workspace:
+            check(lib.hotrg_workspace_size(d, Dcut, byref(o), byref(n)), "hotrg_workspace_size")
         self.stream = stream if stream is not None else torch.cuda.current_stream()
-        self._ws = torch.empty(int(n.value), dtype=torch.uint8, device=self.stream.device)
+        while True:
+            try:
+                self._ws = torch.empty(int(n.value), dtype=torch.uint8, device=self.stream.device)
+                break
+            except torch.cuda.OutOfMemoryError:
+                least = c_size_t(0)
+                check(lib.hotrg_workspace_min(d, Dcut, byref(o), byref(least)), "hotrg_workspace_min")
+                if workspace or n.value <= least.value:
+                    raise
+                n.value = max(n.value // 2, least.value)
         self._beta_buf = (c_double * batch)(*betas)
         self._h_buf = (c_double * batch)(*hs)
         o.beta = ctypes.cast(self._beta_buf, ctypes.POINTER(c_double))

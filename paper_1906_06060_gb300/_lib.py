@@ -46,6 +46,7 @@ class Tuning(ctypes.Structure):
 _SIGS = {
     "hotrg_opts_default": (None, [POINTER(Opts)]),
     "hotrg_workspace_size": (c_int, [c_int, c_int, POINTER(Opts), POINTER(c_size_t)]),
+    "hotrg_workspace_min": (c_int, [c_int, c_int, POINTER(Opts), POINTER(c_size_t)]),
     "hotrg_init": (c_int, [POINTER(c_void_p), c_int, c_double, c_double, c_int, POINTER(Opts)]),
     "hotrg_step": (c_int, [c_void_p, c_int]),
     "hotrg_free_energy": (c_int, [c_void_p, POINTER(c_double), POINTER(c_double)]),

@@ -382,7 +382,7 @@ size_t gram_partial_doubles(int nr_max, int batch) {
 }
 
 void launch_half_gram(const double* T, long long t_stride, int batch, Geom g, int l1, int l2, double* partial,
-                      double* Q, long long q_stride, cudaStream_t s, const double* TA, const int* z2ev) {
+                      size_t partial_doubles, double* Q, long long q_stride, cudaStream_t s, const double* TA, const int* z2ev) {
   const int d = g.d;
   auto leg_dim = [&](int l) { return g.D[l % d]; };
   auto leg_stride = [&](int l) { return l < d ? g.Sn[l] * g.P : g.Sn[l - d]; };
@@ -405,7 +405,9 @@ void launch_half_gram(const double* T, long long t_stride, int batch, Geom g, in
   // hold up to nr rows: ntile covers that, the tiles beyond the actual class exit)
   const int gt = z2ev ? gram_tile((nr + 1) / 2, sym) : gram_tile(nr, sym);
   const int ntile = (nr + gt - 1) / gt;
-  const int nsplit = z2ev ? nsplit_for((nr + 1) / 2, K / 2, batch, sym) : nsplit_for(nr, K, batch, sym);
+  const long long room = std::max(1LL, (long long)(partial_doubles / ((size_t)batch * nr * nr)));
+  const int nsplit = (int)std::min<long long>(
+      room, z2ev ? nsplit_for((nr + 1) / 2, K / 2, batch, sym) : nsplit_for(nr, K, batch, sym));
   dim3 grid((z2ev ? 2 : 1) * (sym ? ntile * (ntile + 1) / 2 : ntile * ntile), nsplit, batch);
   const double* A = TA ? TA : T;
   switch (gt) {

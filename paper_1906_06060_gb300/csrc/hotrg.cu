@@ -90,8 +90,8 @@ struct StepSizes {
   }
 };
 
-// Contexts whose workspace would pass this size with the digit planes (16 bytes an entry for FP64's 8) keep the FP64
-// operands and the FP64 units: what fitted the card before still does.
+// Plans with the digit planes (16 bytes an entry for FP64's 8) stay below this size: a context keeps more than half of
+// the card free for others, or else its FP64 operands and the FP64 units (see plan_workspace).
 constexpr size_t kSliceWorkspaceLimit = (size_t)128 << 30;
 
 // Chunks in flight: as many of the `inner` chunks as keep the group's chunk buffers within this size, in equal parts.
@@ -245,6 +245,10 @@ struct hotrg_ctx {
   // instances squeezed together (one GEMM launch per chunk batch for all of them): every per-step buffer holds `group`
   // times the bytes sz lists
   int group = 1;
+  // what plan_workspace gave up: most chunks in flight, and a quarter of the Gram sums' splits
+  int chunks = kMaxGemmBatch;
+  bool few_gram_splits = false;
+  size_t gpartial_doubles = 0;
   StepSizes sz;
   size_t st_Tnext = 0;
   long long spec_stride = 0;  // doubles per instance in spec_log
@@ -334,7 +338,7 @@ bool f16_planes(int precision, int planes) {
 }
 
 StepSizes plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int max_steps, bool slices, int group,
-               int nblk, long long* Pmax_out) {
+               int chunks, int nblk, long long* Pmax_out) {
   // breadth-first: minimal number of steps after which each bond-dimension state is reached
   std::vector<std::vector<int>> states{std::vector<int>(d, 2)};
   std::vector<int> depth{0};
@@ -363,7 +367,7 @@ StepSizes plan(int d, int Dcut, int precision, int fp64_steps, int x6_steps, int
         if (step >= first && step <= max_steps)
           acc.max_with(StepSizes::of(needs_for(d, states[i].data(), a, Dcut,
                                                planes_for_step(precision, step, fp64_steps, x6_steps, P), slices, group,
-                                               nblk)));
+                                               nblk, chunks)));
   }
   *Pmax_out = Pmax;
   return acc;
@@ -398,7 +402,7 @@ bool step_needs(const hotrg_ctx* c, const int* dims, int a, int planes, StepNeed
 size_t carve(hotrg_ctx* c, char* base) {
   long long Pmax = 1;
   // with tangents the operands hold three column blocks per row (see squeeze)
-  c->sz = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, c->slices, c->group,
+  c->sz = plan(c->d, c->Dcut, c->precision, c->fp64_steps, c->x6_steps, c->max_steps, c->slices, c->group, c->chunks,
                c->deriv ? 3 : 1, &Pmax);
   c->Pmax = Pmax;
   const long long P2 = Pmax * Pmax;
@@ -426,7 +430,9 @@ size_t carve(hotrg_ctx* c, char* base) {
   c->q_stride = (long long)nrm * nrm;
   c->g_stride = (long long)kMaxD * nmax * nmax;
   c->u_stride = (long long)kMaxD * kMaxBond * kMaxGram;
-  c->gpartial = k.take<double>(sizeof(double) * gram_partial_doubles(nrm, c->batch));
+  c->gpartial_doubles = c->few_gram_splits ? std::max((size_t)c->batch * nrm * nrm, gram_partial_doubles(nrm, c->batch) / 4)
+                                           : gram_partial_doubles(nrm, c->batch);
+  c->gpartial = k.take<double>(sizeof(double) * c->gpartial_doubles);
   c->Q1 = k.take<double>(sizeof(double) * c->q_stride * c->batch);
   c->Q2 = k.take<double>(sizeof(double) * c->q_stride * c->batch);
   c->G = k.take<double>(sizeof(double) * c->g_stride * c->batch);
@@ -494,15 +500,40 @@ size_t carve(hotrg_ctx* c, char* base) {
   return k.off;
 }
 
-// Workspace bytes, with digit slices for the FP64 products unless that would pass kSliceWorkspaceLimit.
-size_t plan_workspace(hotrg_ctx* c) {
-  c->slices = true;
-  size_t n = carve(c, nullptr);
-  if (n > kSliceWorkspaceLimit) {
-    c->slices = false;
-    n = carve(c, nullptr);
+// Lays the context out within `most` bytes and returns what that takes: the first of these forms that fits, or, where none
+// does, the size of the last, the least that holds the context. Digit slices for the FP64 products (up to
+// kSliceWorkspaceLimit), all instances of a group and up to 256 chunks in flight; then fewer chunks (the gradient of two 4D
+// flows at bond dimension 5: 75 ms in 2.2 GB, 100 in 1.0, 189 in 0.4, 1570 without digits); then a smaller group or no
+// digits, and last of all Gram sums in fewer splits. An FP64 context gives up the group first: FP64 products run 30 times
+// slower on the FP64 units.
+size_t plan_workspace(hotrg_ctx* c, size_t most) {
+  const int group = c->group;
+  size_t n = 0;
+  c->few_gram_splits = false;
+  auto fits = [&](bool slices, int g) {
+    for (int chunks : {kMaxGemmBatch, 32, 8, 1}) {
+      c->slices = slices;
+      c->group = g;
+      c->chunks = chunks;
+      n = carve(c, nullptr);
+      if (n <= (slices ? std::min(most, kSliceWorkspaceLimit) : most)) return true;
+    }
+    return false;
+  };
+  std::vector<int> groups;
+  for (int g = group; g > 1; g = (g + 1) / 2) groups.push_back(g);
+  groups.push_back(1);
+  if (c->precision == HOTRG_FP64) {
+    for (bool slices : {true, false})
+      for (int g : groups)
+        if (fits(slices, g)) return n;
+  } else {
+    for (int g : groups)
+      for (bool slices : {true, false})
+        if (fits(slices, g)) return n;
   }
-  return n;
+  c->few_gram_splits = true;
+  return carve(c, nullptr);
 }
 
 int cuda_err(hotrg_ctx* c) {
@@ -1096,7 +1127,7 @@ void hotrg_opts_default(hotrg_opts* o) {
   o->max_sweeps = 40;
 }
 
-int hotrg_workspace_size(int d, int Dcut, const hotrg_opts* opt, size_t* bytes) {
+static int workspace_query(int d, int Dcut, const hotrg_opts* opt, size_t most, size_t* bytes) {
   if (!bytes || d < 1 || d > kMaxD || Dcut < 2 || Dcut > kMaxBond) return HOTRG_EINVAL;
   hotrg_opts def;
   hotrg_opts_default(&def);
@@ -1117,8 +1148,16 @@ int hotrg_workspace_size(int d, int Dcut, const hotrg_opts* opt, size_t* bytes) 
   c.impure = opt->impurities != 0;
   c.z2 = opt->z2 != 0;
   c.group = group_for(opt);
-  *bytes = plan_workspace(&c);
+  *bytes = plan_workspace(&c, most);
   return HOTRG_OK;
+}
+
+int hotrg_workspace_size(int d, int Dcut, const hotrg_opts* opt, size_t* bytes) {
+  return workspace_query(d, Dcut, opt, SIZE_MAX, bytes);
+}
+
+int hotrg_workspace_min(int d, int Dcut, const hotrg_opts* opt, size_t* bytes) {
+  return workspace_query(d, Dcut, opt, 0, bytes);
 }
 
 int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const hotrg_opts* opt) {
@@ -1177,7 +1216,7 @@ int hotrg_init(hotrg_ctx** out, int d, double beta, double h, int Dcut, const ho
   c->stream = static_cast<cudaStream_t>(opt->stream);
   c->beta = vb;
   c->h = vh;
-  const size_t need = plan_workspace(c);
+  const size_t need = plan_workspace(c, opt->workspace_bytes);
   if (!opt->workspace || opt->workspace_bytes < need ||
       (reinterpret_cast<uintptr_t>(opt->workspace) % kAlign)) {
     delete c;
@@ -1277,8 +1316,10 @@ static int enqueue_step(hotrg_ctx* c, int a, int step) {
       for (int t = 0; t < nt; ++t) {
         const int b = trans[t];
         double* Gb = c->G + (long long)b * (c->g_stride / kMaxD);
-        launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->Q1, c->q_stride, s, nullptr, zev);
-        launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->Q2, c->q_stride, s, nullptr, zev);
+        launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->gpartial_doubles,
+                         c->Q1, c->q_stride, s, nullptr, zev);
+        launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->gpartial_doubles,
+                         c->Q2, c->q_stride, s, nullptr, zev);
         launch_gram_combine(c->Q1, c->Q2, c->q_stride, c->batch, g.D[b], g.D[a], Gb, c->g_stride, s);
         ea.ax[t] = EigAxis{Gb, g.D[b] * g.D[b], chi[b], b, g.D[b], c->spec_log + (long long)b * kSpecCap,
                            c->U + (long long)b * kMaxBond * kMaxGram, c->ework + t * c->ework_axis};
@@ -1290,8 +1331,10 @@ static int enqueue_step(hotrg_ctx* c, int a, int step) {
       const int n = g.D[b] * g.D[b];
       double* Gb = c->G + (long long)b * (c->g_stride / kMaxD);
       double* Ub = c->U + (long long)b * kMaxBond * kMaxGram;
-      launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->Q1, c->q_stride, s, nullptr, zev);
-      launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->Q2, c->q_stride, s, nullptr, zev);
+      launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->gpartial_doubles,
+                       c->Q1, c->q_stride, s, nullptr, zev);
+      launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->gpartial_doubles,
+                       c->Q2, c->q_stride, s, nullptr, zev);
       launch_gram_combine(c->Q1, c->Q2, c->q_stride, c->batch, g.D[b], g.D[a], Gb, c->g_stride, s);
       EigOut eo{c->spec_log + (long long)b * kSpecCap, c->spec_stride, (long long)c->d * kSpecCap, c->dstep,
                 c->max_steps};
@@ -1301,8 +1344,9 @@ static int enqueue_step(hotrg_ctx* c, int a, int step) {
         for (int w = 0; w < 2; ++w) {
           // dG from the half-Gram tangents, then dU from the eigensystem still in ework
           const double* dTw = c->dT + w * P2max * c->batch;
-          launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->H1, c->q_stride, s, dTw);
-          launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->H2, c->q_stride, s, dTw);
+          launch_half_gram(c->T, P2max, c->batch, g, b, c->d + a, c->gpartial, c->gpartial_doubles,
+                           c->H1, c->q_stride, s, dTw);
+          launch_half_gram(c->T, P2max, c->batch, g, b, a, c->gpartial, c->gpartial_doubles, c->H2, c->q_stride, s, dTw);
           launch_gram_combine_tangent(c->Q1, c->Q2, c->H1, c->H2, c->q_stride, c->batch, g.D[b], g.D[a], c->dG,
                                       c->dg_stride, s);
           launch_eig_tangent(c->ework, Ub, c->u_stride, c->dG, c->dg_stride, c->batch, n, chi[b],
