@@ -286,6 +286,11 @@ def effective_cta_group(a, tuned):
     return a.cta_group or (2 if use_z2(a) else 1)
 
 
+def timed_cta_group(a, tuned):
+    """effective_cta_group with the library's default, pairs for both squeezes, where nothing chose otherwise."""
+    return effective_cta_group(a, list(tuned or []) + [{"cta_group": a.cta_group or 2}])
+
+
 def traffic_from_profile(z2, cta_group):
     """Per-launch DRAM bytes of the squeeze GEMM (dense or block-sparse launch) from the
     committed ncu summary, valid only if the kernel source is unchanged since the capture and the
@@ -412,7 +417,7 @@ def run_ours(a, rank, world, dist):
             "frac": achieved / peak,
             # the committed ncu summaries are of the steady-step three-product GEMM (fp16 and bf16
             # planes move the same bytes), scaled to Dcut = 10
-            "traffic": (traffic_from_profile(use_z2(a), effective_cta_group(a, tuned))
+            "traffic": (traffic_from_profile(use_z2(a), timed_cta_group(a, tuned))
                         if (a.workload == "flow" and a.dcut == 10 and a.precision in ("bf16x3", "fp16x3"))
                         else None),
             "peak_source": f"{src} bf16 sustained (kernel timed inside long steps)",

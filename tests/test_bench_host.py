@@ -124,3 +124,17 @@ def test_scan_group_is_the_largest_that_fits(monkeypatch):
     assert bench.squeeze_group(a, FakeTorch(1e6)) == 1
     assert bench.squeeze_group(args(monkeypatch, "--workload", "scan", "--group", "4"), FakeTorch(1e6)) == 4
     assert bench.squeeze_group(args(monkeypatch), FakeTorch(1e6)) == 0      # single flow: library default
+
+
+@pytest.mark.parametrize("z2", [True, False])
+def test_lines_without_the_autotuner_name_the_librarys_cta_group(monkeypatch, z2):
+    """hotrg_init runs CTA pairs by default, block-sparse or dense."""
+    class A:
+        cta_group = 0
+    a = A()
+    monkeypatch.setattr(bench, "use_z2", lambda _: z2)
+    assert bench.timed_cta_group(a, []) == 2
+    assert bench.timed_cta_group(a, [{"kblock": 64, "cta_group": 1}]) == 1
+    assert bench.timed_cta_group(a, [{"skipped": "FP64"}]) == 2
+    a.cta_group = 1
+    assert bench.timed_cta_group(a, []) == 1
