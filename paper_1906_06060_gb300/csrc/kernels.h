@@ -125,7 +125,7 @@ struct EigOut {
   const int* step;
   int max_steps;
 };
-// Symmetric eigendecomposition of G (n x n, n <= 256) by cyclic Jacobi, one CTA per instance;
+// Symmetric eigendecomposition of G (n x n, n <= 256) by cyclic Jacobi, one cluster of up to 16 CTAs per instance;
 // eigenvalues sorted descending, the leading chi eigenvectors, sign-fixed, into U[k][0..n).
 // work: batch * 2*n*n doubles. Sets ST_NOCONV on the sweep limit.
 // Several axes in one launch (blockIdx.y = axis): per axis its Gram matrices G (+ instance x
